@@ -278,8 +278,8 @@ int emu_batch_diagnostics(emu_box* box, double* out, int on_host);
  * that cannot run on this device).  A candidate is a step form
  * (emu_batch_step), a grid of blocks of 256 threads whose warps split the
  * work (the number of particles each warp and block takes follows from it),
- * and the RK stage's tile: 30 cells and two halo lanes per warp (form 0) or
- * 32 cells per warp (form 1):
+ * and the RK stage's work split: single 32-cell tiles (form 0) or slabs of up
+ * to 8 tiles per block (form 1):
  *   c = 0..5  one launch per phase, grid {304, 152, 608}[c / 2], RK form c % 2
  *   c = 6..9  one cooperative launch per step, grid {304, 152}[(c - 6) / 2],
  *             RK form c % 2;
@@ -353,19 +353,19 @@ int emu_set_barrier_timeout(emu_box* box, int64_t ns);
  * step in progress). */
 int emu_set_deposit_form(emu_box* box, int32_t form);
 
-/* Form of the RK stage kernel: 1 = 32 cells per warp, 0 = the halo-lane form
- * (both give bitwise the same results), -1 = chosen by units per warp (the
- * default; emu_autotune and emu_set_grid set it too).  Errors: EMU_EINVAL. */
+/* Work split of the RK stage kernel: 1 = a block takes slabs of up to 8
+ * consecutive 32-cell tiles, 0 = single tiles (both give bitwise the same
+ * results), -1 = chosen by 32-cell units per block (the default; emu_autotune
+ * and emu_set_grid set it too).  Errors: EMU_EINVAL. */
 int emu_set_rk_form(emu_box* box, int32_t form);
 
 /* Set the grid of the step kernels to `blocks` blocks of 256 threads (1..608;
  * the default is 304, two per SM; emu_autotune picks among 152, 304 and 608),
  * for callers that share the GPU with other work.  The blocks' warps split the
  * work, so the choice changes the deposit's summation order (results stay
- * bitwise reproducible for a fixed choice) and whether the RK stage runs with
- * 32 cells per warp (every warp walking at least 8 units) or the halo-lane
- * form (the same results); it drops the RK form emu_autotune chose, and the
- * fused step form if not every block of the new grid could be resident.
+ * bitwise reproducible for a fixed choice); it drops the RK form emu_autotune
+ * chose, and the fused step form if not every block of the new grid could be
+ * resident.
  * Errors: EMU_EINVAL. */
 int emu_set_grid(emu_box* box, int32_t blocks);
 

@@ -37,7 +37,7 @@ size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 // Geometry of a batch, from its configurations only (no device needed).
 struct Shape {
   int nbox = 0;
-  int64_t Ptot = 0, U = 0, U32 = 0;
+  int64_t Ptot = 0, U = 0, U32 = 0, US = 0;
   int NZ = 0, MT = 0, NT = 0;
   int NT32 = 0;    // 32-cell tiles of all boxes
   int order = 2;   // shape order of every box (Sec. 2.2.1)
@@ -78,6 +78,15 @@ const char* config_problem(const emu_config* c) {
   return nullptr;
 }
 
+// Tiles of a slab of the RK stage for a box of nt 32-cell tiles: the most (a
+// power of two, at most one per warp of a block) that leave no more than a
+// sixteenth of the slabs' tiles beyond the box, since their warps idle.
+int slab_tiles(int nt) {
+  int sw = kWarps;
+  while (sw > 1 && (int64_t)((nt + sw - 1) / sw) * sw * 16 > (int64_t)nt * 17) sw >>= 1;
+  return sw;
+}
+
 const char* make_shape(const emu_config* cfgs, int nbox, Shape& S) {
   if (!cfgs) return "config array is NULL";
   if (nbox < 1 || nbox > kMaxBoxes) return "nbox out of range";
@@ -101,6 +110,8 @@ const char* make_shape(const emu_config* cfgs, int nbox, Shape& S) {
     g.uoff = S.U;
     g.ntiles32 = (c->nz + kLanes - 1) / kLanes;
     g.uoff32 = S.U32;
+    g.sw = slab_tiles(g.ntiles32);
+    g.soff = S.US;
     g.toff32 = S.NT32;
     g.coff = (int)NZ;
     g.toff = (int)NT;
@@ -121,6 +132,7 @@ const char* make_shape(const emu_config* cfgs, int nbox, Shape& S) {
     S.Ptot += g.P;
     S.U += (int64_t)g.ntiles * g.M;
     S.U32 += (int64_t)g.ntiles32 * g.M;
+    S.US += (int64_t)((g.ntiles32 + g.sw - 1) / g.sw) * g.sw * g.M;
     S.Mmax = g.M > S.Mmax ? g.M : S.Mmax;
     NZ += c->nz;
     MT += c->ndir;
@@ -210,7 +222,7 @@ struct emu_box {
   double* wtab = nullptr;   // the rings' shape weights at each shift row [5 x kWSlots][MT] (k_shifts)
   unsigned* bar = nullptr;
   int blocks = kPersistBlocks;  // grid of the step kernels (autotuned); its warps split the units
-  int rk_form = -1;             // RK stage: 0 halo-lane, 1 32-cell, -1 by units per warp (autotuned)
+  int rk_form = -1;             // RK stage: 0 single tiles, 1 slabs of tiles, -1 by units per block (autotuned)
   int dep_form = 0;             // the form-0 step's deposit: 0 per-warp partials and their combination,
                                 // 1, 2 thread-block clusters of 8, 16 blocks writing the potential
   int dep_clusters[2] = {-1, -1};   // clusters of 8, 16 blocks resident at once (-1: not asked yet)
@@ -285,6 +297,14 @@ int cuda_check(emu_box* b, cudaError_t e, const char* what) {
   return fail(b, EMU_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+// Whether the RK stage's blocks take slabs of several tiles (rings read in
+// pieces of up to 2 KB) or single tiles: slabs when the batch has at least 16
+// 32-cell units per block of the default grid, unless a form was chosen; below
+// that single tiles spread the few units over all SMs.
+int use_slabs(const emu_box* b) {
+  return b->rk_form >= 0 ? b->rk_form : b->S.U32 >= 16 * (int64_t)kPersistBlocks;
+}
+
 Batch batch_view(const emu_box* b) {
   Batch B;
   B.box = b->geo_d;
@@ -300,6 +320,8 @@ Batch batch_view(const emu_box* b) {
   B.U32 = b->S.U32;
   B.nw32 = (int)(b->S.U32 < nw ? b->S.U32 : nw);
   B.Ptot = b->S.Ptot;
+  B.slabs = use_slabs(b);
+  B.US = B.slabs ? b->S.US : b->S.U32;
   return B;
 }
 
@@ -702,12 +724,17 @@ int launch_stage(emu_box* b, int s, int dry) {
   return launch_rk(b, s, srow, dry);
 }
 
-// Whether the RK stage runs with 32 cells per warp (no halo lanes): when every
-// warp walks at least 8 units (the tile ends at ring and range boundaries are
-// computed directly), unless a form was chosen; otherwise the halo-lane form,
-// which gives bitwise the same results.
-bool use_rk32(const emu_box* b, const Batch& Bv) {
-  return b->rk_form >= 0 ? b->rk_form == 1 : Bv.U32 >= 8 * (int64_t)Bv.nw32;
+// Raises a kernel's dynamic shared memory limit, once per device and kernel
+// (`done`: one bit per device).
+template <typename K>
+cudaError_t raise_smem(K kernel, int bytes, std::atomic<unsigned>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 32 && ((done.load() >> dev) & 1u)) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && dev < 32) done.fetch_or(1u << dev);
+  return e;
 }
 
 // Most blocks of the fused step kernel that can be resident at once (its
@@ -718,10 +745,12 @@ int fused_max_blocks(const emu_box* b) {
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
   int coop = 0;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
-  // every instantiation has the same launch bounds; the largest (cubic shape,
-  // vacuum terms, 32-cell RK stage) stands for all
+  // every instantiation has the same launch bounds and shared memory; one
+  // (cubic shape, vacuum terms) stands for all
   (void)b;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<true, 3, true>, kThreads, 0) != cudaSuccess)
+  static std::atomic<unsigned> done{0};
+  if (raise_smem(k_step<true, 3>, kSlabSmem, done) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<true, 3>, kThreads, kSlabSmem) != cudaSuccess)
     return 0;
   return per_sm * sms;
 }
@@ -746,11 +775,10 @@ int launch_fused(emu_box* b, int dry, int64_t nsteps) {
   a.nsteps = nsteps;
   a.split = combine_split(b->S, B.nw);
   a.dry = dry;
-  const bool r32 = use_rk32(b, B);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = persist_grid(b);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = kSlabSmem;
   cfg.stream = b->stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -760,13 +788,13 @@ int launch_fused(emu_box* b, int dry, int64_t nsteps) {
   before_launch(b, CLS_STEP);
   by_order(b->S.order, [&](auto O) {
     constexpr int R = decltype(O)::value;
-    if (b->pot) {
-      if (r32) (void)cudaLaunchKernelEx(&cfg, k_step<true, R, true>, B, b->pt, a);
-      else (void)cudaLaunchKernelEx(&cfg, k_step<true, R, false>, B, b->pt, a);
-    } else {
-      if (r32) (void)cudaLaunchKernelEx(&cfg, k_step<false, R, true>, B, b->pt, a);
-      else (void)cudaLaunchKernelEx(&cfg, k_step<false, R, false>, B, b->pt, a);
-    }
+    auto launch = [&](auto POT) {
+      static std::atomic<unsigned> done{0};
+      auto k = k_step<decltype(POT)::value, R>;
+      if (raise_smem(k, kSlabSmem, done) == cudaSuccess) (void)cudaLaunchKernelEx(&cfg, k, B, b->pt, a);
+    };
+    if (b->pot) launch(std::true_type{});
+    else launch(std::false_type{});
     return 0;
   });
   return after_launch(b, "fused step kernel");
@@ -780,23 +808,21 @@ int launch_rk_on(emu_box* b, int s, const int* srow, int dry, const Parts& pt, c
   before_launch(b, CLS_RK);
   by_order(b->S.order, [&](auto O) {
     constexpr int R = decltype(O)::value;
-    // 32 cells per warp, no halo lanes, when every warp walks at least 8 units (the
-    // tile ends at ring and range boundaries are computed directly); otherwise
-    // the halo-lane kernel, which gives bitwise the same results
     const Batch Bv = batch_view(b);
-    const dim3 grid = persist_grid(b);
-    const bool use32 = use_rk32(b, Bv);
-    if (!use32) {
-      if (b->pot)
-        pdl(b->stream, k_rk_stage<true, R>, grid, Bv, pt, W, b->dirtab, srow, At, stage_src, s, dry);
-      else
-        pdl(b->stream, k_rk_stage<false, R>, grid, Bv, pt, W, b->dirtab, srow, At, stage_src, s, dry);
-      return 0;
-    }
-    if (b->pot)
-      pdl(b->stream, k_rk_stage32<true, R>, grid, Bv, pt, W, b->dirtab, srow, At, stage_src, s, dry);
-    else
-      pdl(b->stream, k_rk_stage32<false, R>, grid, Bv, pt, W, b->dirtab, srow, At, stage_src, s, dry);
+    const double* wrow = weight_row(b, srow);
+    auto launch = [&](auto POT, auto STAGE) {
+      static std::atomic<unsigned> done{0};
+      auto k = k_rk_stage<decltype(POT)::value, R, decltype(STAGE)::value>;
+      if (raise_smem(k, kSlabSmem, done) == cudaSuccess)
+        pdl_smem(b->stream, k, persist_grid(b), kSlabSmem, Bv, pt, W, wrow, b->dirtab, srow, At, stage_src, s, dry);
+    };
+    auto stage = [&](auto POT) {
+      if (s == 1) launch(POT, std::integral_constant<int, 1>{});
+      else if (s == 4) launch(POT, std::integral_constant<int, 4>{});
+      else launch(POT, std::integral_constant<int, 2>{});
+    };
+    if (b->pot) stage(std::true_type{});
+    else stage(std::false_type{});
     return 0;
   });
   return after_launch(b, "RK stage kernel");

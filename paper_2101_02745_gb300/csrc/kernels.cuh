@@ -22,8 +22,8 @@
 // common offset, Sec. 3.1 and Eq. 4), the particle on cell j is ring entry
 // (j - shift_d) mod nz and its stencil neighbours sit on the adjacent lanes:
 // deposit (Eq. 5) and interpolation (Eq. 6) are warp-shuffle gathers.  The
-// RK stage also has a form without halo lanes (k_rk_stage32: 32-cell tiles,
-// the tile ends through shared memory).
+// RK stage has no halo lanes (32-cell tiles, the tile ends through shared
+// memory); its commutators and stencil sums run on the integer pipe (wide.cuh).
 //
 // Persistent schedule.  The step kernels run a fixed grid (2 blocks of 8 warps
 // per SM); the first nw warps split the U units of the batch into equal
@@ -35,6 +35,8 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+
+#include "wide.cuh"
 
 namespace emu_dev {
 
@@ -78,8 +80,10 @@ struct Sten {
 struct BoxGeo {
   int nz, M, ntiles, use_dirs;
   int coff, toff, doff, ntiles32;  // ntiles32: 32-cell tiles of the RK stage
-  int toff32, reserved_;           // toff32: first 32-cell tile of the box among all boxes'
+  int toff32, sw;                  // toff32: first 32-cell tile of the box among all boxes'; sw: 32-cell tiles of a
+                                   // slab of the RK stage (1, 2, 4 or 8)
   int64_t P, poff, uoff, uoff32;   // uoff32: first 32-cell unit of the box
+  int64_t soff;                    // first tile unit of the box's slabs (sw per slab and direction)
   double Lz, dz, inv_dz, nz_d, dV, c_light;
   double kappa_dV;   // kappa / dV: scale of the grid potential
   double inv_dV;     // 1 / dV: scale of the moments
@@ -105,6 +109,8 @@ struct Batch {
   int64_t U, Ptot;     // total units, particles
   int64_t U32;         // total 32-cell units of the RK stage (shape orders 0-2)
   int nw32;            // warps that split them
+  int64_t US;          // total tile units of the RK stage's slabs
+  int slabs;           // its slabs: 1 = BoxGeo::sw tiles, 0 = one tile
 };
 
 struct Parts {
@@ -269,6 +275,16 @@ __device__ __forceinline__ double ldp(const double* p) {
   else return *p;
 }
 
+// Element k of an array of rows of P doubles, at row pointer p (P < 2^32: the
+// address is one IMAD.WIDE; with a 64-bit P each cost about seven
+// instructions, a fifth of the RK stage's).
+__device__ __forceinline__ const double* row(const double* p, unsigned P, unsigned k) {
+  return (const double*)((const char*)p + (uint64_t)P * (8u * k));
+}
+__device__ __forceinline__ double* row(double* p, unsigned P, unsigned k) {
+  return (double*)((char*)p + (uint64_t)P * (8u * k));
+}
+
 // Index of this warp among the warps of a persistent grid: warp i of every
 // block comes before warp i + 1 of any block.  Units are split into
 // contiguous ranges in this order, so when a batch has fewer units than the
@@ -348,13 +364,21 @@ struct Spread {
   }
 };
 
-// Bulk prefetch of the doubles [i0, i0 + n) of array a into L2 (a hint; the
-// range is rounded inwards to 16-byte boundaries so it never leaves the array).
-__device__ __forceinline__ void prefetch_l2(const double* a, int64_t i0, int n) {
-  uintptr_t lo = ((uintptr_t)(a + i0) + 15) & ~(uintptr_t)15;
-  uintptr_t hi = ((uintptr_t)(a + i0 + n)) & ~(uintptr_t)15;
-  if (hi > lo)
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"((unsigned)(hi - lo)) : "memory");
+// Prefetch into L2 by a whole warp: of `narr` arrays (array(a) the first double
+// of array a) the doubles [i0, i0 + n), n <= 32.  One lane takes one 128-byte
+// line: at most three per array.  (The bulk form, one cp.async.bulk.prefetch per
+// array, is a uniform instruction: a warp whose lanes name different arrays
+// runs it once per lane, ~17 instructions each; 57 arrays cost a unit of the
+// RK stage a quarter of its 3750 instructions.)
+__device__ __forceinline__ void prefetch_line(const double* a) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
+}
+template <typename F>
+__device__ __forceinline__ void prefetch_l2(int lane, int narr, int64_t i0, int n, F array) {
+  for (int t = lane; t < 4 * narr; t += kLanes) {
+    const int a = t >> 2, q = t & 3;
+    if (q < 3) prefetch_line(array(a) + i0 + min(16 * q, n - 1));
+  }
 }
 
 // Periodic wrap into [0, Lz).
@@ -602,6 +626,10 @@ __device__ __forceinline__ void deposit_tile_dirs(const Batch& B, int b, int til
   }
 }
 
+// A value of lane `src` as limbs in every lane.
+__device__ __forceinline__ emu_wide::Limbs bcast(emu_wide::Limbs v, int src) {
+  return emu_wide::Limbs{__shfl_sync(kFull, v.h, src), __shfl_sync(kFull, v.l, src)};
+}
 // Deposit (Eq. 5), first phase.  MODE 0: B = N rho - Nbar rhobar^* (the
 // combination that enters H, Eq. 2); MODE 1: B = N rho; MODE 2: B = Nbar rhobar;
 // MODE 3: B = r_nu (packed matrices given per particle: the adjoint's Gamma);
@@ -885,118 +913,105 @@ k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ 
   if (bad) atomicOr(err, ERR_LATTICE);
 }
 
-// The RK4 update (Sec. 2.3) of particle p (ring direction gd) of box g at
-// stage s, given its interpolated self-interaction Hamiltonian Hm (Eq. 6,
-// Eq. 2) and its neutrino source matrix r (already loaded): K = -i[H, rho],
-// Kbar = -i[Hbar, rhobar] (Eq. 4) with Hbar = -H^* (plus the vacuum and
-// matter terms with POT), then the accumulator and next stage state (stage 4:
-// the new state and position).  vz points at the particle's v_z in the
-// direction table.  With KEEP
-// the state it stores (the next stage's, or at stage 4 the new one), rho and
-// rhobar, is also combined as B = n1 rho - n2 rhobar^* into keep[9] (the
-// arithmetic of the deposit, Eq. 5) and the new position returned in *zkeep.
-template <bool POT, bool COH, bool KEEP = false>
-__device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, const double* src_b, int64_t P,
-                                            int64_t p, int s, int dry, double bdt, double cdt, double dtb,
-                                            const double* __restrict__ vz, double (&Hm)[kNC], const double (&r)[9],
-                                            double* keep = nullptr, double* zkeep = nullptr, double n1 = 0.0,
-                                            double n2 = 0.0) {
-  const double bdt2 = 2.0 * bdt, cdt2 = 2.0 * cdt;   // diagonal K are returned halved
-  // Hm: H in the traceless components.  Antineutrinos: Hbar = -H^* (diagonal
-  // differences and real parts flip sign, imaginary parts stay)
-  double Hb[kNC];
-  if (POT) {
-    const double* vn = g.vnu;
-    const double* vb = g.vnubar;
-#pragma unroll
-    for (int c = 0; c < kNC; ++c) {
-      const bool im = (c == 3 || c == 5 || c == 7);
-      Hb[c] = (im ? Hm[c] : -Hm[c]) + __ldg(vb + c);
-      Hm[c] += __ldg(vn + c);
-    }
-  }
-  const double d12 = Hm[0], d23 = Hm[1], d13 = d12 + d23;
-#pragma unroll
+// The RK4 update (Sec. 2.3) of particle p at stage s: K =
+// -i[H, rho], Kbar = -i[Hbar, rhobar] (Eq. 4) from the operand hm of H (Eq. 6,
+// Eq. 2; OWNBAR: hb of Hbar, otherwise Hbar = -H^*) and the neutrino source
+// matrix r (already loaded; the antineutrinos' source is src_b), then the
+// accumulator and next stage state (stage 4: the new state and position, from
+// *vz).  S is the stage as a template parameter (2 stands for 2 and 3), or 0
+// for the run-time s.  With KEEP the state it stores (the next stage's, or at
+// stage 4 the new one), rho and rhobar, is also combined as
+// B = n1 rho - n2 rhobar^* into keep[9] (the arithmetic of the deposit, Eq. 5)
+// and the new position returned in *zkeep.
+// The commutators run on the integer pipe (wide.cuh), the updates as FP64
+// multiply-adds: 36 + 31 FP64 instructions a particle instead of 144 (at
+// 16 cycles each the FP64 pipe bound the stage).
+template <int S, bool OWNBAR, bool COH, bool KEEP = false>
+__device__ __forceinline__ void rk_update(double Lz, const Parts& pt, const double* src_b, int64_t P_, int64_t p,
+                                          int s, int dry, double bdt, double cdt, double dtb,
+                                          const double* vz, const emu_wide::Ham& hm, const emu_wide::Ham& hb,
+                                          double (&r)[9], double* keep = nullptr, double* zkeep = nullptr,
+                                          double n1 = 0.0, double n2 = 0.0) {
+  namespace w = emu_wide;
+  const unsigned P = (unsigned)P_;
+  const bool first = S == 0 ? s == 1 : S == 1, last = S == 0 ? s == 4 : S == 4;
+  // Sums of products have an exponent of at least emin, so that the
+  // coefficients that take it (below) stay normal; infinite and NaN inputs
+  // raise it to kInfExp, and the coefficients, held at the infinities'
+  // exponent field, then make every result infinite or NaN
+  constexpr int kInfExp = 1 << 16;
+  const int bmax = 2047 - w::exponent(bdt), cmax = 2047 - w::exponent(cdt);
+  const int emin = w::kBiasP - 2046 + w::max_i(bmax, cmax);
+  const int htop = w::top(hm);
+  // one pass per species: a loop, not unrolled (the commutator's ~600
+  // instructions once keep the stage in the instruction cache)
+#pragma unroll 1
   for (int which = 0; which < 2; ++which) {
-    double* __restrict__ yv = which ? pt.rhobar : pt.rho;
-    double* __restrict__ av = pt.acc + which * 9 * P;
-    double* __restrict__ sv = pt.stage + which * 9 * P;
-    // all loads of this matrix before any store (the arrays do not alias)
-    double a[9], y[9], rb[9];
-    if (which == 1) {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) rb[k] = ldp<COH>(src_b + k * P + p);
-    }
-    if (s >= 2) {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) a[k] = ldp<COH>(av + k * P + p);
-    }
-    if (s == 2 || s == 3) {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) y[k] = ldp<COH>(yv + k * P + p);
-    }
-    const double* rr = which ? rb : r;
-    double kd[3], ko[6];
-    if (which == 0) commutator(d12, d13, d23, Hm[2], Hm[3], Hm[4], Hm[5], Hm[6], Hm[7], rr, kd, ko);
-    else if (POT) commutator(Hb[0], Hb[0] + Hb[1], Hb[1], Hb[2], Hb[3], Hb[4], Hb[5], Hb[6], Hb[7], rr, kd, ko);
-    else commutator(-d12, -d13, -d23, -Hm[2], Hm[3], -Hm[4], Hm[5], -Hm[6], Hm[7], rr, kd, ko);
-    if constexpr (!KEEP) {
-      if (s == 1) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          av[k * P + p] = fma(bdt2, kd[k], rr[k]);
-          sv[k * P + p] = fma(cdt2, kd[k], rr[k]);
-        }
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-          av[(k + 3) * P + p] = fma(bdt, ko[k], rr[k + 3]);
-          sv[(k + 3) * P + p] = fma(cdt, ko[k], rr[k + 3]);
-        }
-      } else if (s < 4) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          av[k * P + p] = fma(bdt2, kd[k], a[k]);
-          sv[k * P + p] = fma(cdt2, kd[k], y[k]);
-        }
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-          av[(k + 3) * P + p] = fma(bdt, ko[k], a[k + 3]);
-          sv[(k + 3) * P + p] = fma(cdt, ko[k], y[k + 3]);
-        }
-      } else {
-        double* __restrict__ dst = dry ? sv : yv;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) dst[k * P + p] = fma(bdt2, kd[k], a[k]);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) dst[(k + 3) * P + p] = fma(bdt, ko[k], a[k + 3]);
-      }
+    // K = -i[H, r]: neutrinos K_12.. = (Im C, -Re C).  Antineutrinos with
+    // Hbar = -H^*: conj(rhobar) obeys the neutrinos' equation with the same H,
+    // and Kbar = conj(K): (Im C, Re C)
+    w::Comm C;
+    if (OWNBAR) {
+      const w::Ham& h = which ? hb : hm;
+      const w::Mat m = w::mat(r, false);
+      const int top = w::max_i(w::top(m), which ? w::top(hb) : htop);
+      w::commutator(h, m, top < w::kExpNonFinite ? emin : kInfExp, C);
     } else {
-      double nv[9];   // the state stored as the next stage's (stage 4: the new state)
-      if (s == 1) {
+      const w::Mat m = w::mat(r, which != 0);
+      const int top = w::max_i(w::top(m), htop);
+      w::commutator(hm, m, top < w::kExpNonFinite ? emin : kInfExp, C);
+    }
+    // the accumulator and the step's start (after the commutator: the operands
+    // it keeps in registers leave no room for them; the caller prefetches them
+    // into L2), before any store
+    double* __restrict__ yv = (which ? pt.rhobar : pt.rho) + p;
+    double* __restrict__ av = row(pt.acc, P, which * 9) + p;
+    double* __restrict__ sv = row(pt.stage, P, which * 9) + p;
+    double a[9], y[9];
+    if (first) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) { av[k * P + p] = fma(bdt2, kd[k], rr[k]); nv[k] = fma(cdt2, kd[k], rr[k]); }
+      for (int k = 0; k < 9; ++k) a[k] = y[k] = r[k];
+    } else {
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-          av[(k + 3) * P + p] = fma(bdt, ko[k], rr[k + 3]);
-          nv[k + 3] = fma(cdt, ko[k], rr[k + 3]);
-        }
-      } else if (s < 4) {
+      for (int k = 0; k < 9; ++k) a[k] = ldp<COH>(row(av, P, k));
+      if (!last) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) { av[k * P + p] = fma(bdt2, kd[k], a[k]); nv[k] = fma(cdt2, kd[k], y[k]); }
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-          av[(k + 3) * P + p] = fma(bdt, ko[k], a[k + 3]);
-          nv[k + 3] = fma(cdt, ko[k], y[k + 3]);
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) nv[k] = fma(bdt2, kd[k], a[k]);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) nv[k + 3] = fma(bdt, ko[k], a[k + 3]);
+        for (int k = 0; k < 9; ++k) y[k] = ldp<COH>(row(yv, P, k));
       }
-      double* __restrict__ dst = (s < 4 || dry) ? sv : yv;
+    }
+    if (which == 0) {   // the other species' source
 #pragma unroll
-      for (int k = 0; k < 9; ++k) dst[k * P + p] = nv[k];
+      for (int k = 0; k < 9; ++k) r[k] = ldp<COH>(row(src_b + p, P, k));
+    }
+    // K_k = kv[k] 2^(its exponent): the coefficients bdt, cdt take the exponent
+    // (at most the infinities' field)
+    double kv[9], kb[9], kc[9];
+    const int flip = (which == 1 && !OWNBAR) ? 0 : (int)0x80000000;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int ed = C.ke[q] - w::kBiasP + 1, eo = C.oe[q] - w::kBiasP;   // (diagonal K are halved)
+      kv[q] = C.kd[q];
+      kb[q] = w::scale(bdt, w::min_i(ed, bmax));
+      kc[q] = w::scale(cdt, w::min_i(ed, cmax));
+      kv[3 + 2 * q] = C.ci[q];
+      kv[4 + 2 * q] = w::from_words(w::hi_word(C.cr[q]) ^ flip, w::lo_word(C.cr[q]));
+      kb[3 + 2 * q] = kb[4 + 2 * q] = w::scale(bdt, w::min_i(eo, bmax));
+      kc[3 + 2 * q] = kc[4 + 2 * q] = w::scale(cdt, w::min_i(eo, cmax));
+    }
+    double nv[9];   // the state stored: the next stage's, or at stage 4 the new one
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      if (last) {
+        nv[k] = fma(kb[k], kv[k], a[k]);
+      } else {
+        *row(av, P, k) = fma(kb[k], kv[k], a[k]);
+        nv[k] = fma(kc[k], kv[k], y[k]);
+      }
+    }
+    double* __restrict__ dst = (!last || dry) ? sv : yv;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) *row(dst, P, k) = nv[k];
+    if constexpr (KEEP) {
       // B = n1 rho - n2 rhobar^*: conj(rhobar) flips the sign of the imaginary components 4, 6, 8
       if (which == 0) {
 #pragma unroll
@@ -1007,13 +1022,64 @@ __device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, co
       }
     }
   }
-  if (s == 4) {
+  if (last) {
     const double vzv = *vz;   // (a plain load: vz may point at a caller's local value)
-    const double zn = wrap_z(fma(dtb, vzv, ldp<COH>(pt.z + p)), g.Lz);
+    const double zn = wrap_z(fma(dtb, vzv, ldp<COH>(pt.z + p)), Lz);
     if (dry) pt.stage[p] = zn;  // (only to keep the work of the real stage)
     else pt.z[p] = zn;
     if constexpr (KEEP) *zkeep = zn;
   }
+}
+
+// Coefficients of K at stage s (Sec. 2.3): bdt in the accumulator, cdt in the
+// next stage's state (at least the smallest normal number: rk_update scales
+// them by powers of two).
+__device__ __forceinline__ void rk_coefficients(int s, double dt, double& bdt, double& cdt) {
+  bdt = fmax((s == 1 || s == 4) ? dt / 6.0 : dt / 3.0, 0x1p-1022);
+  cdt = fmax(s == 3 ? dt : 0.5 * dt, 0x1p-1022);
+}
+
+// H + V and Hbar = -H^* + Vbar with the box's vacuum and matter terms (Eq. 2):
+// in the traceless components the diagonal differences and real parts of -H^*
+// flip sign, the imaginary parts stay.
+__device__ __forceinline__ void add_potentials(const BoxGeo& g, double (&Hm)[kNC], double (&Hb)[kNC]) {
+#pragma unroll
+  for (int c = 0; c < kNC; ++c) {
+    const bool im = (c == 3 || c == 5 || c == 7);
+    Hb[c] = (im ? Hm[c] : -Hm[c]) + __ldg(g.vnubar + c);
+    Hm[c] += __ldg(g.vnu + c);
+  }
+}
+
+// rk_update of particle p of box g from H in the traceless components.
+template <bool POT, bool COH, bool KEEP = false>
+__device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, const double* src_b, int64_t P,
+                                            int64_t p, int s, int dry, double bdt, double cdt, double dtb,
+                                            const double* __restrict__ vz, double (&Hm)[kNC], double (&r)[9],
+                                            double* keep = nullptr, double* zkeep = nullptr, double n1 = 0.0,
+                                            double n2 = 0.0) {
+  if constexpr (POT) {
+    double Hb[kNC];
+    add_potentials(g, Hm, Hb);
+    const emu_wide::Ham hm = emu_wide::ham(Hm), hb = emu_wide::ham(Hb);
+    rk_update<0, true, COH, KEEP>(g.Lz, pt, src_b, P, p, s, dry, bdt, cdt, dtb, vz, hm, hb, r, keep, zkeep, n1, n2);
+  } else {
+    const emu_wide::Ham hm = emu_wide::ham(Hm);
+    rk_update<0, false, COH, KEEP>(g.Lz, pt, src_b, P, p, s, dry, bdt, cdt, dtb, vz, hm, hm, r, keep, zkeep, n1,
+                                   n2);
+  }
+}
+
+// Tiles before box g's first slab, and the box of tile unit x (a pair of a
+// slab and a direction counts as its sw tile units).
+__device__ __forceinline__ int64_t slab_offset(const Batch& B, const BoxGeo& g) { return B.slabs ? g.soff : g.uoff32; }
+__device__ __forceinline__ int box_of_slab_unit(const Batch& B, int64_t x) {
+  int lo = 0, hi = B.nbox - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (slab_offset(B, B.box[mid]) <= x) lo = mid; else hi = mid - 1;
+  }
+  return lo;
 }
 
 // One RK4 stage s (1..4) after the deposit of the stage state: interpolate
@@ -1024,297 +1090,270 @@ __device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, co
 //   s = 3: acc += dt/3 K,     stage = y + dt K
 //   s = 4: y = acc + dt/6 K,  z = wrap(z + dt v_z)   (dry: into the stage buffer instead)
 // With POT the constant vacuum and matter terms of the box are added:
-// H = H_self + V, Hbar = -H_self^* + Vbar (Eq. 2, Sec. 2.1).
-// Persistent: each warp walks its contiguous range of units, direction-major
-// within a box (unit = direction * ntiles + tile) so it streams along each
-// ring, and prefetches the next unit's particle data into L2.  The shape
-// weights come from the deposit.  Stages 2-4 read their state from stage_src
-// (normally the stage buffer itself, updated in place; a separate buffer when
-// the stage states are kept for the adjoint).
-template <bool POT, int ORDER, bool COH>
-__device__ __forceinline__ void rk_phase(const Batch& B, int64_t w, int lane, const Parts& pt, const double* W,
+// H = H_self + V, Hbar = -H_self^* + Vbar (Eq. 2, Sec. 2.1).  Stages 2-4 read
+// their state from stage_src (normally the stage buffer itself, updated in
+// place; a separate buffer when the stage states are kept for the adjoint).
+//
+// Work split.  A block takes a contiguous range of (slab, direction) pairs of
+// the batch (an equal share of their tile units), slab by slab; a slab is 1, 2, 4 or 8 (BoxGeo::sw; Batch::slabs 0:
+// 1) consecutive 32-cell tiles.  It converts the slab's potential once to integer operands
+// in shared memory (per cell and moment the 8 traceless components, one
+// exponent per cell for the diagonal pair and for each complex component),
+// and its warps walk the slab's directions: with sw tiles, warp i takes tile
+// i mod sw and every (8 / sw)-th direction, so the warps of a block read
+// adjacent pieces of the same rings (sw = 8: 2 KB of every array).  Per unit a
+// warp forms G = A0 - Omega . A of its cells, the neighbours' G come from
+// shared memory, and the stencil sum is the commutator's operand: everything
+// up to the update runs on the integer pipe.
+constexpr int kSlabCells = kWarps * kLanes + 4;    // cells of the widest slab, two neighbours a side
+constexpr int kRowCells = kLanes + 4;              // cells of a unit, likewise
+struct SlabTable {
+  int2 a[kNT][kSlabCells];                         // the potential: A0 / 4 as int64, limbs of A_x, A_y, A_z
+  int e[4][kSlabCells];                            // exponents: diagonal pair, three complex components
+  int2 g[kWarps][kNC][kRowCells];                  // limbs of G of each warp's unit
+  const double* pf[64];                            // the arrays a stage reads, for the L2 prefetch
+};
+constexpr int kSlabSmem = (int)sizeof(SlabTable);
+
+// Potential of cells c0 .. c0 + n - 1 (modulo nz) of box g into the table, by
+// the whole block: one (cell, exponent group) per thread and round.
+template <bool COH>
+__device__ __forceinline__ void slab_table(SlabTable& t, const double* A, int NZ, const BoxGeo& g, int c0, int n) {
+  namespace w = emu_wide;
+  for (int q = threadIdx.x; q < 4 * n; q += kThreads) {
+    const int grp = q / n, c = q - grp * n;
+    const double* Aj = A + g.coff + wrapc(c0 + c, g.nz) + (int64_t)2 * grp * NZ;
+    double v[8];
+    int e[8], top = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {   // moment k / 2, component 2 grp + k % 2
+      v[k] = ldd<COH>(Aj + (int64_t)((k >> 1) * kNC + (k & 1)) * NZ);
+      e[k] = w::exponent(v[k]);
+      top = max(top, e[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const w::Limbs l = w::limbs(v[k], e[k], top);
+      int2 x = make_int2(l.h, l.l);
+      if (k < 2) {   // A0: a quarter of the operand as an int64 (dot3's addend)
+        const int64_t q = w::join(l) >> 2;
+        x = make_int2((int)q, (int)(q >> 32));
+      }
+      t.a[(k >> 1) * kNC + 2 * grp + (k & 1)][c] = x;
+    }
+    t.e[grp][c] = top;
+  }
+}
+
+__device__ __forceinline__ emu_wide::Limbs limbs_of(int2 v) { return emu_wide::Limbs{v.x, v.y}; }
+
+// Component c of G = A0 - Omega . A at table cell j (o: limbs of -Omega).
+// Directions scaled by 2^-ko: so is G.
+__device__ __forceinline__ int2 table_G(const SlabTable& t, int c, int j, const emu_wide::Limbs (&o)[3], int ko) {
+  const int2 q = t.a[c][j];
+  const int64_t a0 = (int64_t)(((uint64_t)(uint32_t)q.y << 32) | (uint32_t)q.x);
+  const emu_wide::Limbs g = emu_wide::split(
+      emu_wide::dot3(emu_wide::align(a0, ko, 0), limbs_of(t.a[kNC + c][j]), o[0], limbs_of(t.a[2 * kNC + c][j]), o[1],
+                     limbs_of(t.a[3 * kNC + c][j]), o[2]));
+  return make_int2(g.h, g.l);
+}
+
+template <bool POT, int ORDER, int S, bool COH>
+__device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const double* W, const double* wrow,
                                          const double* __restrict__ dirtab, const int* shift, const double* A,
-                                         const double* stage_src, int s, int dry) {
-  const int64_t u0 = unit_begin(w, B), u1 = unit_begin(w + 1, B);
-  if (u0 >= u1) return;
-  const int64_t P = B.Ptot;
-  const int MT = B.MT, NZ = B.NZ;
-  const double* src_r = (s == 1) ? pt.rho : stage_src;
-  const double* src_b = (s == 1) ? pt.rhobar : stage_src + 9 * P;
-  // arrays this stage reads, for the prefetch: source (18), y (18, s = 2, 3), acc (18, s >= 2), W (NWS), z (s = 4)
-  constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T, NWS = Sten<ORDER>::NWS;
-  const int nsrc = 18, ny = (s == 2 || s == 3) ? 18 : 0, nacc = (s >= 2) ? 18 : 0;
-  const int narr = nsrc + ny + nacc + NWS + (s == 4 ? 1 : 0);
-  int b = box_of_unit(B, u0);
-  double bdt = 0.0, cdt = 0.0;
-  int bcur = -1;
-  for (int64_t u = u0; u < u1; ++u) {
-    while (u >= B.box[b].uoff + (int64_t)B.box[b].ntiles * B.box[b].M) ++b;
-    const BoxGeo& g = B.box[b];
-    const int nz = g.nz, nt = g.ntiles;
-    if (b != bcur) {
-      bcur = b;
-      const double dt = B.dt[b];
-      bdt = (s == 1 || s == 4) ? dt / 6.0 : dt / 3.0;   // weight of K in acc
-      cdt = (s == 3) ? dt : 0.5 * dt;                   // offset of the next stage
-    }
-    const int lu = (int)(u - g.uoff);        // unit within the box: direction-major
-    const int d = lu / nt, tile = lu - d * nt;
-    if (u + 1 < u1 && lu + 1 < nt * g.M) {   // prefetch the next unit of the same box
-      const int dn = (lu + 1) / nt, tn = lu + 1 - dn * nt;
-      const int i0 = tn * T - ldi<COH>(shift + g.doff + dn);   // ring index of the next unit's first cell
-      const int n = min(T, nz - tn * T);
-      if (i0 >= 0 && i0 + n <= nz) {
-        const int64_t base = g.poff + (int64_t)dn * nz + i0;
-        for (int a = lane; a < narr; a += kLanes) {
-          const double* arr;
-          if (a < nsrc) arr = (a < 9 ? src_r + (int64_t)a * P : src_b + (int64_t)(a - 9) * P);
-          else if (a < nsrc + ny) arr = (a - nsrc < 9 ? pt.rho + (int64_t)(a - nsrc) * P
-                                                      : pt.rhobar + (int64_t)(a - nsrc - 9) * P);
-          else if (a < nsrc + ny + nacc) arr = pt.acc + (int64_t)(a - nsrc - ny) * P;
-          else if (a < nsrc + ny + nacc + NWS) arr = W + (int64_t)(a - nsrc - ny - nacc) * P;
-          else arr = pt.z;
-          prefetch_l2(arr, base, n);
-        }
-      }
-    }
-    const int craw = tile * T - H + lane, j = wrapc(craw, nz);
-    const bool active = lane >= H && lane < H + T && craw < nz;
-    const int gd = g.doff + d;
-    const double ox = __ldg(dirtab + gd), oy = __ldg(dirtab + MT + gd), oz = __ldg(dirtab + 2 * MT + gd);
-    const int64_t p = g.poff + (int64_t)d * nz + wrapc(j - ldi<COH>(shift + gd), nz);
-    double wt[Sten<ORDER>::NW];
-    zero_weights<ORDER>(wt);
-    // the neutrino source matrix first, so its latency overlaps the interpolation
-    double r[9];
-    if (active) {
-      load_weights<ORDER, COH>(W, P, p, wt);
-#pragma unroll
-      for (int k = 0; k < 9; ++k) r[k] = ldp<COH>(src_r + k * P + p);
-    }
-    double Hm[kNC];
-    const double* Aj = A + g.coff + j;
-#pragma unroll
-    for (int c = 0; c < kNC; ++c) {
-      const double G = fma(-oz, ldd<COH>(Aj + (int64_t)(3 * kNC + c) * NZ),
-                           fma(-oy, ldd<COH>(Aj + (int64_t)(2 * kNC + c) * NZ),
-                               fma(-ox, ldd<COH>(Aj + (int64_t)(kNC + c) * NZ), ldd<COH>(Aj + (int64_t)c * NZ))));
-      Hm[c] = gather<ORDER>(wt, G);
-    }
-    if (!active) continue;
-    rk_particle<POT, COH>(g, pt, src_b, P, p, s, dry, bdt, cdt, B.dt[b], dirtab + 3 * MT + gd, Hm, r);
-  }
-}
-
-template <bool POT, int ORDER>
-__global__ void __launch_bounds__(kThreads, 2)
-k_rk_stage(Batch B, Parts pt, const double* __restrict__ W, const double* __restrict__ dirtab,
-           const int* __restrict__ shift, const double* __restrict__ A, const double* stage_src, int s, int dry) {
-  griddep_wait();
-  rk_phase<POT, ORDER, false>(B, logical_warp(), threadIdx.x & 31, pt, W, dirtab, shift, A, stage_src, s, dry);
-}
-
-// The RK stage with 32 cells per warp: the same arithmetic as k_rk_stage,
-// without its halo lanes (two for shape orders 0-2, four for the cubic
-// shape).  Units are (32-cell tile, direction), direction-major, split evenly
-// over the warps.  A warp writes G = A0 - Omega . A of a unit's cells into
-// shared memory and finishes that unit one iteration later, when the next
-// tile's first cells are known: the stencil neighbours of its end cells (H on
-// each side) come from the adjacent tiles of the same ring when the warp
-// handles them in order, and are computed directly (one cell at a time, by the
-// whole warp) at ring and range boundaries.
-template <bool COH>
-__device__ __forceinline__ void ring_cell_G(const double* A, int NZ, int coff, int cell, double ox, double oy,
-                                            double oz, double (&G)[kNC]) {
-  const double* Aj = A + coff + cell;
-#pragma unroll
-  for (int c = 0; c < kNC; ++c)
-    G[c] = fma(-oz, ldd<COH>(Aj + (int64_t)(3 * kNC + c) * NZ),
-               fma(-oy, ldd<COH>(Aj + (int64_t)(2 * kNC + c) * NZ),
-                   fma(-ox, ldd<COH>(Aj + (int64_t)(kNC + c) * NZ), ldd<COH>(Aj + (int64_t)c * NZ))));
-}
-
-// Component c of G at one cell, the arithmetic of ring_cell_G (for one lane
-// per component).
-template <bool COH>
-__device__ __forceinline__ double cell_G_component(const double* A, int NZ, int coff, int cell, int c, double ox,
-                                                   double oy, double oz) {
-  const double* Aj = A + coff + cell;
-  return fma(-oz, ldd<COH>(Aj + (int64_t)(3 * kNC + c) * NZ),
-             fma(-oy, ldd<COH>(Aj + (int64_t)(2 * kNC + c) * NZ),
-                 fma(-ox, ldd<COH>(Aj + (int64_t)(kNC + c) * NZ), ldd<COH>(Aj + (int64_t)c * NZ))));
-}
-
-// Cell index on a ring of nz cells for cells within two rings of it (the
-// stencil reaches at most two cells past a tile; rings may be shorter).
-__device__ __forceinline__ int ring_wrap(int cell, int nz) {
-  while (cell < 0) cell += nz;
-  while (cell >= nz) cell -= nz;
-  return cell;
-}
-
-template <bool POT, int ORDER, bool COH>
-__device__ __forceinline__ void rk32_phase(const Batch& B, int64_t w, const Parts& pt, const double* W,
-                                           const double* __restrict__ dirtab, const int* shift, const double* A,
-                                           const double* stage_src, int s, int dry) {
-  constexpr int H = Sten<ORDER>::H, NW = Sten<ORDER>::NW;
-  __shared__ double gsm[kWarps][2][kNC][kLanes];   // G of the last two units, per warp
-  __shared__ double edge[kWarps][2][H][kNC];       // the H cells left / right of the unit being finished
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t u0 = unit32_begin(w, B), u1 = unit32_begin(w + 1, B);
-  if (u0 >= u1) return;
-  const int64_t P = B.Ptot;
-  const int MT = B.MT, NZ = B.NZ;
-  const double* src_r = (s == 1) ? pt.rho : stage_src;
-  const double* src_b = (s == 1) ? pt.rhobar : stage_src + 9 * P;
+                                         const double* stage_src, int s, int dry, SlabTable& t) {
+  namespace w = emu_wide;
+  constexpr int H = ORDER == 0 ? 0 : Sten<ORDER>::H, NW = ORDER == 0 ? 1 : Sten<ORDER>::NW;
   constexpr int NWS = Sten<ORDER>::NWS;
-  const int nsrc = 18, ny = (s == 2 || s == 3) ? 18 : 0, nacc = (s >= 2) ? 18 : 0;
-  const int narr = nsrc + ny + nacc + NWS + (s == 4 ? 1 : 0);
-  // the unit being finished (previous iteration's)
-  int pb = -1, pd = 0, pt_ = 0, pn = 0, pgd = 0;
-  int bcur = -1;                    // box of the RK coefficients below (divisions once per box)
-  double dtb = 0.0, bdt = 0.0, cdt = 0.0;
-  int b = box_of_unit32(B, u0);
-  for (int64_t u = u0; u <= u1; ++u) {
-    const int slot = (int)((u - u0) & 1);
-    int cb = -1, cd = 0, ct = 0, cn = 0, cgd = 0;   // this iteration's unit (none at u == u1)
-    if (u < u1) {
-      while (u >= B.box[b].uoff32 + (int64_t)B.box[b].ntiles32 * B.box[b].M) ++b;
-      const BoxGeo& g = B.box[b];
-      const int lu = (int)(u - g.uoff32);
-      cb = b;
-      cd = lu / g.ntiles32;
-      ct = lu - cd * g.ntiles32;
-      cn = min(kLanes, g.nz - ct * kLanes);
-      cgd = g.doff + cd;
-      // prefetch this unit's particle data into L2 (it is finished next iteration)
-      const int i0 = ct * kLanes - ldi<COH>(shift + cgd);
-      if (i0 >= 0 && i0 + cn <= g.nz) {
-        const int64_t base = g.poff + (int64_t)cd * g.nz + i0;
-        for (int a = lane; a < narr; a += kLanes) {
-          const double* arr;
-          if (a < nsrc) arr = (a < 9 ? src_r + (int64_t)a * P : src_b + (int64_t)(a - 9) * P);
-          else if (a < nsrc + ny) arr = (a - nsrc < 9 ? pt.rho + (int64_t)(a - nsrc) * P
-                                                      : pt.rhobar + (int64_t)(a - nsrc - 9) * P);
-          else if (a < nsrc + ny + nacc) arr = pt.acc + (int64_t)(a - nsrc - ny) * P;
-          else if (a < nsrc + ny + nacc + NWS) arr = W + (int64_t)(a - nsrc - ny - nacc) * P;
-          else arr = pt.z;
-          prefetch_l2(arr, base, cn);
-        }
-      }
-      // G of this unit's cells
-      if (lane < cn) {
-        double G[kNC];
-        ring_cell_G<COH>(A, NZ, g.coff, ct * kLanes + lane, __ldg(dirtab + cgd), __ldg(dirtab + MT + cgd),
-                         __ldg(dirtab + 2 * MT + cgd), G);
-#pragma unroll
-        for (int k = 0; k < kNC; ++k) gsm[wib][slot][k][lane] = G[k];
-      }
+  const int lane = threadIdx.x & 31;
+  const int wib = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+  const int64_t P = B.Ptot;
+  const int MT = B.MT;
+  const double* src_r = S == 1 ? pt.rho : stage_src;
+  const double* src_b = S == 1 ? pt.rhobar : stage_src + 9 * P;
+  // the arrays this stage reads per particle
+  constexpr int ny = S == 2 ? 18 : 0, nacc = S == 1 ? 0 : 18, nz_ = S == 4 ? 1 : 0;
+  const int narr = 18 + ny + nacc + nz_ + (wrow != nullptr ? 0 : NWS);
+  __syncthreads();
+  if (threadIdx.x < (unsigned)narr) {
+    const int a = threadIdx.x;
+    const double* arr;
+    if (a < 18) arr = a < 9 ? src_r + a * P : src_b + (a - 9) * P;
+    else if (a < 18 + nacc) arr = pt.acc + (a - 18) * P;
+    else if (a < 18 + nacc + ny) arr = a - 18 - nacc < 9 ? pt.rho + (a - 18 - nacc) * P
+                                                         : pt.rhobar + (a - 18 - nacc - 9) * P;
+    else if (a < 18 + nacc + ny + nz_) arr = pt.z;
+    else arr = W + (a - 18 - nacc - ny - nz_) * P;
+    t.pf[a] = arr;
+  }
+  // this block's tile units [x, x1); a (slab, direction) pair belongs to the
+  // block its first unit falls to
+  int64_t x = (int64_t)blockIdx.x * B.US / gridDim.x;
+  const int64_t x1 = ((int64_t)blockIdx.x + 1) * B.US / gridDim.x;
+  if (x >= x1) return;
+  int b = box_of_slab_unit(B, x);
+  while (x < x1 && b < B.nbox) {
+    const BoxGeo* gp = &B.box[b];
+    const int nz = gp->nz, M = gp->M, sw = B.slabs ? gp->sw : 1;
+    const int nslab = (gp->ntiles32 + sw - 1) / sw;
+    const int64_t off = slab_offset(B, *gp);
+    const int64_t q = (x - off + sw - 1) / sw;                            // first pair, box-local
+    const int64_t q1 = min((int64_t)nslab * M, (x1 - off + sw - 1) / sw);   // and the end of this block's
+    if (q >= q1) {   // (the box's pairs left start in later blocks, or it has none left)
+      x = off + (int64_t)nslab * M * sw;
+      ++b;
+      continue;
     }
-    // does this unit continue the ring of the one being finished?
-    const bool next_in_ring = pb >= 0 && cb == pb && cd == pd && ct == pt_ + 1;
-    if (pb >= 0) {
-      const BoxGeo& g = B.box[pb];
-      const double ox = __ldg(dirtab + pgd), oy = __ldg(dirtab + MT + pgd), oz = __ldg(dirtab + 2 * MT + pgd);
-      // the H cells right of the finished unit's last cell: from this unit's
-      // first cells when it continues the ring and has them, else computed
-      // (lane k < 8 forms component k, in ring_cell_G's order)
-#pragma unroll
-      for (int o = 0; o < H; ++o) {
-        if (!(next_in_ring && (H == 1 || o < cn))) {   // (a unit that continues a ring has a first cell)
-          const int cell = pt_ * kLanes + pn + o;
-          if (lane < kNC)
-            edge[wib][1][o][lane] = cell_G_component<COH>(
-                A, NZ, g.coff, H == 1 ? (cell >= g.nz ? cell - g.nz : cell) : ring_wrap(cell, g.nz), lane, ox, oy, oz);
+    const int slab = (int)(q / M), d0 = (int)(q - (int64_t)slab * M);
+    const int d1 = (int)min((int64_t)M, (int64_t)d0 + (q1 - q));
+    x = off + (q + (d1 - d0)) * sw;
+    const BoxGeo& g = *gp;
+    const int c0 = slab * sw * kLanes;
+    __syncthreads();   // (the previous slab's table is free, and pf is written)
+    slab_table<COH>(t, A, B.NZ, g, c0 - H, min(sw * kLanes, nz - c0) + 2 * H);
+    __syncthreads();
+    const int tile0 = (wib & (sw - 1)) * kLanes;       // this warp's tile within the slab, in cells
+    const int n = min(kLanes, nz - c0 - tile0);
+    if (n <= 0) continue;
+    const int dstep = kWarps / sw;
+    double bdt, cdt;
+    const double dtb = B.dt[b];
+    rk_coefficients(S == 2 ? s : S, dtb, bdt, cdt);
+    const int64_t poff = g.poff;
+    const int doff = g.doff;
+    const int tc = tile0 + H + lane;                   // table cell of this lane
+    for (int d = d0 + wib / sw; d < d1; d += dstep) {
+      const int gd = doff + d;
+      const int sh = ldi<COH>(shift + gd);
+      if (d + dstep < d1) {   // prefetch the next unit's particle data into L2
+        int i0 = c0 + tile0 - ldi<COH>(shift + gd + dstep);
+        if (i0 < 0) i0 += nz;
+        const int cnt = min(n, nz - i0);
+        const int64_t nb = poff + (int64_t)(d + dstep) * nz + i0;
+        for (int x = lane; x < 3 * narr; x += kLanes) {
+          const int a = (x * 171) >> 9, l = x - 3 * a;   // x / 3, x % 3 (exact below 256)
+          prefetch_line(t.pf[a] + nb + min(16 * l, cnt - 1));
         }
       }
+      int i = c0 + tile0 + lane - sh;
+      if (i < 0) i += nz;
+      const bool active = lane < n;
+      if (!active) i = 0;
+      const int64_t p = poff + (int64_t)d * nz + i;
+      // the neutrino source matrix and the weights first, so their latency
+      // overlaps the interpolation
+      double r[9], wd[NW];
+#pragma unroll
+      for (int k = 0; k < 9; ++k) r[k] = ldp<COH>(row(src_r + p, (unsigned)P, k));
+      // -Omega, and the ring's weights when every particle takes them: lane q
+      // converts one of them
+      double u = 0.0;
+      if (lane < 3) u = -__ldg(dirtab + lane * MT + gd);
+      if constexpr (ORDER > 0) {
+        if (wrow != nullptr) {
+          if (lane >= 3 && lane < 3 + NW) u = ldp<COH>(wrow + (lane - 3) * MT + gd);
+        } else {
+#pragma unroll
+          for (int o = 0; o < NW; ++o) wd[o] = ldp<COH>(row(W + p, (unsigned)P, o));
+        }
+      }
+      // directions above 1 (not unit vectors) are scaled by 2^-ko
+      const int ko = __reduce_max_sync(kFull, lane < 3 ? w::unit_excess(u) : 0);
+      const w::Limbs ul = w::unit_limbs(u, lane < 3 ? ko : 0);
+      const w::Limbs om[3] = {bcast(ul, 0), bcast(ul, 1), bcast(ul, 2)};
+      // G of this lane's cell and of the H cells on each side of the tile
+      if (active) {
+        if (ko == 0) {
+#pragma unroll
+          for (int c = 0; c < kNC; ++c) t.g[wib][c][H + lane] = table_G(t, c, tc, om, 0);
+        } else {
+#pragma unroll 1
+          for (int c = 0; c < kNC; ++c) t.g[wib][c][H + lane] = table_G(t, c, tc, om, ko);
+        }
+      }
+      if constexpr (H > 0) {
+        if (lane < 2 * H * kNC) {
+          const int c = lane & (kNC - 1), h = lane >> 3;
+          const int x = h < H ? h : n + h;            // position among the unit's cells
+          t.g[wib][c][x] = table_G(t, c, tile0 + x, om, ko);
+        }
+      }
+      w::Limbs wl[NW];
+      if constexpr (ORDER > 0) {
+#pragma unroll
+        for (int o = 0; o < NW; ++o) wl[o] = wrow != nullptr ? bcast(ul, 3 + o) : w::unit_limbs(wd[o]);
+      }
       __syncwarp();
-      if (next_in_ring && lane == 0) {
+      if (active) {
+        // interpolation (Eq. 6): per component the taps at the largest exponent
+        int64_t hv[kNC];
+        int he[4];
 #pragma unroll
-        for (int o = 0; o < H; ++o)
-          if (H == 1 || o < cn) {
+        for (int grp = 0; grp < 4; ++grp) {
+          int e[NW], dd[NW], df[NW];
+          he[grp] = 0;
 #pragma unroll
-            for (int k = 0; k < kNC; ++k) edge[wib][1][o][k] = gsm[wib][slot][k][o];
+          for (int o = 0; o < NW; ++o) {
+            e[o] = t.e[grp][tc - H + o];
+            he[grp] = max(he[grp], e[o]);
           }
-      }
-      __syncwarp();
-      // finish the previous unit: interpolation (the taps in k_rk_stage's
-      // order), commutators, RK update
-      const int psl = slot ^ 1;
-      if (lane < pn) {
-        const int64_t p =
-            g.poff + (int64_t)pd * g.nz + wrapc(pt_ * kLanes + lane - ldi<COH>(shift + pgd), g.nz);
-        double wt[NW];
-        double r[9];
-        load_weights<ORDER, COH>(W, P, p, wt);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) r[k] = ldp<COH>(src_r + k * P + p);
-        double Hm[kNC];
+          for (int o = 0; o < NW; ++o) {
+            dd[o] = he[grp] - e[o];
+            df[o] = max(dd[o] - 32, 0);
+          }
 #pragma unroll
-        for (int k = 0; k < kNC; ++k) {
-          if (ORDER == 0) {
-            Hm[k] = gsm[wib][psl][k][lane];
-          } else if (H == 1) {
-            const double gl = lane == 0 ? edge[wib][0][0][k] : gsm[wib][psl][k][lane - 1];
-            const double gr = lane == pn - 1 ? edge[wib][1][0][k] : gsm[wib][psl][k][lane + 1];
-            Hm[k] = fma(wt[0], gl, fma(wt[1], gsm[wib][psl][k][lane], wt[2] * gr));
-          } else {
-            // value of G at tap offset o: this unit's cells, or the edges
-            auto gv = [&](int o) {
-              const int i = lane + o;
-              return i < 0 ? edge[wib][0][-i - 1][k] : i >= pn ? edge[wib][1][i - pn][k] : gsm[wib][psl][k][i];
-            };
-            double h = wt[NW - 1] * gv(H);
+          for (int c = 2 * grp; c < 2 * grp + 2; ++c) {
+            if constexpr (ORDER == 0) {
+              hv[c] = w::join(limbs_of(t.g[wib][c][lane]));
+            } else {
+              int64_t v = 0;
 #pragma unroll
-            for (int t = NW - 2; t >= 0; --t) h = fma(wt[t], gv(t - H), h);
-            Hm[k] = h;
+              for (int o = 0; o < NW; ++o)
+                v += w::align(w::mul(limbs_of(t.g[wib][c][lane + o]), wl[o]), dd[o], df[o]);
+              hv[c] = v * 4;
+            }
           }
         }
-        if (pb != bcur) {
-          bcur = pb;
-          dtb = B.dt[pb];
-          bdt = (s == 1 || s == 4) ? dtb / 6.0 : dtb / 3.0;   // weight of K in acc
-          cdt = (s == 3) ? dtb : 0.5 * dtb;                   // offset of the next stage
+        // hv[c] 2^(he + 2 - kBiasV) = H_c
+        if (ko != 0) {
+#pragma unroll
+          for (int grp = 0; grp < 4; ++grp) he[grp] = ko <= w::kMaxExcess ? he[grp] + ko : w::kExpNonFinite;
         }
-        rk_particle<POT, COH>(g, pt, src_b, P, p, s, dry, bdt, cdt, dtb, dirtab + 3 * MT + pgd, Hm, r);
+        const double* vz = dirtab + 3 * MT + gd;
+        if constexpr (POT) {
+          double Hm[kNC], Hb[kNC];
+#pragma unroll
+          for (int c = 0; c < kNC; ++c)
+            Hm[c] = (double)hv[c] * w::scale(1.0, he[c >> 1] < w::kExpNonFinite ? max(he[c >> 1] + 2 - w::kBiasV, -1022)
+                                                                               : 1024);
+          add_potentials(g, Hm, Hb);
+          const w::Ham hm = w::ham(Hm), hb = w::ham(Hb);
+          rk_update<S, true, COH>(g.Lz, pt, src_b, P, p, s, dry, bdt, cdt, dtb, vz, hm, hb, r);
+        } else {
+          w::Ham hm;
+          hm.d12 = w::Real{w::split(hv[0]), he[0] + 2};
+          hm.d13 = w::Real{w::split(hv[0] + hv[1]), he[0] + 2};
+          hm.d23 = w::Real{w::split(hv[1]), he[0] + 2};
+          hm.a = w::Cplx{w::split(hv[2]), w::split(hv[3]), he[1] + 2};
+          hm.b = w::Cplx{w::split(hv[4]), w::split(hv[5]), he[2] + 2};
+          hm.c = w::Cplx{w::split(hv[6]), w::split(hv[7]), he[3] + 2};
+          rk_update<S, false, COH>(g.Lz, pt, src_b, P, p, s, dry, bdt, cdt, dtb, vz, hm, hm, r);
+        }
       }
-      __syncwarp();
+      __syncwarp();   // (the unit's G are rewritten by the next)
     }
-    // the H cells left of this unit's first cell, for when it is finished:
-    // the previous unit's last cells when this one continues its ring (that
-    // unit then has all 32 cells), else computed
-    if (cb >= 0) {
-      if (next_in_ring) {
-        if (lane == 0) {
-#pragma unroll
-          for (int o = 1; o <= H; ++o) {
-#pragma unroll
-            for (int k = 0; k < kNC; ++k) edge[wib][0][o - 1][k] = gsm[wib][slot ^ 1][k][kLanes - o];
-          }
-        }
-      } else {
-        const BoxGeo& g = B.box[cb];
-#pragma unroll
-        for (int o = 1; o <= H; ++o) {
-          const int cell = ct * kLanes - o;
-          if (lane < kNC)
-            edge[wib][0][o - 1][lane] = cell_G_component<COH>(
-                A, NZ, g.coff, H == 1 ? (cell < 0 ? cell + g.nz : cell) : ring_wrap(cell, g.nz), lane,
-                __ldg(dirtab + cgd), __ldg(dirtab + MT + cgd), __ldg(dirtab + 2 * MT + cgd));
-        }
-      }
-      __syncwarp();
-    }
-    pb = cb; pd = cd; pt_ = ct; pn = cn; pgd = cgd;
   }
 }
 
-template <bool POT, int ORDER>
+template <bool POT, int ORDER, int S>
 __global__ void __launch_bounds__(kThreads, 2)
-k_rk_stage32(Batch B, Parts pt, const double* __restrict__ W, const double* __restrict__ dirtab,
-             const int* __restrict__ shift, const double* __restrict__ A, const double* stage_src, int s, int dry) {
+k_rk_stage(Batch B, Parts pt, const double* __restrict__ W, const double* __restrict__ wrow,
+           const double* __restrict__ dirtab, const int* __restrict__ shift, const double* __restrict__ A,
+           const double* stage_src, int s, int dry) {
+  extern __shared__ char smem[];
   griddep_wait();
-  rk32_phase<POT, ORDER, false>(B, logical_warp(), pt, W, dirtab, shift, A, stage_src, s, dry);
+  rk_phase<POT, ORDER, S, false>(B, pt, W, wrow, dirtab, shift, A, stage_src, s, dry, *(SlabTable*)smem);
 }
 
 // ------------------------------------------- RK stage with the next deposit
@@ -1413,8 +1452,8 @@ __device__ __forceinline__ double frame_value(const double* __restrict__ Fr, con
   return v;
 }
 
-// Stage s (1..4) of every box: the RK4 update of k_rk_stage32 (same
-// arithmetic; the potential of a cell is the sum of the frame entries of
+// Stage s (1..4) of every box: the RK4 update of k_rk_stage (its commutators
+// and update; interpolation in FP64; the potential of a cell is the sum of the frame entries of
 // k_frame_sum that cover it, Fr), then the
 // deposit of its result at the next stage's positions: the shape weights
 // (kept in W for the next stage), B = N rho - Nbar rhobar^* in the traceless
@@ -1476,8 +1515,7 @@ k_rk_deposit(Batch B, Parts pt, double* __restrict__ W, const double* __restrict
     if (b != bcur) {
       bcur = b;
       dtb = B.dt[b];
-      bdt = (s == 1 || s == 4) ? dtb / 6.0 : dtb / 3.0;   // weight of K in acc
-      cdt = (s == 3) ? dtb : 0.5 * dtb;                   // offset of the next stage
+      rk_coefficients(s, dtb, bdt, cdt);
     }
     if (u + 1 < u1 && lu + 1 < g.ntiles32 * M) {   // prefetch the next unit of the same box
       const int tn = (lu + 1) / M, dn = lu + 1 - tn * M;
@@ -1485,7 +1523,7 @@ k_rk_deposit(Batch B, Parts pt, double* __restrict__ W, const double* __restrict
       const int cnt = min(kLanes, nz - tn * kLanes);
       if (i0 >= 0 && i0 + cnt <= nz) {
         const int64_t base = g.poff + (int64_t)dn * nz + i0;
-        for (int a = lane; a < narr; a += kLanes) {
+        prefetch_l2(lane, narr, base, cnt, [&](int a) {
           const double* arr;
           if (a < 18) arr = a < 9 ? src_r + (int64_t)a * P : src_b + (int64_t)(a - 9) * P;
           else if (a < 18 + ny) arr = a - 18 < 9 ? pt.rho + (int64_t)(a - 18) * P : pt.rhobar + (int64_t)(a - 27) * P;
@@ -1495,8 +1533,8 @@ k_rk_deposit(Batch B, Parts pt, double* __restrict__ W, const double* __restrict
             const int k = a - 18 - ny - nacc - nw_;
             arr = k == 0 ? pt.z : k == 1 ? pt.N : pt.Nbar;
           }
-          prefetch_l2(arr, base, cnt);
-        }
+          return arr;
+        });
       }
     }
     const int n = min(kLanes, nz - tile * kLanes);
@@ -1820,15 +1858,17 @@ __device__ __forceinline__ void fused_combine(const Batch& B, const StepArgs& a)
   combine_phase(B, a.partial, a.At, kNT, 1, a.split, a.err);
 }
 
-template <bool POT, int ORDER, bool RK32>
-__device__ __forceinline__ void fused_rk(const Batch& B, int64_t w, int lane, const Parts& pt, const StepArgs& a,
-                                     const int* srow, int s) {
-  if constexpr (RK32) rk32_phase<POT, ORDER, true>(B, w, pt, a.W, a.dirtab, srow, a.At, pt.stage, s, a.dry);
-  else rk_phase<POT, ORDER, true>(B, w, lane, pt, a.W, a.dirtab, srow, a.At, pt.stage, s, a.dry);
+template <bool POT, int ORDER>
+__device__ __forceinline__ void fused_rk(const Batch& B, const Parts& pt, const StepArgs& a, const int* srow,
+                                         const double* wrow, int s, SlabTable& t) {
+  if (s == 1) rk_phase<POT, ORDER, 1, true>(B, pt, a.W, wrow, a.dirtab, srow, a.At, pt.stage, s, a.dry, t);
+  else if (s == 4) rk_phase<POT, ORDER, 4, true>(B, pt, a.W, wrow, a.dirtab, srow, a.At, pt.stage, s, a.dry, t);
+  else rk_phase<POT, ORDER, 2, true>(B, pt, a.W, wrow, a.dirtab, srow, a.At, pt.stage, s, a.dry, t);
 }
 
-template <bool POT, int ORDER, bool RK32>
+template <bool POT, int ORDER>
 __global__ void __launch_bounds__(kThreads, 2) k_step(Batch B, Parts pt, StepArgs a) {
+  extern __shared__ char smem[];
   __shared__ int aborted;
   if (threadIdx.x == 0) aborted = ld_acquire_u32(a.bar + 1) != 0u;
   __syncthreads();
@@ -1853,7 +1893,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_step(Batch B, Parts pt, StepArg
       if (grid_barrier(a.bar, a.limit_ns, a.err)) return;
       fused_combine(B, a);
       if (grid_barrier(a.bar, a.limit_ns, a.err)) return;
-      fused_rk<POT, ORDER, RK32>(B, w, lane, pt, a, srow, s);
+      fused_rk<POT, ORDER>(B, pt, a, srow, wrow, s, *(SlabTable*)smem);
       if (grid_barrier(a.bar, a.limit_ns, a.err)) return;
     }
   }
@@ -2153,7 +2193,7 @@ k_adj_b(Batch B, Parts pt, const double* __restrict__ W, const double* __restric
       const int n = min(T, nz - tn * T);
       if (i0 >= 0 && i0 + n <= nz) {
         const int64_t base = g.poff + (int64_t)dn * nz + i0;
-        for (int a = lane; a < narr; a += kLanes) {
+        prefetch_l2(lane, narr, base, n, [&](int a) {
           const double* arr;
           if (a < 9) arr = rho + (int64_t)a * P;
           else if (a < 18) arr = rhobar + (int64_t)(a - 9) * P;
@@ -2164,8 +2204,8 @@ k_adj_b(Batch B, Parts pt, const double* __restrict__ W, const double* __restric
           else if (a == 56) arr = gN;
           else if (a == 57) arr = gNbar;
           else arr = W + (int64_t)(a - 58) * P;
-          prefetch_l2(arr, base, n);
-        }
+          return arr;
+        });
       }
     }
     const int craw = tile * T - Hh + lane, j = wrapc(craw, nz);

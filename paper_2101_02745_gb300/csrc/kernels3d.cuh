@@ -451,8 +451,8 @@ k3_rk_stage(Box3 b, Parts pt, double* __restrict__ x, double* __restrict__ y, co
   const int64_t P = b.P;
   const int M = b.M, ny = b.n[1], nz = b.n[2];
   const double dt = *b.dt;
-  const double bdt = (s == 1 || s == 4) ? dt / 6.0 : dt / 3.0;
-  const double cdt = (s == 3) ? dt : 0.5 * dt;
+  double bdt, cdt;
+  rk_coefficients(s, dt, bdt, cdt);
   const double* src_b = (s == 1) ? pt.rhobar : pt.stage + 9 * P;
   const double* src_r = (s == 1) ? pt.rho : pt.stage;
   for (int64_t u = u0; u < u1; ++u) {

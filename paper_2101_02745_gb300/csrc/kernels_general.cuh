@@ -431,8 +431,8 @@ k_grk_stage(Batch B, Parts pt, const double* __restrict__ At, int s, int dry) {
   const BoxGeo& g = B.box[b];
   const int64_t P = B.Ptot;
   const double dt = B.dt[b];
-  const double bdt = (s == 1 || s == 4) ? dt / 6.0 : dt / 3.0;
-  const double cdt = (s == 3) ? dt : 0.5 * dt;
+  double bdt, cdt;
+  rk_coefficients(s, dt, bdt, cdt);
   const double ox = pt.ox[p], oy = pt.oy[p], oz = pt.oz[p];
   const double vz = g.c_light * oz;
   const double zs = fma(stage_frac(s - 1) * dt, vz, pt.z[p]);

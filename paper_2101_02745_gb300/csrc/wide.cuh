@@ -1,0 +1,320 @@
+// wide.cuh -- sums of products of doubles on the integer pipe.
+//
+// GB300 issues one FP64 instruction per SM every ~16 cycles (measured: DFMA
+// 16.4, DADD and DMUL 19), and in that time ~33 half-rate integer instructions
+// (IMAD.WIDE, SHF, LOP3) or ~65 full-rate ones (IADD, IMNMX); the two pipes
+// run side by side.  The bilinear parts of the step (commutators, stencil
+// sums) therefore run as fixed-point sums of 61-bit products with explicit
+// exponents, at a third to a sixth of the FP64 pipe's time.
+//
+// Representation.  An operand is a signed integer V = h 2^32 + 2 l with
+// |V| < 2^61 (h: the upper word; l: 31 bits with the sign of V) and an exponent
+// e, the IEEE exponent field it is aligned to: the double x becomes
+// V = x 2^(kBiasV - e), its 53 bits left-justified when e is x's own exponent
+// field.  A complex operand has one exponent, the larger of its parts'.
+// Products are (a b) / 2^64 = ah bh + 2 (ah bl + al bh) / 2^32 in an int64; the
+// dropped al bl and the rounded middle term cost at most two units of 2^-56 of
+// the product of the left-justified magnitudes.  A sum aligns its products to
+// the largest exponent among them (arithmetic shifts, one unit each): the four
+// groups of a commutator entry err by at most 12 units of 2^-56 of the largest
+// product, a third to a half of a chain of FP64 multiply-adds in the mean
+// (tests/test_wide_host.py measures both against exact sums: rms 3.7e-17 to
+// 6e-17 of the entry against 5.5e-17 to 1.3e-16).
+// Zero operands stay exactly zero, so zero products add exactly nothing.
+// Subnormal inputs count with their exponent field's value.  An infinite or
+// NaN input is not represented: callers test exponents for kExpNonFinite.
+//
+// The same code compiles for the host (g++), where the test runs it.
+#pragma once
+
+#include <cstdint>
+#ifndef __CUDACC__
+#define __host__
+#define __device__
+#define __forceinline__ inline
+#endif
+#define EMU_HD __host__ __device__ __forceinline__
+
+namespace emu_wide {
+
+struct Limbs { int h, l; };            // h 2^32 + 2 l
+struct Real { Limbs v; int e; };       // v 2^(e - kBiasV)
+struct Cplx { Limbs r, i; int e; };
+
+constexpr int kBiasV = 1083;           // 1023 + 52 + 8: 53 bits shifted up by 8
+constexpr int kBiasP = 2 * kBiasV - 64;   // a product of operands of exponents ea, eb: int64 2^(ea + eb - kBiasP)
+constexpr int kExpNonFinite = 2047;
+
+EMU_HD int hi_word(double x) {
+#ifdef __CUDA_ARCH__
+  return __double2hiint(x);
+#else
+  int64_t b;
+  __builtin_memcpy(&b, &x, 8);
+  return (int)(b >> 32);
+#endif
+}
+EMU_HD int lo_word(double x) {
+#ifdef __CUDA_ARCH__
+  return __double2loint(x);
+#else
+  int64_t b;
+  __builtin_memcpy(&b, &x, 8);
+  return (int)b;
+#endif
+}
+EMU_HD double from_words(int hi, int lo) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(hi, lo);
+#else
+  const int64_t b = (int64_t)(((uint64_t)(uint32_t)hi << 32) | (uint32_t)lo);
+  double x;
+  __builtin_memcpy(&x, &b, 8);
+  return x;
+#endif
+}
+// Low word of (hi:lo) >> min(s, 32), s >= 0.
+EMU_HD unsigned funnel_r(unsigned lo, unsigned hi, int s) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_rc(lo, hi, s);
+#else
+  return s >= 32 ? hi : (unsigned)((((uint64_t)hi << 32) | lo) >> s);
+#endif
+}
+// x >> s for any s >= 0 (the PTX shifts clamp s).
+EMU_HD int sar(int x, int s) {
+#ifdef __CUDA_ARCH__
+  int r;
+  asm("shr.s32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(s));
+  return r;
+#else
+  return x >> (s > 31 ? 31 : s);
+#endif
+}
+EMU_HD unsigned shr(unsigned x, int s) {
+#ifdef __CUDA_ARCH__
+  unsigned r;
+  asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(s));
+  return r;
+#else
+  return s > 31 ? 0u : x >> s;
+#endif
+}
+EMU_HD int min_i(int a, int b) { return a < b ? a : b; }
+EMU_HD int max_i(int a, int b) { return a > b ? a : b; }
+// a b + c and a b: one IMAD.WIDE each.  (Written out in PTX: where the compiler
+// moves an operand's sign extension away from the product it multiplies 64 by
+// 64 bits, four instructions for one.)
+EMU_HD int64_t mad(int a, int b, int64_t c) {
+#ifdef __CUDA_ARCH__
+  int64_t d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+#else
+  return (int64_t)a * b + c;
+#endif
+}
+EMU_HD int64_t prod(int a, int b) {
+#ifdef __CUDA_ARCH__
+  int64_t d;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+  return d;
+#else
+  return (int64_t)a * b;
+#endif
+}
+
+EMU_HD int exponent(double x) { return (hi_word(x) >> 20) & 0x7ff; }
+
+EMU_HD Limbs negate(Limbs a) { return Limbs{-a.h, -a.l}; }
+
+// x (exponent field e) left-justified / aligned to exponent E >= e.
+EMU_HD Limbs limbs(double x, int e) {
+  const int hi = hi_word(x), lo = lo_word(x), s = hi >> 31;
+  const unsigned m = (unsigned)(hi & 0xfffff) + ((unsigned)min_i(e, 1) << 20);   // (no leading one at e = 0)
+  return Limbs{((int)((m << 8) | ((unsigned)lo >> 24)) ^ s) - s, ((int)(((unsigned)lo << 7) & 0x7fffffffu) ^ s) - s};
+}
+EMU_HD Limbs limbs(double x, int e, int E) {
+  const int hi = hi_word(x), lo = lo_word(x), s = hi >> 31, d = E - e;
+  const unsigned m = (unsigned)(hi & 0xfffff) + ((unsigned)min_i(e, 1) << 20);
+  const unsigned v1 = (m << 8) | ((unsigned)lo >> 24), v0 = (unsigned)lo << 8;
+  const unsigned h = shr(v1, d), l = funnel_r(funnel_r(v0, v1, d), h, max_i(d - 32, 0));
+  return Limbs{((int)h ^ s) - s, ((int)(l >> 1) ^ s) - s};
+}
+
+// x, |x| <= 1, as V = x 2^62 (direction components, shape weights), whatever
+// its exponent field; with k > 0 V = x 2^(62 - k).
+EMU_HD Limbs unit_limbs(double x, int k = 0) {
+  const int hi = hi_word(x), lo = lo_word(x), s = hi >> 31, e = (hi >> 20) & 0x7ff, d = 1023 + k - e;
+  const unsigned m = (unsigned)(hi & 0xfffff) + ((unsigned)min_i(e, 1) << 20);
+  const unsigned v1 = (m << 10) | ((unsigned)lo >> 22), v0 = (unsigned)lo << 10;
+  const unsigned h = shr(v1, d), l = funnel_r(funnel_r(v0, v1, d), h, max_i(d - 32, 0));
+  return Limbs{((int)h ^ s) - s, ((int)(l >> 1) ^ s) - s};
+}
+// The k a component x of a direction needs: 0 up to 1 (and its rounding),
+// otherwise such that three scaled components stay below 1/2 each.
+EMU_HD int unit_excess(double x) {
+  const int a = hi_word(x) & 0x7fffffff;
+  return a > 0x3ff00001 ? (a >> 20) - 1021 : 0;
+}
+constexpr int kMaxExcess = 29;   // larger directions (above 2^27) count as infinite
+// Limbs of an int64 below 2^61 in magnitude, and back.
+EMU_HD Limbs split(int64_t v) { return Limbs{(int)(v >> 32), (int)((unsigned)v >> 1)}; }
+EMU_HD int64_t join(Limbs a) { return (int64_t)(((uint64_t)(uint32_t)a.h << 32) + 2 * (int64_t)a.l); }
+
+EMU_HD Real real(double x) {
+  const int e = exponent(x);
+  return Real{limbs(x, e), e};
+}
+EMU_HD Cplx cplx(double re, double im) {
+  const int er = exponent(re), ei = exponent(im), e = max_i(er, ei);
+  return Cplx{limbs(re, er, e), limbs(im, ei, e), e};
+}
+
+// Rounding addend of the middle term and the factor that folds it in.  From
+// constant memory, so that they stay register operands of IMAD.WIDE: as
+// literals the compiler turns them into 64-bit adds and shifts (mul 8 instead of
+// 4 instructions, mul2 12 instead of 7).
+#ifdef __CUDACC__
+__constant__ int64_t c_half = (int64_t)1 << 31;
+__constant__ int c_two = 2;
+#endif
+EMU_HD int64_t half_unit() {
+#ifdef __CUDA_ARCH__
+  return c_half;
+#else
+  return (int64_t)1 << 31;
+#endif
+}
+EMU_HD int two() {
+#ifdef __CUDA_ARCH__
+  return c_two;
+#else
+  return 2;
+#endif
+}
+// a b / 2^64 and (a b + c d) / 2^64.  |V| < 2^61 keeps every partial sum in 63 bits.
+EMU_HD int64_t mul(Limbs a, Limbs b) {
+  const int64_t m = mad(a.h, b.l, mad(a.l, b.h, half_unit()));
+  return mad((int)(m >> 32), two(), prod(a.h, b.h));
+}
+EMU_HD int64_t mul_add(Limbs a, Limbs b, int64_t c) {   // c + a b / 2^64
+  const int64_t m = mad(a.h, b.l, mad(a.l, b.h, half_unit()));
+  return mad((int)(m >> 32), two(), mad(a.h, b.h, c));
+}
+EMU_HD int64_t mul2(Limbs a, Limbs b, Limbs c, Limbs d) {
+  const int64_t m = mad(a.h, b.l, mad(a.l, b.h, mad(c.h, d.l, mad(c.l, d.h, half_unit()))));
+  return mad((int)(m >> 32), two(), mad(a.h, b.h, prod(c.h, d.h)));
+}
+
+// q + (a1 b1 + a2 b2 + a3 b3) / 2^64 for |a| < 2^61, |q| < 2^59 and |b| <= 2^62
+// with b1^2 + b2^2 + b3^2 <= 2^124: below 2^60.6.
+EMU_HD int64_t dot3(int64_t q, Limbs a1, Limbs b1, Limbs a2, Limbs b2, Limbs a3, Limbs b3) {
+  const int64_t m =
+      mad(a1.h, b1.l, mad(a1.l, b1.h, mad(a2.h, b2.l, mad(a2.l, b2.h, mad(a3.h, b3.l, mad(a3.l, b3.h, half_unit()))))));
+  const int64_t p = mad(a1.h, b1.h, mad(a2.h, b2.h, mad(a3.h, b3.h, q)));
+  return mad((int)(m >> 32), two(), p);
+}
+
+// v >> d, arithmetic, for any d >= 0; d2 = max(d - 32, 0) (shared by values of one shift).
+EMU_HD int64_t align(int64_t v, int d, int d2) {
+  const int hi = (int)(v >> 32), h = sar(hi, d);
+  const unsigned l = funnel_r(funnel_r((unsigned)v, (unsigned)hi, d), (unsigned)h, d2);
+  return (int64_t)(((uint64_t)(uint32_t)h << 32) | l);
+}
+EMU_HD int64_t align(int64_t v, int d) { return align(v, d, max_i(d - 32, 0)); }
+
+// c 2^k for a normal c whose exponent stays normal.
+EMU_HD double scale(double c, int k) { return from_words(hi_word(c) + (int)((unsigned)k << 20), lo_word(c)); }
+
+// x 2^k for x = 0 or a normal x whose exponent stays normal.
+EMU_HD double scale_nz(double x, int k) {
+  const int hi = hi_word(x);
+  return from_words(hi != 0 ? hi + (int)((unsigned)k << 20) : hi, lo_word(x));
+}
+
+// A traceless Hermitian matrix H as the commutator's left operand: diagonal
+// differences H_11 - H_22, H_11 - H_33, H_22 - H_33 and off-diagonals.
+struct Ham {
+  Real d12, d13, d23;
+  Cplx a, b, c;
+};
+// From the traceless components (H_11 - H_22, H_22 - H_33, off-diagonal reals).
+EMU_HD Ham ham(const double (&H)[8]) {
+  return Ham{real(H[0]), real(H[0] + H[1]), real(H[1]), cplx(H[2], H[3]), cplx(H[4], H[5]), cplx(H[6], H[7])};
+}
+
+// A Hermitian matrix r (or its conjugate) as the right operand.
+struct Mat {
+  Real e21, e31, e32;    // r_22 - r_11, r_33 - r_11, r_33 - r_22
+  Cplx x, y, z;
+  Limbs nx, ny, nz;      // minus the imaginary parts
+};
+EMU_HD Mat mat(const double* r, bool conj) {
+  Mat m;
+  m.e21 = real(r[1] - r[0]);
+  m.e31 = real(r[2] - r[0]);
+  m.e32 = real(r[2] - r[1]);
+  m.x = cplx(r[3], r[4]);
+  m.y = cplx(r[5], r[6]);
+  m.z = cplx(r[7], r[8]);
+  const int c = conj ? -1 : 0;
+  m.x.i = Limbs{(m.x.i.h ^ c) - c, (m.x.i.l ^ c) - c};
+  m.y.i = Limbs{(m.y.i.h ^ c) - c, (m.y.i.l ^ c) - c};
+  m.z.i = Limbs{(m.z.i.h ^ c) - c, (m.z.i.l ^ c) - c};
+  m.nx = negate(m.x.i);
+  m.ny = negate(m.y.i);
+  m.nz = negate(m.z.i);
+  return m;
+}
+// Largest exponent field among the operands (kExpNonFinite: an input is infinite or NaN).
+EMU_HD int top(const Ham& H) {
+  return max_i(max_i(max_i(H.d12.e, H.d13.e), max_i(H.d23.e, H.a.e)), max_i(H.b.e, H.c.e));
+}
+EMU_HD int top(const Mat& m) {
+  return max_i(max_i(max_i(m.e21.e, m.e31.e), max_i(m.e32.e, m.x.e)), max_i(m.y.e, m.z.e));
+}
+
+// C = [H, r], rounded to doubles up to a power of two each:
+//   C_12, C_13, C_23 = (or[q] + i oi[q]) 2^(oe[q] - kBiasP),
+//   K_11 / 2, K_22 / 2, K_33 / 2 of K = -i C = kd[q] 2^(ke[q] - kBiasP).
+struct Comm {
+  double cr[3], ci[3], kd[3];
+  int oe[3], ke[3];
+};
+
+// D x + E a + (g1) + (g2) at the largest exponent (at least emin).
+EMU_HD void off_diagonal(const Real& D, const Cplx& x, const Real& E, const Cplx& a, int64_t g1r, int64_t g1i, int e1,
+                         int64_t g2r, int64_t g2i, int e2, int emin, double& cr, double& ci, int& oe) {
+  const int ea = D.e + x.e, eb = E.e + a.e;
+  const int e = max_i(max_i(max_i(ea, eb), max_i(e1, e2)), emin);
+  const int da = e - ea, db = e - eb, d1 = e - e1, d2 = e - e2;
+  const int fa = max_i(da - 32, 0), fb = max_i(db - 32, 0), f1 = max_i(d1 - 32, 0), f2 = max_i(d2 - 32, 0);
+  cr = (double)(align(mul(D.v, x.r), da, fa) + align(mul(E.v, a.r), db, fb) + align(g1r, d1, f1) + align(g2r, d2, f2));
+  ci = (double)(align(mul(D.v, x.i), da, fa) + align(mul(E.v, a.i), db, fb) + align(g1i, d1, f1) + align(g2i, d2, f2));
+  oe = e;
+}
+
+EMU_HD void commutator(const Ham& H, const Mat& m, int emin, Comm& o) {
+  const Cplx &x = m.x, &y = m.y, &z = m.z, &a = H.a, &b = H.b, &c = H.c;
+  // C_12 = d12 x + e21 a + b z^* - y c^*
+  off_diagonal(H.d12, x, m.e21, a, mul2(b.r, z.r, b.i, z.i), mul2(b.i, z.r, b.r, m.nz), b.e + z.e,
+               -mul2(c.r, y.r, c.i, y.i), mul2(c.i, y.r, c.r, m.ny), c.e + y.e, emin, o.cr[0], o.ci[0], o.oe[0]);
+  // C_13 = d13 y + e31 b + a z - x c
+  off_diagonal(H.d13, y, m.e31, b, mul2(a.r, z.r, a.i, m.nz), mul2(a.r, z.i, a.i, z.r), a.e + z.e,
+               -mul2(c.r, x.r, c.i, m.nx), -mul2(c.r, x.i, c.i, x.r), c.e + x.e, emin, o.cr[1], o.ci[1], o.oe[1]);
+  // C_23 = d23 z + e32 c + a^* y - x^* b
+  off_diagonal(H.d23, z, m.e32, c, mul2(a.r, y.r, a.i, y.i), -mul2(a.r, m.ny, a.i, y.r), a.e + y.e,
+               -mul2(b.r, x.r, b.i, x.i), -mul2(b.i, x.r, b.r, m.nx), b.e + x.e, emin, o.cr[2], o.ci[2], o.oe[2]);
+  // K_11 / 2 = Im(a x^*) + Im(b y^*), K_22 / 2 = Im(c z^*) - Im(a x^*), K_33 / 2 = -Im(b y^*) - Im(c z^*)
+  const int64_t p = mul2(a.i, x.r, a.r, m.nx), q = mul2(b.i, y.r, b.r, m.ny), t = mul2(c.i, z.r, c.r, m.nz);
+  const int ep = a.e + x.e, eq = b.e + y.e, et = c.e + z.e;
+  o.ke[0] = max_i(max_i(ep, eq), emin);
+  o.ke[1] = max_i(max_i(ep, et), emin);
+  o.ke[2] = max_i(max_i(eq, et), emin);
+  o.kd[0] = (double)(align(p, o.ke[0] - ep) + align(q, o.ke[0] - eq));
+  o.kd[1] = (double)(align(t, o.ke[1] - et) - align(p, o.ke[1] - ep));
+  o.kd[2] = (double)(-align(q, o.ke[2] - eq) - align(t, o.ke[2] - et));
+}
+
+}  // namespace emu_wide

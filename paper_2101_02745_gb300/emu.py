@@ -620,7 +620,7 @@ class Box:
         emu_set_grid(self.box, blocks)
 
     def set_rk_form(self, form: int):
-        """1: RK stage with 32 cells per warp, 0: halo-lane form, -1: by units per warp."""
+        """Work split of the RK stage, 1: slabs of up to 8 tiles per block, 0: single tiles, -1: by units per block."""
         emu_set_rk_form(self.box, form)
 
     def set_step_form(self, form: int):
