@@ -79,10 +79,10 @@ const char* config_problem(const emu_config* c) {
 }
 
 // Tiles of a slab of the RK stage for a box of nt 32-cell tiles: the most (a
-// power of two, at most one per warp of a block) that leave no more than a
+// power of two, at most kSlabTiles) that leave no more than a
 // sixteenth of the slabs' tiles beyond the box, since their warps idle.
 int slab_tiles(int nt) {
-  int sw = kWarps;
+  int sw = kSlabTiles;
   while (sw > 1 && (int64_t)((nt + sw - 1) / sw) * sw * 16 > (int64_t)nt * 17) sw >>= 1;
   return sw;
 }
@@ -504,6 +504,19 @@ void pdl(cudaStream_t st, void (*kernel)(KArgs...), dim3 grid, Args... args) {
   (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Raises a kernel's dynamic shared memory limit, once per device and kernel
+// (`done`: one bit per device).
+template <typename K>
+cudaError_t raise_smem(K kernel, int bytes, std::atomic<unsigned>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 32 && ((done.load() >> dev) & 1u)) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && dev < 32) done.fetch_or(1u << dev);
+  return e;
+}
+
 template <typename... KArgs, typename... Args>
 void pdl_smem(cudaStream_t st, void (*kernel)(KArgs...), dim3 grid, int smem, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -583,7 +596,7 @@ int dep_cluster_size(int form) { return form == 2 ? 16 : 8; }
 
 // The cluster deposit's instance for the box's shape order, the weight table
 // and the cluster size of deposit form `form` (1: 8 blocks, 2: 16), with its
-// attributes set for the current device (64 KB of shared memory; 16-block
+// attributes set for the current device (86 KB of shared memory; 16-block
 // clusters are beyond the portable size).
 DepClusterKernel dep_cluster_kernel(const emu_box* b, int form, bool tab, cudaError_t* e) {
   DepClusterKernel k = nullptr;
@@ -593,7 +606,7 @@ DepClusterKernel dep_cluster_kernel(const emu_box* b, int form, bool tab, cudaEr
     else k = tab ? k_deposit_cluster<R, true, 8> : k_deposit_cluster<R, false, 8>;
     return 0;
   });
-  *e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kDepClusterSmem);
+  *e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kDepSmem);
   if (*e == cudaSuccess && form == 2) *e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   return k;
 }
@@ -611,7 +624,7 @@ int dep_cluster_capacity(emu_box* b, int form) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(64 * cl));
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kDepClusterSmem;
+    cfg.dynamicSmemBytes = kDepSmem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)cl;
@@ -641,7 +654,7 @@ int launch_deposit_cluster(emu_box* b, const double* rnu, const double* rnb, con
   DepClusterKernel k = dep_cluster_kernel(b, form, wrow != nullptr, &e);
   if (e != cudaSuccess) return cuda_check(b, e, "cluster deposit attributes");
   before_launch(b, CLS_DEPOSIT);
-  e = cluster_pdl(b->stream, k, clusters, dep_cluster_size(form), kDepClusterSmem, B, b->pt.z, b->pt.N, b->pt.Nbar,
+  e = cluster_pdl(b->stream, k, clusters, dep_cluster_size(form), kDepSmem, B, b->pt.z, b->pt.N, b->pt.Nbar,
                   rnu, rnb, b->dirtab, shift_row, wrow, frac, out, W, b->err);
   const int rc = after_launch(b, "cluster deposit kernel");   // (closes the timing record either way)
   return e != cudaSuccess ? cuda_check(b, e, "cluster deposit launch") : rc;
@@ -651,8 +664,9 @@ int launch_deposit_cluster(emu_box* b, const double* rnu, const double* rnb, con
 // with the shift row shift_row, into out ([36][NZ]; mode 5: [32][NZ]).  Modes as k_deposit; the
 // potential scale kappa/dV for modes 0 and 3, 1/dV for the moments.
 int launch_deposit(emu_box* b, int mode, const double* rnu, const double* rnb, const int* shift_row, double frac,
-                   double* out, double* W = nullptr) {
-  if (!W) W = b->W;   // where modes 0 and 5 keep the shape weights
+                   double* out, double* W = nullptr, bool keep = true) {
+  // where modes 0 and 5 keep the shape weights
+  if (!W) W = keep || weight_row(b, shift_row) == nullptr ? b->W : nullptr;
   if (mode == 5 && b->dep_form != 0) return launch_deposit_cluster(b, rnu, rnb, shift_row, frac, out, W);
   const Batch B = batch_view(b);
   before_launch(b, CLS_DEPOSIT);
@@ -681,11 +695,17 @@ int launch_deposit(emu_box* b, int mode, const double* rnu, const double* rnb, c
     else if (mode == 4)
       pdl(st, k_deposit<4, R>, grid, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, nullptr,
           b->err);
-    else if (wrow != nullptr)
-      pdl(st, k_deposit<5, R, true>, grid, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, W,
-          b->err);
-    else
-      pdl(st, k_deposit<5, R>, grid, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, W, b->err);
+    else {
+      auto step = [&](auto TAB) {
+        static std::atomic<unsigned> done{0};
+        auto k = k_deposit<5, R, decltype(TAB)::value>;
+        if (raise_smem(k, kDepSmem, done) == cudaSuccess)
+          pdl_smem(st, k, grid, kDepSmem, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, W,
+                   b->err);
+      };
+      if (wrow != nullptr) step(std::true_type{});
+      else step(std::false_type{});
+    }
     return 0;
   });
   if (int rc = after_launch(b, "deposit kernel")) return rc;
@@ -715,26 +735,16 @@ int launch_gstep(emu_box* b, int dry);
 int launch_gstage(emu_box* b, int s, int dry);
 int launch_gdeposit(emu_box* b, int mode, const double* rnu, const double* rnb, double frac, double* out);
 
-int launch_stage(emu_box* b, int s, int dry) {
+// keep: the stage's shape weights stay in b->W (the adjoint reads them);
+// otherwise, when every particle takes its ring's weights from the table, they
+// are not stored (the RK stage reads the table: 48 bytes a particle less).
+int launch_stage(emu_box* b, int s, int dry, bool keep = false) {
   const size_t P = (size_t)b->S.Ptot;
   const double* rnu = (s == 1) ? b->pt.rho : b->pt.stage;
   const double* rnb = (s == 1) ? b->pt.rhobar : b->pt.stage + 9 * P;
   const int* srow = b->shift + (size_t)(s - 1) * b->S.MT;
-  if (int rc = launch_deposit(b, 5, rnu, rnb, srow, kStageFrac[s - 1], b->At)) return rc;
+  if (int rc = launch_deposit(b, 5, rnu, rnb, srow, kStageFrac[s - 1], b->At, nullptr, keep)) return rc;
   return launch_rk(b, s, srow, dry);
-}
-
-// Raises a kernel's dynamic shared memory limit, once per device and kernel
-// (`done`: one bit per device).
-template <typename K>
-cudaError_t raise_smem(K kernel, int bytes, std::atomic<unsigned>& done) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 32 && ((done.load() >> dev) & 1u)) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess && dev < 32) done.fetch_or(1u << dev);
-  return e;
 }
 
 // Most blocks of the fused step kernel that can be resident at once (its
@@ -749,8 +759,8 @@ int fused_max_blocks(const emu_box* b) {
   // (cubic shape, vacuum terms) stands for all
   (void)b;
   static std::atomic<unsigned> done{0};
-  if (raise_smem(k_step<true, 3>, kSlabSmem, done) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<true, 3>, kThreads, kSlabSmem) != cudaSuccess)
+  if (raise_smem(k_step<true, 3>, kStepSmem, done) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<true, 3>, kThreads, kStepSmem) != cudaSuccess)
     return 0;
   return per_sm * sms;
 }
@@ -778,7 +788,7 @@ int launch_fused(emu_box* b, int dry, int64_t nsteps) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = persist_grid(b);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSlabSmem;
+  cfg.dynamicSmemBytes = kStepSmem;
   cfg.stream = b->stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -791,7 +801,7 @@ int launch_fused(emu_box* b, int dry, int64_t nsteps) {
     auto launch = [&](auto POT) {
       static std::atomic<unsigned> done{0};
       auto k = k_step<decltype(POT)::value, R>;
-      if (raise_smem(k, kSlabSmem, done) == cudaSuccess) (void)cudaLaunchKernelEx(&cfg, k, B, b->pt, a);
+      if (raise_smem(k, kStepSmem, done) == cudaSuccess) (void)cudaLaunchKernelEx(&cfg, k, B, b->pt, a);
     };
     if (b->pot) launch(std::true_type{});
     else launch(std::false_type{});
@@ -2288,7 +2298,7 @@ int adjoint_body(emu_box* b, double* lambda, double* gN, double* gNbar, void* ad
   // forward stages 1..3: y2, y3 copied out, y4 left in the stage buffer; each
   // stage's weights and potential kept for the backward pass
   for (int s = 1; s <= 3; ++s) {
-    if (int rc = launch_stage(b, s, 0)) return rc;
+    if (int rc = launch_stage(b, s, 0, true)) return rc;
     if (nws)
       if (int rc = cuda_check(b, cudaMemcpyAsync(Wk + (s - 1) * nws, b->W, sizeof(double) * nws,
                                                  cudaMemcpyDeviceToDevice, b->stream), "keep stage weights"))

@@ -559,36 +559,13 @@ __device__ __forceinline__ void deposit_tile_dirs(const Batch& B, int b, int til
     } else {
       bad |= shape_weights<ORDER>(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d), wt);
     }
-    if ((MODE == 0 || MODE == 5) && W != nullptr && own) {   // the RK stage of these positions reads them back
+    if (MODE == 0 && W != nullptr && own) {   // the RK stage of these positions reads them back
 #pragma unroll
       for (int q = 0; q < Sten<ORDER>::NWS; ++q) W[q * P + p] = wt[q];
     }
     Spread<ORDER> spread;
     spread.init(wt);
-    if constexpr (MODE == 5) {
-      const double n1 = __ldg(N + p), n2 = __ldg(Nbar + p);
-      double bprev = 0.0;   // B of the previous diagonal entry
-#pragma unroll
-      for (int c = 0; c < kNC; ++c) {
-        double bv;
-        if (c < 2) {
-          if (c == 0) bprev = fma(-n2, ldd<COH>(r_nb + p), n1 * ldd<COH>(r_nu + p));
-          const double bn =
-              fma(-n2, ldd<COH>(r_nb + (c + 1) * P + p), n1 * ldd<COH>(r_nu + (c + 1) * P + p));
-          bv = bprev - bn;
-          bprev = bn;
-        } else {
-          const int k = c + 1;
-          const double x = ldd<COH>(r_nu + k * P + p), y = ldd<COH>(r_nb + k * P + p);
-          bv = (k == 4 || k == 6 || k == 8) ? fma(n2, y, n1 * x) : fma(-n2, y, n1 * x);
-        }
-        const double cc = spread.apply(bv);
-        acc[c] += cc;
-        acc[kNC + c] = fma(ox, cc, acc[kNC + c]);
-        acc[2 * kNC + c] = fma(oy, cc, acc[2 * kNC + c]);
-        acc[3 * kNC + c] = fma(oz, cc, acc[3 * kNC + c]);
-      }
-    } else if constexpr (MODE == 4) {
+    if constexpr (MODE == 4) {
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
         const double c1 = spread.apply(__ldg(N + p) * ldd<COH>(r_nu + k * P + p));
@@ -630,6 +607,226 @@ __device__ __forceinline__ void deposit_tile_dirs(const Batch& B, int b, int til
 __device__ __forceinline__ emu_wide::Limbs bcast(emu_wide::Limbs v, int src) {
   return emu_wide::Limbs{__shfl_sync(kFull, v.h, src), __shfl_sync(kFull, v.l, src)};
 }
+// Limbs of the lane o to the left (o > 0) or right (o < 0).
+__device__ __forceinline__ emu_wide::Limbs from_lane(emu_wide::Limbs v, int o) {
+  return o > 0 ? emu_wide::Limbs{__shfl_up_sync(kFull, v.h, o), __shfl_up_sync(kFull, v.l, o)}
+               : emu_wide::Limbs{__shfl_down_sync(kFull, v.h, -o), __shfl_down_sync(kFull, v.l, -o)};
+}
+__device__ __forceinline__ int from_lane(int v, int o) {
+  return o > 0 ? __shfl_up_sync(kFull, v, o) : __shfl_down_sync(kFull, v, -o);
+}
+
+// Asynchronous copies of 8 bytes from global to shared memory, by the thread
+// that reads them: its copies of all but the last N groups are done after
+// cp_async_wait<N>.
+__device__ __forceinline__ void cp_async8(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+constexpr int kDepRows = 21;   // doubles of a particle the step's deposit reads
+constexpr int kDepBuf = 2 * kDepRows * kLanes;                                // of one warp's buffers
+constexpr int kDepSmem = kWarps * kDepBuf * (int)sizeof(double);              // 86 KB a block
+
+// deposit_tile_dirs for the step's deposit (MODE 5), on the integer pipe.  B is
+// formed in FP64 (20 instructions a particle, against 85 for the whole
+// deposit: at 16 cycles each the FP64 pipe bound it); its spread over the
+// stencil and the four moments' sums are fixed-point (wide.cuh).  A sum is an
+// int64 per lane; the components of one exponent group (B_11 - B_22,
+// B_22 - B_33 and the three complex off-diagonals) share the exponent ea of
+// their sums, which grows when a direction's contribution asks for it (the
+// sums are then shifted).  A tile's sums of n directions leave ceil(log2 n)
+// bits of headroom, so a contribution keeps 61 - ceil(log2 n) bits below the
+// largest one's leading bit: less error than FP64 sums of n terms, whose
+// rounding follows the partial sums.  Zero contributions add exactly nothing.
+// (buf: this warp's two buffers of kDepRows x 32 doubles in shared memory.)
+template <int ORDER, bool COH>
+__device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int tile, int dfirst, int dlast, int lane,
+                                                  const double* z, const double* __restrict__ N,
+                                                  const double* __restrict__ Nbar, const double* r_nu,
+                                                  const double* r_nb, const double* __restrict__ dirtab,
+                                                  const int* shift, const double* wrow, double frac, double* W,
+                                                  double* buf, double (&out)[kNT], int& bad) {
+  namespace w = emu_wide;
+  constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T, NW = Sten<ORDER>::NW, kGroups = 5;
+  const BoxGeo& g = B.box[b];
+  const int nz = g.nz;
+  const unsigned P = (unsigned)B.Ptot;
+  const int MT = B.MT;
+  const int craw = tile * T - H + lane;
+  const int j = wrapc(craw, nz);
+  const double hp = (double)j + 0.5;
+  const bool own = lane >= H && lane < H + T && craw < nz;
+  const double pos_dt = frac * B.dt[b];
+  const int dbase = g.doff;
+  const int head = max(32 - __clz(dlast - dfirst), 2) - 2;   // headroom beyond the two bits a contribution leaves
+  int64_t acc[kNT];
+  int ea[kGroups];
+#pragma unroll
+  for (int c = 0; c < kNT; ++c) acc[c] = 0;
+#pragma unroll
+  for (int q = 0; q < kGroups; ++q) ea[q] = 0;
+  // direction d's particle data into buffer d & 1, asynchronously (each lane
+  // its own particle's: no exchange between lanes): z, N, Nbar, rho, rhobar
+  auto fetch = [&](int d, int sh) -> int64_t {
+    int i = j - sh;
+    if (i < 0) i += nz;
+    const int64_t p = g.poff + (int64_t)d * nz + i;
+    double* dst = buf + (d & 1) * kDepRows * kLanes + lane;
+    cp_async8(dst, z + p);
+    cp_async8(dst + kLanes, N + p);
+    cp_async8(dst + 2 * kLanes, Nbar + p);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      cp_async8(dst + (3 + k) * kLanes, row(r_nu + p, P, k));
+      cp_async8(dst + (12 + k) * kLanes, row(r_nb + p, P, k));
+    }
+    cp_async_commit();
+    return p;
+  };
+  // a direction's own numbers, loaded a direction ahead: Omega in lanes 0-2,
+  // the ring's weights (when every particle takes them) in the next NW, v_z
+  const bool ring = ORDER > 0 && wrow != nullptr;
+  const double* utab = lane < 3 ? dirtab + lane * MT : wrow + (lane - 3) * MT;
+  const bool uload = lane < 3 || (ring && lane < 3 + NW);
+  auto own_number = [&](int gd) { return uload ? ldp<COH>(utab + gd) : 0.0; };
+  int64_t pnext = fetch(dfirst, ldi<COH>(shift + dbase + dfirst));
+  double unext = own_number(dbase + dfirst), vnext = __ldg(dirtab + 3 * MT + dbase + dfirst);
+  int shnext = dfirst + 1 < dlast ? ldi<COH>(shift + dbase + dfirst + 1) : 0;
+  for (int d = dfirst; d < dlast; ++d) {
+    const int gd = dbase + d;
+    const int64_t p = pnext;
+    const double u = unext, vz = vnext;
+    if (d + 1 < dlast) {
+      pnext = fetch(d + 1, shnext);
+      unext = own_number(gd + 1);
+      vnext = __ldg(dirtab + 3 * MT + gd + 1);
+      if (d + 2 < dlast) shnext = ldi<COH>(shift + gd + 2);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    const double* x = buf + (d & 1) * kDepRows * kLanes + lane;
+    auto rnu = [&](int k) { return x[(3 + k) * kLanes]; };
+    auto rnb = [&](int k) { return x[(12 + k) * kLanes]; };
+    const double n1 = x[kLanes], n2 = x[2 * kLanes];
+    const double zs = fma(pos_dt, vz, x[0]);
+    w::Limbs wl[NW];   // the weight slot o of the particle that gives it to this lane's cell
+    double wt[NW];
+    if (wrow != nullptr) {
+      bad |= off_site(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d));
+    } else {
+      bad |= shape_weights<ORDER>(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d), wt);
+      if (W != nullptr && own) {   // the RK stage of these positions reads them back
+#pragma unroll
+        for (int q = 0; q < Sten<ORDER>::NWS; ++q) *row(W + p, P, q) = wt[q];
+      }
+    }
+    // directions above 1 (not unit vectors) are scaled by 2^-ko
+    const int ko = __reduce_max_sync(kFull, lane < 3 ? w::unit_excess(u) : 0);
+    const w::Limbs ul = w::unit_limbs(u, lane < 3 ? ko : 0);
+    const w::Limbs om[3] = {bcast(ul, 0), bcast(ul, 1), bcast(ul, 2)};
+    if constexpr (ORDER > 0) {
+      if (wrow != nullptr) {
+        if (W != nullptr && own) {
+#pragma unroll
+          for (int q = 0; q < NW; ++q) *row(W + p, P, q) = ldp<COH>(wrow + q * MT + gd);
+        }
+#pragma unroll
+        for (int o = 0; o < NW; ++o) wl[o] = bcast(ul, 3 + o);
+      } else {
+#pragma unroll
+        for (int o = 0; o < NW; ++o) {   // from the lane o - H to the left
+          wl[o] = w::unit_limbs(wt[o]);
+          if (o != H) wl[o] = from_lane(wl[o], o - H);
+        }
+      }
+    }
+    double bprev = fma(-n2, rnb(0), n1 * rnu(0));   // B of the previous diagonal entry
+#pragma unroll
+    for (int q = 0; q < kGroups; ++q) {
+      const int nc = q < 2 ? 1 : 2, c0 = q < 2 ? q : 2 * q - 2;   // the group's components c0 .. c0 + nc - 1
+      double bv[2];
+      if (q < 2) {
+        const double bn = fma(-n2, rnb(q + 1), n1 * rnu(q + 1));
+        bv[0] = bprev - bn;
+        bprev = bn;
+        bv[1] = 0.0;
+      } else {
+        const int k = c0 + 1;   // conj(rhobar) flips the sign of the imaginary part
+        bv[0] = fma(-n2, rnb(k), n1 * rnu(k));
+        bv[1] = fma(n2, rnb(k + 1), n1 * rnu(k + 1));
+      }
+      const int e0 = w::exponent(bv[0]), e1 = nc > 1 ? w::exponent(bv[1]) : 0, e = max(e0, e1);
+      w::Limbs bl[2];
+      bl[0] = nc > 1 ? w::limbs(bv[0], e0, e) : w::limbs(bv[0], e);
+      if (nc > 1) bl[1] = w::limbs(bv[1], e1, e);
+      // the spread (Eq. 5): taps at the largest exponent of the contributing particles
+      int64_t cv[2];
+      int et = e;
+      if constexpr (ORDER == 0) {
+        for (int c = 0; c < nc; ++c) cv[c] = w::join(bl[c]) >> 2;
+      } else {
+        int en[NW];
+#pragma unroll
+        for (int o = 0; o < NW; ++o) {
+          en[o] = o == H ? e : from_lane(e, o - H);
+          et = max(et, en[o]);
+        }
+        for (int c = 0; c < nc; ++c) cv[c] = 0;
+#pragma unroll
+        for (int o = 0; o < NW; ++o) {
+          const int dd = et - en[o], df = max(dd - 32, 0);
+#pragma unroll
+          for (int c = 0; c < nc; ++c) {
+            const w::Limbs v = o == H ? bl[c] : from_lane(bl[c], o - H);
+            cv[c] += w::align(w::mul(v, wl[o]), dd, df);
+          }
+        }
+      }
+      // the sums' exponent
+      const int es = ko <= w::kMaxExcess ? et + ko : w::kExpNonFinite;
+      if (es + head > ea[q]) {
+        const int sh = es + head - ea[q], sf = max(sh - 32, 0);
+        ea[q] += sh;
+#pragma unroll
+        for (int c = 0; c < nc; ++c) {
+#pragma unroll
+          for (int m = 0; m < 4; ++m) acc[m * kNC + c0 + c] = w::align(acc[m * kNC + c0 + c], sh, sf);
+        }
+      }
+      const int dd = ea[q] - es, df = max(dd - 32, 0);
+#pragma unroll
+      for (int c = 0; c < nc; ++c) {
+        const int64_t v = w::align(cv[c], dd, df);
+        const w::Limbs l = w::split(v);
+        acc[c0 + c] += w::align(v, 2 + ko, 0);
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+          acc[(m + 1) * kNC + c0 + c] = w::mul_add(l, om[m], acc[(m + 1) * kNC + c0 + c]);
+      }
+    }
+  }
+  // acc 2^(ea + 4 - kBiasV)
+#pragma unroll
+  for (int q = 0; q < kGroups; ++q) {
+    const int nc = q < 2 ? 1 : 2, c0 = q < 2 ? q : 2 * q - 2;
+    const int k = min(max(ea[q] + 4 - w::kBiasV, -1022), 959);
+#pragma unroll
+    for (int c = 0; c < nc; ++c) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const double v = (double)acc[m * kNC + c0 + c];
+        out[m * kNC + c0 + c] = ea[q] >= w::kExpNonFinite ? nan("") : w::scale_nz(v, k);
+      }
+    }
+  }
+}
+
 // Deposit (Eq. 5), first phase.  MODE 0: B = N rho - Nbar rhobar^* (the
 // combination that enters H, Eq. 2); MODE 1: B = N rho; MODE 2: B = Nbar rhobar;
 // MODE 3: B = r_nu (packed matrices given per particle: the adjoint's Gamma);
@@ -652,7 +849,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
                                               const double* r_nu, const double* r_nb,
                                               const double* __restrict__ dirtab, const int* shift,
                                               const double* wrow, double frac, double* __restrict__ partial,
-                                              double* W, int* err) {
+                                              double* W, int* err, double* buf = nullptr) {
   const int64_t u0 = unit_begin(w, B), u1 = unit_begin(w + 1, B);
   if (u0 >= u1) return;
   int bad = 0;
@@ -670,8 +867,12 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
     double acc[NA];
 #pragma unroll
     for (int c = 0; c < NA; ++c) acc[c] = 0.0;
-    deposit_tile_dirs<MODE, ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow,
-                                        frac, W, acc, bad);
+    if constexpr (MODE == 5)
+      deposit_tile_wide<ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow, frac,
+                                    W, buf, acc, bad);
+    else
+      deposit_tile_dirs<MODE, ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow,
+                                          frac, W, acc, bad);
     constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T;
     flush_tile<ORDER>(acc, g.toff + tile, tile * T - H + lane, g.nz, w, lane, partial);
   }
@@ -686,9 +887,10 @@ k_deposit(Batch B, const double* __restrict__ z, const double* __restrict__ N, c
           const double* __restrict__ r_nu, const double* __restrict__ r_nb, const double* __restrict__ dirtab,
           const int* __restrict__ shift, const double* __restrict__ wrow, double frac, double* __restrict__ partial,
           double* __restrict__ W, int* __restrict__ err) {
+  extern __shared__ double dep_sm[];   // (MODE 5: kDepSmem bytes)
   griddep_wait();
   deposit_phase<MODE, ORDER, false>(B, logical_warp(), threadIdx.x & 31, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                    TAB ? wrow : nullptr, frac, partial, W, err);
+                                    TAB ? wrow : nullptr, frac, partial, W, err, dep_sm + (threadIdx.x >> 5) * kDepBuf);
 }
 
 // ------------------------------------------------------- cluster deposit
@@ -704,7 +906,7 @@ k_deposit(Batch B, const double* __restrict__ z, const double* __restrict__ N, c
 // box and the cluster size, not on the grid: results are bitwise reproducible.
 // All blocks of a cluster walk the same tiles, so every block reaches every
 // cluster barrier (hardware barriers, as __syncthreads: no spin on memory).
-constexpr int kDepClusterSmem = kWarps * kNT * kLanes * (int)sizeof(double);   // 64 KB
+static_assert(kDepBuf >= kNT * kLanes, "a warp's sums of a tile fit its buffers");
 
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
@@ -754,7 +956,8 @@ k_deposit_cluster(Batch B, const double* __restrict__ z, const double* __restric
                   const double* __restrict__ dirtab, const int* __restrict__ shift, const double* __restrict__ wrow,
                   double frac, double* __restrict__ out, double* __restrict__ W, int* __restrict__ err) {
   griddep_wait();
-  extern __shared__ double red[];   // [kWarps][kNT][kLanes]: each warp's sums of the tile
+  // each warp's particle data, then its sums of the tile ([kNT][kLanes])
+  extern __shared__ double red[];
   constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T;
   constexpr int NE = kNT * kLanes, per = NE / CL, nwc = CL * kWarps;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -770,15 +973,15 @@ k_deposit_cluster(Batch B, const double* __restrict__ z, const double* __restric
 #pragma unroll
     for (int c = 0; c < kNT; ++c) acc[c] = 0.0;
     if (d0 < d1)
-      deposit_tile_dirs<5, ORDER, false>(B, b, tile, d0, d1, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                         TAB ? wrow : nullptr, frac, W, acc, bad);
+      deposit_tile_wide<ORDER, false>(B, b, tile, d0, d1, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
+                                      TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, acc, bad);
 #pragma unroll
-    for (int c = 0; c < kNT; ++c) red[(wib * kNT + c) * kLanes + lane] = acc[c];
+    for (int c = 0; c < kNT; ++c) red[wib * kDepBuf + c * kLanes + lane] = acc[c];
     __syncthreads();
     for (int e = threadIdx.x; e < NE; e += kThreads) {   // the block's warps, in warp order
       double v = red[e];
 #pragma unroll
-      for (int i = 1; i < kWarps; ++i) v += red[i * NE + e];
+      for (int i = 1; i < kWarps; ++i) v += red[i * kDepBuf + e];
       red[e] = v;
     }
     cluster_sync();
@@ -1105,7 +1308,8 @@ __device__ __forceinline__ int box_of_slab_unit(const Batch& B, int64_t x) {
 // warp forms G = A0 - Omega . A of its cells, the neighbours' G come from
 // shared memory, and the stencil sum is the commutator's operand: everything
 // up to the update runs on the integer pipe.
-constexpr int kSlabCells = kWarps * kLanes + 4;    // cells of the widest slab, two neighbours a side
+constexpr int kSlabTiles = 8;                      // most tiles of a slab
+constexpr int kSlabCells = kSlabTiles * kLanes + 4;   // cells of the widest slab, two neighbours a side
 constexpr int kRowCells = kLanes + 4;              // cells of a unit, likewise
 struct SlabTable {
   int2 a[kNT][kSlabCells];                         // the potential: A0 / 4 as int64, limbs of A_x, A_y, A_z
@@ -1114,6 +1318,7 @@ struct SlabTable {
   const double* pf[64];                            // the arrays a stage reads, for the L2 prefetch
 };
 constexpr int kSlabSmem = (int)sizeof(SlabTable);
+constexpr int kStepSmem = kSlabSmem > kDepSmem ? kSlabSmem : kDepSmem;   // of k_step: either phase's
 
 // Potential of cells c0 .. c0 + n - 1 (modulo nz) of box g into the table, by
 // the whole block: one (cell, exponent group) per thread and round.
@@ -1222,11 +1427,28 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
     const int64_t poff = g.poff;
     const int doff = g.doff;
     const int tc = tile0 + H + lane;                   // table cell of this lane
-    for (int d = d0 + wib / sw; d < d1; d += dstep) {
+    // a direction's own numbers, loaded a unit ahead: -Omega in lanes 0-2, the
+    // ring's weights (when every particle takes them) in the next NW, the shift
+    const bool ring = ORDER > 0 && wrow != nullptr;
+    const double* utab = lane < 3 ? dirtab + lane * MT : wrow + (lane - 3) * MT;
+    const bool uload = lane < 3 || (ring && lane < 3 + NW);
+    auto own_number = [&](int gd) {
+      const double v = uload ? ldp<COH>(utab + gd) : 0.0;
+      return lane < 3 ? -v : v;
+    };
+    const int dw = d0 + wib / sw;
+    if (dw >= d1) continue;
+    const bool active = lane < n;
+    double unext = own_number(doff + dw);
+    int shnext = ldi<COH>(shift + doff + dw);
+    for (int d = dw; d < d1; d += dstep) {
       const int gd = doff + d;
-      const int sh = ldi<COH>(shift + gd);
+      const int sh = shnext;
+      const double u = unext;
       if (d + dstep < d1) {   // prefetch the next unit's particle data into L2
-        int i0 = c0 + tile0 - ldi<COH>(shift + gd + dstep);
+        unext = own_number(gd + dstep);
+        shnext = ldi<COH>(shift + gd + dstep);
+        int i0 = c0 + tile0 - shnext;
         if (i0 < 0) i0 += nz;
         const int cnt = min(n, nz - i0);
         const int64_t nb = poff + (int64_t)(d + dstep) * nz + i0;
@@ -1237,25 +1459,15 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
       }
       int i = c0 + tile0 + lane - sh;
       if (i < 0) i += nz;
-      const bool active = lane < n;
-      if (!active) i = 0;
-      const int64_t p = poff + (int64_t)d * nz + i;
+      const int64_t p = poff + (int64_t)d * nz + (active ? i : 0);
       // the neutrino source matrix and the weights first, so their latency
       // overlaps the interpolation
       double r[9], wd[NW];
 #pragma unroll
       for (int k = 0; k < 9; ++k) r[k] = ldp<COH>(row(src_r + p, (unsigned)P, k));
-      // -Omega, and the ring's weights when every particle takes them: lane q
-      // converts one of them
-      double u = 0.0;
-      if (lane < 3) u = -__ldg(dirtab + lane * MT + gd);
-      if constexpr (ORDER > 0) {
-        if (wrow != nullptr) {
-          if (lane >= 3 && lane < 3 + NW) u = ldp<COH>(wrow + (lane - 3) * MT + gd);
-        } else {
+      if (ORDER > 0 && !ring) {
 #pragma unroll
-          for (int o = 0; o < NW; ++o) wd[o] = ldp<COH>(row(W + p, (unsigned)P, o));
-        }
+        for (int o = 0; o < NW; ++o) wd[o] = ldp<COH>(row(W + p, (unsigned)P, o));
       }
       // directions above 1 (not unit vectors) are scaled by 2^-ko
       const int ko = __reduce_max_sync(kFull, lane < 3 ? w::unit_excess(u) : 0);
@@ -1849,9 +2061,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned long long l
 template <int ORDER>
 __device__ __forceinline__ void fused_deposit(const Batch& B, int64_t w, int lane, const Parts& pt, const double* rnu,
                                            const double* rnb, const StepArgs& a, const int* srow,
-                                           const double* wrow, double frac) {
+                                           const double* wrow, double frac, double* buf) {
   deposit_phase<5, ORDER, true>(B, w, lane, pt.z, pt.N, pt.Nbar, rnu, rnb, a.dirtab, srow, wrow, frac, a.partial,
-                                a.W, a.err);
+                                wrow != nullptr ? nullptr : a.W, a.err, buf);
 }
 
 __device__ __forceinline__ void fused_combine(const Batch& B, const StepArgs& a) {
@@ -1868,7 +2080,7 @@ __device__ __forceinline__ void fused_rk(const Batch& B, const Parts& pt, const 
 
 template <bool POT, int ORDER>
 __global__ void __launch_bounds__(kThreads, 2) k_step(Batch B, Parts pt, StepArgs a) {
-  extern __shared__ char smem[];
+  extern __shared__ char smem[];   // the deposit's buffers, then the RK stage's table
   __shared__ int aborted;
   if (threadIdx.x == 0) aborted = ld_acquire_u32(a.bar + 1) != 0u;
   __syncthreads();
@@ -1889,7 +2101,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_step(Batch B, Parts pt, StepArg
       const double* wrow = a.wtab != nullptr ? a.wtab + (s - 1) * kWSlots * MT : nullptr;
       const double* rnu = s == 1 ? pt.rho : pt.stage;
       const double* rnb = s == 1 ? pt.rhobar : pt.stage + 9 * P;
-      fused_deposit<ORDER>(B, w, lane, pt, rnu, rnb, a, srow, wrow, stage_frac(s - 1));
+      fused_deposit<ORDER>(B, w, lane, pt, rnu, rnb, a, srow, wrow, stage_frac(s - 1),
+                           (double*)smem + (threadIdx.x >> 5) * kDepBuf);
       if (grid_barrier(a.bar, a.limit_ns, a.err)) return;
       fused_combine(B, a);
       if (grid_barrier(a.bar, a.limit_ns, a.err)) return;
