@@ -4,6 +4,7 @@ from __future__ import annotations
 import os
 import shutil
 import subprocess
+import tempfile
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
@@ -29,15 +30,22 @@ def stale() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:
-    """Compile every CUDA source into one shared library (static cudart)."""
+    """Compile every CUDA source (in parallel) into one shared library (static cudart)."""
     if not force and not stale():
         return LIB
     tmp = LIB.with_name(f".{LIB.name}.{os.getpid()}.tmp")
-    cmd = [nvcc(), *ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-shared",
-           f"-I{ROOT / 'include'}", "-o", str(tmp), *map(str, SOURCES)]
+    # (kernel templates are instantiated in one translation unit and launched from another)
+    flags = [*ARCH, "-O3", "-lineinfo", "-std=c++17", "-static-global-template-stub=false", "-Xcompiler", "-fPIC",
+             f"-I{ROOT / 'include'}"]
     if verbose:
-        cmd.insert(1, "-Xptxas=-v")
-    subprocess.check_call(cmd)
+        flags.insert(0, "-Xptxas=-v")
+    with tempfile.TemporaryDirectory() as d:   # the translation units side by side
+        objs = [Path(d) / (p.stem + ".o") for p in SOURCES]
+        jobs = [subprocess.Popen([nvcc(), *flags, "-c", "-o", str(o), str(p)]) for o, p in zip(objs, SOURCES)]
+        bad = [p.name for j, p in zip(jobs, SOURCES) if j.wait() != 0]
+        if bad:
+            raise RuntimeError(f"nvcc failed on {', '.join(bad)}")
+        subprocess.check_call([nvcc(), *ARCH, "-shared", "-o", str(tmp), *map(str, objs)])
     os.replace(tmp, LIB)
     return LIB
 

@@ -22,9 +22,17 @@
 #include <type_traits>
 #include <vector>
 
-#include "kernels.cuh"
-#include "kernels3d.cuh"
-#include "kernels_general.cuh"
+#include "instances.cuh"
+
+namespace emu_dev {   // compiled in instances_<R>.cu
+EMU_ORDER_INSTANCES(extern, 0)
+EMU_ORDER_INSTANCES(extern, 1)
+EMU_ORDER_INSTANCES(extern, 2)
+EMU_ORDER_INSTANCES(extern, 3)
+EMU_RD_INSTANCES(extern, 0)
+EMU_RD_INSTANCES(extern, 1)
+EMU_RD_INSTANCES(extern, 2)
+}  // namespace emu_dev
 
 using namespace emu_dev;
 

@@ -431,7 +431,7 @@ __device__ __forceinline__ void commutator(double d12, double d13, double d23, d
 
 // Per-direction table from each ring's first particle: Omega and v_z = c Omega_z
 // ([4][MT]); also checks that every particle of a ring carries its direction.
-__global__ void k_dirtable(Batch B, Parts pt, double* __restrict__ dirtab, int* __restrict__ err) {
+static __global__ void k_dirtable(Batch B, Parts pt, double* __restrict__ dirtab, int* __restrict__ err) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= B.Ptot) return;
   const BoxGeo& g = B.box[box_of_particle(B, p)];
@@ -672,8 +672,8 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
   for (int q = 0; q < kGroups; ++q) ea[q] = 0;
   // direction d's particle data into buffer d & 1, asynchronously (each lane
   // its own particle's: no exchange between lanes): z, N, Nbar, rho, rhobar
-  auto fetch = [&](int d, int sh) -> int64_t {
-    int i = j - sh;
+  auto fetch = [&](int d) -> int64_t {
+    int i = j - ldi<COH>(shift + dbase + d);
     if (i < 0) i += nz;
     const int64_t p = g.poff + (int64_t)d * nz + i;
     double* dst = buf + (d & 1) * kDepRows * kLanes + lane;
@@ -688,24 +688,12 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
     cp_async_commit();
     return p;
   };
-  // a direction's own numbers, loaded a direction ahead: Omega in lanes 0-2,
-  // the ring's weights (when every particle takes them) in the next NW, v_z
-  const bool ring = ORDER > 0 && wrow != nullptr;
-  const double* utab = lane < 3 ? dirtab + lane * MT : wrow + (lane - 3) * MT;
-  const bool uload = lane < 3 || (ring && lane < 3 + NW);
-  auto own_number = [&](int gd) { return uload ? ldp<COH>(utab + gd) : 0.0; };
-  int64_t pnext = fetch(dfirst, ldi<COH>(shift + dbase + dfirst));
-  double unext = own_number(dbase + dfirst), vnext = __ldg(dirtab + 3 * MT + dbase + dfirst);
-  int shnext = dfirst + 1 < dlast ? ldi<COH>(shift + dbase + dfirst + 1) : 0;
+  int64_t pnext = fetch(dfirst);
   for (int d = dfirst; d < dlast; ++d) {
     const int gd = dbase + d;
     const int64_t p = pnext;
-    const double u = unext, vz = vnext;
     if (d + 1 < dlast) {
-      pnext = fetch(d + 1, shnext);
-      unext = own_number(gd + 1);
-      vnext = __ldg(dirtab + 3 * MT + gd + 1);
-      if (d + 2 < dlast) shnext = ldi<COH>(shift + gd + 2);
+      pnext = fetch(d + 1);
       cp_async_wait<1>();
     } else {
       cp_async_wait<0>();
@@ -714,10 +702,15 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
     auto rnu = [&](int k) { return x[(3 + k) * kLanes]; };
     auto rnb = [&](int k) { return x[(12 + k) * kLanes]; };
     const double n1 = x[kLanes], n2 = x[2 * kLanes];
-    const double zs = fma(pos_dt, vz, x[0]);
+    // Omega, and the ring's weights when every particle takes them: lane q
+    // converts one of them
+    double u = 0.0;
+    if (lane < 3) u = __ldg(dirtab + lane * MT + gd);
+    const double zs = fma(pos_dt, __ldg(dirtab + 3 * MT + gd), x[0]);
     w::Limbs wl[NW];   // the weight slot o of the particle that gives it to this lane's cell
     double wt[NW];
     if (wrow != nullptr) {
+      if (ORDER > 0 && lane >= 3 && lane < 3 + NW) u = ldp<COH>(wrow + (lane - 3) * MT + gd);
       bad |= off_site(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d));
     } else {
       bad |= shape_weights<ORDER>(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d), wt);
@@ -1068,7 +1061,7 @@ __device__ __forceinline__ void combine_phase(const Batch& B, const double* part
   if (bad) atomicOr(err, ERR_NONFINITE);
 }
 
-__global__ void k_combine(Batch B, const double* __restrict__ partial, double* __restrict__ out, int rows,
+static __global__ void k_combine(Batch B, const double* __restrict__ partial, double* __restrict__ out, int rows,
                           int potential, int split, int* __restrict__ err) {
   griddep_wait();
   combine_phase(B, partial, out, rows, potential, split, err);
@@ -1935,7 +1928,7 @@ __device__ __forceinline__ int box_of_tile32(const Batch& B, int64_t t) {
 // lane of a warp walks the same warps.  Split over warps and running sums as
 // in combine_phase.  The potential at a cell is the sum of the frame entries
 // that cover it (frame_sources).
-__global__ void k_frame_sum(Batch B, const double* __restrict__ partial, double* __restrict__ Fr, int64_t NT32,
+static __global__ void k_frame_sum(Batch B, const double* __restrict__ partial, double* __restrict__ Fr, int64_t NT32,
                             int split, int* __restrict__ err) {
   __shared__ double sums[kWarps][kLanes];
   griddep_wait();
@@ -2131,7 +2124,7 @@ __device__ __forceinline__ double uniform_pm1(uint64_t seed, int64_t p, int k) {
 // fused multiply-add) so the weights and states round like the formulas read.
 // Box-local particle numbers key the random draws.  species: per box, at
 // 8 * coff_b: n_nu[nz], n_nubar[nz], f_nu[3 nz], f_nubar[3 nz]; dirs[3 * MT].
-__global__ void k_init(Batch B, Parts pt, const double* __restrict__ species, const double* __restrict__ dirs,
+static __global__ void k_init(Batch B, Parts pt, const double* __restrict__ species, const double* __restrict__ dirs,
                        int* __restrict__ err) {
   const int64_t gp = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (gp >= B.Ptot) return;
@@ -2190,7 +2183,7 @@ __global__ void k_init(Batch B, Parts pt, const double* __restrict__ species, co
 
 // Per box: maximum over cells of the diagonal components of n and nbar (Eq. 7).
 // One block per box.
-__global__ void k_max_diag(Batch B, const double* __restrict__ mom, double* __restrict__ out) {
+static __global__ void k_max_diag(Batch B, const double* __restrict__ mom, double* __restrict__ out) {
   __shared__ double sm[kThreads];
   const BoxGeo& g = B.box[blockIdx.x];
   double m = 0.0;
@@ -2209,7 +2202,7 @@ __global__ void k_max_diag(Batch B, const double* __restrict__ mom, double* __re
 }
 
 // Eq. 7 per box from the maxima: dt_b = min(C dz / c, C_F / (kappa n_max)).
-__global__ void k_dt_from_max(Batch B, const double* __restrict__ nmax, double* __restrict__ dt_out) {
+static __global__ void k_dt_from_max(Batch B, const double* __restrict__ nmax, double* __restrict__ dt_out) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B.nbox) return;
   const BoxGeo& g = B.box[b];
@@ -2221,7 +2214,7 @@ __global__ void k_dt_from_max(Batch B, const double* __restrict__ nmax, double* 
 
 // Writes one box descriptor and step size from kernel parameters (used where
 // no host-to-device copy may be issued).
-__global__ void k_write_geo(BoxGeo g, double dt, BoxGeo* __restrict__ dst, double* __restrict__ dt_dst) {
+static __global__ void k_write_geo(BoxGeo g, double dt, BoxGeo* __restrict__ dst, double* __restrict__ dt_dst) {
   *dst = g;
   *dt_dst = dt;
 }
@@ -2238,7 +2231,7 @@ __device__ __forceinline__ double abs_entry(const double* __restrict__ m, int64_
   return sqrt(re * re + im * im);
 }
 
-__global__ void k_diagnostics(Batch B, const double* __restrict__ mom, double* __restrict__ out) {
+static __global__ void k_diagnostics(Batch B, const double* __restrict__ mom, double* __restrict__ out) {
   __shared__ double sm[kThreads];
   const BoxGeo& g = B.box[blockIdx.x];
   const int64_t NZ = B.NZ;
@@ -2537,7 +2530,7 @@ k_adj_seed(Batch B, Parts pt, const double* __restrict__ dirtab, const int* __re
 // Chain rule through Eq. 8, N_p = (n_c + 3 f_c . Omega_p) dV / M with c the
 // particle's initial cell: per cell (thread) and in direction order,
 // out[0] dL/dn_nu, out[1] dL/dn_nubar, out[2..4] dL/df_nu, out[5..7] dL/df_nubar ([8][NZ]).
-__global__ void k_weight_grad(Batch B, const double* __restrict__ gN, const double* __restrict__ gNbar,
+static __global__ void k_weight_grad(Batch B, const double* __restrict__ gN, const double* __restrict__ gNbar,
                               const double* __restrict__ dirtab, double* __restrict__ out) {
   const int gc = blockIdx.x * blockDim.x + threadIdx.x;
   if (gc >= B.NZ) return;

@@ -75,7 +75,7 @@ __device__ __forceinline__ double pick(const double (&w)[NW], int i) {
 
 // Direction table ([6][M]: Omega, then c Omega) from each direction's site-0
 // particle; every particle of a direction must carry its direction.
-__global__ void k3_dirtable(Box3 b, Parts pt, double* __restrict__ dirtab, int* __restrict__ err) {
+static __global__ void k3_dirtable(Box3 b, Parts pt, double* __restrict__ dirtab, int* __restrict__ err) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= b.P) return;
   const int d = (int)(p / b.C);
@@ -243,7 +243,7 @@ k3_deposit(Box3 b, const double* __restrict__ x, const double* __restrict__ y, c
 // stage (ERR_LATTICE) and writes the 8 traceless components of
 // B = N rho - Nbar rhobar^* (Eq. 5) at that cell of its direction's field:
 // Bf[c * P + d * C + cell].
-__global__ void __launch_bounds__(kThreads)
+static __global__ void __launch_bounds__(kThreads)
 k3_prep(Box3 b, const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
         const double* __restrict__ N, const double* __restrict__ Nbar, const double* __restrict__ r_nu,
         const double* __restrict__ r_nb, const double* __restrict__ dirtab, const int* __restrict__ srow,
@@ -381,7 +381,7 @@ k3_spread_x_sum(Box3 b, const double* __restrict__ in, const double* __restrict_
 // potential, once per stage: Gf[c][d][cell] (component c, M C values each).
 // The RK stage's interpolation reads the G of its neighbour rows instead of
 // forming it for each of the (2H+1)^2 rows that need it.
-__global__ void __launch_bounds__(kThreads)
+static __global__ void __launch_bounds__(kThreads)
 k3_gfield(Box3 b, const double* __restrict__ At, const double* __restrict__ dirtab, double* __restrict__ Gf) {
   griddep_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -537,7 +537,7 @@ k3_interpolate(Box3 b, const double* __restrict__ x, const double* __restrict__ 
 // Initial particles on the 3D lattice (Sec. 3.1, Eq. 8, 9; as k_init):
 // particle p = d C + c0 at the centre of cell c0.  species: n_nu[C],
 // n_nubar[C], f_nu[3C], f_nubar[3C]; dirs[3M] (with use_dirs).
-__global__ void k3_init(Box3 b, Parts pt, double* __restrict__ x, double* __restrict__ y,
+static __global__ void k3_init(Box3 b, Parts pt, double* __restrict__ x, double* __restrict__ y,
                         const double* __restrict__ species, const double* __restrict__ dirs, int* __restrict__ err) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= b.P) return;

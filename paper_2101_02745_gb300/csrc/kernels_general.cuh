@@ -32,7 +32,7 @@ constexpr int kRadixTile = kThreads * kRadixItems;   // items per block
 
 // Containing cell (global index) of every particle at z + frac dt_b c Omega_z;
 // ids[p] = p.  Non-finite positions are an error (key 0).
-__global__ void k_gkeys(Batch B, const double* __restrict__ z, const double* __restrict__ oz, double frac,
+static __global__ void k_gkeys(Batch B, const double* __restrict__ z, const double* __restrict__ oz, double frac,
                         unsigned* __restrict__ keys, int* __restrict__ ids, int* __restrict__ err) {
   griddep_wait();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -48,7 +48,7 @@ __global__ void k_gkeys(Batch B, const double* __restrict__ z, const double* __r
 }
 
 // Radix sort, pass histogram: hist[d * nblk + block] = count of digit d in the block's tile.
-__global__ void k_radix_hist(const unsigned* __restrict__ keys, int64_t n, int shift, int* __restrict__ hist,
+static __global__ void k_radix_hist(const unsigned* __restrict__ keys, int64_t n, int shift, int* __restrict__ hist,
                              int nblk) {
   __shared__ int cnt[kRadixBuckets];
   if (threadIdx.x < kRadixBuckets) cnt[threadIdx.x] = 0;
@@ -63,7 +63,7 @@ __global__ void k_radix_hist(const unsigned* __restrict__ keys, int64_t n, int s
 
 // Exclusive scan of v[0, n) in place by one block of kThreads threads (each
 // takes a contiguous chunk; the chunk sums are scanned in shared memory).
-__global__ void k_scan_exclusive(int* __restrict__ v, int64_t n) {
+static __global__ void k_scan_exclusive(int* __restrict__ v, int64_t n) {
   __shared__ int64_t part[kThreads];
   const int64_t chunk = (n + kThreads - 1) / kThreads;
   const int64_t lo = min(n, (int64_t)threadIdx.x * chunk), hi = min(n, lo + chunk);
@@ -87,7 +87,7 @@ __global__ void k_scan_exclusive(int* __restrict__ v, int64_t n) {
 
 // Radix sort, pass scatter: stable ranks within the block (a thread's items in
 // index order, threads in order), offsets from the scanned histogram.
-__global__ void k_radix_scatter(const unsigned* __restrict__ keys, const int* __restrict__ vals, int64_t n,
+static __global__ void k_radix_scatter(const unsigned* __restrict__ keys, const int* __restrict__ vals, int64_t n,
                                 int shift, const int* __restrict__ offs, int nblk, unsigned* __restrict__ keys_out,
                                 int* __restrict__ vals_out) {
   __shared__ int cnt[kRadixBuckets][kThreads];
@@ -146,7 +146,7 @@ __global__ void k_radix_scatter(const unsigned* __restrict__ keys, const int* __
 
 // start[c] = first index of sorted key c (start[NZ] = n): a cell without
 // particles starts where the next non-empty one does.
-__global__ void k_cell_start(const unsigned* __restrict__ keys, int64_t n, int NZ, int* __restrict__ start) {
+static __global__ void k_cell_start(const unsigned* __restrict__ keys, int64_t n, int NZ, int* __restrict__ start) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i > n) return;
   const int lo = i == 0 ? -1 : (int)keys[i - 1];
@@ -464,7 +464,7 @@ __global__ void k_ginterpolate(Batch B, Parts pt, const double* __restrict__ A, 
 // Lattice contract check (the lattice path's precondition): every particle of
 // a ring carries the ring's direction and sits in the cell its ring index
 // assigns (within the lattice tolerance).  Sets *bad_out to 1 otherwise.
-__global__ void k_lattice_check(Batch B, Parts pt, int* __restrict__ bad_out) {
+static __global__ void k_lattice_check(Batch B, Parts pt, int* __restrict__ bad_out) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= B.Ptot) return;
   const BoxGeo& g = B.box[box_of_particle(B, p)];

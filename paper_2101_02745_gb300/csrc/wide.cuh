@@ -176,8 +176,8 @@ EMU_HD Cplx cplx(double re, double im) {
 // literals the compiler turns them into 64-bit adds and shifts (mul 8 instead of
 // 4 instructions, mul2 12 instead of 7).
 #ifdef __CUDACC__
-__constant__ int64_t c_half = (int64_t)1 << 31;
-__constant__ int c_two = 2;
+static __constant__ int64_t c_half = (int64_t)1 << 31;
+static __constant__ int c_two = 2;
 #endif
 EMU_HD int64_t half_unit() {
 #ifdef __CUDA_ARCH__
