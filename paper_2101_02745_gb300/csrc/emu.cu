@@ -305,12 +305,24 @@ int cuda_check(emu_box* b, cudaError_t e, const char* what) {
   return fail(b, EMU_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
-// Whether the RK stage's blocks take slabs of several tiles (rings read in
-// pieces of up to 2 KB) or single tiles: slabs when the batch has at least 16
-// 32-cell units per block of the default grid, unless a form was chosen; below
-// that single tiles spread the few units over all SMs.
+// Whether the RK stage's blocks take ranges of slabs (several tiles, rings read
+// in pieces of up to 2 KB) or parts of single tiles: slabs when the batch has
+// at least 16 32-cell units per block of the default grid or more tiles than
+// blocks, unless a form was chosen; parts spread few units evenly.
 int use_slabs(const emu_box* b) {
-  return b->rk_form >= 0 ? b->rk_form : b->S.U32 >= 16 * (int64_t)kPersistBlocks;
+  return b->rk_form >= 0 ? b->rk_form : b->S.U32 >= 16 * (int64_t)kPersistBlocks || b->S.NT32 > b->blocks;
+}
+
+// Directions of a block's part of a tile: the fewest that leave no more parts
+// than blocks (all of a tile's directions when the tiles alone are more).
+int part_directions(const emu_box* b) {
+  int64_t upb = (b->S.U32 + b->blocks - 1) / b->blocks;
+  for (; upb < b->S.Mmax; ++upb) {
+    int64_t parts = 0;
+    for (const BoxGeo& g : b->S.geo) parts += (int64_t)g.ntiles32 * ((g.M + upb - 1) / upb);
+    if (parts <= b->blocks) break;
+  }
+  return (int)(upb < 1 ? 1 : upb);
 }
 
 Batch batch_view(const emu_box* b) {
@@ -329,7 +341,8 @@ Batch batch_view(const emu_box* b) {
   B.nw32 = (int)(b->S.U32 < nw ? b->S.U32 : nw);
   B.Ptot = b->S.Ptot;
   B.slabs = use_slabs(b);
-  B.US = B.slabs ? b->S.US : b->S.U32;
+  B.US = b->S.US;
+  B.upb = B.slabs ? 0 : part_directions(b);
   return B;
 }
 
@@ -708,7 +721,7 @@ int launch_deposit(emu_box* b, int mode, const double* rnu, const double* rnb, c
         static std::atomic<unsigned> done{0};
         auto k = k_deposit<5, R, decltype(TAB)::value>;
         if (raise_smem(k, kDepSmem, done) == cudaSuccess)
-          pdl_smem(st, k, grid, kDepSmem, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, W,
+          pdl_smem(st, k, grid, B.U > B.nw ? kDepSmem : kDepSmem / 2, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, W,
                    b->err);
       };
       if (wrow != nullptr) step(std::true_type{});
@@ -828,11 +841,16 @@ int launch_rk_on(emu_box* b, int s, const int* srow, int dry, const Parts& pt, c
     constexpr int R = decltype(O)::value;
     const Batch Bv = batch_view(b);
     const double* wrow = weight_row(b, srow);
-    auto launch = [&](auto POT, auto STAGE) {
+    auto launch_tiles = [&](auto POT, auto STAGE, auto TILES) {
       static std::atomic<unsigned> done{0};
-      auto k = k_rk_stage<decltype(POT)::value, R, decltype(STAGE)::value>;
-      if (raise_smem(k, kSlabSmem, done) == cudaSuccess)
-        pdl_smem(b->stream, k, persist_grid(b), kSlabSmem, Bv, pt, W, wrow, b->dirtab, srow, At, stage_src, s, dry);
+      constexpr int T = decltype(TILES)::value, smem = (int)sizeof(SlabTable<T>);
+      auto k = k_rk_stage<decltype(POT)::value, R, decltype(STAGE)::value, T>;
+      if (raise_smem(k, smem, done) == cudaSuccess)
+        pdl_smem(b->stream, k, persist_grid(b), smem, Bv, pt, W, wrow, b->dirtab, srow, At, stage_src, s, dry);
+    };
+    auto launch = [&](auto POT, auto STAGE) {
+      if (Bv.slabs) launch_tiles(POT, STAGE, std::integral_constant<int, kSlabTiles>{});
+      else launch_tiles(POT, STAGE, std::integral_constant<int, 1>{});
     };
     auto stage = [&](auto POT) {
       if (s == 1) launch(POT, std::integral_constant<int, 1>{});

@@ -7,9 +7,10 @@
 #include "kernels3d.cuh"
 #include "kernels_general.cuh"
 
-#define EMU_RK_STAGE(X, POT, R, S)                                                                                  \
-  X template __global__ void k_rk_stage<POT, R, S>(Batch, Parts, const double*, const double*, const double*,       \
-                                                   const int*, const double*, const double*, int, int);
+#define EMU_RK_STAGE(X, POT, R, S, TILES)                                                                           \
+  X template __global__ void k_rk_stage<POT, R, S, TILES>(Batch, Parts, const double*, const double*,               \
+                                                          const double*, const int*, const double*, const double*,  \
+                                                          int, int);
 #define EMU_RK_DEPOSIT(X, POT, R, S)                                                                                \
   X template __global__ void k_rk_deposit<POT, R, S>(Batch, Parts, double*, const double*, const int*,              \
                                                      const double*, int, double*, int*);
@@ -22,9 +23,12 @@
                                                            const double*, const double*, const double*, const int*, \
                                                            const double*, double, double*, double*, int*);
 #define EMU_POT_INSTANCES(X, POT, R)                                                                                \
-  EMU_RK_STAGE(X, POT, R, 1)                                                                                        \
-  EMU_RK_STAGE(X, POT, R, 2)                                                                                        \
-  EMU_RK_STAGE(X, POT, R, 4)                                                                                        \
+  EMU_RK_STAGE(X, POT, R, 1, 1)                                                                                     \
+  EMU_RK_STAGE(X, POT, R, 2, 1)                                                                                     \
+  EMU_RK_STAGE(X, POT, R, 4, 1)                                                                                     \
+  EMU_RK_STAGE(X, POT, R, 1, kSlabTiles)                                                                            \
+  EMU_RK_STAGE(X, POT, R, 2, kSlabTiles)                                                                            \
+  EMU_RK_STAGE(X, POT, R, 4, kSlabTiles)                                                                            \
   X template __global__ void k_step<POT, R>(Batch, Parts, StepArgs);                                                \
   X template __global__ void k3_rk_stage<POT, R>(Box3, Parts, double*, double*, const double*, const int*,          \
                                                  const double*, const double*, int, int);                           \

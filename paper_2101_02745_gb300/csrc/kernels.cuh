@@ -110,7 +110,8 @@ struct Batch {
   int64_t U32;         // total 32-cell units of the RK stage (shape orders 0-2)
   int nw32;            // warps that split them
   int64_t US;          // total tile units of the RK stage's slabs
-  int slabs;           // its slabs: 1 = BoxGeo::sw tiles, 0 = one tile
+  int slabs;           // its work split: 1 = ranges of slabs, 0 = parts of one tile
+  int upb;             // directions of a part (slabs 0)
 };
 
 struct Parts {
@@ -643,14 +644,15 @@ constexpr int kDepSmem = kWarps * kDepBuf * (int)sizeof(double);              //
 // bits of headroom, so a contribution keeps 61 - ceil(log2 n) bits below the
 // largest one's leading bit: less error than FP64 sums of n terms, whose
 // rounding follows the partial sums.  Zero contributions add exactly nothing.
-// (buf: this warp's two buffers of kDepRows x 32 doubles in shared memory.)
+// (buf: this warp's two buffers of kDepRows x 32 doubles in shared memory;
+// ring2 0: only one, when no warp takes more than one direction of a tile.)
 template <int ORDER, bool COH>
 __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int tile, int dfirst, int dlast, int lane,
                                                   const double* z, const double* __restrict__ N,
                                                   const double* __restrict__ Nbar, const double* r_nu,
                                                   const double* r_nb, const double* __restrict__ dirtab,
                                                   const int* shift, const double* wrow, double frac, double* W,
-                                                  double* buf, double (&out)[kNT], int& bad) {
+                                                  double* buf, int ring2, double (&out)[kNT], int& bad) {
   namespace w = emu_wide;
   constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T, NW = Sten<ORDER>::NW, kGroups = 5;
   const BoxGeo& g = B.box[b];
@@ -676,7 +678,7 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
     int i = j - ldi<COH>(shift + dbase + d);
     if (i < 0) i += nz;
     const int64_t p = g.poff + (int64_t)d * nz + i;
-    double* dst = buf + (d & 1) * kDepRows * kLanes + lane;
+    double* dst = buf + (d & ring2) * kDepRows * kLanes + lane;
     cp_async8(dst, z + p);
     cp_async8(dst + kLanes, N + p);
     cp_async8(dst + 2 * kLanes, Nbar + p);
@@ -692,13 +694,13 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
   for (int d = dfirst; d < dlast; ++d) {
     const int gd = dbase + d;
     const int64_t p = pnext;
-    if (d + 1 < dlast) {
+    if (d + 1 < dlast && ring2) {
       pnext = fetch(d + 1);
       cp_async_wait<1>();
     } else {
       cp_async_wait<0>();
     }
-    const double* x = buf + (d & 1) * kDepRows * kLanes + lane;
+    const double* x = buf + (d & ring2) * kDepRows * kLanes + lane;
     auto rnu = [&](int k) { return x[(3 + k) * kLanes]; };
     auto rnb = [&](int k) { return x[(12 + k) * kLanes]; };
     const double n1 = x[kLanes], n2 = x[2 * kLanes];
@@ -862,7 +864,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
     for (int c = 0; c < NA; ++c) acc[c] = 0.0;
     if constexpr (MODE == 5)
       deposit_tile_wide<ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow, frac,
-                                    W, buf, acc, bad);
+                                    W, buf, B.U > B.nw, acc, bad);
     else
       deposit_tile_dirs<MODE, ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow,
                                           frac, W, acc, bad);
@@ -883,7 +885,7 @@ k_deposit(Batch B, const double* __restrict__ z, const double* __restrict__ N, c
   extern __shared__ double dep_sm[];   // (MODE 5: kDepSmem bytes)
   griddep_wait();
   deposit_phase<MODE, ORDER, false>(B, logical_warp(), threadIdx.x & 31, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                    TAB ? wrow : nullptr, frac, partial, W, err, dep_sm + (threadIdx.x >> 5) * kDepBuf);
+                                    TAB ? wrow : nullptr, frac, partial, W, err, dep_sm + (threadIdx.x >> 5) * (B.U > B.nw ? kDepBuf : kDepBuf / 2));
 }
 
 // ------------------------------------------------------- cluster deposit
@@ -967,7 +969,7 @@ k_deposit_cluster(Batch B, const double* __restrict__ z, const double* __restric
     for (int c = 0; c < kNT; ++c) acc[c] = 0.0;
     if (d0 < d1)
       deposit_tile_wide<ORDER, false>(B, b, tile, d0, d1, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                      TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, acc, bad);
+                                      TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, 1, acc, bad);
 #pragma unroll
     for (int c = 0; c < kNT; ++c) red[wib * kDepBuf + c * kLanes + lane] = acc[c];
     __syncthreads();
@@ -1266,14 +1268,13 @@ __device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, co
   }
 }
 
-// Tiles before box g's first slab, and the box of tile unit x (a pair of a
-// slab and a direction counts as its sw tile units).
-__device__ __forceinline__ int64_t slab_offset(const Batch& B, const BoxGeo& g) { return B.slabs ? g.soff : g.uoff32; }
+// Box of tile unit x of the slabs (a pair of a slab and a direction counts as
+// its sw tile units).
 __device__ __forceinline__ int box_of_slab_unit(const Batch& B, int64_t x) {
   int lo = 0, hi = B.nbox - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (slab_offset(B, B.box[mid]) <= x) lo = mid; else hi = mid - 1;
+    if (B.box[mid].soff <= x) lo = mid; else hi = mid - 1;
   }
   return lo;
 }
@@ -1290,9 +1291,13 @@ __device__ __forceinline__ int box_of_slab_unit(const Batch& B, int64_t x) {
 // their state from stage_src (normally the stage buffer itself, updated in
 // place; a separate buffer when the stage states are kept for the adjoint).
 //
-// Work split.  A block takes a contiguous range of (slab, direction) pairs of
-// the batch (an equal share of their tile units), slab by slab; a slab is 1, 2, 4 or 8 (BoxGeo::sw; Batch::slabs 0:
-// 1) consecutive 32-cell tiles.  It converts the slab's potential once to integer operands
+// Work split.  Batch::slabs 1: a block takes a contiguous range of (slab,
+// direction) pairs of the batch (an equal share of their tile units), slab by
+// slab; a slab is 1, 2, 4 or 8 (BoxGeo::sw) consecutive 32-cell tiles.  Batch::
+// slabs 0 (few units): a block takes a part of one tile's directions (at most
+// upb), so that no block does two tiles one after the other while others idle
+// (256 x 96: 3 units a block on 256 blocks).  The block converts the slab's (tile's)
+// potential once to integer operands
 // in shared memory (per cell and moment the 8 traceless components, one
 // exponent per cell for the diagonal pair and for each complex component),
 // and its warps walk the slab's directions: with sw tiles, warp i takes tile
@@ -1302,21 +1307,22 @@ __device__ __forceinline__ int box_of_slab_unit(const Batch& B, int64_t x) {
 // shared memory, and the stencil sum is the commutator's operand: everything
 // up to the update runs on the integer pipe.
 constexpr int kSlabTiles = 8;                      // most tiles of a slab
-constexpr int kSlabCells = kSlabTiles * kLanes + 4;   // cells of the widest slab, two neighbours a side
 constexpr int kRowCells = kLanes + 4;              // cells of a unit, likewise
+template <int TILES>                               // of the widest slab
 struct SlabTable {
+  static constexpr int kSlabCells = TILES * kLanes + 4;   // its cells, two neighbours a side
   int2 a[kNT][kSlabCells];                         // the potential: A0 / 4 as int64, limbs of A_x, A_y, A_z
   int e[4][kSlabCells];                            // exponents: diagonal pair, three complex components
   int2 g[kWarps][kNC][kRowCells];                  // limbs of G of each warp's unit
   const double* pf[64];                            // the arrays a stage reads, for the L2 prefetch
 };
-constexpr int kSlabSmem = (int)sizeof(SlabTable);
+constexpr int kSlabSmem = (int)sizeof(SlabTable<kSlabTiles>);
 constexpr int kStepSmem = kSlabSmem > kDepSmem ? kSlabSmem : kDepSmem;   // of k_step: either phase's
 
 // Potential of cells c0 .. c0 + n - 1 (modulo nz) of box g into the table, by
 // the whole block: one (cell, exponent group) per thread and round.
-template <bool COH>
-__device__ __forceinline__ void slab_table(SlabTable& t, const double* A, int NZ, const BoxGeo& g, int c0, int n) {
+template <bool COH, class Table>
+__device__ __forceinline__ void slab_table(Table& t, const double* A, int NZ, const BoxGeo& g, int c0, int n) {
   namespace w = emu_wide;
   for (int q = threadIdx.x; q < 4 * n; q += kThreads) {
     const int grp = q / n, c = q - grp * n;
@@ -1347,7 +1353,8 @@ __device__ __forceinline__ emu_wide::Limbs limbs_of(int2 v) { return emu_wide::L
 
 // Component c of G = A0 - Omega . A at table cell j (o: limbs of -Omega).
 // Directions scaled by 2^-ko: so is G.
-__device__ __forceinline__ int2 table_G(const SlabTable& t, int c, int j, const emu_wide::Limbs (&o)[3], int ko) {
+template <class Table>
+__device__ __forceinline__ int2 table_G(const Table& t, int c, int j, const emu_wide::Limbs (&o)[3], int ko) {
   const int2 q = t.a[c][j];
   const int64_t a0 = (int64_t)(((uint64_t)(uint32_t)q.y << 32) | (uint32_t)q.x);
   const emu_wide::Limbs g = emu_wide::split(
@@ -1356,10 +1363,10 @@ __device__ __forceinline__ int2 table_G(const SlabTable& t, int c, int j, const 
   return make_int2(g.h, g.l);
 }
 
-template <bool POT, int ORDER, int S, bool COH>
+template <bool POT, int ORDER, int S, bool COH, class Table>
 __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const double* W, const double* wrow,
                                          const double* __restrict__ dirtab, const int* shift, const double* A,
-                                         const double* stage_src, int s, int dry, SlabTable& t) {
+                                         const double* stage_src, int s, int dry, Table& t) {
   namespace w = emu_wide;
   constexpr int H = ORDER == 0 ? 0 : Sten<ORDER>::H, NW = ORDER == 0 ? 1 : Sten<ORDER>::NW;
   constexpr int NWS = Sten<ORDER>::NWS;
@@ -1384,28 +1391,49 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
     else arr = W + (a - 18 - nacc - ny - nz_) * P;
     t.pf[a] = arr;
   }
-  // this block's tile units [x, x1); a (slab, direction) pair belongs to the
-  // block its first unit falls to
+  // slabs: this block's tile units [x, x1), a (slab, direction) pair belonging
+  // to the block its first unit falls to; otherwise its parts part, part + grid, ..
   int64_t x = (int64_t)blockIdx.x * B.US / gridDim.x;
   const int64_t x1 = ((int64_t)blockIdx.x + 1) * B.US / gridDim.x;
-  if (x >= x1) return;
-  int b = box_of_slab_unit(B, x);
-  while (x < x1 && b < B.nbox) {
-    const BoxGeo* gp = &B.box[b];
-    const int nz = gp->nz, M = gp->M, sw = B.slabs ? gp->sw : 1;
-    const int nslab = (gp->ntiles32 + sw - 1) / sw;
-    const int64_t off = slab_offset(B, *gp);
-    const int64_t q = (x - off + sw - 1) / sw;                            // first pair, box-local
-    const int64_t q1 = min((int64_t)nslab * M, (x1 - off + sw - 1) / sw);   // and the end of this block's
-    if (q >= q1) {   // (the box's pairs left start in later blocks, or it has none left)
-      x = off + (int64_t)nslab * M * sw;
-      ++b;
-      continue;
+  int64_t part = blockIdx.x;
+  int b = B.slabs && x < x1 ? box_of_slab_unit(B, x) : 0;
+  while (true) {
+    int slab, d0, d1, sw = 1;
+    if (B.slabs) {
+      if (x >= x1 || b >= B.nbox) break;
+      const BoxGeo& g = B.box[b];
+      const int M = g.M;
+      sw = g.sw;
+      const int nslab = (g.ntiles32 + sw - 1) / sw;
+      const int64_t q = (x - g.soff + sw - 1) / sw;                             // first pair, box-local
+      const int64_t q1 = min((int64_t)nslab * M, (x1 - g.soff + sw - 1) / sw);   // and the end of this block's
+      if (q >= q1) {   // (the box's pairs left start in later blocks, or it has none left)
+        x = g.soff + (int64_t)nslab * M * sw;
+        ++b;
+        continue;
+      }
+      slab = (int)(q / M);
+      d0 = (int)(q - (int64_t)slab * M);
+      d1 = (int)min((int64_t)M, (int64_t)d0 + (q1 - q));
+      x = g.soff + (q + (d1 - d0)) * sw;
+    } else {
+      int64_t k = part;
+      int per = 0;
+      for (b = 0; b < B.nbox; ++b) {
+        per = (B.box[b].M + B.upb - 1) / B.upb;   // parts of a tile
+        const int64_t all = (int64_t)per * B.box[b].ntiles32;
+        if (k < all) break;
+        k -= all;
+      }
+      if (b == B.nbox) break;
+      part += gridDim.x;
+      slab = (int)(k / per);
+      const int i = (int)(k - (int64_t)slab * per), M = B.box[b].M;
+      d0 = (int)((int64_t)i * M / per);
+      d1 = (int)((int64_t)(i + 1) * M / per);
     }
-    const int slab = (int)(q / M), d0 = (int)(q - (int64_t)slab * M);
-    const int d1 = (int)min((int64_t)M, (int64_t)d0 + (q1 - q));
-    x = off + (q + (d1 - d0)) * sw;
-    const BoxGeo& g = *gp;
+    const BoxGeo& g = B.box[b];
+    const int nz = g.nz;
     const int c0 = slab * sw * kLanes;
     __syncthreads();   // (the previous slab's table is free, and pf is written)
     slab_table<COH>(t, A, B.NZ, g, c0 - H, min(sw * kLanes, nz - c0) + 2 * H);
@@ -1551,14 +1579,16 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
   }
 }
 
-template <bool POT, int ORDER, int S>
+// TILES: of the widest slab (kSlabTiles, or 1 when Batch::slabs is 0: the
+// smaller table leaves the SM room for the next kernel's blocks).
+template <bool POT, int ORDER, int S, int TILES>
 __global__ void __launch_bounds__(kThreads, 2)
 k_rk_stage(Batch B, Parts pt, const double* __restrict__ W, const double* __restrict__ wrow,
            const double* __restrict__ dirtab, const int* __restrict__ shift, const double* __restrict__ A,
            const double* stage_src, int s, int dry) {
   extern __shared__ char smem[];
   griddep_wait();
-  rk_phase<POT, ORDER, S, false>(B, pt, W, wrow, dirtab, shift, A, stage_src, s, dry, *(SlabTable*)smem);
+  rk_phase<POT, ORDER, S, false>(B, pt, W, wrow, dirtab, shift, A, stage_src, s, dry, *(SlabTable<TILES>*)smem);
 }
 
 // ------------------------------------------- RK stage with the next deposit
@@ -2065,7 +2095,7 @@ __device__ __forceinline__ void fused_combine(const Batch& B, const StepArgs& a)
 
 template <bool POT, int ORDER>
 __device__ __forceinline__ void fused_rk(const Batch& B, const Parts& pt, const StepArgs& a, const int* srow,
-                                         const double* wrow, int s, SlabTable& t) {
+                                         const double* wrow, int s, SlabTable<kSlabTiles>& t) {
   if (s == 1) rk_phase<POT, ORDER, 1, true>(B, pt, a.W, wrow, a.dirtab, srow, a.At, pt.stage, s, a.dry, t);
   else if (s == 4) rk_phase<POT, ORDER, 4, true>(B, pt, a.W, wrow, a.dirtab, srow, a.At, pt.stage, s, a.dry, t);
   else rk_phase<POT, ORDER, 2, true>(B, pt, a.W, wrow, a.dirtab, srow, a.At, pt.stage, s, a.dry, t);
@@ -2099,7 +2129,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_step(Batch B, Parts pt, StepArg
       if (grid_barrier(a.bar, a.limit_ns, a.err)) return;
       fused_combine(B, a);
       if (grid_barrier(a.bar, a.limit_ns, a.err)) return;
-      fused_rk<POT, ORDER>(B, pt, a, srow, wrow, s, *(SlabTable*)smem);
+      fused_rk<POT, ORDER>(B, pt, a, srow, wrow, s, *(SlabTable<kSlabTiles>*)smem);
       if (grid_barrier(a.bar, a.limit_ns, a.err)) return;
     }
   }
