@@ -71,6 +71,19 @@ int by_order(int order, F&& f) {
   }
 }
 
+// Calls f(vacuum and matter terms, stage) with the constants the RK stage
+// kernels are instantiated for (stage 2 stands for 2 and 3).
+template <typename F>
+void by_stage(bool pot, int s, F&& f) {
+  auto stage = [&](auto POT) {
+    if (s == 1) f(POT, std::integral_constant<int, 1>{});
+    else if (s == 4) f(POT, std::integral_constant<int, 4>{});
+    else f(POT, std::integral_constant<int, 2>{});
+  };
+  if (pot) stage(std::true_type{});
+  else stage(std::false_type{});
+}
+
 const char* config_problem(const emu_config* c) {
   if (!c) return "config is NULL";
   if (c->nz < 1) return "nz must be >= 1";
@@ -848,17 +861,10 @@ int launch_rk_on(emu_box* b, int s, const int* srow, int dry, const Parts& pt, c
       if (raise_smem(k, smem, done) == cudaSuccess)
         pdl_smem(b->stream, k, persist_grid(b), smem, Bv, pt, W, wrow, b->dirtab, srow, At, stage_src, s, dry);
     };
-    auto launch = [&](auto POT, auto STAGE) {
+    by_stage(b->pot, s, [&](auto POT, auto STAGE) {
       if (Bv.slabs) launch_tiles(POT, STAGE, std::integral_constant<int, kSlabTiles>{});
       else launch_tiles(POT, STAGE, std::integral_constant<int, 1>{});
-    };
-    auto stage = [&](auto POT) {
-      if (s == 1) launch(POT, std::integral_constant<int, 1>{});
-      else if (s == 4) launch(POT, std::integral_constant<int, 4>{});
-      else launch(POT, std::integral_constant<int, 2>{});
-    };
-    if (b->pot) stage(std::true_type{});
-    else stage(std::false_type{});
+    });
     return 0;
   });
   return after_launch(b, "RK stage kernel");
@@ -1333,12 +1339,10 @@ int launch3_rk(emu_box* b, int s, const int* srow, int dry) {
   before_launch(b, CLS_RK);
   by_order(b->S.order, [&](auto O) {
     constexpr int R = decltype(O)::value;
-    if (b->pot)
-      pdl(b->stream, k3_rk_stage<true, R>, persist_grid(b), v, b->pt, b->x3, b->y3, b->dirtab, srow,
-          (const double*)F1, wrow, s, dry);
-    else
-      pdl(b->stream, k3_rk_stage<false, R>, persist_grid(b), v, b->pt, b->x3, b->y3, b->dirtab, srow,
-          (const double*)F1, wrow, s, dry);
+    by_stage(b->pot, s, [&](auto POT, auto STAGE) {
+      pdl(b->stream, k3_rk_stage<decltype(POT)::value, R, decltype(STAGE)::value>, persist_grid(b), v, b->pt, b->x3,
+          b->y3, b->dirtab, srow, (const double*)F1, wrow, s, dry);
+    });
     return 0;
   });
   return after_launch(b, "3D RK stage kernel");
@@ -1508,8 +1512,10 @@ int launch_gstage(emu_box* b, int s, int dry) {
   by_order(b->S.order, [&](auto O) {
     constexpr int R = decltype(O)::value;
     const dim3 grid((unsigned)((P + kThreads - 1) / kThreads));
-    if (b->pot) pdl(b->stream, k_grk_stage<true, R>, grid, batch_view(b), b->pt, (const double*)b->At, s, dry);
-    else pdl(b->stream, k_grk_stage<false, R>, grid, batch_view(b), b->pt, (const double*)b->At, s, dry);
+    by_stage(b->pot, s, [&](auto POT, auto STAGE) {
+      pdl(b->stream, k_grk_stage<decltype(POT)::value, R, decltype(STAGE)::value>, grid, batch_view(b), b->pt,
+          (const double*)b->At, s, dry);
+    });
     return 0;
   });
   return after_launch(b, "RK stage kernel (particles anywhere)");

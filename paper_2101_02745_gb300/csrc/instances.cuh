@@ -11,6 +11,10 @@
   X template __global__ void k_rk_stage<POT, R, S, TILES>(Batch, Parts, const double*, const double*,               \
                                                           const double*, const int*, const double*, const double*,  \
                                                           int, int);
+#define EMU_RK_OTHER(X, POT, R, S)                                                                                  \
+  X template __global__ void k3_rk_stage<POT, R, S>(Box3, Parts, double*, double*, const double*, const int*,       \
+                                                    const double*, const double*, int, int);                        \
+  X template __global__ void k_grk_stage<POT, R, S>(Batch, Parts, const double*, int, int);
 #define EMU_RK_DEPOSIT(X, POT, R, S)                                                                                \
   X template __global__ void k_rk_deposit<POT, R, S>(Batch, Parts, double*, const double*, const int*,              \
                                                      const double*, int, double*, int*);
@@ -30,9 +34,9 @@
   EMU_RK_STAGE(X, POT, R, 2, kSlabTiles)                                                                            \
   EMU_RK_STAGE(X, POT, R, 4, kSlabTiles)                                                                            \
   X template __global__ void k_step<POT, R>(Batch, Parts, StepArgs);                                                \
-  X template __global__ void k3_rk_stage<POT, R>(Box3, Parts, double*, double*, const double*, const int*,          \
-                                                 const double*, const double*, int, int);                           \
-  X template __global__ void k_grk_stage<POT, R>(Batch, Parts, const double*, int, int);
+  EMU_RK_OTHER(X, POT, R, 1)                                                                                        \
+  EMU_RK_OTHER(X, POT, R, 2)                                                                                        \
+  EMU_RK_OTHER(X, POT, R, 4)
 #define EMU_ORDER_INSTANCES(X, R)                                                                                   \
   EMU_POT_INSTANCES(X, false, R)                                                                                    \
   EMU_POT_INSTANCES(X, true, R)                                                                                     \

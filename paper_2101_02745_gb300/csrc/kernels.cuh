@@ -1116,108 +1116,97 @@ k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ 
 // Eq. 2; OWNBAR: hb of Hbar, otherwise Hbar = -H^*) and the neutrino source
 // matrix r (already loaded; the antineutrinos' source is src_b), then the
 // accumulator and next stage state (stage 4: the new state and position, from
-// *vz).  S is the stage as a template parameter (2 stands for 2 and 3), or 0
-// for the run-time s.  With KEEP the state it stores (the next stage's, or at
+// *vz).  S is the stage (2 stands for 2 and 3).  With KEEP the state it stores (the next stage's, or at
 // stage 4 the new one), rho and rhobar, is also combined as
 // B = n1 rho - n2 rhobar^* into keep[9] (the arithmetic of the deposit, Eq. 5)
 // and the new position returned in *zkeep.
 // The commutators run on the integer pipe (wide.cuh), the updates as FP64
 // multiply-adds: 36 + 31 FP64 instructions a particle instead of 144 (at
 // 16 cycles each the FP64 pipe bound the stage).
+template <int N>
+struct Int {
+  static constexpr int value = N;
+};
+
 template <int S, bool OWNBAR, bool COH, bool KEEP = false>
 __device__ __forceinline__ void rk_update(double Lz, const Parts& pt, const double* src_b, int64_t P_, int64_t p,
-                                          int s, int dry, double bdt, double cdt, double dtb,
+                                          int dry, double bdt, double cdt, double dtb,
                                           const double* vz, const emu_wide::Ham& hm, const emu_wide::Ham& hb,
                                           double (&r)[9], double* keep = nullptr, double* zkeep = nullptr,
                                           double n1 = 0.0, double n2 = 0.0) {
   namespace w = emu_wide;
   const unsigned P = (unsigned)P_;
-  const bool first = S == 0 ? s == 1 : S == 1, last = S == 0 ? s == 4 : S == 4;
+  static_assert(S == 1 || S == 2 || S == 4, "stage 1, 2 (and 3) or 4");
+  constexpr bool first = S == 1, last = S == 4;
   // Sums of products have an exponent of at least emin, so that the
   // coefficients that take it (below) stay normal; infinite and NaN inputs
-  // raise it to kInfExp, and the coefficients, held at the infinities'
-  // exponent field, then make every result infinite or NaN
+  // raise it to kInfExp, and the coefficients, out of range, then make every
+  // result NaN
   constexpr int kInfExp = 1 << 16;
-  const int bmax = 2047 - w::exponent(bdt), cmax = 2047 - w::exponent(cdt);
-  const int emin = w::kBiasP - 2046 + w::max_i(bmax, cmax);
+  const int emin0 = w::kBiasP + 1 - w::min_i(w::exponent(bdt), w::exponent(cdt));
   const int htop = w::top(hm);
   // one pass per species: a loop, not unrolled (the commutator's ~600
   // instructions once keep the stage in the instruction cache)
 #pragma unroll 1
   for (int which = 0; which < 2; ++which) {
-    // K = -i[H, r]: neutrinos K_12.. = (Im C, -Re C).  Antineutrinos with
-    // Hbar = -H^*: conj(rhobar) obeys the neutrinos' equation with the same H,
-    // and Kbar = conj(K): (Im C, Re C)
-    w::Comm C;
-    if (OWNBAR) {
-      const w::Ham& h = which ? hb : hm;
-      const w::Mat m = w::mat(r, false);
-      const int top = w::max_i(w::top(m), which ? w::top(hb) : htop);
-      w::commutator(h, m, top < w::kExpNonFinite ? emin : kInfExp, C);
-    } else {
-      const w::Mat m = w::mat(r, which != 0);
-      const int top = w::max_i(w::top(m), htop);
-      w::commutator(hm, m, top < w::kExpNonFinite ? emin : kInfExp, C);
-    }
-    // the accumulator and the step's start (after the commutator: the operands
-    // it keeps in registers leave no room for them; the caller prefetches them
-    // into L2), before any store
+    const w::Ham& h = OWNBAR && which ? hb : hm;
+    const w::Mat m = w::mat(r, !OWNBAR && which);
+    const int top = w::max_i(w::top(m), OWNBAR && which ? w::top(hb) : htop);
+    const int emin = top < w::kExpNonFinite ? emin0 : kInfExp;
     double* __restrict__ yv = (which ? pt.rhobar : pt.rho) + p;
     double* __restrict__ av = row(pt.acc, P, which * 9) + p;
     double* __restrict__ sv = row(pt.stage, P, which * 9) + p;
-    double a[9], y[9];
-    if (first) {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) a[k] = y[k] = r[k];
-    } else {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) a[k] = ldp<COH>(row(av, P, k));
-      if (!last) {
-#pragma unroll
-        for (int k = 0; k < 9; ++k) y[k] = ldp<COH>(row(yv, P, k));
-      }
-    }
-    if (which == 0) {   // the other species' source
-#pragma unroll
-      for (int k = 0; k < 9; ++k) r[k] = ldp<COH>(row(src_b + p, P, k));
-    }
-    // K_k = kv[k] 2^(its exponent): the coefficients bdt, cdt take the exponent
-    // (at most the infinities' field)
-    double kv[9], kb[9], kc[9];
-    const int flip = (which == 1 && !OWNBAR) ? 0 : (int)0x80000000;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const int ed = C.ke[q] - w::kBiasP + 1, eo = C.oe[q] - w::kBiasP;   // (diagonal K are halved)
-      kv[q] = C.kd[q];
-      kb[q] = w::scale(bdt, w::min_i(ed, bmax));
-      kc[q] = w::scale(cdt, w::min_i(ed, cmax));
-      kv[3 + 2 * q] = C.ci[q];
-      kv[4 + 2 * q] = w::from_words(w::hi_word(C.cr[q]) ^ flip, w::lo_word(C.cr[q]));
-      kb[3 + 2 * q] = kb[4 + 2 * q] = w::scale(bdt, w::min_i(eo, bmax));
-      kc[3 + 2 * q] = kc[4 + 2 * q] = w::scale(cdt, w::min_i(eo, cmax));
-    }
-    double nv[9];   // the state stored: the next stage's, or at stage 4 the new one
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      if (last) {
-        nv[k] = fma(kb[k], kv[k], a[k]);
-      } else {
-        *row(av, P, k) = fma(kb[k], kv[k], a[k]);
-        nv[k] = fma(kc[k], kv[k], y[k]);
-      }
-    }
     double* __restrict__ dst = (!last || dry) ? sv : yv;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) *row(dst, P, k) = nv[k];
-    if constexpr (KEEP) {
-      // B = n1 rho - n2 rhobar^*: conj(rhobar) flips the sign of the imaginary components 4, 6, 8
-      if (which == 0) {
-#pragma unroll
-        for (int k = 0; k < 9; ++k) keep[k] = n1 * nv[k];
+    // the accumulator and the step's start of component k
+    auto load = [&](int k, double& a, double& y) {
+      a = first ? r[k] : ldp<COH>(row(av, P, k));
+      y = first ? r[k] : last ? 0.0 : ldp<COH>(row(yv, P, k));
+    };
+    // its update from K_k = kv 2^e: the coefficients bdt, cdt take the exponent
+    auto update = [&](int k, double kv, int e, double a, double y) {
+      double nv;   // the state stored: the next stage's, or at stage 4 the new one
+      if (last) {
+        nv = fma(w::scale_up(bdt, e), kv, a);
       } else {
-#pragma unroll
-        for (int k = 0; k < 9; ++k) keep[k] = fma((k == 4 || k == 6 || k == 8) ? n2 : -n2, nv[k], keep[k]);
+        *row(av, P, k) = fma(w::scale_up(bdt, e), kv, a);
+        nv = fma(w::scale_up(cdt, e), kv, y);
       }
+      *row(dst, P, k) = nv;
+      if constexpr (KEEP)   // B = n1 rho - n2 rhobar^*: conj(rhobar) flips the sign of the imaginary components
+        keep[k] = which == 0 ? n1 * nv : fma((k == 4 || k == 6 || k == 8) ? n2 : -n2, nv, keep[k]);
+    };
+    // K = -i[H, r]: neutrinos K_12.. = (Im C, -Re C).  Antineutrinos with
+    // Hbar = -H^*: conj(rhobar) obeys the neutrinos' equation with the same H,
+    // and Kbar = conj(K): (Im C, Re C).  Entry by entry, each with its loads
+    // issued before its products and finished before the next: few registers
+    // wait, and the products cover the loads' latency.
+    const int flip = (which == 1 && !OWNBAR) ? 0 : (int)0x80000000;
+    auto off = [&](auto Q) {
+      constexpr int q = decltype(Q)::value, k = 3 + 2 * q;
+      double a0, a1, y0, y1, cr, ci;
+      int e;
+      load(k, a0, y0);
+      load(k + 1, a1, y1);
+      w::commutator_off<q>(h, m, emin, cr, ci, e);
+      e = w::min_i(e - w::kBiasP, 3000);
+      update(k, ci, e, a0, y0);
+      update(k + 1, w::from_words(w::hi_word(cr) ^ flip, w::lo_word(cr)), e, a1, y1);
+    };
+    off(Int<0>{});
+    off(Int<1>{});
+    off(Int<2>{});
+    {
+      double a[3], y[3], kd[3];
+      int ke[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) load(k, a[k], y[k]);
+      if (which == 0) {   // the other species' source
+#pragma unroll
+        for (int k = 0; k < 9; ++k) r[k] = ldp<COH>(row(src_b + p, P, k));
+      }
+      w::commutator_diag(h, m, emin, kd, ke);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) update(k, kd[k], w::min_i(ke[k] - w::kBiasP + 1, 3000), a[k], y[k]);   // (halved)
     }
   }
   if (last) {
@@ -1250,9 +1239,9 @@ __device__ __forceinline__ void add_potentials(const BoxGeo& g, double (&Hm)[kNC
 }
 
 // rk_update of particle p of box g from H in the traceless components.
-template <bool POT, bool COH, bool KEEP = false>
+template <bool POT, int S, bool COH, bool KEEP = false>
 __device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, const double* src_b, int64_t P,
-                                            int64_t p, int s, int dry, double bdt, double cdt, double dtb,
+                                            int64_t p, int dry, double bdt, double cdt, double dtb,
                                             const double* __restrict__ vz, double (&Hm)[kNC], double (&r)[9],
                                             double* keep = nullptr, double* zkeep = nullptr, double n1 = 0.0,
                                             double n2 = 0.0) {
@@ -1260,10 +1249,10 @@ __device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, co
     double Hb[kNC];
     add_potentials(g, Hm, Hb);
     const emu_wide::Ham hm = emu_wide::ham(Hm), hb = emu_wide::ham(Hb);
-    rk_update<0, true, COH, KEEP>(g.Lz, pt, src_b, P, p, s, dry, bdt, cdt, dtb, vz, hm, hb, r, keep, zkeep, n1, n2);
+    rk_update<S, true, COH, KEEP>(g.Lz, pt, src_b, P, p, dry, bdt, cdt, dtb, vz, hm, hb, r, keep, zkeep, n1, n2);
   } else {
     const emu_wide::Ham hm = emu_wide::ham(Hm);
-    rk_update<0, false, COH, KEEP>(g.Lz, pt, src_b, P, p, s, dry, bdt, cdt, dtb, vz, hm, hm, r, keep, zkeep, n1,
+    rk_update<S, false, COH, KEEP>(g.Lz, pt, src_b, P, p, dry, bdt, cdt, dtb, vz, hm, hm, r, keep, zkeep, n1,
                                    n2);
   }
 }
@@ -1562,7 +1551,7 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
                                                                                : 1024);
           add_potentials(g, Hm, Hb);
           const w::Ham hm = w::ham(Hm), hb = w::ham(Hb);
-          rk_update<S, true, COH>(g.Lz, pt, src_b, P, p, s, dry, bdt, cdt, dtb, vz, hm, hb, r);
+          rk_update<S, true, COH>(g.Lz, pt, src_b, P, p, dry, bdt, cdt, dtb, vz, hm, hb, r);
         } else {
           w::Ham hm;
           hm.d12 = w::Real{w::split(hv[0]), he[0] + 2};
@@ -1571,7 +1560,7 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
           hm.a = w::Cplx{w::split(hv[2]), w::split(hv[3]), he[1] + 2};
           hm.b = w::Cplx{w::split(hv[4]), w::split(hv[5]), he[2] + 2};
           hm.c = w::Cplx{w::split(hv[6]), w::split(hv[7]), he[3] + 2};
-          rk_update<S, false, COH>(g.Lz, pt, src_b, P, p, s, dry, bdt, cdt, dtb, vz, hm, hm, r);
+          rk_update<S, false, COH>(g.Lz, pt, src_b, P, p, dry, bdt, cdt, dtb, vz, hm, hm, r);
         }
       }
       __syncwarp();   // (the unit's G are rewritten by the next)
@@ -1861,7 +1850,7 @@ k_rk_deposit(Batch B, Parts pt, double* __restrict__ W, const double* __restrict
           }
         }
         double zn = 0.0;
-        rk_particle<POT, false, true>(g, pt, src_b, P, p, s, dry, bdt, cdt, dtb, dirtab + 3 * MT + gd, Hm, r,
+        rk_particle<POT, s == 3 ? 2 : s, false, true>(g, pt, src_b, P, p, dry, bdt, cdt, dtb, dirtab + 3 * MT + gd, Hm, r,
                                       bm, &zn, n1, n2);
         zs = s < 4 ? fma(stage_frac(s) * dtb, vz, pt.z[p]) : zn;
       }

@@ -437,7 +437,7 @@ __device__ __forceinline__ void interp3(const Box3& b, const double* A, int jx, 
 // Units are (row, 32-cell z tile, direction), every lane on its own cell: the
 // z neighbours' G come from the field in memory (L1), not from halo lanes, so
 // no lane idles except past the end of a row.
-template <bool POT, int ORDER>
+template <bool POT, int ORDER, int S>   // S: as rk_update's
 __global__ void __launch_bounds__(kThreads, 2)
 k3_rk_stage(Box3 b, Parts pt, double* __restrict__ x, double* __restrict__ y, const double* __restrict__ dirtab,
             const int* __restrict__ srow, const double* __restrict__ Gxy, const double* __restrict__ wrow, int s,
@@ -483,7 +483,7 @@ k3_rk_stage(Box3 b, Parts pt, double* __restrict__ x, double* __restrict__ y, co
     double r[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) r[k] = src_r[k * P + p];
-    rk_particle<POT, false>(*b.g, pt, src_b, P, p, s, dry, bdt, cdt, dt, dirtab + 5 * M + d, Hm, r);
+    rk_particle<POT, S, false>(*b.g, pt, src_b, P, p, dry, bdt, cdt, dt, dirtab + 5 * M + d, Hm, r);
     if (s == 4) {   // x and y move as z does (rk_particle moved z; dry: into the RK scratch)
       const double xn = wrap_z(fma(dt, vx, x[p]), b.L[0]), yn = wrap_z(fma(dt, vy, y[p]), b.L[1]);
       if (dry) { pt.acc[p] = xn; pt.acc[P + p] = yn; }

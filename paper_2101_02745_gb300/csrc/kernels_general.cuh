@@ -421,7 +421,7 @@ __device__ __forceinline__ void ginterp(const BoxGeo& g, int NZ, const double* _
 }
 
 // One RK4 stage of particles anywhere (as k_rk_stage): one thread per particle.
-template <bool POT, int ORDER>
+template <bool POT, int ORDER, int S>   // S: as rk_update's
 __global__ void __launch_bounds__(kThreads, 2)
 k_grk_stage(Batch B, Parts pt, const double* __restrict__ At, int s, int dry) {
   griddep_wait();
@@ -443,7 +443,7 @@ k_grk_stage(Batch B, Parts pt, const double* __restrict__ At, int s, int dry) {
   double r[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) r[k] = src_r[k * P + p];
-  rk_particle<POT, false>(g, pt, src_b, P, p, s, dry, bdt, cdt, dt, &vz, Hm, r);
+  rk_particle<POT, S, false>(g, pt, src_b, P, p, dry, bdt, cdt, dt, &vz, Hm, r);
 }
 
 // Interpolation only (Eq. 6 then Eq. 2) for particles anywhere: H[k * P + p].

@@ -193,17 +193,24 @@ EMU_HD int two() {
   return 2;
 #endif
 }
-// a b / 2^64 and (a b + c d) / 2^64.  |V| < 2^61 keeps every partial sum in 63 bits.
+// a b / 2^64 and c + a b / 2^64.  |V| < 2^61 keeps every partial sum in 63 bits.
 EMU_HD int64_t mul(Limbs a, Limbs b) {
   const int64_t m = mad(a.h, b.l, mad(a.l, b.h, half_unit()));
   return mad((int)(m >> 32), two(), prod(a.h, b.h));
 }
-EMU_HD int64_t mul_add(Limbs a, Limbs b, int64_t c) {   // c + a b / 2^64
+EMU_HD int64_t mul_add(Limbs a, Limbs b, int64_t c) {
   const int64_t m = mad(a.h, b.l, mad(a.l, b.h, half_unit()));
   return mad((int)(m >> 32), two(), mad(a.h, b.h, c));
 }
-EMU_HD int64_t mul2(Limbs a, Limbs b, Limbs c, Limbs d) {
-  const int64_t m = mad(a.h, b.l, mad(a.l, b.h, mad(c.h, d.l, mad(c.l, d.h, half_unit()))));
+// The same with the middle term rounded down (two instructions less each: the
+// rounding addend costs a 64-bit add).  For sums with as many subtracted as
+// added products, in which the bias cancels.
+EMU_HD int64_t mul_down(Limbs a, Limbs b) {
+  const int64_t m = mad(a.h, b.l, prod(a.l, b.h));
+  return mad((int)(m >> 32), two(), prod(a.h, b.h));
+}
+EMU_HD int64_t mul2_down(Limbs a, Limbs b, Limbs c, Limbs d) {
+  const int64_t m = mad(a.h, b.l, mad(a.l, b.h, mad(c.h, d.l, prod(c.l, d.h))));
   return mad((int)(m >> 32), two(), mad(a.h, b.h, prod(c.h, d.h)));
 }
 
@@ -226,7 +233,12 @@ EMU_HD int64_t align(int64_t v, int d) { return align(v, d, max_i(d - 32, 0)); }
 
 // c 2^k for a normal c whose exponent stays normal.
 EMU_HD double scale(double c, int k) { return from_words(hi_word(c) + (int)((unsigned)k << 20), lo_word(c)); }
-
+// c 2^k for a positive normal c, k not below its smallest normal result; NaN
+// where the result is out of range (k at most 3000).
+EMU_HD double scale_up(double c, int k) {
+  const unsigned h = (unsigned)hi_word(c) + ((unsigned)k << 20);
+  return from_words((int)(h < 0x7ff80000u ? h : 0x7ff80000u), lo_word(c));
+}
 // x 2^k for x = 0 or a normal x whose exponent stays normal.
 EMU_HD double scale_nz(double x, int k) {
   const int hi = hi_word(x);
@@ -241,20 +253,27 @@ struct Ham {
 };
 // From the traceless components (H_11 - H_22, H_22 - H_33, off-diagonal reals).
 EMU_HD Ham ham(const double (&H)[8]) {
-  return Ham{real(H[0]), real(H[0] + H[1]), real(H[1]), cplx(H[2], H[3]), cplx(H[4], H[5]), cplx(H[6], H[7])};
+  Ham h;
+  h.d12 = real(H[0]);
+  h.d13 = real(H[0] + H[1]);
+  h.d23 = real(H[1]);
+  h.a = cplx(H[2], H[3]);
+  h.b = cplx(H[4], H[5]);
+  h.c = cplx(H[6], H[7]);
+  return h;
 }
 
 // A Hermitian matrix r (or its conjugate) as the right operand.
 struct Mat {
-  Real e21, e31, e32;    // r_22 - r_11, r_33 - r_11, r_33 - r_22
+  Real e12, e13, e23;    // r_11 - r_22, r_11 - r_33, r_22 - r_33
   Cplx x, y, z;
-  Limbs nx, ny, nz;      // minus the imaginary parts
+  Limbs nx, nz;          // minus the imaginary parts of x, z
 };
 EMU_HD Mat mat(const double* r, bool conj) {
   Mat m;
-  m.e21 = real(r[1] - r[0]);
-  m.e31 = real(r[2] - r[0]);
-  m.e32 = real(r[2] - r[1]);
+  m.e12 = real(r[0] - r[1]);
+  m.e13 = real(r[0] - r[2]);
+  m.e23 = real(r[1] - r[2]);
   m.x = cplx(r[3], r[4]);
   m.y = cplx(r[5], r[6]);
   m.z = cplx(r[7], r[8]);
@@ -263,7 +282,6 @@ EMU_HD Mat mat(const double* r, bool conj) {
   m.y.i = Limbs{(m.y.i.h ^ c) - c, (m.y.i.l ^ c) - c};
   m.z.i = Limbs{(m.z.i.h ^ c) - c, (m.z.i.l ^ c) - c};
   m.nx = negate(m.x.i);
-  m.ny = negate(m.y.i);
   m.nz = negate(m.z.i);
   return m;
 }
@@ -272,49 +290,53 @@ EMU_HD int top(const Ham& H) {
   return max_i(max_i(max_i(H.d12.e, H.d13.e), max_i(H.d23.e, H.a.e)), max_i(H.b.e, H.c.e));
 }
 EMU_HD int top(const Mat& m) {
-  return max_i(max_i(max_i(m.e21.e, m.e31.e), max_i(m.e32.e, m.x.e)), max_i(m.y.e, m.z.e));
+  return max_i(max_i(max_i(m.e12.e, m.e13.e), max_i(m.e23.e, m.x.e)), max_i(m.y.e, m.z.e));
 }
 
-// C = [H, r], rounded to doubles up to a power of two each:
-//   C_12, C_13, C_23 = (or[q] + i oi[q]) 2^(oe[q] - kBiasP),
-//   K_11 / 2, K_22 / 2, K_33 / 2 of K = -i C = kd[q] 2^(ke[q] - kBiasP).
-struct Comm {
-  double cr[3], ci[3], kd[3];
-  int oe[3], ke[3];
-};
-
-// D x + E a + (g1) + (g2) at the largest exponent (at least emin).
+// Entries of C = [H, r], rounded to doubles up to a power of two each, so that a
+// caller can finish one before it forms the next:
+//   commutator_off<q>: C_12, C_13, C_23 (q = 0, 1, 2) = (cr + i ci) 2^(e - kBiasP),
+//   commutator_diag:   K_11 / 2, K_22 / 2, K_33 / 2 of K = -i C = kd[q] 2^(ke[q] - kBiasP).
+// D x - E a + (g1) - (g2) at the largest exponent (at least emin).  Two products
+// are added and two subtracted: their rounding down cancels in the mean.
 EMU_HD void off_diagonal(const Real& D, const Cplx& x, const Real& E, const Cplx& a, int64_t g1r, int64_t g1i, int e1,
                          int64_t g2r, int64_t g2i, int e2, int emin, double& cr, double& ci, int& oe) {
   const int ea = D.e + x.e, eb = E.e + a.e;
   const int e = max_i(max_i(max_i(ea, eb), max_i(e1, e2)), emin);
   const int da = e - ea, db = e - eb, d1 = e - e1, d2 = e - e2;
   const int fa = max_i(da - 32, 0), fb = max_i(db - 32, 0), f1 = max_i(d1 - 32, 0), f2 = max_i(d2 - 32, 0);
-  cr = (double)(align(mul(D.v, x.r), da, fa) + align(mul(E.v, a.r), db, fb) + align(g1r, d1, f1) + align(g2r, d2, f2));
-  ci = (double)(align(mul(D.v, x.i), da, fa) + align(mul(E.v, a.i), db, fb) + align(g1i, d1, f1) + align(g2i, d2, f2));
+  cr = (double)(align(mul_down(D.v, x.r), da, fa) - align(mul_down(E.v, a.r), db, fb) + align(g1r, d1, f1) -
+                align(g2r, d2, f2));
+  ci = (double)(align(mul_down(D.v, x.i), da, fa) - align(mul_down(E.v, a.i), db, fb) + align(g1i, d1, f1) -
+                align(g2i, d2, f2));
   oe = e;
 }
 
-EMU_HD void commutator(const Ham& H, const Mat& m, int emin, Comm& o) {
+template <int Q>
+EMU_HD void commutator_off(const Ham& H, const Mat& m, int emin, double& cr, double& ci, int& e) {
   const Cplx &x = m.x, &y = m.y, &z = m.z, &a = H.a, &b = H.b, &c = H.c;
-  // C_12 = d12 x + e21 a + b z^* - y c^*
-  off_diagonal(H.d12, x, m.e21, a, mul2(b.r, z.r, b.i, z.i), mul2(b.i, z.r, b.r, m.nz), b.e + z.e,
-               -mul2(c.r, y.r, c.i, y.i), mul2(c.i, y.r, c.r, m.ny), c.e + y.e, emin, o.cr[0], o.ci[0], o.oe[0]);
-  // C_13 = d13 y + e31 b + a z - x c
-  off_diagonal(H.d13, y, m.e31, b, mul2(a.r, z.r, a.i, m.nz), mul2(a.r, z.i, a.i, z.r), a.e + z.e,
-               -mul2(c.r, x.r, c.i, m.nx), -mul2(c.r, x.i, c.i, x.r), c.e + x.e, emin, o.cr[1], o.ci[1], o.oe[1]);
-  // C_23 = d23 z + e32 c + a^* y - x^* b
-  off_diagonal(H.d23, z, m.e32, c, mul2(a.r, y.r, a.i, y.i), -mul2(a.r, m.ny, a.i, y.r), a.e + y.e,
-               -mul2(b.r, x.r, b.i, x.i), -mul2(b.i, x.r, b.r, m.nx), b.e + x.e, emin, o.cr[2], o.ci[2], o.oe[2]);
-  // K_11 / 2 = Im(a x^*) + Im(b y^*), K_22 / 2 = Im(c z^*) - Im(a x^*), K_33 / 2 = -Im(b y^*) - Im(c z^*)
-  const int64_t p = mul2(a.i, x.r, a.r, m.nx), q = mul2(b.i, y.r, b.r, m.ny), t = mul2(c.i, z.r, c.r, m.nz);
+  if (Q == 0)   // C_12 = d12 x - e12 a + b z^* - y c^*
+    off_diagonal(H.d12, x, m.e12, a, mul2_down(b.r, z.r, b.i, z.i), mul2_down(b.i, z.r, b.r, m.nz), b.e + z.e,
+                 mul2_down(c.r, y.r, c.i, y.i), mul2_down(c.r, y.i, negate(c.i), y.r), c.e + y.e, emin, cr, ci, e);
+  else if (Q == 1)   // C_13 = d13 y - e13 b + a z - x c
+    off_diagonal(H.d13, y, m.e13, b, mul2_down(a.r, z.r, a.i, m.nz), mul2_down(a.r, z.i, a.i, z.r), a.e + z.e,
+                 mul2_down(c.r, x.r, c.i, m.nx), mul2_down(c.r, x.i, c.i, x.r), c.e + x.e, emin, cr, ci, e);
+  else   // C_23 = d23 z - e23 c + a^* y - x^* b
+    off_diagonal(H.d23, z, m.e23, c, mul2_down(a.r, y.r, a.i, y.i), mul2_down(a.r, y.i, negate(a.i), y.r), a.e + y.e,
+                 mul2_down(b.r, x.r, b.i, x.i), mul2_down(b.i, x.r, b.r, m.nx), b.e + x.e, emin, cr, ci, e);
+}
+EMU_HD void commutator_diag(const Ham& H, const Mat& m, int emin, double (&kd)[3], int (&ke)[3]) {
+  const Cplx &x = m.x, &y = m.y, &z = m.z, &a = H.a, &b = H.b, &c = H.c;
+  // p = Im(a x^*), q = -Im(b y^*), t = Im(c z^*): K_11 / 2 = p - q, K_22 / 2 = t - p, K_33 / 2 = q - t
+  const int64_t p = mul2_down(a.i, x.r, a.r, m.nx), q = mul2_down(b.r, y.i, negate(b.i), y.r),
+                t = mul2_down(c.i, z.r, c.r, m.nz);
   const int ep = a.e + x.e, eq = b.e + y.e, et = c.e + z.e;
-  o.ke[0] = max_i(max_i(ep, eq), emin);
-  o.ke[1] = max_i(max_i(ep, et), emin);
-  o.ke[2] = max_i(max_i(eq, et), emin);
-  o.kd[0] = (double)(align(p, o.ke[0] - ep) + align(q, o.ke[0] - eq));
-  o.kd[1] = (double)(align(t, o.ke[1] - et) - align(p, o.ke[1] - ep));
-  o.kd[2] = (double)(-align(q, o.ke[2] - eq) - align(t, o.ke[2] - et));
+  ke[0] = max_i(max_i(ep, eq), emin);
+  ke[1] = max_i(max_i(ep, et), emin);
+  ke[2] = max_i(max_i(eq, et), emin);
+  kd[0] = (double)(align(p, ke[0] - ep) - align(q, ke[0] - eq));
+  kd[1] = (double)(align(t, ke[1] - et) - align(p, ke[1] - ep));
+  kd[2] = (double)(align(q, ke[2] - eq) - align(t, ke[2] - et));
 }
 
 }  // namespace emu_wide

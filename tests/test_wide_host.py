@@ -17,12 +17,15 @@ extern "C" {
 void comm(const double* H, const double* r, int conj, int emin, double* v, int* e) {
   double h[8];
   for (int k = 0; k < 8; ++k) h[k] = H[k];
-  Comm C;
-  commutator(ham(h), mat(r, conj != 0), emin, C);
-  for (int q = 0; q < 3; ++q) {
-    v[2 * q] = C.cr[q]; v[2 * q + 1] = C.ci[q]; v[6 + q] = C.kd[q];
-    e[2 * q] = e[2 * q + 1] = C.oe[q] - kBiasP; e[6 + q] = C.ke[q] - kBiasP;
-  }
+  const Ham hm = ham(h);
+  const Mat m = mat(r, conj != 0);
+  int o, ke[3];
+  double kd[3];
+  commutator_off<0>(hm, m, emin, v[0], v[1], o); e[0] = e[1] = o - kBiasP;
+  commutator_off<1>(hm, m, emin, v[2], v[3], o); e[2] = e[3] = o - kBiasP;
+  commutator_off<2>(hm, m, emin, v[4], v[5], o); e[4] = e[5] = o - kBiasP;
+  commutator_diag(hm, m, emin, kd, ke);
+  for (int q = 0; q < 3; ++q) { v[6 + q] = kd[q]; e[6 + q] = ke[q] - kBiasP; }
 }
 int top_of(const double* H, const double* r) {
   double h[8];
