@@ -712,34 +712,24 @@ int launch_deposit(emu_box* b, int mode, const double* rnu, const double* rnb, c
   const double* wrow = weight_row(b, shift_row);
   by_order(b->S.order, [&](auto O) {
     constexpr int R = decltype(O)::value;
-    if (mode == 0)
-      pdl(st, k_deposit<0, R>, grid, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, W, b->err);
-    else if (mode == 1)
-      pdl(st, k_deposit<1, R>, grid, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, nullptr,
-          b->err);
-    else if (mode == 2)
-      pdl(st, k_deposit<2, R>, grid, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, nullptr,
-          b->err);
+    auto go = [&](auto MODE, auto TAB) {
+      static std::atomic<unsigned> done{0};
+      auto k = k_deposit<decltype(MODE)::value, R, decltype(TAB)::value>;
+      if (raise_smem(k, kDepSmem, done) == cudaSuccess)
+        pdl_smem(st, k, grid, B.U > B.nw ? kDepSmem : kDepSmem / 2, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow,
+                 frac, b->partial, mode == 0 || mode == 5 ? W : nullptr, b->err);
+    };
+    using std::false_type;
+    using std::true_type;
+    if (mode == 0) go(std::integral_constant<int, 0>{}, false_type{});
+    else if (mode == 1) go(std::integral_constant<int, 1>{}, false_type{});
+    else if (mode == 2) go(std::integral_constant<int, 2>{}, false_type{});
     else if (mode == 3 && wrow != nullptr)   // (the adjoint's deposit: the weights its forward step used)
-      pdl(st, k_deposit<3, R, true>, grid, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial,
-          nullptr, b->err);
-    else if (mode == 3)
-      pdl(st, k_deposit<3, R>, grid, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, nullptr,
-          b->err);
-    else if (mode == 4)
-      pdl(st, k_deposit<4, R>, grid, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, nullptr,
-          b->err);
-    else {
-      auto step = [&](auto TAB) {
-        static std::atomic<unsigned> done{0};
-        auto k = k_deposit<5, R, decltype(TAB)::value>;
-        if (raise_smem(k, kDepSmem, done) == cudaSuccess)
-          pdl_smem(st, k, grid, B.U > B.nw ? kDepSmem : kDepSmem / 2, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow, frac, b->partial, W,
-                   b->err);
-      };
-      if (wrow != nullptr) step(std::true_type{});
-      else step(std::false_type{});
-    }
+      go(std::integral_constant<int, 3>{}, true_type{});
+    else if (mode == 3) go(std::integral_constant<int, 3>{}, false_type{});
+    else if (mode == 4) go(std::integral_constant<int, 4>{}, false_type{});
+    else if (wrow != nullptr) go(std::integral_constant<int, 5>{}, true_type{});
+    else go(std::integral_constant<int, 5>{}, false_type{});
     return 0;
   });
   if (int rc = after_launch(b, "deposit kernel")) return rc;
@@ -2684,8 +2674,11 @@ extern "C" int emu_deposit_static(const emu_config* cfg, const double* z, const 
   f.v[0] = 1.0;
   k_shifts<2><<<(S.MT + kThreads - 1) / kThreads, kThreads, 0, st>>>(B, z, dirtab, f, 1, shift, nullptr);
   if (int rc = check(cudaGetLastError(), "shift kernel")) return rc;
-  k_deposit<0, 2><<<dim3(kPersistBlocks), kThreads, 0, st>>>(B, z, N, Nbar, rho, rhobar, dirtab, shift, nullptr, 1.0,
-                                                            partial, nullptr, err);
+  static std::atomic<unsigned> smem_raised{0};
+  if (int rc = check(raise_smem(k_deposit<0, 2, false>, kDepSmem, smem_raised), "deposit kernel's shared memory"))
+    return rc;
+  k_deposit<0, 2, false><<<dim3(kPersistBlocks), kThreads, kDepSmem, st>>>(B, z, N, Nbar, rho, rhobar, dirtab, shift,
+                                                                          nullptr, 1.0, partial, nullptr, err);
   if (int rc = check(cudaGetLastError(), "deposit kernel")) return rc;
   const int split = combine_split(S, B.nw);
   k_combine<<<combine_blocks(kNA, S.NZ, split), kThreads, 0, st>>>(B, partial, A_out, kNA, 1, split, err);

@@ -519,91 +519,6 @@ __device__ __forceinline__ void flush_tile(const double (&acc)[NA], int64_t gtil
   }
 }
 
-// The direction loop of the deposit for one tile: warp lane `lane` of a tile
-// of box b (lane l owns cell tile * T - H + l) adds the rings dfirst..dlast-1
-// of the tile, in order, to acc (MODES as deposit_phase).  Shared by the
-// per-warp deposit and the cluster deposit.
-template <int MODE, int ORDER, bool COH, int NA>
-__device__ __forceinline__ void deposit_tile_dirs(const Batch& B, int b, int tile, int dfirst, int dlast, int lane,
-                                                  const double* z, const double* __restrict__ N,
-                                                  const double* __restrict__ Nbar, const double* r_nu,
-                                                  const double* r_nb, const double* __restrict__ dirtab,
-                                                  const int* shift, const double* wrow, double frac, double* W,
-                                                  double (&acc)[NA], int& bad) {
-  const BoxGeo& g = B.box[b];
-  const int nz = g.nz;
-  const int64_t P = B.Ptot;
-  const int MT = B.MT;
-  constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T;
-  const int craw = tile * T - H + lane;
-  const int j = wrapc(craw, nz);
-  const double hp = (double)j + 0.5;
-  const bool own = lane >= H && lane < H + T && craw < nz;
-  const double pos_dt = frac * B.dt[b];
-  const int64_t pbase = g.poff;
-  const int dbase = g.doff;
-  for (int d = dfirst; d < dlast; ++d) {
-    const int gd = dbase + d;
-    const double ox = __ldg(dirtab + gd), oy = __ldg(dirtab + MT + gd), oz = __ldg(dirtab + 2 * MT + gd);
-    const double vz = __ldg(dirtab + 3 * MT + gd);
-    const int64_t p = pbase + (int64_t)d * nz + wrapc(j - ldi<COH>(shift + gd), nz);
-    double wt[Sten<ORDER>::NW];
-    const double zs = fma(pos_dt, vz, ldd<COH>(z + p));
-    if (wrow != nullptr) {
-      bad |= off_site(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d));
-      if constexpr (ORDER == 0) {
-        wt[0] = 0.0; wt[1] = 1.0; wt[2] = 0.0;
-      } else {
-#pragma unroll
-        for (int q = 0; q < Sten<ORDER>::NW; ++q) wt[q] = ldp<COH>(wrow + q * B.MT + gd);
-      }
-    } else {
-      bad |= shape_weights<ORDER>(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d), wt);
-    }
-    if (MODE == 0 && W != nullptr && own) {   // the RK stage of these positions reads them back
-#pragma unroll
-      for (int q = 0; q < Sten<ORDER>::NWS; ++q) W[q * P + p] = wt[q];
-    }
-    Spread<ORDER> spread;
-    spread.init(wt);
-    if constexpr (MODE == 4) {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        const double c1 = spread.apply(__ldg(N + p) * ldd<COH>(r_nu + k * P + p));
-        const double c2 = spread.apply(__ldg(Nbar + p) * ldd<COH>(r_nb + k * P + p));
-        acc[k] += c1;
-        acc[9 + k] = fma(ox, c1, acc[9 + k]);
-        acc[18 + k] += c2;
-        acc[27 + k] = fma(ox, c2, acc[27 + k]);
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        // (the weights are read inside the loop: fewer live registers across it)
-        const double n1 = (MODE == 0 || MODE == 1) ? __ldg(N + p) : 0.0;
-        const double n2 = (MODE == 0 || MODE == 2) ? __ldg(Nbar + p) : 0.0;
-        double bv;
-        if (MODE == 0) {
-          const double x = ldd<COH>(r_nu + k * P + p), y = ldd<COH>(r_nb + k * P + p);
-          // conj(rhobar) flips the sign of the imaginary components 4, 6, 8
-          bv = (k == 4 || k == 6 || k == 8) ? fma(n2, y, n1 * x) : fma(-n2, y, n1 * x);
-        } else if (MODE == 1) {
-          bv = n1 * ldd<COH>(r_nu + k * P + p);
-        } else if (MODE == 2) {
-          bv = n2 * ldd<COH>(r_nb + k * P + p);
-        } else {
-          bv = ldd<COH>(r_nu + k * P + p);
-        }
-        const double c = spread.apply(bv);
-        acc[k] += c;
-        acc[9 + k] = fma(ox, c, acc[9 + k]);
-        acc[18 + k] = fma(oy, c, acc[18 + k]);
-        acc[27 + k] = fma(oz, c, acc[27 + k]);
-      }
-    }
-  }
-}
-
 // A value of lane `src` as limbs in every lane.
 __device__ __forceinline__ emu_wide::Limbs bcast(emu_wide::Limbs v, int src) {
   return emu_wide::Limbs{__shfl_sync(kFull, v.h, src), __shfl_sync(kFull, v.l, src)};
@@ -629,16 +544,31 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
-constexpr int kDepRows = 21;   // doubles of a particle the step's deposit reads
+constexpr int kDepRows = 21;   // doubles of a particle a deposit reads
 constexpr int kDepBuf = 2 * kDepRows * kLanes;                                // of one warp's buffers
 constexpr int kDepSmem = kWarps * kDepBuf * (int)sizeof(double);              // 86 KB a block
 
-// deposit_tile_dirs for the step's deposit (MODE 5), on the integer pipe.  B is
-// formed in FP64 (20 instructions a particle, against 85 for the whole
-// deposit: at 16 cycles each the FP64 pipe bound it); its spread over the
-// stencil and the four moments' sums are fixed-point (wide.cuh).  A sum is an
-// int64 per lane; the components of one exponent group (B_11 - B_22,
-// B_22 - B_33 and the three complex off-diagonals) share the exponent ea of
+// What a deposit of mode MODE (deposit_phase) sums: SETS fields of COMP
+// components with MOM moments each (row (set * MOM + m) * COMP + c), and which
+// of a particle's arrays it reads.
+template <int MODE>
+struct DepMode {
+  static constexpr int SETS = MODE == 4 ? 2 : 1, MOM = MODE == 4 ? 2 : 4, COMP = MODE == 5 ? kNC : 9;
+  static constexpr int NA = SETS * MOM * COMP;
+  static constexpr bool N1 = MODE != 2 && MODE != 3, N2 = MODE != 1 && MODE != 3, RNU = MODE != 2,
+                        RNB = MODE != 1 && MODE != 3;
+  // components that share the exponent of their sums: single diagonal entries (or
+  // their differences), then the real and imaginary part of an off-diagonal
+  static constexpr int SINGLE = MODE == 5 ? 2 : 3, GROUPS = SINGLE + 3;
+};
+
+// The direction loop of the deposit for one tile: warp lane `lane` of a tile
+// of box b (lane l owns cell tile * T - H + l) adds the rings dfirst..dlast-1
+// of the tile, in order, to out (MODES as deposit_phase), on the integer pipe.
+// B is formed in FP64 (20 instructions a particle, against 85-100 for a deposit
+// with FP64 sums: at 16 cycles each the FP64 pipe bound it); its spread over the
+// stencil and the moments' sums are fixed-point (wide.cuh).  A sum is an
+// int64 per lane; the components of one group share the exponent ea of
 // their sums, which grows when a direction's contribution asks for it (the
 // sums are then shifted).  A tile's sums of n directions leave ceil(log2 n)
 // bits of headroom, so a contribution keeps 61 - ceil(log2 n) bits below the
@@ -646,15 +576,16 @@ constexpr int kDepSmem = kWarps * kDepBuf * (int)sizeof(double);              //
 // rounding follows the partial sums.  Zero contributions add exactly nothing.
 // (buf: this warp's two buffers of kDepRows x 32 doubles in shared memory;
 // ring2 0: only one, when no warp takes more than one direction of a tile.)
-template <int ORDER, bool COH>
-__device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int tile, int dfirst, int dlast, int lane,
+template <int MODE, int ORDER, bool COH>
+__device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, int dfirst, int dlast, int lane,
                                                   const double* z, const double* __restrict__ N,
                                                   const double* __restrict__ Nbar, const double* r_nu,
                                                   const double* r_nb, const double* __restrict__ dirtab,
                                                   const int* shift, const double* wrow, double frac, double* W,
-                                                  double* buf, int ring2, double (&out)[kNT], int& bad) {
+                                                  double* buf, int ring2, double (&out)[DepMode<MODE>::NA], int& bad) {
   namespace w = emu_wide;
-  constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T, NW = Sten<ORDER>::NW, kGroups = 5;
+  constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T, NW = Sten<ORDER>::NW;
+  using D = DepMode<MODE>;
   const BoxGeo& g = B.box[b];
   const int nz = g.nz;
   const unsigned P = (unsigned)B.Ptot;
@@ -666,12 +597,12 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
   const double pos_dt = frac * B.dt[b];
   const int dbase = g.doff;
   const int head = max(32 - __clz(dlast - dfirst), 2) - 2;   // headroom beyond the two bits a contribution leaves
-  int64_t acc[kNT];
-  int ea[kGroups];
+  int64_t acc[D::NA];
+  int ea[D::SETS * D::GROUPS];
 #pragma unroll
-  for (int c = 0; c < kNT; ++c) acc[c] = 0;
+  for (int c = 0; c < D::NA; ++c) acc[c] = 0;
 #pragma unroll
-  for (int q = 0; q < kGroups; ++q) ea[q] = 0;
+  for (int q = 0; q < D::SETS * D::GROUPS; ++q) ea[q] = 0;
   // direction d's particle data into buffer d & 1, asynchronously (each lane
   // its own particle's: no exchange between lanes): z, N, Nbar, rho, rhobar
   auto fetch = [&](int d) -> int64_t {
@@ -680,12 +611,12 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
     const int64_t p = g.poff + (int64_t)d * nz + i;
     double* dst = buf + (d & ring2) * kDepRows * kLanes + lane;
     cp_async8(dst, z + p);
-    cp_async8(dst + kLanes, N + p);
-    cp_async8(dst + 2 * kLanes, Nbar + p);
+    if (D::N1) cp_async8(dst + kLanes, N + p);
+    if (D::N2) cp_async8(dst + 2 * kLanes, Nbar + p);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      cp_async8(dst + (3 + k) * kLanes, row(r_nu + p, P, k));
-      cp_async8(dst + (12 + k) * kLanes, row(r_nb + p, P, k));
+      if (D::RNU) cp_async8(dst + (3 + k) * kLanes, row(r_nu + p, P, k));
+      if (D::RNB) cp_async8(dst + (12 + k) * kLanes, row(r_nb + p, P, k));
     }
     cp_async_commit();
     return p;
@@ -701,9 +632,17 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
       cp_async_wait<0>();
     }
     const double* x = buf + (d & ring2) * kDepRows * kLanes + lane;
-    auto rnu = [&](int k) { return x[(3 + k) * kLanes]; };
-    auto rnb = [&](int k) { return x[(12 + k) * kLanes]; };
-    const double n1 = x[kLanes], n2 = x[2 * kLanes];
+    const double n1 = D::N1 ? x[kLanes] : 0.0, n2 = D::N2 ? x[2 * kLanes] : 0.0;
+    // component k of the deposited matrix (conj(rhobar) flips the sign of the
+    // imaginary components 4, 6, 8)
+    auto value = [&](int set, int k) -> double {
+      const bool im = k == 4 || k == 6 || k == 8;
+      const double a = D::RNU ? x[(3 + k) * kLanes] : 0.0, c = D::RNB ? x[(12 + k) * kLanes] : 0.0;
+      if (MODE == 3) return a;
+      if (MODE == 1 || (MODE == 4 && set == 0)) return n1 * a;
+      if (MODE == 2 || MODE == 4) return n2 * c;
+      return fma(im ? n2 : -n2, c, n1 * a);
+    };
     // Omega, and the ring's weights when every particle takes them: lane q
     // converts one of them
     double u = 0.0;
@@ -716,7 +655,7 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
       bad |= off_site(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d));
     } else {
       bad |= shape_weights<ORDER>(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d), wt);
-      if (W != nullptr && own) {   // the RK stage of these positions reads them back
+      if ((MODE == 0 || MODE == 5) && W != nullptr && own) {   // the RK stage of these positions reads them back
 #pragma unroll
         for (int q = 0; q < Sten<ORDER>::NWS; ++q) *row(W + p, P, q) = wt[q];
       }
@@ -727,7 +666,7 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
     const w::Limbs om[3] = {bcast(ul, 0), bcast(ul, 1), bcast(ul, 2)};
     if constexpr (ORDER > 0) {
       if (wrow != nullptr) {
-        if (W != nullptr && own) {
+        if ((MODE == 0 || MODE == 5) && W != nullptr && own) {
 #pragma unroll
           for (int q = 0; q < NW; ++q) *row(W + p, P, q) = ldp<COH>(wrow + q * MT + gd);
         }
@@ -741,20 +680,21 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
         }
       }
     }
-    double bprev = fma(-n2, rnb(0), n1 * rnu(0));   // B of the previous diagonal entry
+    double bprev = MODE == 5 ? value(0, 0) : 0.0;   // B of the previous diagonal entry
 #pragma unroll
-    for (int q = 0; q < kGroups; ++q) {
-      const int nc = q < 2 ? 1 : 2, c0 = q < 2 ? q : 2 * q - 2;   // the group's components c0 .. c0 + nc - 1
-      double bv[2];
-      if (q < 2) {
-        const double bn = fma(-n2, rnb(q + 1), n1 * rnu(q + 1));
+    for (int sq = 0; sq < D::SETS * D::GROUPS; ++sq) {
+      const int set = sq / D::GROUPS, q = sq % D::GROUPS, nc = q < D::SINGLE ? 1 : 2;
+      const int c0 = q < D::SINGLE ? q : 2 * q - D::SINGLE;   // the group's components c0 .. c0 + nc - 1
+      const int r0 = set * D::MOM * D::COMP + c0;             // and the row of its first sum
+      double bv[2] = {0.0, 0.0};
+      if (MODE == 5 && nc == 1) {
+        const double bn = value(0, q + 1);
         bv[0] = bprev - bn;
         bprev = bn;
-        bv[1] = 0.0;
       } else {
-        const int k = c0 + 1;   // conj(rhobar) flips the sign of the imaginary part
-        bv[0] = fma(-n2, rnb(k), n1 * rnu(k));
-        bv[1] = fma(n2, rnb(k + 1), n1 * rnu(k + 1));
+        const int k = c0 + (MODE == 5 ? 1 : 0);
+        bv[0] = value(set, k);
+        if (nc > 1) bv[1] = value(set, k + 1);
       }
       const int e0 = w::exponent(bv[0]), e1 = nc > 1 ? w::exponent(bv[1]) : 0, e = max(e0, e1);
       w::Limbs bl[2];
@@ -785,38 +725,39 @@ __device__ __forceinline__ void deposit_tile_wide(const Batch& B, int b, int til
       }
       // the sums' exponent
       const int es = ko <= w::kMaxExcess ? et + ko : w::kExpNonFinite;
-      if (es + head > ea[q]) {
-        const int sh = es + head - ea[q], sf = max(sh - 32, 0);
-        ea[q] += sh;
+      if (es + head > ea[sq]) {
+        const int sh = es + head - ea[sq], sf = max(sh - 32, 0);
+        ea[sq] += sh;
 #pragma unroll
         for (int c = 0; c < nc; ++c) {
 #pragma unroll
-          for (int m = 0; m < 4; ++m) acc[m * kNC + c0 + c] = w::align(acc[m * kNC + c0 + c], sh, sf);
+          for (int m = 0; m < D::MOM; ++m) acc[m * D::COMP + r0 + c] = w::align(acc[m * D::COMP + r0 + c], sh, sf);
         }
       }
-      const int dd = ea[q] - es, df = max(dd - 32, 0);
+      const int dd = ea[sq] - es, df = max(dd - 32, 0);
 #pragma unroll
       for (int c = 0; c < nc; ++c) {
         const int64_t v = w::align(cv[c], dd, df);
         const w::Limbs l = w::split(v);
-        acc[c0 + c] += w::align(v, 2 + ko, 0);
+        acc[r0 + c] += w::align(v, 2 + ko, 0);
 #pragma unroll
-        for (int m = 0; m < 3; ++m)
-          acc[(m + 1) * kNC + c0 + c] = w::mul_add(l, om[m], acc[(m + 1) * kNC + c0 + c]);
+        for (int m = 1; m < D::MOM; ++m)
+          acc[m * D::COMP + r0 + c] = w::mul_add(l, om[m - 1], acc[m * D::COMP + r0 + c]);
       }
     }
   }
   // acc 2^(ea + 4 - kBiasV)
 #pragma unroll
-  for (int q = 0; q < kGroups; ++q) {
-    const int nc = q < 2 ? 1 : 2, c0 = q < 2 ? q : 2 * q - 2;
-    const int k = min(max(ea[q] + 4 - w::kBiasV, -1022), 959);
+  for (int sq = 0; sq < D::SETS * D::GROUPS; ++sq) {
+    const int set = sq / D::GROUPS, q = sq % D::GROUPS, nc = q < D::SINGLE ? 1 : 2;
+    const int r0 = set * D::MOM * D::COMP + (q < D::SINGLE ? q : 2 * q - D::SINGLE);
+    const int k = min(max(ea[sq] + 4 - w::kBiasV, -1022), 959);
 #pragma unroll
     for (int c = 0; c < nc; ++c) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const double v = (double)acc[m * kNC + c0 + c];
-        out[m * kNC + c0 + c] = ea[q] >= w::kExpNonFinite ? nan("") : w::scale_nz(v, k);
+      for (int m = 0; m < D::MOM; ++m) {
+        const double v = (double)acc[m * D::COMP + r0 + c];
+        out[m * D::COMP + r0 + c] = ea[sq] >= w::kExpNonFinite ? nan("") : w::scale_nz(v, k);
       }
     }
   }
@@ -858,16 +799,9 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
     const int64_t ubase = g.uoff + (int64_t)tile * M;
     const int dfirst = (int)(u - ubase), dlast = (int)(uend - ubase);
     u = uend;
-    constexpr int NA = MODE == 5 ? kNT : kNA;
-    double acc[NA];
-#pragma unroll
-    for (int c = 0; c < NA; ++c) acc[c] = 0.0;
-    if constexpr (MODE == 5)
-      deposit_tile_wide<ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow, frac,
-                                    W, buf, B.U > B.nw, acc, bad);
-    else
-      deposit_tile_dirs<MODE, ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow,
-                                          frac, W, acc, bad);
+    double acc[DepMode<MODE>::NA];
+    deposit_tile<MODE, ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow, frac, W,
+                                   buf, B.U > B.nw, acc, bad);
     constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T;
     flush_tile<ORDER>(acc, g.toff + tile, tile * T - H + lane, g.nz, w, lane, partial);
   }
@@ -882,7 +816,7 @@ k_deposit(Batch B, const double* __restrict__ z, const double* __restrict__ N, c
           const double* __restrict__ r_nu, const double* __restrict__ r_nb, const double* __restrict__ dirtab,
           const int* __restrict__ shift, const double* __restrict__ wrow, double frac, double* __restrict__ partial,
           double* __restrict__ W, int* __restrict__ err) {
-  extern __shared__ double dep_sm[];   // (MODE 5: kDepSmem bytes)
+  extern __shared__ double dep_sm[];   // kDepSmem bytes (half with one buffer)
   griddep_wait();
   deposit_phase<MODE, ORDER, false>(B, logical_warp(), threadIdx.x & 31, z, N, Nbar, r_nu, r_nb, dirtab, shift,
                                     TAB ? wrow : nullptr, frac, partial, W, err, dep_sm + (threadIdx.x >> 5) * (B.U > B.nw ? kDepBuf : kDepBuf / 2));
@@ -968,8 +902,8 @@ k_deposit_cluster(Batch B, const double* __restrict__ z, const double* __restric
 #pragma unroll
     for (int c = 0; c < kNT; ++c) acc[c] = 0.0;
     if (d0 < d1)
-      deposit_tile_wide<ORDER, false>(B, b, tile, d0, d1, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                      TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, 1, acc, bad);
+      deposit_tile<5, ORDER, false>(B, b, tile, d0, d1, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
+                                    TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, 1, acc, bad);
 #pragma unroll
     for (int c = 0; c < kNT; ++c) red[wib * kDepBuf + c * kLanes + lane] = acc[c];
     __syncthreads();
