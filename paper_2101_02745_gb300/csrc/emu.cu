@@ -177,7 +177,8 @@ struct Layout {
   size_t frame = 0; // step form 2: the frame sums of every 32-cell tile (k_frame_sum)
   size_t bw3 = 0;   // 3D boxes: 8-component field of every (direction, cell): B, its spread passes (k3_prep, k3_pass)
   size_t gf3 = 0;   // 3D boxes: a second such field: G = A0 - Omega . A and its gather passes (k3_gfield, k3_pass)
-  size_t wdir3 = 0; // 3D boxes: every direction's shape weights per stage and axis (k3_shifts)
+  size_t wdir3 = 0; // 3D boxes: every direction's shape weights per stage and axis, and Omega, as operands (k3_shifts)
+  size_t ae3 = 0;   // 3D boxes: exponents of the potential's operands (At holds the operands)
 };
 
 Layout layout(const Shape& S) {
@@ -1199,9 +1200,10 @@ Layout layout3(const Shape& S, size_t nrows) {
   L.diag = take(sizeof(double) * 63);
   L.scalar = take(sizeof(double) * 4);
   L.rowgeo = take(sizeof(BoxGeo) * nrows);
-  L.bw3 = take(sizeof(double) * (size_t)kNC * (size_t)S.Ptot);
-  L.gf3 = take(sizeof(double) * (size_t)kNC * (size_t)S.Ptot);
-  L.wdir3 = take(sizeof(double) * 4 * 3 * 5 * MT);
+  L.bw3 = take(sizeof(int2) * (size_t)(kNC + 1) * (size_t)S.Ptot);   // (operands, and their exponents)
+  L.gf3 = take(sizeof(int2) * (size_t)(kNC + 1) * (size_t)S.Ptot);
+  L.wdir3 = take(sizeof(int2) * kOpRows * MT);
+  L.ae3 = take(sizeof(int2) * NZ);
   L.total = off;
   return L;
 }
@@ -1254,7 +1256,7 @@ Batch row_view(const emu_box* b) {
 int launch3_shifts(emu_box* b, const double* fracs, int nrows) {
   Fracs f{};
   for (int s = 0; s < nrows; ++s) f.v[s] = fracs[s];
-  double* wtab = (double*)(b->ws + b->L.wdir3);
+  int2* wtab = (int2*)(b->ws + b->L.wdir3);
   before_launch(b, CLS_SHIFT);
   by_order(b->S.order, [&](auto O) {
     pdl(b->stream, k3_shifts<decltype(O)::value>, dim3((unsigned)((b->c3.ndir + kThreads - 1) / kThreads)),
@@ -1265,13 +1267,18 @@ int launch3_shifts(emu_box* b, const double* fracs, int nrows) {
 }
 
 // The stage's rows of the direction weight table (k3_shifts).
-const double* wrow3(const emu_box* b, int s) {
-  return (const double*)(b->ws + b->L.wdir3) + (size_t)(s - 1) * 3 * 5 * b->S.MT;
+const int2* wrow3(const emu_box* b, int s) {
+  return (const int2*)(b->ws + b->L.wdir3) + (size_t)(s - 1) * 3 * 5 * b->S.MT;
+}
+// The two fields the separable passes write in turn.
+Field3 field3(const emu_box* b, size_t at) {
+  int2* f = (int2*)(b->ws + at);
+  return Field3{f, f + (size_t)kNC * b->S.Ptot};
 }
 
 // One separable pass (k3_pass) over every (direction, cell).
 template <int AXIS, bool SPREAD>
-int launch3_pass(emu_box* b, const double* in, const double* wrow, double* out) {
+int launch3_pass(emu_box* b, Field3 in, const int2* wrow, Field3 out) {
   before_launch(b, CLS_OTHER);
   by_order(b->S.order, [&](auto O) {
     pdl(b->stream, k3_pass<decltype(O)::value, AXIS, SPREAD>, dim3((unsigned)((b->S.Ptot + kThreads - 1) / kThreads)),
@@ -1317,12 +1324,16 @@ int launch3_deposit(emu_box* b, int mode, const double* rnu, const double* rnb, 
 // (along z, commutators, RK update).
 int launch3_rk(emu_box* b, int s, const int* srow, int dry) {
   const Box3 v = box3_view(b);
-  double* F0 = (double*)(b->ws + b->L.bw3);
-  double* F1 = (double*)(b->ws + b->L.gf3);
-  const double* wrow = wrow3(b, s);
+  const Field3 F0 = field3(b, b->L.bw3), F1 = field3(b, b->L.gf3);
+  const int2* wrow = wrow3(b, s);
+  const int2* ops = wrow3(b, 1);
+  int2* At = (int2*)b->At;
+  int2* Ae = (int2*)(b->ws + b->L.ae3);
   before_launch(b, CLS_OTHER);
-  pdl(b->stream, k3_gfield, dim3((unsigned)((b->S.Ptot + kThreads - 1) / kThreads)), v, (const double*)b->At,
-      (const double*)b->dirtab, F1);
+  // (enough threads for two blocks per SM, at most one per direction and cell)
+  const int64_t cb = ((int64_t)v.C + kThreads - 1) / kThreads, want = (2 * kPersistBlocks + cb - 1) / cb;
+  pdl(b->stream, k3_gfield, dim3((unsigned)cb, (unsigned)std::min<int64_t>(want, std::min(v.M, 65535))), v,
+      (const int2*)At, (const int2*)Ae, ops, F1);
   if (int rc = after_launch(b, "3D G field kernel")) return rc;
   if (int rc = launch3_pass<0, false>(b, F1, wrow, F0)) return rc;
   if (int rc = launch3_pass<1, false>(b, F0, wrow, F1)) return rc;
@@ -1331,7 +1342,7 @@ int launch3_rk(emu_box* b, int s, const int* srow, int dry) {
     constexpr int R = decltype(O)::value;
     by_stage(b->pot, s, [&](auto POT, auto STAGE) {
       pdl(b->stream, k3_rk_stage<decltype(POT)::value, R, decltype(STAGE)::value>, persist_grid(b), v, b->pt, b->x3,
-          b->y3, b->dirtab, srow, (const double*)F1, wrow, s, dry);
+          b->y3, b->dirtab, srow, F1, wrow, s, dry);
     });
     return 0;
   });
@@ -1346,9 +1357,11 @@ int launch3_step_deposit(emu_box* b, int s, const int* srow) {
   const size_t P = (size_t)b->S.Ptot;
   const double* rnu = (s == 1) ? b->pt.rho : b->pt.stage;
   const double* rnb = (s == 1) ? b->pt.rhobar : b->pt.stage + 9 * P;
-  double* F0 = (double*)(b->ws + b->L.bw3);
-  double* F1 = (double*)(b->ws + b->L.gf3);
-  const double* wrow = wrow3(b, s);
+  const Field3 F0 = field3(b, b->L.bw3), F1 = field3(b, b->L.gf3);
+  const int2* wrow = wrow3(b, s);
+  const int2* ops = wrow3(b, 1);
+  int2* At = (int2*)b->At;
+  int2* Ae = (int2*)(b->ws + b->L.ae3);
   const Box3 v = box3_view(b);
   before_launch(b, CLS_OTHER);
   pdl(b->stream, k3_prep, dim3((unsigned)((P + kThreads - 1) / kThreads)), v, (const double*)b->x3,
@@ -1359,8 +1372,8 @@ int launch3_step_deposit(emu_box* b, int s, const int* srow) {
   if (int rc = launch3_pass<1, true>(b, F1, wrow, F0)) return rc;
   before_launch(b, CLS_DEPOSIT);
   by_order(b->S.order, [&](auto O) {
-    pdl(b->stream, k3_spread_x_sum<decltype(O)::value>, dim3((unsigned)((v.C + kThreads - 1) / kThreads)), v,
-        (const double*)F0, wrow, (const double*)b->dirtab, b->At, b->err);
+    pdl(b->stream, k3_spread_x_sum<decltype(O)::value>, dim3((unsigned)((v.C + kThreads - 1) / kThreads), 2), v,
+        F0, wrow, ops, At, Ae, b->err);
     return 0;
   });
   return after_launch(b, "3D deposit sum kernel");

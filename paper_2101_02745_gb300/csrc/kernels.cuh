@@ -183,6 +183,10 @@ __device__ __forceinline__ int box_of_direction(const Batch& B, int d) {
   return lo;
 }
 
+// |d| >= 1/2 (or NaN) from the upper word: the FP64 comparison of the lattice
+// test, one more instruction of the FP64 pipe, only behind it.
+__device__ __forceinline__ bool half_or_more(double d) { return (__double2hiint(d) & 0x7fffffff) >= 0x3fe00000; }
+
 // Shape weights (Sec. 2.2.1) of order ORDER of a particle at (unwrapped)
 // position zs whose lattice site is cell h (hp = h + 1/2): the offset
 // d = zs/dz - hp, reduced to the nearest periodic image, lies in [-1/2, 1/2),
@@ -201,7 +205,7 @@ __device__ __forceinline__ int shape_weights(double zs, double hp, double inv_dz
                                              double (&w)[Sten<ORDER>::NW]) {
   double d = fma(zs, inv_dz, -hp);
   int bad = 0;
-  if (fabs(d) > 0.5 + kLatticeTol) {
+  if (half_or_more(d) && fabs(d) > 0.5 + kLatticeTol) {
     d -= nz_d * rint(d / nz_d);
     bad = fabs(d) > 0.5 + kLatticeTol;
   }
@@ -236,7 +240,7 @@ __device__ __forceinline__ int shape_weights(double zs, double hp, double inv_dz
 // off the cell whose centre is hp (in cells), up to the periodic image.
 __device__ __forceinline__ int off_site(double zs, double hp, double inv_dz, double nz_d) {
   double d = fma(zs, inv_dz, -hp);
-  if (fabs(d) > 0.5 + kLatticeTol) {
+  if (half_or_more(d) && fabs(d) > 0.5 + kLatticeTol) {
     d -= nz_d * rint(d / nz_d);
     return fabs(d) > 0.5 + kLatticeTol;
   }
@@ -1191,6 +1195,31 @@ __device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, co
   }
 }
 
+// rk_update of particle p of box g from H in the traceless components as
+// hv[c] 2^(he[c / 2] - kBiasV), |hv| < 2^60.6.
+template <bool POT, int S, bool COH>
+__device__ __forceinline__ void rk_from_H(const BoxGeo& g, const Parts& pt, const double* src_b, int64_t P, int64_t p,
+                                          int dry, double bdt, double cdt, double dtb, const double* vz,
+                                          const int64_t (&hv)[kNC], const int (&he)[4], double (&r)[9]) {
+  namespace w = emu_wide;
+  if constexpr (POT) {
+    double Hm[kNC];
+#pragma unroll
+    for (int c = 0; c < kNC; ++c)
+      Hm[c] = (double)hv[c] * w::scale(1.0, he[c >> 1] < w::kExpNonFinite ? max(he[c >> 1] - w::kBiasV, -1022) : 1024);
+    rk_particle<POT, S, COH>(g, pt, src_b, P, p, dry, bdt, cdt, dtb, vz, Hm, r);
+  } else {
+    w::Ham hm;
+    hm.d12 = w::Real{w::split(hv[0]), he[0]};
+    hm.d13 = w::Real{w::split(hv[0] + hv[1]), he[0]};
+    hm.d23 = w::Real{w::split(hv[1]), he[0]};
+    hm.a = w::Cplx{w::split(hv[2]), w::split(hv[3]), he[1]};
+    hm.b = w::Cplx{w::split(hv[4]), w::split(hv[5]), he[2]};
+    hm.c = w::Cplx{w::split(hv[6]), w::split(hv[7]), he[3]};
+    rk_update<S, false, COH>(g.Lz, pt, src_b, P, p, dry, bdt, cdt, dtb, vz, hm, hm, r);
+  }
+}
+
 // Box of tile unit x of the slabs (a pair of a slab and a direction counts as
 // its sw tile units).
 __device__ __forceinline__ int box_of_slab_unit(const Batch& B, int64_t x) {
@@ -1242,48 +1271,59 @@ struct SlabTable {
 constexpr int kSlabSmem = (int)sizeof(SlabTable<kSlabTiles>);
 constexpr int kStepSmem = kSlabSmem > kDepSmem ? kSlabSmem : kDepSmem;   // of k_step: either phase's
 
+// The operands of one exponent group of the potential at a cell: v[k] moment
+// k / 2, component k % 2 of the group; put(k, operand): A0 / 4 as an int64 (low,
+// high word; dot3's addend), limbs of A_x, A_y, A_z.  Returns their exponent.
+template <typename F>
+__device__ __forceinline__ int potential_operands(const double (&v)[8], F put) {
+  namespace w = emu_wide;
+  int e[8], top = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    e[k] = w::exponent(v[k]);
+    top = max(top, e[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const w::Limbs l = w::limbs(v[k], e[k], top);
+    int2 x = make_int2(l.h, l.l);
+    if (k < 2) {
+      const int64_t q = w::join(l) >> 2;
+      x = make_int2((int)q, (int)(q >> 32));
+    }
+    put(k, x);
+  }
+  return top;
+}
+
 // Potential of cells c0 .. c0 + n - 1 (modulo nz) of box g into the table, by
 // the whole block: one (cell, exponent group) per thread and round.
 template <bool COH, class Table>
 __device__ __forceinline__ void slab_table(Table& t, const double* A, int NZ, const BoxGeo& g, int c0, int n) {
-  namespace w = emu_wide;
   for (int q = threadIdx.x; q < 4 * n; q += kThreads) {
     const int grp = q / n, c = q - grp * n;
     const double* Aj = A + g.coff + wrapc(c0 + c, g.nz) + (int64_t)2 * grp * NZ;
     double v[8];
-    int e[8], top = 0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {   // moment k / 2, component 2 grp + k % 2
-      v[k] = ldd<COH>(Aj + (int64_t)((k >> 1) * kNC + (k & 1)) * NZ);
-      e[k] = w::exponent(v[k]);
-      top = max(top, e[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const w::Limbs l = w::limbs(v[k], e[k], top);
-      int2 x = make_int2(l.h, l.l);
-      if (k < 2) {   // A0: a quarter of the operand as an int64 (dot3's addend)
-        const int64_t q = w::join(l) >> 2;
-        x = make_int2((int)q, (int)(q >> 32));
-      }
-      t.a[(k >> 1) * kNC + 2 * grp + (k & 1)][c] = x;
-    }
-    t.e[grp][c] = top;
+    for (int k = 0; k < 8; ++k) v[k] = ldd<COH>(Aj + (int64_t)((k >> 1) * kNC + (k & 1)) * NZ);
+    t.e[grp][c] = potential_operands(
+        v, [&](int k, int2 x) { t.a[(k >> 1) * kNC + 2 * grp + (k & 1)][c] = x; });
   }
 }
 
 __device__ __forceinline__ emu_wide::Limbs limbs_of(int2 v) { return emu_wide::Limbs{v.x, v.y}; }
 
-// Component c of G = A0 - Omega . A at table cell j (o: limbs of -Omega).
-// Directions scaled by 2^-ko: so is G.
-template <class Table>
-__device__ __forceinline__ int2 table_G(const Table& t, int c, int j, const emu_wide::Limbs (&o)[3], int ko) {
-  const int2 q = t.a[c][j];
+// G = A0 - Omega . A from the operands of one component (o: limbs of -Omega;
+// directions scaled by 2^-ko: so is G); component c of it at table cell j.
+__device__ __forceinline__ int2 operand_G(int2 q, int2 a1, int2 a2, int2 a3, const emu_wide::Limbs (&o)[3], int ko) {
   const int64_t a0 = (int64_t)(((uint64_t)(uint32_t)q.y << 32) | (uint32_t)q.x);
   const emu_wide::Limbs g = emu_wide::split(
-      emu_wide::dot3(emu_wide::align(a0, ko, 0), limbs_of(t.a[kNC + c][j]), o[0], limbs_of(t.a[2 * kNC + c][j]), o[1],
-                     limbs_of(t.a[3 * kNC + c][j]), o[2]));
+      emu_wide::dot3(emu_wide::align(a0, ko, 0), limbs_of(a1), o[0], limbs_of(a2), o[1], limbs_of(a3), o[2]));
   return make_int2(g.h, g.l);
+}
+template <class Table>
+__device__ __forceinline__ int2 table_G(const Table& t, int c, int j, const emu_wide::Limbs (&o)[3], int ko) {
+  return operand_G(t.a[c][j], t.a[kNC + c][j], t.a[2 * kNC + c][j], t.a[3 * kNC + c][j], o, ko);
 }
 
 template <bool POT, int ORDER, int S, bool COH, class Table>
@@ -1471,31 +1511,14 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
             }
           }
         }
-        // hv[c] 2^(he + 2 - kBiasV) = H_c
+        // hv[c] 2^(he + 2 - kBiasV) = H_c, then he + 2 -> he
         if (ko != 0) {
 #pragma unroll
           for (int grp = 0; grp < 4; ++grp) he[grp] = ko <= w::kMaxExcess ? he[grp] + ko : w::kExpNonFinite;
         }
-        const double* vz = dirtab + 3 * MT + gd;
-        if constexpr (POT) {
-          double Hm[kNC], Hb[kNC];
 #pragma unroll
-          for (int c = 0; c < kNC; ++c)
-            Hm[c] = (double)hv[c] * w::scale(1.0, he[c >> 1] < w::kExpNonFinite ? max(he[c >> 1] + 2 - w::kBiasV, -1022)
-                                                                               : 1024);
-          add_potentials(g, Hm, Hb);
-          const w::Ham hm = w::ham(Hm), hb = w::ham(Hb);
-          rk_update<S, true, COH>(g.Lz, pt, src_b, P, p, dry, bdt, cdt, dtb, vz, hm, hb, r);
-        } else {
-          w::Ham hm;
-          hm.d12 = w::Real{w::split(hv[0]), he[0] + 2};
-          hm.d13 = w::Real{w::split(hv[0] + hv[1]), he[0] + 2};
-          hm.d23 = w::Real{w::split(hv[1]), he[0] + 2};
-          hm.a = w::Cplx{w::split(hv[2]), w::split(hv[3]), he[1] + 2};
-          hm.b = w::Cplx{w::split(hv[4]), w::split(hv[5]), he[2] + 2};
-          hm.c = w::Cplx{w::split(hv[6]), w::split(hv[7]), he[3] + 2};
-          rk_update<S, false, COH>(g.Lz, pt, src_b, P, p, dry, bdt, cdt, dtb, vz, hm, hm, r);
-        }
+        for (int grp = 0; grp < 4; ++grp) he[grp] += 2;
+        rk_from_H<POT, S, COH>(g, pt, src_b, P, p, dry, bdt, cdt, dtb, dirtab + 3 * MT + gd, hv, he, r);
       }
       __syncwarp();   // (the unit's G are rewritten by the next)
     }

@@ -97,11 +97,13 @@ static __global__ void k3_dirtable(Box3 b, Parts pt, double* __restrict__ dirtab
 // Omega; shift[(s * 3 + axis) * M + d].  With wtab, also that particle's
 // shape weights there, the direction's weights on each axis (all its
 // particles share the offset inside their cells): wtab[((s * 3 + axis) * 5 +
-// q) * M + d], q < NW.
+// q) * M + d], q < NW, as operands (unit_limbs); then the directions as
+// operands, rows 60-62 Omega and row 63 (their scale 2^-x, 0).
+constexpr int kOpRows = 64;   // rows of the operand table
 template <int ORDER>
 __global__ void k3_shifts(Box3 b, const double* __restrict__ x, const double* __restrict__ y,
                           const double* __restrict__ z, const double* __restrict__ dirtab, Fracs fr, int nrows,
-                          int* __restrict__ shift, double* __restrict__ wtab) {
+                          int* __restrict__ shift, int2* __restrict__ wtab) {
   griddep_wait();
   constexpr int NW = Sten<ORDER>::NW;
   const int d = blockIdx.x * blockDim.x + threadIdx.x;
@@ -121,11 +123,40 @@ __global__ void k3_shifts(Box3 b, const double* __restrict__ x, const double* __
         double w[NW];
         (void)shape_weights<ORDER>(xs, (double)cell + 0.5, b.inv_h[a], b.n_d[a], w);
 #pragma unroll
-        for (int q = 0; q < NW; ++q) wtab[((s * 3 + a) * 5 + q) * b.M + d] = w[q];
+        for (int q = 0; q < NW; ++q) {
+          const emu_wide::Limbs l = emu_wide::unit_limbs(w[q]);
+          wtab[((s * 3 + a) * 5 + q) * b.M + d] = make_int2(l.h, l.l);
+        }
       }
     }
   }
+  if (wtab != nullptr) {
+    const double om[3] = {dirtab[d], dirtab[b.M + d], dirtab[2 * b.M + d]};
+    const int ko = max(max(emu_wide::unit_excess(om[0]), emu_wide::unit_excess(om[1])), emu_wide::unit_excess(om[2]));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const emu_wide::Limbs l = emu_wide::unit_limbs(om[a], ko);
+      wtab[(60 + a) * b.M + d] = make_int2(l.h, l.l);
+    }
+    wtab[63 * b.M + d] = make_int2(ko, 0);
+  }
 }
+
+// A field of 8 components per (direction, cell) i = d C + cell as operands
+// (wide.cuh): limbs at f[c * P + i], and at e[i] the exponents of the diagonal
+// pair and the three complex components, 16 bits each.
+struct Field3 {
+  int2* f;
+  int2* e;
+};
+__device__ __forceinline__ int2 pack_exponents(const int (&e)[4]) {
+  return make_int2(e[0] | e[1] << 16, e[2] | e[3] << 16);
+}
+__device__ __forceinline__ void unpack_exponents(int2 v, int (&e)[4]) {
+  e[0] = v.x & 0xffff; e[1] = v.x >> 16; e[2] = v.y & 0xffff; e[3] = v.y >> 16;
+}
+// A row of the operand table at direction d.
+__device__ __forceinline__ emu_wide::Limbs operand(const int2* row, int d) { return limbs_of(__ldg(row + d)); }
 
 // Site of the particle of direction d on cell (jx, jy, jz) for shifts (sx, sy, sz).
 __device__ __forceinline__ int64_t site3(const Box3& b, int d, int jx, int jy, int jz, int sx, int sy, int sz) {
@@ -238,59 +269,127 @@ k3_deposit(Box3 b, const double* __restrict__ x, const double* __restrict__ y, c
   if (bad) atomicOr(err, ERR_LATTICE);
 }
 
+// off_site for cell j: first whether the position lies in the cell itself, from
+// the bits of its coordinate in cells (one FP64 instruction; off_site and its
+// operand take four).
+__device__ __forceinline__ int off_cell(double zs, int j, double inv_h, double n_d) {
+  const int hi = __double2hiint(zs * inv_h), e = (hi >> 20) - 1023;
+  if (hi >= 0 && e <= 20 && (int)emu_wide::shr((unsigned)(hi & 0xfffff) | 0x100000u, 20 - e) == j) return 0;
+  return off_site(zs, (double)j + 0.5, inv_h, n_d);
+}
+
 // The step's deposit (MODE 5 of k3_deposit), separable.  k3_prep: one thread
 // per particle; checks its position against the cell its site assigns at the
 // stage (ERR_LATTICE) and writes the 8 traceless components of
 // B = N rho - Nbar rhobar^* (Eq. 5) at that cell of its direction's field:
-// Bf[c * P + d * C + cell].
+// the field Bf (operands, wide.cuh: the passes that follow run on the integer
+// pipe; as FP64 sums of three taps each of them took the FP64 pipe's whole time).
 static __global__ void __launch_bounds__(kThreads)
 k3_prep(Box3 b, const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
         const double* __restrict__ N, const double* __restrict__ Nbar, const double* __restrict__ r_nu,
         const double* __restrict__ r_nb, const double* __restrict__ dirtab, const int* __restrict__ srow,
-        double frac, double* __restrict__ Bf, int* __restrict__ err) {
+        double frac, Field3 Bf, int* __restrict__ err) {
   griddep_wait();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= b.P) return;
   const int64_t P = b.P;
   const int M = b.M;
-  const int d = (int)(p / b.C);
+  const int d = (int)((unsigned)p / (unsigned)b.C);
   const int c0 = (int)(p - (int64_t)d * b.C);
   const int iz = c0 % b.n[2], iy = (c0 / b.n[2]) % b.n[1], ix = c0 / (b.n[2] * b.n[1]);
   const int jx = wrapn(ix + __ldg(srow + d), b.n[0]);
   const int jy = wrapn(iy + __ldg(srow + M + d), b.n[1]);
   const int jz = wrapn(iz + __ldg(srow + 2 * M + d), b.n[2]);
   const double pos_dt = frac * *b.dt;
-  int bad = off_site(fma(pos_dt, __ldg(dirtab + 3 * M + d), x[p]), (double)jx + 0.5, b.inv_h[0], b.n_d[0]);
-  bad |= off_site(fma(pos_dt, __ldg(dirtab + 4 * M + d), y[p]), (double)jy + 0.5, b.inv_h[1], b.n_d[1]);
-  bad |= off_site(fma(pos_dt, __ldg(dirtab + 5 * M + d), z[p]), (double)jz + 0.5, b.inv_h[2], b.n_d[2]);
+  int bad = off_cell(fma(pos_dt, __ldg(dirtab + 3 * M + d), x[p]), jx, b.inv_h[0], b.n_d[0]);
+  bad |= off_cell(fma(pos_dt, __ldg(dirtab + 4 * M + d), y[p]), jy, b.inv_h[1], b.n_d[1]);
+  bad |= off_cell(fma(pos_dt, __ldg(dirtab + 5 * M + d), z[p]), jz, b.inv_h[2], b.n_d[2]);
   const int64_t out = (int64_t)d * b.C + ((int64_t)jx * b.n[1] + jy) * b.n[2] + jz;
   const double n1 = N[p], n2 = Nbar[p];
-  double bprev = 0.0;
+  const unsigned P32 = (unsigned)P;
+  // conj(rhobar) flips the sign of the imaginary components 4, 6, 8
+  auto value = [&](int k) {
+    const double xv = *row(r_nu + p, P32, k), yv = *row(r_nb + p, P32, k);
+    return fma((k == 4 || k == 6 || k == 8) ? n2 : -n2, yv, n1 * xv);
+  };
+  double bprev = value(0);
+  int eg[4];
 #pragma unroll
-  for (int c = 0; c < kNC; ++c) {
-    double bv;
-    if (c < 2) {
-      if (c == 0) bprev = fma(-n2, r_nb[p], n1 * r_nu[p]);
-      const double bn = fma(-n2, r_nb[(c + 1) * P + p], n1 * r_nu[(c + 1) * P + p]);
-      bv = bprev - bn;
+  for (int q = 0; q < 4; ++q) {
+    double bv[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const double bn = value(q == 0 ? c + 1 : 2 * q + 1 + c);
+      bv[c] = q == 0 ? bprev - bn : bn;
       bprev = bn;
-    } else {
-      const int k = c + 1;
-      const double xv = r_nu[k * P + p], yv = r_nb[k * P + p];
-      bv = (k == 4 || k == 6 || k == 8) ? fma(n2, yv, n1 * xv) : fma(-n2, yv, n1 * xv);
     }
-    Bf[c * P + out] = bv;
+    const emu_wide::Cplx l = emu_wide::cplx(bv[0], bv[1]);
+    Bf.f[(int64_t)(2 * q) * P + out] = make_int2(l.r.h, l.r.l);
+    Bf.f[(int64_t)(2 * q + 1) * P + out] = make_int2(l.i.h, l.i.l);
+    eg[q] = l.e;
   }
+  Bf.e[out] = pack_exponents(eg);
   if (bad) atomicOr(err, ERR_LATTICE);
 }
 
-// Neighbour of cell (jx, jy, jz) at offset o along AXIS (periodic).
-template <int AXIS>
-__device__ __forceinline__ int64_t cell_along(const Box3& b, int jx, int jy, int jz, int o) {
-  if (AXIS == 0) jx = wrapn(jx + o, b.n[0]);
-  else if (AXIS == 1) jy = wrapn(jy + o, b.n[1]);
-  else jz = wrapn(jz + o, b.n[2]);
-  return ((int64_t)jx * b.n[1] + jy) * b.n[2] + jz;
+// sum_q w[q] V_q of a field's values at the sites nb, for its NG exponent groups
+// from g0 on: per component an int64 of 4 x the operands' scale / 2^64, and the
+// exponents (the largest of the taps').
+template <int NW, int BATCH, int NG = 4>
+__device__ __forceinline__ void field_taps(const Field3& in, int64_t P, int64_t base, const int (&nb)[NW],
+                                           const emu_wide::Limbs (&w)[NW], int64_t (&v)[2 * NG], int (&eg)[NG],
+                                           int g0 = 0) {
+  static_assert(NG % BATCH == 0, "whole batches");
+  // loads ahead of their use, BATCH groups of components at a time: the passes wait on them
+  int2 raw[BATCH][NW][2];
+  int e[NW][4];
+  auto load = [&](int g) {
+#pragma unroll
+    for (int q = 0; q < NW; ++q) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        raw[g % BATCH][q][c] =
+            __ldg((const int2*)row((const double*)in.f + base + nb[q], (unsigned)P, 2 * (g0 + g) + c));
+    }
+  };
+  if (NG == 4) {
+    int2 ex[NW];
+#pragma unroll
+    for (int q = 0; q < NW; ++q) ex[q] = __ldg(in.e + base + nb[q]);
+#pragma unroll
+    for (int g = 0; g < BATCH; ++g) load(g);
+#pragma unroll
+    for (int q = 0; q < NW; ++q) unpack_exponents(ex[q], e[q]);
+  } else {   // (two groups: one word of the packed exponents)
+    int ex[NW];
+#pragma unroll
+    for (int q = 0; q < NW; ++q) ex[q] = __ldg((const int*)(in.e + base + nb[q]) + (g0 >> 1));
+#pragma unroll
+    for (int g = 0; g < BATCH; ++g) load(g);
+#pragma unroll
+    for (int q = 0; q < NW; ++q) {
+      e[q][0] = ex[q] & 0xffff;
+      e[q][1] = ex[q] >> 16;
+    }
+  }
+#pragma unroll
+  for (int g = 0; g < NG; ++g) {
+    if (g > 0 && g % BATCH == 0) {
+#pragma unroll
+      for (int k = 0; k < BATCH; ++k) load(g + k);
+    }
+    eg[g] = e[0][g];
+#pragma unroll
+    for (int q = 1; q < NW; ++q) eg[g] = max(eg[g], e[q][g]);
+    v[2 * g] = v[2 * g + 1] = 0;
+#pragma unroll
+    for (int q = 0; q < NW; ++q) {
+      const int dd = eg[g] - e[q][g], df = max(dd - 32, 0);
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        v[2 * g + c] += emu_wide::align(emu_wide::mul(limbs_of(raw[g % BATCH][q][c]), w[q]), dd, df);
+    }
+  }
 }
 
 // One 3-tap (NW-tap) pass along AXIS of the 8-component field of every
@@ -298,104 +397,158 @@ __device__ __forceinline__ int64_t cell_along(const Box3& b, int jx, int jy, int
 //   SPREAD (deposit, Eq. 5): out(cell) = sum_q w_d[q] in(cell - (q - H))
 //     (a particle's weight q goes to the cell q - H away from its own);
 //   otherwise (interpolation, Eq. 6): out(cell) = sum_q w_d[q] in(cell + q - H).
-// w_d: the direction's weights on AXIS at the stage (wrow = wtab + stage rows).
+// w_d: the direction's weights on AXIS at the stage (operand table rows wrow).
+// Bound by memory: 72 bytes read (three taps, two from L1 or L2) and 72 written
+// (as FP64 sums by the FP64 pipe: 197 us for 64^3 x 16).
 template <int ORDER, int AXIS, bool SPREAD>
-__global__ void __launch_bounds__(kThreads)
-k3_pass(Box3 b, const double* __restrict__ in, const double* __restrict__ wrow, double* __restrict__ out) {
+__global__ void __launch_bounds__(kThreads, 2)
+k3_pass(Box3 b, Field3 in, const int2* __restrict__ wrow, Field3 out) {
   griddep_wait();
   constexpr int H = Sten<ORDER>::H, NW = Sten<ORDER>::NW;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t P = b.P;
   if (i >= P) return;
-  const int d = (int)(i / b.C);
-  const int cell = (int)(i - (int64_t)d * b.C);
-  const int jz = cell % b.n[2], jy = (cell / b.n[2]) % b.n[1], jx = cell / (b.n[2] * b.n[1]);
-  const double* src = in + (int64_t)d * b.C;
-  double w[NW];
-  int64_t nb[NW];
+  const int d = (int)((unsigned)i / (unsigned)b.C);
+  const int64_t base = (int64_t)d * b.C;
+  const int cell = (int)(i - base);
+  // position along AXIS and the distance of neighbours there
+  const int stride = AXIS == 0 ? b.n[1] * b.n[2] : AXIS == 1 ? b.n[2] : 1;
+  const int j = AXIS == 0 ? cell / stride : (cell / stride) % b.n[AXIS];
+  emu_wide::Limbs w[NW];
+  int nb[NW];
 #pragma unroll
   for (int q = 0; q < NW; ++q) {
-    w[q] = __ldg(wrow + ((AXIS * 5) + q) * b.M + d);
-    nb[q] = cell_along<AXIS>(b, jx, jy, jz, SPREAD ? H - q : q - H);
+    w[q] = operand(wrow + ((AXIS * 5) + q) * b.M, d);
+    const int o = SPREAD ? H - q : q - H;
+    int jn = j + o;
+    if (jn < 0 || jn >= b.n[AXIS]) jn = wrapn(jn, b.n[AXIS]);
+    nb[q] = cell + (jn - j) * stride;
   }
+  int64_t v[kNC];
+  int eg[4];
+  field_taps<NW, NW == 3 ? 4 : 2>(in, P, base, nb, w, v, eg);
 #pragma unroll
   for (int c = 0; c < kNC; ++c) {
-    const double* sc = src + c * P;
-    double v = w[0] * __ldg(sc + nb[0]);
-#pragma unroll
-    for (int q = 1; q < NW; ++q) v = fma(w[q], __ldg(sc + nb[q]), v);
-    out[c * P + i] = v;
+    const emu_wide::Limbs l = emu_wide::split(v[c] * 4);
+    out.f[(int64_t)c * P + i] = make_int2(l.h, l.l);
   }
+  out.e[i] = pack_exponents(eg);
 }
 
 // The last deposit pass: along x, summed over directions in order with
-// (1, Omega_x, Omega_y, Omega_z) into the traceless potential (thread per
-// cell): At[(m * 8 + c) * C + cell] = kappa / dV sum_d Omega~_m,d (the
-// direction's x-spread of its y- and z-spread B field).  No partial sums.
+// (1, Omega_x, Omega_y, Omega_z) into the traceless potential, kappa / dV
+// sum_d Omega~_m,d (the direction's x-spread of its y- and z-spread B field),
+// thread per cell, sums as in deposit_tile.  The potential is written as the
+// operands k3_gfield reads: At[(m * 8 + c) * C + cell], their exponents Ae[cell].
+// No partial sums.  Two threads a cell (blockIdx.y), two exponent groups each:
+// half the sums in registers, three blocks an SM instead of two.
 template <int ORDER>
-__global__ void __launch_bounds__(kThreads)
-k3_spread_x_sum(Box3 b, const double* __restrict__ in, const double* __restrict__ wrow,
-                const double* __restrict__ dirtab, double* __restrict__ At, int* __restrict__ err) {
+__global__ void __launch_bounds__(kThreads, 3)
+k3_spread_x_sum(Box3 b, Field3 in, const int2* __restrict__ wrow, const int2* __restrict__ ops,
+                int2* __restrict__ At, int2* __restrict__ Ae, int* __restrict__ err) {
   griddep_wait();
-  constexpr int H = Sten<ORDER>::H, NW = Sten<ORDER>::NW;
+  namespace w = emu_wide;
+  constexpr int H = Sten<ORDER>::H, NW = Sten<ORDER>::NW, NG = 2;
+  const int g0 = NG * blockIdx.y;   // this thread's groups g0, g0 + 1
   const int cell = blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= b.C) return;
   const int64_t P = b.P;
   const int M = b.M;
-  const int jz = cell % b.n[2], jy = (cell / b.n[2]) % b.n[1], jx = cell / (b.n[2] * b.n[1]);
-  int64_t nb[NW];
+  const int stride = b.n[1] * b.n[2], jx = cell / stride;
+  int nb[NW];
 #pragma unroll
-  for (int q = 0; q < NW; ++q) nb[q] = cell_along<0>(b, jx, jy, jz, H - q);
-  double acc[kNT];
+  for (int q = 0; q < NW; ++q) {
+    int jn = jx + H - q;
+    if (jn < 0 || jn >= b.n[0]) jn = wrapn(jn, b.n[0]);
+    nb[q] = cell + (jn - jx) * stride;
+  }
+  const int head = max(32 - __clz(M), 2) - 2;   // headroom (deposit_tile)
+  int64_t acc[4 * 2 * NG];
+  int ea[NG];
 #pragma unroll
-  for (int c = 0; c < kNT; ++c) acc[c] = 0.0;
+  for (int c = 0; c < 4 * 2 * NG; ++c) acc[c] = 0;
+#pragma unroll
+  for (int g = 0; g < NG; ++g) ea[g] = 0;
   for (int d = 0; d < M; ++d) {
-    const double ox = __ldg(dirtab + d), oy = __ldg(dirtab + M + d), oz = __ldg(dirtab + 2 * M + d);
-    double w[NW];
+    w::Limbs wl[NW];
 #pragma unroll
-    for (int q = 0; q < NW; ++q) w[q] = __ldg(wrow + q * M + d);
-    const double* src = in + (int64_t)d * b.C;
+    for (int q = 0; q < NW; ++q) wl[q] = operand(wrow + q * M, d);
+    const w::Limbs om[3] = {operand(ops + 60 * M, d), operand(ops + 61 * M, d), operand(ops + 62 * M, d)};
+    const int ko = __ldg(&ops[63 * M + d].x);
+    int64_t cv[2 * NG];
+    int eg[NG];
+    field_taps<NW, NW == 3 ? 2 : 1, NG>(in, P, (int64_t)d * b.C, nb, wl, cv, eg, g0);
 #pragma unroll
-    for (int c = 0; c < kNC; ++c) {
-      const double* sc = src + c * P;
-      double v = w[0] * __ldg(sc + nb[0]);
+    for (int g = 0; g < NG; ++g) {
+      const int es = ko <= w::kMaxExcess ? eg[g] + ko : w::kExpNonFinite;
+      if (es + head > ea[g]) {
+        const int sh = es + head - ea[g], sf = max(sh - 32, 0);
+        ea[g] += sh;
 #pragma unroll
-      for (int q = 1; q < NW; ++q) v = fma(w[q], __ldg(sc + nb[q]), v);
-      acc[c] += v;
-      acc[kNC + c] = fma(ox, v, acc[kNC + c]);
-      acc[2 * kNC + c] = fma(oy, v, acc[2 * kNC + c]);
-      acc[3 * kNC + c] = fma(oz, v, acc[3 * kNC + c]);
+        for (int c = 2 * g; c < 2 * g + 2; ++c) {
+#pragma unroll
+          for (int m = 0; m < 4; ++m) acc[m * 2 * NG + c] = w::align(acc[m * 2 * NG + c], sh, sf);
+        }
+      }
+      const int dd = ea[g] - es, df = max(dd - 32, 0);
+#pragma unroll
+      for (int c = 2 * g; c < 2 * g + 2; ++c) {
+        const int64_t v = w::align(cv[c], dd, df);
+        const w::Limbs l = w::split(v);
+        acc[c] += w::align(v, 2 + ko, 0);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) acc[(m + 1) * 2 * NG + c] = w::mul_add(l, om[m], acc[(m + 1) * 2 * NG + c]);
+      }
     }
   }
-  int bad = 0;
+  int bad = 0, eo[NG];
 #pragma unroll
-  for (int c = 0; c < kNT; ++c) {
-    const double v = acc[c] * b.kappa_dV;
-    bad |= !isfinite(v);
-    At[(int64_t)c * b.C + cell] = v;
+  for (int g = 0; g < NG; ++g) {
+    const int k = min(max(ea[g] + 4 - w::kBiasV, -1022), 959);
+    double v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const double x = w::scale_nz((double)acc[(q >> 1) * 2 * NG + 2 * g + (q & 1)], k) * b.kappa_dV;
+      v[q] = ea[g] >= w::kExpNonFinite ? nan("") : x;
+      bad |= !isfinite(v[q]);
+    }
+    eo[g] = potential_operands(
+        v, [&](int q, int2 x) { At[(int64_t)((q >> 1) * kNC + 2 * (g0 + g) + (q & 1)) * b.C + cell] = x; });
   }
+  ((int*)(Ae + cell))[blockIdx.y] = eo[0] | eo[1] << 16;   // (as pack_exponents)
   if (bad) atomicOr(err, ERR_NONFINITE);
 }
 
-// G = A0 - Omega_d . A of every (direction, cell) from the traceless
-// potential, once per stage: Gf[c][d][cell] (component c, M C values each).
-// The RK stage's interpolation reads the G of its neighbour rows instead of
-// forming it for each of the (2H+1)^2 rows that need it.
-static __global__ void __launch_bounds__(kThreads)
-k3_gfield(Box3 b, const double* __restrict__ At, const double* __restrict__ dirtab, double* __restrict__ Gf) {
+// G = A0 - Omega_d . A of every (direction, cell) from the potential's operands,
+// once per stage.  Thread per cell, over the directions blockIdx.y, blockIdx.y +
+// gridDim.y, ..: a cell's 32 operands are read once.  The RK stage's
+// interpolation reads the G of its neighbour rows instead of forming it for
+// each of the (2H+1)^2 rows that need it.
+static __global__ void __launch_bounds__(kThreads, 2)
+k3_gfield(Box3 b, const int2* __restrict__ At, const int2* __restrict__ Ae, const int2* __restrict__ ops, Field3 G) {
   griddep_wait();
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t MC = (int64_t)b.M * b.C;
-  if (i >= MC) return;
-  const int d = (int)(i / b.C);
-  const int64_t cell = i - (int64_t)d * b.C;
-  const double ox = __ldg(dirtab + d), oy = __ldg(dirtab + b.M + d), oz = __ldg(dirtab + 2 * b.M + d);
-  const double* Aj = At + cell;
-  const int64_t Cn = b.C;
+  namespace w = emu_wide;
+  const int cell = blockIdx.x * blockDim.x + threadIdx.x;
+  if (cell >= b.C) return;
+  const int M = b.M;
+  int2 a[kNT];
 #pragma unroll
-  for (int c = 0; c < kNC; ++c)
-    Gf[c * MC + i] = fma(-oz, Aj[(3 * kNC + c) * Cn],
-                         fma(-oy, Aj[(2 * kNC + c) * Cn], fma(-ox, Aj[(kNC + c) * Cn], Aj[c * Cn])));
+  for (int c = 0; c < kNT; ++c) a[c] = At[(int64_t)c * b.C + cell];
+  int e[4];
+  unpack_exponents(Ae[cell], e);
+  for (int d = blockIdx.y; d < M; d += gridDim.y) {
+    const w::Limbs om[3] = {w::negate(operand(ops + 60 * M, d)), w::negate(operand(ops + 61 * M, d)),
+                            w::negate(operand(ops + 62 * M, d))};
+    const int ko = __ldg(&ops[63 * M + d].x);
+    const int64_t i = (int64_t)d * b.C + cell;
+#pragma unroll
+    for (int c = 0; c < kNC; ++c)
+      G.f[(int64_t)c * b.P + i] = operand_G(a[c], a[kNC + c], a[2 * kNC + c], a[3 * kNC + c], om, ko);
+    int eg[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) eg[g] = ko <= w::kMaxExcess ? min(e[g] + 2 + ko, w::kExpNonFinite) : w::kExpNonFinite;
+    G.e[i] = pack_exponents(eg);
+  }
 }
 
 // H of the lane's particle (traceless components, Eq. 6 then Eq. 2): its
@@ -440,8 +593,7 @@ __device__ __forceinline__ void interp3(const Box3& b, const double* A, int jx, 
 template <bool POT, int ORDER, int S>   // S: as rk_update's
 __global__ void __launch_bounds__(kThreads, 2)
 k3_rk_stage(Box3 b, Parts pt, double* __restrict__ x, double* __restrict__ y, const double* __restrict__ dirtab,
-            const int* __restrict__ srow, const double* __restrict__ Gxy, const double* __restrict__ wrow, int s,
-            int dry) {
+            const int* __restrict__ srow, Field3 Gxy, const int2* __restrict__ wrow, int s, int dry) {
   griddep_wait();
   constexpr int H = Sten<ORDER>::H, NW = Sten<ORDER>::NW;
   const int lane = threadIdx.x & 31;
@@ -464,27 +616,25 @@ k3_rk_stage(Box3 b, Parts pt, double* __restrict__ x, double* __restrict__ y, co
     if (jz >= nz) continue;
     const double vx = __ldg(dirtab + 3 * M + d), vy = __ldg(dirtab + 4 * M + d);
     const int64_t p = site3(b, d, jx, jy, jz, __ldg(srow + d), __ldg(srow + M + d), __ldg(srow + 2 * M + d));
-    double wz[NW];
-#pragma unroll
-    for (int q = 0; q < NW; ++q) wz[q] = __ldg(wrow + (2 * 5 + q) * M + d);
-    const double* G = Gxy + (int64_t)d * b.C + (int64_t)row * nz;
-    int cz[NW];   // the stencil's z cells, cell jz + q - H (periodic)
-#pragma unroll
-    for (int q = 0; q < NW; ++q) cz[q] = wrapn(jz + q - H, nz);
-    double Hm[kNC];
-#pragma unroll
-    for (int c = 0; c < kNC; ++c) {   // (the taps in gather's order)
-      const double* Gc = G + c * P;
-      double h = wz[NW - 1] * __ldg(Gc + cz[NW - 1]);
-#pragma unroll
-      for (int q = NW - 2; q >= 0; --q) h = fma(wz[q], __ldg(Gc + cz[q]), h);
-      Hm[c] = h;
-    }
     double r[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) r[k] = src_r[k * P + p];
-    rk_particle<POT, S, false>(*b.g, pt, src_b, P, p, dry, bdt, cdt, dt, dirtab + 5 * M + d, Hm, r);
-    if (s == 4) {   // x and y move as z does (rk_particle moved z; dry: into the RK scratch)
+    for (int k = 0; k < 9; ++k) r[k] = *emu_dev::row(src_r + p, (unsigned)P, k);
+    emu_wide::Limbs wz[NW];
+#pragma unroll
+    for (int q = 0; q < NW; ++q) wz[q] = operand(wrow + (2 * 5 + q) * M, d);
+    int cz[NW];   // the stencil's z cells, cell jz + q - H (periodic)
+#pragma unroll
+    for (int q = 0; q < NW; ++q) {
+      const int jn = jz + q - H;
+      cz[q] = row * nz + (jn < 0 || jn >= nz ? wrapn(jn, nz) : jn);
+    }
+    int64_t hv[kNC];
+    int he[4];
+    field_taps<NW, 2>(Gxy, P, (int64_t)d * b.C, cz, wz, hv, he);
+#pragma unroll
+    for (int c = 0; c < kNC; ++c) hv[c] *= 4;
+    rk_from_H<POT, S, false>(*b.g, pt, src_b, P, p, dry, bdt, cdt, dt, dirtab + 5 * M + d, hv, he, r);
+    if (S == 4) {   // x and y move as z does (rk_update moved z; dry: into the RK scratch)
       const double xn = wrap_z(fma(dt, vx, x[p]), b.L[0]), yn = wrap_z(fma(dt, vy, y[p]), b.L[1]);
       if (dry) { pt.acc[p] = xn; pt.acc[P + p] = yn; }
       else { x[p] = xn; y[p] = yn; }
