@@ -173,7 +173,8 @@ struct Layout {
   // particles anywhere (kernels_general.cuh): sort keys and values (two of
   // each), digit histogram, cell starts, lattice-check flag
   size_t gkeys = 0, gkeys2 = 0, gids = 0, gids2 = 0, ghist = 0, gstart = 0, gflag = 0;
-  size_t gprep = 0;  // particles anywhere: B (8) and Omega (3) of every particle in sorted order (k_gprep)
+  size_t gprep = 0;  // particles anywhere: B (8), Omega (3) and exponents of every particle in sorted order (k_gprep)
+  size_t gae = 0;    // particles anywhere: exponents of the potential's operands (At holds the operands)
   size_t frame = 0; // step form 2: the frame sums of every 32-cell tile (k_frame_sum)
   size_t bw3 = 0;   // 3D boxes: 8-component field of every (direction, cell): B, its spread passes (k3_prep, k3_pass)
   size_t gf3 = 0;   // 3D boxes: a second such field: G = A0 - Omega . A and its gather passes (k3_gfield, k3_pass)
@@ -214,7 +215,8 @@ Layout layout(const Shape& S) {
   L.ghist = take(sizeof(int) * kRadixBuckets * (nblk ? nblk : 1));
   L.gstart = take(sizeof(int) * ((size_t)NZ + 1));
   L.gflag = take(sizeof(int));
-  L.gprep = take(sizeof(double) * (size_t)(kNC + 3) * P);
+  L.gprep = take(sizeof(int2) * (size_t)(kNC + 4) * P);
+  L.gae = take(sizeof(int2) * NZ);
   L.total = off;
   return L;
 }
@@ -1486,12 +1488,12 @@ int launch_gstep_deposit(emu_box* b, const double* rnu, const double* rnb, doubl
   const Batch B = batch_view(b);
   const int64_t P = b->S.Ptot;
   const int* start = (const int*)(b->ws + b->L.gstart);
-  double* Bs = (double*)(b->ws + b->L.gprep);
-  double* Os = Bs + (size_t)kNC * P;
+  int2* base = (int2*)(b->ws + b->L.gprep);
+  const Sorted sorted{base, base + (size_t)kNC * P, base + (size_t)(kNC + 3) * P};
   before_launch(b, CLS_OTHER);
   by_order(b->S.order, [&](auto O) {
     pdl(b->stream, k_gprep<decltype(O)::value>, dim3((unsigned)((P + kThreads - 1) / kThreads)), B, b->pt, rnu, rnb,
-        frac, ids, b->W, Bs, Os, b->err);
+        frac, ids, (int2*)b->W, sorted, b->err);
     return 0;
   });
   if (int rc = after_launch(b, "deposit prep kernel (particles anywhere)")) return rc;
@@ -1499,8 +1501,8 @@ int launch_gstep_deposit(emu_box* b, const double* rnu, const double* rnb, doubl
   before_launch(b, CLS_DEPOSIT);
   by_order(b->S.order, [&](auto O) {
     pdl(b->stream, k_gdeposit_sorted<decltype(O)::value>,
-        dim3((unsigned)(nb < 8 * kPersistBlocks ? nb : 8 * kPersistBlocks)), B, (const double*)b->W,
-        (const double*)Bs, (const double*)Os, start, b->At, b->err);
+        dim3((unsigned)(nb < 8 * kPersistBlocks ? nb : 8 * kPersistBlocks)), B, (const int2*)b->W, sorted, start,
+        (int2*)b->At, (int2*)(b->ws + b->L.gae), b->err);
     return 0;
   });
   return after_launch(b, "deposit kernel (particles anywhere)");
@@ -1517,7 +1519,7 @@ int launch_gstage(emu_box* b, int s, int dry) {
     const dim3 grid((unsigned)((P + kThreads - 1) / kThreads));
     by_stage(b->pot, s, [&](auto POT, auto STAGE) {
       pdl(b->stream, k_grk_stage<decltype(POT)::value, R, decltype(STAGE)::value>, grid, batch_view(b), b->pt,
-          (const double*)b->At, s, dry);
+          (const int2*)b->At, (const int2*)(b->ws + b->L.gae), s, dry);
     });
     return 0;
   });

@@ -14,7 +14,7 @@
 #define EMU_RK_OTHER(X, POT, R, S)                                                                                  \
   X template __global__ void k3_rk_stage<POT, R, S>(Box3, Parts, double*, double*, const double*, const int*,       \
                                                     Field3, const int2*, int, int);                                 \
-  X template __global__ void k_grk_stage<POT, R, S>(Batch, Parts, const double*, int, int);
+  X template __global__ void k_grk_stage<POT, R, S>(Batch, Parts, const int2*, const int2*, int, int);
 #define EMU_RK_DEPOSIT(X, POT, R, S)                                                                                \
   X template __global__ void k_rk_deposit<POT, R, S>(Batch, Parts, double*, const double*, const int*,              \
                                                      const double*, int, double*, int*);

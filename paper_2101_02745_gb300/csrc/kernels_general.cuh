@@ -268,15 +268,21 @@ k_gdeposit(Batch B, Parts pt, const double* __restrict__ r_nu, const double* __r
 // The step's deposit (MODE 5) in two parts.  k_gprep: one thread per sorted
 // position i (particle p = ids[i]): its weights at its stage position (as
 // k_gdeposit forms them), the 8 traceless components of B = N rho - Nbar
-// rhobar^* (Eq. 5) and its direction, stored in sorted order (Ws[q][i],
-// Bs[c][i], Os[a][i]) so that the deposit reads each particle's data once per
-// stage and contiguously instead of forming it for every cell that gathers it.
+// rhobar^* (Eq. 5) and its direction, as operands (wide.cuh) in sorted order
+// (Ws[q][i], S.b[c][i], S.o[a][i]), so that the deposit reads each particle's
+// data once per stage and contiguously instead of forming it for every cell
+// that gathers it.
+struct Sorted {
+  int2* b;   // [kNC][P] B
+  int2* o;   // [3][P] Omega 2^-ko
+  int2* e;   // [P] exponents of B (diagonal pair, three complex components), 16 bits each; ko in bits 11-15
+};
 template <int ORDER>
 __global__ void __launch_bounds__(kThreads)
 k_gprep(Batch B, Parts pt, const double* __restrict__ r_nu, const double* __restrict__ r_nb, double frac,
-        const int* __restrict__ ids, double* __restrict__ Ws, double* __restrict__ Bs, double* __restrict__ Os,
-        int* __restrict__ err) {
+        const int* __restrict__ ids, int2* __restrict__ Ws, Sorted S, int* __restrict__ err) {
   griddep_wait();
+  namespace w = emu_wide;
   constexpr int NW = Sten<ORDER>::NW, NWS = Sten<ORDER>::NWS;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t P = B.Ptot;
@@ -284,51 +290,64 @@ k_gprep(Batch B, Parts pt, const double* __restrict__ r_nu, const double* __rest
   const int64_t p = ids[i];
   const int b = box_of_particle(B, p);
   const BoxGeo& g = B.box[b];
-  const double ox = pt.ox[p], oy = pt.oy[p], oz = pt.oz[p];
-  const double zs = fma(frac * B.dt[b], g.c_light * oz, pt.z[p]);
+  const double om[3] = {pt.ox[p], pt.oy[p], pt.oz[p]};
+  const double zs = fma(frac * B.dt[b], g.c_light * om[2], pt.z[p]);
   const int h = wrapc((int)floor(zs * g.inv_dz), g.nz);
   double wt[NW];
   const int bad = shape_weights<ORDER>(zs, (double)h + 0.5, g.inv_dz, g.nz_d, wt);
+  auto put = [](int2* dst, w::Limbs l) { *dst = make_int2(l.h, l.l); };
 #pragma unroll
-  for (int q = 0; q < NWS; ++q) Ws[q * P + i] = wt[q];
-  Os[i] = ox;
-  Os[P + i] = oy;
-  Os[2 * P + i] = oz;
+  for (int q = 0; q < NWS; ++q) put(Ws + q * P + i, w::unit_limbs(wt[q]));
+  int ko = max(max(w::unit_excess(om[0]), w::unit_excess(om[1])), w::unit_excess(om[2]));
+#pragma unroll
+  for (int a = 0; a < 3; ++a) put(S.o + a * P + i, w::unit_limbs(om[a], ko));
   const double n1 = pt.N[p], n2 = pt.Nbar[p];
-  double bprev = 0.0;
+  // conj(rhobar) flips the sign of the imaginary components 4, 6, 8
+  auto value = [&](int k) {
+    const double xv = *row(r_nu + p, (unsigned)P, k), yv = *row(r_nb + p, (unsigned)P, k);
+    return fma((k == 4 || k == 6 || k == 8) ? n2 : -n2, yv, n1 * xv);
+  };
+  double bprev = value(0);
+  int eg[4];
 #pragma unroll
-  for (int c = 0; c < kNC; ++c) {
-    double bv;
-    if (c < 2) {
-      if (c == 0) bprev = fma(-n2, r_nb[p], n1 * r_nu[p]);
-      const double bn = fma(-n2, r_nb[(c + 1) * P + p], n1 * r_nu[(c + 1) * P + p]);
-      bv = bprev - bn;
+  for (int q = 0; q < 4; ++q) {
+    double bv[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const double bn = value(q == 0 ? c + 1 : 2 * q + 1 + c);
+      bv[c] = q == 0 ? bprev - bn : bn;
       bprev = bn;
-    } else {
-      const int k = c + 1;
-      const double xv = r_nu[k * P + p], yv = r_nb[k * P + p];
-      bv = (k == 4 || k == 6 || k == 8) ? fma(n2, yv, n1 * xv) : fma(-n2, yv, n1 * xv);
     }
-    Bs[c * P + i] = bv;
+    const w::Cplx l = w::cplx(bv[0], bv[1]);
+    put(S.b + (int64_t)(2 * q) * P + i, l.r);
+    put(S.b + (int64_t)(2 * q + 1) * P + i, l.i);
+    eg[q] = ko <= w::kMaxExcess ? l.e : w::kExpNonFinite;
   }
+  if (ko > w::kMaxExcess) ko = 0;
+  S.e[i] = make_int2(eg[0] | ko << 11 | eg[1] << 16, eg[2] | eg[3] << 16);
   if (bad) atomicOr(err, ERR_LATTICE);
 }
 
 // The step's deposit from k_gprep's sorted data: kGSplit warps per global
 // cell (one group of warps of a block), warp k of a group taking every
-// kGSplit-th run of 32 particles of each source cell; each warp's sums are
-// added over its lanes in a fixed order (a transpose through shared memory)
-// and the group's warps in warp order: no float atomics, the same order on
-// every run.
-// out as k_gdeposit<5>: the traceless potential (kNT rows x NZ, kappa / dV).
+// kGSplit-th run of 32 particles of each source cell.  A lane's sums are
+// fixed-point as in deposit_tile, with headroom for all particles the cell
+// gathers; at the end the lanes', then the warps' sums are shifted to their
+// largest exponent and added as integers (through a transpose in shared
+// memory): exact, no float atomics, the same result on every run.
+// The traceless potential (kappa / dV) is written as the operands the RK stage
+// reads: At[(m * 8 + c) * NZ + cell], their exponents Ae[cell].
+// (As FP64 sums 35 instructions a visit, 102 us for 387072 particles in 1024
+// cells, bound by the FP64 pipe.)
 constexpr int kGSplit = 4;
 template <int ORDER>
-__global__ void __launch_bounds__(kThreads)
-k_gdeposit_sorted(Batch B, const double* __restrict__ Ws, const double* __restrict__ Bs,
-                  const double* __restrict__ Os, const int* __restrict__ start, double* __restrict__ out,
-                  int* __restrict__ err) {
-  __shared__ double part[kWarps][kNT];
-  __shared__ double tr[kWarps][kLanes][17];   // a warp's sums, 16 rows at a time (padded: no bank conflicts)
+__global__ void __launch_bounds__(kThreads, 2)
+k_gdeposit_sorted(Batch B, const int2* __restrict__ Ws, Sorted S, const int* __restrict__ start, int2* __restrict__ At,
+                  int2* __restrict__ Ae, int* __restrict__ err) {
+  namespace w = emu_wide;
+  __shared__ int64_t part[kWarps][kNT];
+  __shared__ int parte[kWarps][4];
+  __shared__ int64_t tr[kWarps][kLanes][17];   // a warp's sums, 16 rows at a time (padded: no bank conflicts)
   griddep_wait();
   constexpr int H = Sten<ORDER>::H;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -339,30 +358,69 @@ k_gdeposit_sorted(Batch B, const double* __restrict__ Ws, const double* __restri
   // every block runs the same number of rounds (it synchronises inside)
   for (int64_t base = (int64_t)blockIdx.x * kGroups; base < B.NZ; base += (int64_t)gridDim.x * kGroups) {
     const int64_t gc = base + grp;
-    double acc[kNT];
+    int64_t acc[kNT];
+    int ea[4];
 #pragma unroll
-    for (int c = 0; c < kNT; ++c) acc[c] = 0.0;
+    for (int c = 0; c < kNT; ++c) acc[c] = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) ea[q] = 0;
     const BoxGeo* g = nullptr;
     if (gc < B.NZ) {
       g = &B.box[box_of_cell(B, (int)gc)];
       const int j = (int)gc - g->coff;
+      int n = 0;   // particles the cell gathers
+      for (int o = -H; o <= H; ++o) {
+        const int sc = g->coff + wrapc(j - o, g->nz);
+        n += start[sc + 1] - start[sc];
+      }
+      const int head = max(32 - __clz(n), 2) - 2;   // headroom (deposit_tile)
       for (int o = -H; o <= H; ++o) {           // source cells j - o: their particles' weight slot H + o
         if (ORDER == 0 && o != 0) continue;
         const int sc = g->coff + wrapc(j - o, g->nz);
         const int i0 = start[sc], i1 = start[sc + 1];
         for (int i = i0 + k * kLanes + lane; i < i1; i += kGSplit * kLanes) {
-          const double w = ORDER == 0 ? 1.0 : __ldg(Ws + (int64_t)(H + o) * P + i);
-          const double wx = w * __ldg(Os + i), wy = w * __ldg(Os + P + i), wz = w * __ldg(Os + 2 * P + i);
+          w::Limbs wl{0, 0};
+          if (ORDER > 0) wl = limbs_of(__ldg(Ws + (int64_t)(H + o) * P + i));
+          const w::Limbs om[3] = {limbs_of(__ldg(S.o + i)), limbs_of(__ldg(S.o + P + i)),
+                                  limbs_of(__ldg(S.o + 2 * P + i))};
+          const int2 ex = __ldg(S.e + i);
+          const int ko = (ex.x >> 11) & 31, e[4] = {ex.x & 0x7ff, ex.x >> 16, ex.y & 0xffff, ex.y >> 16};
 #pragma unroll
-          for (int c = 0; c < kNC; ++c) {
-            const double bv = __ldg(Bs + (int64_t)c * P + i);
-            acc[c] = fma(w, bv, acc[c]);
-            acc[kNC + c] = fma(wx, bv, acc[kNC + c]);
-            acc[2 * kNC + c] = fma(wy, bv, acc[2 * kNC + c]);
-            acc[3 * kNC + c] = fma(wz, bv, acc[3 * kNC + c]);
+          for (int q = 0; q < 4; ++q) {
+            const int es = e[q] + ko;
+            if (es + head > ea[q]) {
+              const int sh = es + head - ea[q], sf = max(sh - 32, 0);
+              ea[q] += sh;
+#pragma unroll
+              for (int c = 2 * q; c < 2 * q + 2; ++c) {
+#pragma unroll
+                for (int m = 0; m < 4; ++m) acc[m * kNC + c] = w::align(acc[m * kNC + c], sh, sf);
+              }
+            }
+            const int dd = ea[q] - es, df = max(dd - 32, 0);
+#pragma unroll
+            for (int c = 2 * q; c < 2 * q + 2; ++c) {
+              const w::Limbs bl = limbs_of(__ldg((const int2*)row((const double*)S.b + i, (unsigned)P, c)));
+              const int64_t v = w::align(ORDER == 0 ? w::join(bl) >> 2 : w::mul(bl, wl), dd, df);
+              const w::Limbs l = w::split(v);
+              acc[c] += w::align(v, 2 + ko, 0);
+#pragma unroll
+              for (int m = 0; m < 3; ++m) acc[(m + 1) * kNC + c] = w::mul_add(l, om[m], acc[(m + 1) * kNC + c]);
+            }
           }
         }
       }
+    }
+    // the lanes' sums at the warp's largest exponent
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int top = __reduce_max_sync(kFull, ea[q]), sh = top - ea[q], sf = max(sh - 32, 0);
+#pragma unroll
+      for (int c = 2 * q; c < 2 * q + 2; ++c) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) acc[m * kNC + c] = w::align(acc[m * kNC + c], sh, sf);
+      }
+      if (lane == q) parte[wib][q] = top;
     }
     // the sum over the lanes of each of the 32 rows, 16 rows at a time through
     // shared memory: lane l adds column l mod 16 over rows 16 (l / 16) .. +15,
@@ -373,7 +431,7 @@ k_gdeposit_sorted(Batch B, const double* __restrict__ Ws, const double* __restri
       for (int c = 0; c < 16; ++c) tr[wib][lane][c] = acc[half * 16 + c];
       __syncwarp();
       const int col = lane & 15, r0 = (lane >> 4) * 16;
-      double v = tr[wib][r0][col];
+      int64_t v = tr[wib][r0][col];
 #pragma unroll
       for (int r = 1; r < 16; ++r) v += tr[wib][r0 + r][col];
       v += __shfl_down_sync(kFull, v, 16);
@@ -382,19 +440,36 @@ k_gdeposit_sorted(Batch B, const double* __restrict__ Ws, const double* __restri
     }
     __syncthreads();
     if (gc < B.NZ && k == 0) {
-      const int c = lane;   // kNT = 32 rows, one per lane
-      double v = part[wib][c];
-      for (int q = 1; q < kGSplit; ++q) v += part[wib + q][c];
-      v *= g->kappa_dV;
-      bad |= !isfinite(v);
-      out[(int64_t)c * B.NZ + gc] = v;
+      const int c = lane, q = (c & (kNC - 1)) >> 1;   // kNT = 32 rows, one per lane, and its exponent group
+      int et = parte[wib][q];
+      for (int x = 1; x < kGSplit; ++x) et = max(et, parte[wib + x][q]);
+      int64_t v = 0;
+      for (int x = 0; x < kGSplit; ++x) v += w::align(part[wib + x][c], et - parte[wib + x][q]);
+      double f = w::scale_nz((double)v, min(max(et + 4 - w::kBiasV, -1022), 959)) * g->kappa_dV;
+      if (et >= w::kExpNonFinite) f = nan("");
+      bad |= !isfinite(f);
+      // its operand at the largest exponent of its group: two components (lane
+      // bit 0) of four moments (lane bits 3, 4)
+      const int fe = w::exponent(f);
+      int top = max(fe, __shfl_xor_sync(kFull, fe, 1));
+      top = max(top, __shfl_xor_sync(kFull, top, 8));
+      top = max(top, __shfl_xor_sync(kFull, top, 16));
+      const w::Limbs l = w::limbs(f, fe, top);
+      int2 x = make_int2(l.h, l.l);
+      if (c < kNC) {   // (A0: potential_operands)
+        const int64_t a0 = w::join(l) >> 2;
+        x = make_int2((int)a0, (int)(a0 >> 32));
+      }
+      At[(int64_t)c * B.NZ + gc] = x;
+      const int t1 = __shfl_sync(kFull, top, 2), t2 = __shfl_sync(kFull, top, 4), t3 = __shfl_sync(kFull, top, 6);
+      if (lane == 0) Ae[gc] = make_int2(top | t1 << 16, t2 | t3 << 16);
     }
     __syncthreads();
   }
   if (bad) atomicOr(err, ERR_NONFINITE);
 }
 
-// H (traceless components, or all 9 with NC = 9) of particle p at its stage
+// H (NC components) of particle p at its stage
 // position from the potential A (NC rows per moment): its weights and
 // G = A0 - Omega_p . A at the cells it reaches.
 template <int ORDER, int NC>
@@ -420,11 +495,14 @@ __device__ __forceinline__ void ginterp(const BoxGeo& g, int NZ, const double* _
   }
 }
 
-// One RK4 stage of particles anywhere (as k_rk_stage): one thread per particle.
+// One RK4 stage of particles anywhere (as k_rk_stage): one thread per particle,
+// interpolating the operands of the potential at the cells it reaches.
 template <bool POT, int ORDER, int S>   // S: as rk_update's
 __global__ void __launch_bounds__(kThreads, 2)
-k_grk_stage(Batch B, Parts pt, const double* __restrict__ At, int s, int dry) {
+k_grk_stage(Batch B, Parts pt, const int2* __restrict__ At, const int2* __restrict__ Ae, int s, int dry) {
   griddep_wait();
+  namespace w = emu_wide;
+  constexpr int H = Sten<ORDER>::H, NW = Sten<ORDER>::NW;
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= B.Ptot) return;
   const int b = box_of_particle(B, p);
@@ -436,14 +514,47 @@ k_grk_stage(Batch B, Parts pt, const double* __restrict__ At, int s, int dry) {
   const double ox = pt.ox[p], oy = pt.oy[p], oz = pt.oz[p];
   const double vz = g.c_light * oz;
   const double zs = fma(stage_frac(s - 1) * dt, vz, pt.z[p]);
-  double Hm[kNC];
-  ginterp<ORDER, kNC>(g, B.NZ, At, zs, ox, oy, oz, Hm);
-  const double* src_r = (s == 1) ? pt.rho : pt.stage;
-  const double* src_b = (s == 1) ? pt.rhobar : pt.stage + 9 * P;
+  const int hc = wrapc((int)floor(zs * g.inv_dz), g.nz);
+  double wt[NW];
+  shape_weights<ORDER>(zs, (double)hc + 0.5, g.inv_dz, g.nz_d, wt);
+  const int ko = max(max(w::unit_excess(ox), w::unit_excess(oy)), w::unit_excess(oz));
+  const w::Limbs om[3] = {w::unit_limbs(-ox, ko), w::unit_limbs(-oy, ko), w::unit_limbs(-oz, ko)};
+  int cell[NW], e[NW][4], he[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int q = 0; q < NW; ++q) {
+    if (ORDER == 0 && q != H) continue;
+    cell[q] = g.coff + wrapc(hc + q - H, g.nz);
+    const int2 ex = __ldg(Ae + cell[q]);
+    e[q][0] = ex.x & 0xffff; e[q][1] = ex.x >> 16; e[q][2] = ex.y & 0xffff; e[q][3] = ex.y >> 16;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) he[c] = max(he[c], e[q][c]);
+  }
+  int64_t hv[kNC];
+#pragma unroll
+  for (int c = 0; c < kNC; ++c) hv[c] = 0;
+#pragma unroll
+  for (int q = 0; q < NW; ++q) {
+    if (ORDER == 0 && q != H) continue;
+    const int2* Aj = At + cell[q];
+    const w::Limbs wl = w::unit_limbs(wt[q]);
+#pragma unroll
+    for (int c = 0; c < kNC; ++c) {
+      const w::Limbs G = limbs_of(operand_G(__ldg(Aj + (int64_t)c * B.NZ), __ldg(Aj + (int64_t)(kNC + c) * B.NZ),
+                                            __ldg(Aj + (int64_t)(2 * kNC + c) * B.NZ),
+                                            __ldg(Aj + (int64_t)(3 * kNC + c) * B.NZ), om, ko));
+      hv[c] += w::align(w::mul(G, wl), he[c >> 1] - e[q][c >> 1]);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < kNC; ++c) hv[c] *= 4;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) he[c] = ko <= w::kMaxExcess ? he[c] + 2 + ko : w::kExpNonFinite;
+  const double* src_r = S == 1 ? pt.rho : pt.stage;
+  const double* src_b = S == 1 ? pt.rhobar : pt.stage + 9 * P;
   double r[9];
 #pragma unroll
-  for (int k = 0; k < 9; ++k) r[k] = src_r[k * P + p];
-  rk_particle<POT, S, false>(g, pt, src_b, P, p, dry, bdt, cdt, dt, &vz, Hm, r);
+  for (int k = 0; k < 9; ++k) r[k] = *row(src_r + p, (unsigned)P, k);
+  rk_from_H<POT, S, false>(g, pt, src_b, P, p, dry, bdt, cdt, dt, &vz, hv, he, r);
 }
 
 // Interpolation only (Eq. 6 then Eq. 2) for particles anywhere: H[k * P + p].
