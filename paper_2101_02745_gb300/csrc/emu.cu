@@ -1813,9 +1813,13 @@ int emu_interpolate_H(emu_box* b, double pos_dt, double* H_out, int on_host) {
     else if (b->is3d)
       k3_interpolate<decltype(O)::value><<<persist_grid(b), kThreads, 0, b->stream>>>(
           box3_view(b), b->x3, b->y3, b->pt.z, b->dirtab, b->shift, b->A, 1.0, dst, b->err);
-    else
-      k_interpolate<decltype(O)::value><<<persist_grid(b), kThreads, 0, b->stream>>>(
-          batch_view(b), b->pt.z, b->dirtab, b->shift, b->A, 1.0, dst, b->err);
+    else {
+      static std::atomic<unsigned> done{0};
+      auto k = k_interpolate<decltype(O)::value>;
+      if (raise_smem(k, kInterpSmem, done) == cudaSuccess)
+        k<<<persist_grid(b), kThreads, kInterpSmem, b->stream>>>(batch_view(b), b->pt.z, b->dirtab, b->shift, b->A, 1.0,
+                                                                 dst, b->err);
+    }
     return 0;
   });
   if (int rc = after_launch(b, "interpolation kernel")) return rc;

@@ -396,33 +396,32 @@ __device__ __forceinline__ double wrap_z(double z, double Lz) {
   return z;
 }
 
-// -i [H, r] for packed Hermitian H and r (Eq. 4 with H in units of hbar).
-// Diagonal outputs are returned HALVED (kd = K_aa / 2); the caller doubles
-// their RK coefficients.  Off-diagonal outputs ko = (Re K12, Im K12, Re K13,
-// Im K13, Re K23, Im K23).  H enters through its diagonal differences
-// d12 = h1 - h2, d13 = h1 - h3, d23 = h2 - h3 and off-diagonals a, b, c.
-__device__ __forceinline__ void commutator(double d12, double d13, double d23, double ar, double ai,
-                                           double br, double bi, double cr, double ci,
-                                           const double r[9], double kd[3], double ko[6]) {
-  const double xr = r[3], xi = r[4], yr = r[5], yi = r[6], zr = r[7], zi = r[8];
-  const double e21 = r[1] - r[0], e31 = r[2] - r[0], e32 = r[2] - r[1];
+// -i [H, r] (Eq. 4 with H in units of hbar) from the operands of wide.cuh.
+// Diagonal outputs are returned HALVED (kd = K_aa / 2).  Off-diagonal outputs
+// ko = (Re K12, Im K12, Re K13, Im K13, Re K23, Im K23).
+__device__ __forceinline__ void commutator(const emu_wide::Ham& H, const emu_wide::Mat& m, double (&kd)[3],
+                                           double (&ko)[6]) {
+  namespace w = emu_wide;
+  // (exponents from the smallest normal results up; out of range: NaN)
+  constexpr int emin = w::kBiasP - 1022;
+  auto value = [](double v, int e) { return e - w::kBiasP > 959 ? nan("") : w::scale_nz(v, e - w::kBiasP); };
+  const bool inf = w::max_i(w::top(H), w::top(m)) >= w::kExpNonFinite;
+  const int e0 = inf ? 1 << 16 : emin;
+  double cr, ci;
+  int e, ke[3];
   // C = [H, r]; K = -i C  =>  Re K = Im C, Im K = -Re C
-  const double c12r = fma(d12, xr, fma(e21, ar, fma(br, zr, fma(bi, zi, fma(-cr, yr, -ci * yi)))));
-  const double c12i = fma(d12, xi, fma(e21, ai, fma(bi, zr, fma(-br, zi, fma(-cr, yi, ci * yr)))));
-  const double c13r = fma(d13, yr, fma(e31, br, fma(ar, zr, fma(-ai, zi, fma(-cr, xr, ci * xi)))));
-  const double c13i = fma(d13, yi, fma(e31, bi, fma(ar, zi, fma(ai, zr, fma(-cr, xi, -ci * xr)))));
-  const double c23r = fma(d23, zr, fma(e32, cr, fma(ar, yr, fma(ai, yi, fma(-br, xr, -bi * xi)))));
-  const double c23i = fma(d23, zi, fma(e32, ci, fma(ar, yi, fma(-ai, yr, fma(-bi, xr, br * xi)))));
-  ko[0] = c12i; ko[1] = -c12r;
-  ko[2] = c13i; ko[3] = -c13r;
-  ko[4] = c23i; ko[5] = -c23r;
-  // K_11 = 2 (Im(a x*) + Im(b y*)), K_22 = 2 (Im(c z*) - Im(a x*)), K_33 = -2 (Im(b y*) + Im(c z*))
-  const double pp = fma(ai, xr, -ar * xi);
-  const double qq = fma(bi, yr, -br * yi);
-  const double tt = fma(ci, zr, -cr * zi);
-  kd[0] = pp + qq;
-  kd[1] = tt - pp;
-  kd[2] = -qq - tt;
+  w::commutator_off<0>(H, m, e0, cr, ci, e);
+  ko[0] = value(ci, e);
+  ko[1] = -value(cr, e);
+  w::commutator_off<1>(H, m, e0, cr, ci, e);
+  ko[2] = value(ci, e);
+  ko[3] = -value(cr, e);
+  w::commutator_off<2>(H, m, e0, cr, ci, e);
+  ko[4] = value(ci, e);
+  ko[5] = -value(cr, e);
+  w::commutator_diag(H, m, e0, kd, ke);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) kd[k] = value(kd[k], ke[k]);
 }
 
 // ------------------------------------------------------------------ kernels
@@ -1007,48 +1006,6 @@ static __global__ void k_combine(Batch B, const double* __restrict__ partial, do
   combine_phase(B, partial, out, rows, potential, split, err);
 }
 
-// Interpolation only (Eq. 6 then Eq. 2): H[k * Ptot + p] at z + frac dt_b v_z.
-template <int ORDER>
-__global__ void __launch_bounds__(kThreads, 2)
-k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ dirtab,
-              const int* __restrict__ shift, const double* __restrict__ A, double frac, double* __restrict__ Hout,
-              int* __restrict__ err) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w = logical_warp();
-  const int64_t u0 = unit_begin(w, B), u1 = unit_begin(w + 1, B);
-  const int64_t P = B.Ptot;
-  const int MT = B.MT, NZ = B.NZ;
-  int bad = 0;
-  if (u0 >= u1) return;
-  int b = box_of_unit(B, u0);
-  for (int64_t u = u0; u < u1; ++u) {
-    while (u >= B.box[b].uoff + (int64_t)B.box[b].ntiles * B.box[b].M) ++b;
-    const BoxGeo& g = B.box[b];
-    const int nz = g.nz, M = g.M;
-    const int tile = (int)((u - g.uoff) / M), d = (int)(u - g.uoff - (int64_t)tile * M);
-    constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T;
-    const int craw = tile * T - H + lane, j = wrapc(craw, nz);
-    const bool active = lane >= H && lane < H + T && craw < nz;
-    const int gd = g.doff + d;
-    const double ox = __ldg(dirtab + gd), oy = __ldg(dirtab + MT + gd), oz = __ldg(dirtab + 2 * MT + gd);
-    const double vz = __ldg(dirtab + 3 * MT + gd);
-    const int64_t p = g.poff + (int64_t)d * nz + wrapc(j - __ldg(shift + gd), nz);
-    double wt[Sten<ORDER>::NW];
-    zero_weights<ORDER>(wt);
-    if (active) bad |= shape_weights<ORDER>(fma(frac * B.dt[b], vz, z[p]), (double)j + 0.5, g.inv_dz, g.nz_d, wt);
-    const double* Aj = A + g.coff + j;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const double G = fma(-oz, __ldg(Aj + (int64_t)(27 + k) * NZ),
-                           fma(-oy, __ldg(Aj + (int64_t)(18 + k) * NZ),
-                               fma(-ox, __ldg(Aj + (int64_t)(9 + k) * NZ), __ldg(Aj + (int64_t)k * NZ))));
-      const double h = gather<ORDER>(wt, G);
-      if (active) Hout[k * P + p] = h;
-    }
-  }
-  if (bad) atomicOr(err, ERR_LATTICE);
-}
-
 // The RK4 update (Sec. 2.3) of particle p at stage s: K =
 // -i[H, rho], Kbar = -i[Hbar, rhobar] (Eq. 4) from the operand hm of H (Eq. 6,
 // Eq. 2; OWNBAR: hb of Hbar, otherwise Hbar = -H^*) and the neutrino source
@@ -1271,23 +1228,24 @@ struct SlabTable {
 constexpr int kSlabSmem = (int)sizeof(SlabTable<kSlabTiles>);
 constexpr int kStepSmem = kSlabSmem > kDepSmem ? kSlabSmem : kDepSmem;   // of k_step: either phase's
 
-// The operands of one exponent group of the potential at a cell: v[k] moment
-// k / 2, component k % 2 of the group; put(k, operand): A0 / 4 as an int64 (low,
-// high word; dot3's addend), limbs of A_x, A_y, A_z.  Returns their exponent.
-template <typename F>
-__device__ __forceinline__ int potential_operands(const double (&v)[8], F put) {
+// The operands of one exponent group of NV / 4 components of the potential at a
+// cell: v[k] moment k / (NV / 4), component k % (NV / 4) of the group; put(k,
+// operand): A0 / 4 as an int64 (low, high word; dot3's addend), limbs of A_x,
+// A_y, A_z.  Returns their exponent.
+template <int NV, typename F>
+__device__ __forceinline__ int potential_operands(const double (&v)[NV], F put) {
   namespace w = emu_wide;
-  int e[8], top = 0;
+  int e[NV], top = 0;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
+  for (int k = 0; k < NV; ++k) {
     e[k] = w::exponent(v[k]);
     top = max(top, e[k]);
   }
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
+  for (int k = 0; k < NV; ++k) {
     const w::Limbs l = w::limbs(v[k], e[k], top);
     int2 x = make_int2(l.h, l.l);
-    if (k < 2) {
+    if (k < NV / 4) {
       const int64_t q = w::join(l) >> 2;
       x = make_int2((int)q, (int)(q >> 32));
     }
@@ -1535,6 +1493,129 @@ k_rk_stage(Batch B, Parts pt, const double* __restrict__ W, const double* __rest
   extern __shared__ char smem[];
   griddep_wait();
   rk_phase<POT, ORDER, S, false>(B, pt, W, wrow, dirtab, shift, A, stage_src, s, dry, *(SlabTable<TILES>*)smem);
+}
+
+// ------------------------------------------------------ interpolation only
+//
+// H[k * Ptot + p] (Eq. 6 then Eq. 2, 9 packed components) of a single box's
+// particles at z + frac dt v_z, each with its own weights, from the potential
+// A[36][NZ].  As rk_phase up to H: a block takes a range of (slab of 4 tiles,
+// direction) pairs and converts the slab's potential once; the diagonal entries
+// have an exponent each.  (With FP64 G and taps 63 FP64 instructions a particle,
+// now 18: 270 us for 2048 x 1000.)
+struct InterpTable {
+  static constexpr int kTiles = 4, kCells = kTiles * kLanes + 4;
+  int2 a[kNA][kCells];
+  int e[6][kCells];              // exponents: three diagonal entries, three complex components
+  int2 g[kWarps][9][kRowCells];
+};
+constexpr int kInterpSmem = (int)sizeof(InterpTable);
+
+template <int ORDER>
+__global__ void __launch_bounds__(kThreads, 2)
+k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ dirtab,
+              const int* __restrict__ shift, const double* __restrict__ A, double frac, double* __restrict__ Hout,
+              int* __restrict__ err) {
+  namespace w = emu_wide;
+  extern __shared__ char smem[];
+  InterpTable& t = *(InterpTable*)smem;
+  constexpr int H = ORDER == 0 ? 0 : Sten<ORDER>::H, NW = ORDER == 0 ? 1 : Sten<ORDER>::NW;
+  const int lane = threadIdx.x & 31, wib = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+  const unsigned P = (unsigned)B.Ptot;
+  const int MT = B.MT, NZ = B.NZ;
+  const BoxGeo& g = B.box[0];
+  const int nz = g.nz, M = g.M, nslab = (g.ntiles32 + InterpTable::kTiles - 1) / InterpTable::kTiles;
+  const double pos_dt = frac * B.dt[0];
+  const int64_t all = (int64_t)nslab * M, q1 = ((int64_t)blockIdx.x + 1) * all / gridDim.x;
+  int bad = 0;
+  for (int64_t q = (int64_t)blockIdx.x * all / gridDim.x; q < q1;) {
+    const int slab = (int)(q / M), d0 = (int)(q - (int64_t)slab * M), d1 = (int)min((int64_t)M, d0 + (q1 - q));
+    q += d1 - d0;
+    const int c0 = slab * InterpTable::kTiles * kLanes, ncell = min(InterpTable::kTiles * kLanes, nz - c0) + 2 * H;
+    __syncthreads();
+    for (int x = threadIdx.x; x < 6 * ncell; x += kThreads) {
+      const int grp = x / ncell, c = x - grp * ncell;
+      const double* Aj = A + wrapc(c0 - H + c, nz);
+      if (grp < 3) {
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = __ldg(Aj + (int64_t)(9 * k + grp) * NZ);
+        t.e[grp][c] = potential_operands<4>(v, [&](int k, int2 o) { t.a[9 * k + grp][c] = o; });
+      } else {
+        const int k0 = 2 * grp - 3;
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = __ldg(Aj + (int64_t)(9 * (k >> 1) + k0 + (k & 1)) * NZ);
+        t.e[grp][c] = potential_operands<8>(v, [&](int k, int2 o) { t.a[9 * (k >> 1) + k0 + (k & 1)][c] = o; });
+      }
+    }
+    __syncthreads();
+    const int tile0 = (wib & (InterpTable::kTiles - 1)) * kLanes, n = min(kLanes, nz - c0 - tile0);
+    if (n <= 0) continue;
+    const int j = c0 + tile0 + lane, tc = tile0 + H + lane;
+    const bool active = lane < n;
+    for (int d = d0 + wib / InterpTable::kTiles; d < d1; d += kWarps / InterpTable::kTiles) {
+      const int gd = g.doff + d;
+      int i = active ? j - __ldg(shift + gd) : 0;
+      if (i < 0) i += nz;
+      const int64_t p = (int64_t)d * nz + i;
+      const double u = lane < 3 ? -__ldg(dirtab + lane * MT + gd) : 0.0;
+      double wt[Sten<ORDER>::NW];
+      zero_weights<ORDER>(wt);
+      if (active)
+        bad |= shape_weights<ORDER>(fma(pos_dt, __ldg(dirtab + 3 * MT + gd), z[p]), (double)j + 0.5, g.inv_dz, g.nz_d,
+                                    wt);
+      const int ko = __reduce_max_sync(kFull, w::unit_excess(u));
+      const w::Limbs ul = w::unit_limbs(u, ko);
+      const w::Limbs om[3] = {bcast(ul, 0), bcast(ul, 1), bcast(ul, 2)};
+      auto G = [&](int c, int x) {
+        return operand_G(t.a[c][x], t.a[9 + c][x], t.a[18 + c][x], t.a[27 + c][x], om, ko);
+      };
+      if (active) {
+#pragma unroll
+        for (int c = 0; c < 9; ++c) t.g[wib][c][H + lane] = G(c, tc);
+      }
+      if constexpr (H > 0) {   // the H cells on each side
+        for (int x = lane; x < 2 * H * 9; x += kLanes) {
+          const int c = x % 9, h = x / 9, at = h < H ? h : n + h;
+          t.g[wib][c][at] = G(c, tile0 + at);
+        }
+      }
+      __syncwarp();
+      if (active) {
+        w::Limbs wl[NW];
+#pragma unroll
+        for (int o = 0; o < NW; ++o) wl[o] = w::unit_limbs(wt[o]);
+#pragma unroll
+        for (int grp = 0; grp < 6; ++grp) {
+          const int nc = grp < 3 ? 1 : 2, k0 = grp < 3 ? grp : 2 * grp - 3;
+          int e[NW], he = 0;
+#pragma unroll
+          for (int o = 0; o < NW; ++o) {
+            e[o] = t.e[grp][tc - H + o];
+            he = max(he, e[o]);
+          }
+          const int k2 = min(max(he + 2 + ko - w::kBiasV, -1022), 959);
+          const bool inf = he >= w::kExpNonFinite || ko > w::kMaxExcess;
+#pragma unroll
+          for (int c = k0; c < k0 + nc; ++c) {
+            int64_t v = 0;
+            if constexpr (ORDER == 0) {
+              v = w::join(limbs_of(t.g[wib][c][lane]));
+            } else {
+#pragma unroll
+              for (int o = 0; o < NW; ++o)
+                v += w::align(w::mul(limbs_of(t.g[wib][c][lane + o]), wl[o]), he - e[o]);
+              v *= 4;
+            }
+            *row(Hout + p, P, c) = inf ? nan("") : w::scale_nz((double)v, k2);
+          }
+        }
+      }
+      __syncwarp();   // (the unit's G are rewritten by the next)
+    }
+  }
+  if (bad) atomicOr(err, ERR_LATTICE);
 }
 
 // ------------------------------------------- RK stage with the next deposit
@@ -2305,7 +2386,7 @@ k_adj_a(Batch B, Parts pt, const double* __restrict__ W, const double* __restric
     double Gm[9];
 #pragma unroll
     for (int which = 0; which < 2; ++which) {
-      double nH[kNC], r[9], m2[9], kd[3], ko[6];
+      double nH[kNC], r[9], m2[9], kd[3], ko[6];   // (the commutators on the integer pipe, as the RK stage's)
 #pragma unroll
       for (int c = 0; c < kNC; ++c) {                                       // -(S H + V), S for antineutrinos
         const bool im = (c == 3 || c == 5 || c == 7);
@@ -2319,12 +2400,16 @@ k_adj_a(Batch B, Parts pt, const double* __restrict__ W, const double* __restric
         m2[k] = k < 3 ? fma(a2, l, bc2 * ln) : fma(a, l, bc * ln);
         r[k] = (which ? pt.rhobar : pt.rho)[k * P + p];
       }
-      commutator(nH[0], nH[0] + nH[1], nH[1], nH[2], nH[3], nH[4], nH[5], nH[6], nH[7], m2, kd, ko);
+      const emu_wide::Mat mm = emu_wide::mat(m2, false);
+      commutator(emu_wide::ham(nH), mm, kd, ko);
 #pragma unroll
       for (int k = 0; k < 3; ++k) lam_out[(which * 9 + k) * P + p] = kd[k];
 #pragma unroll
       for (int k = 0; k < 6; ++k) lam_out[(which * 9 + 3 + k) * P + p] = ko[k];
-      commutator(r[0] - r[1], r[0] - r[2], r[1] - r[2], r[3], r[4], r[5], r[6], r[7], r[8], m2, kd, ko);
+      const double rt[kNC] = {r[0] - r[1], r[1] - r[2], r[3], r[4], r[5], r[6], r[7], r[8]};
+      emu_wide::Ham rh = emu_wide::ham(rt);
+      rh.d13 = emu_wide::real(r[0] - r[2]);
+      commutator(rh, mm, kd, ko);
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
         const bool im = (k == 4 || k == 6 || k == 8);
