@@ -329,16 +329,43 @@ int use_slabs(const emu_box* b) {
   return b->rk_form >= 0 ? b->rk_form : b->S.U32 >= 16 * (int64_t)kPersistBlocks || b->S.NT32 > b->blocks;
 }
 
-// Directions of a block's part of a tile: the fewest that leave no more parts
-// than blocks (all of a tile's directions when the tiles alone are more).
-int part_directions(const emu_box* b) {
-  int64_t upb = (b->S.U32 + b->blocks - 1) / b->blocks;
-  for (; upb < b->S.Mmax; ++upb) {
-    int64_t parts = 0;
-    for (const BoxGeo& g : b->S.geo) parts += (int64_t)g.ntiles32 * ((g.M + upb - 1) / upb);
-    if (parts <= b->blocks) break;
-  }
-  return (int)(upb < 1 ? 1 : upb);
+// Work split of small boxes, in the RK stage and the deposit: a block takes a
+// part of one tile's directions, of no more warps than the part has directions
+// (so that more blocks fit an SM), and the grid has no more blocks than parts.
+// Parts of upb directions: how many there are (of 32-cell tiles in the RK
+// stage, of the deposit's 32 - 2 H cells).
+int64_t parts(const emu_box* b, int64_t upb, bool deposit) {
+  int64_t n = 0;
+  for (const BoxGeo& g : b->S.geo) n += (int64_t)(deposit ? g.ntiles : g.ntiles32) * ((g.M + upb - 1) / upb);
+  return n;
+}
+
+// Directions of a part: the fewest that leave no more parts than blocks (all
+// of a tile's directions when the tiles alone are more), but at least 6 (4 in
+// boxes of less than a unit a block): parts of 3 directions of a 256 x 96 box
+// fill all SMs with half-idle blocks and three such boxes at a time take 254 us
+// per 4 steps, parts of 6 directions 188 us (one box alone the same).
+int part_directions(const emu_box* b, bool deposit) {
+  const int64_t units = deposit ? b->S.U : b->S.U32;
+  int64_t upb = std::max<int64_t>((units + b->blocks - 1) / b->blocks, 1);
+  while (upb < b->S.Mmax && parts(b, upb, deposit) > b->blocks) ++upb;
+  return (int)std::max<int64_t>(upb, std::min(units < b->blocks ? 4 : 6, b->S.Mmax));
+}
+
+// Directions of a block's part in the deposit (Batch::dpb), 0 for ranges of
+// units per warp.  A part writes one partial (the sum of its warps) where each
+// warp of a range writes its own, which shortens the combination and leaves no
+// warp with two tiles: 1024 x 378 deposit + combination 45.5 + 14.6 us with
+// ranges, 41.3 + 8.8 us with parts; 777 x 130 23 + 16.4 -> 18.7 + 9.4 us.  But
+// whole parts split less evenly: ranges where a warp of a part would take more
+// than one direction above its share of a range, and where the tiles alone
+// outnumber the blocks; also with many boxes, which a block would search.
+// (Modes 3 and 5, the adjoint's and the step's; the others have no such kernel.)
+int deposit_part(const emu_box* b, int mode) {
+  if ((mode != 3 && mode != 5) || b->S.nbox > 8 || b->S.NT > b->blocks) return 0;
+  const int64_t nw = (int64_t)b->blocks * kWarps;
+  const int n = part_directions(b, true);
+  return (n + kWarps - 1) / kWarps <= (b->S.U + nw - 1) / nw + 1 ? n : 0;
 }
 
 Batch batch_view(const emu_box* b) {
@@ -358,7 +385,8 @@ Batch batch_view(const emu_box* b) {
   B.Ptot = b->S.Ptot;
   B.slabs = use_slabs(b);
   B.US = b->S.US;
-  B.upb = B.slabs ? 0 : part_directions(b);
+  B.upb = B.slabs ? 0 : part_directions(b, false);
+  B.dpb = 0;
   return B;
 }
 
@@ -393,9 +421,10 @@ dim3 persist_grid(const emu_box* b) { return dim3((unsigned)b->blocks, 1, 1); }
 // over more warps, as far as needed to fill about one wave of the persistent
 // grid (304 blocks x 8 warps); short sums keep one warp (coalesced, latency
 // hidden by the other warps).
-int combine_split(const Shape& S, int64_t nw, bool frame = false) {
+// dpb: directions of a partial when blocks write them (Batch::dpb), else 0.
+int combine_split(const Shape& S, int64_t nw, bool frame = false, int dpb = 0) {
   const int64_t U = frame ? S.U32 : S.U;
-  const int64_t per_warp = nw > 0 && U / nw > 0 ? U / nw : 1;       // fewest units a warp takes
+  const int64_t per_warp = dpb > 0 ? dpb : nw > 0 && U / nw > 0 ? U / nw : 1;       // fewest units of a partial
   const int64_t most = (S.Mmax + per_warp - 1) / per_warp + 1;        // most warps over one tile
   if (most <= 8) return 1;
   const int64_t out_warps = ((int64_t)(frame ? kNT : kNA) * S.NZ + kLanes - 1) / kLanes;
@@ -555,10 +584,10 @@ cudaError_t raise_smem(K kernel, int bytes, std::atomic<unsigned>& done) {
 }
 
 template <typename... KArgs, typename... Args>
-void pdl_smem(cudaStream_t st, void (*kernel)(KArgs...), dim3 grid, int smem, Args... args) {
+void pdl_smem(cudaStream_t st, void (*kernel)(KArgs...), dim3 grid, int threads, int smem, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -705,9 +734,12 @@ int launch_deposit(emu_box* b, int mode, const double* rnu, const double* rnb, c
   // where modes 0 and 5 keep the shape weights
   if (!W) W = keep || weight_row(b, shift_row) == nullptr ? b->W : nullptr;
   if (mode == 5 && b->dep_form != 0) return launch_deposit_cluster(b, rnu, rnb, shift_row, frac, out, W);
-  const Batch B = batch_view(b);
+  Batch B = batch_view(b);
+  B.dpb = deposit_part(b, mode);
   before_launch(b, CLS_DEPOSIT);
-  const dim3 grid = persist_grid(b);
+  const int threads = B.dpb > 0 ? part_warps(B.dpb) * kLanes : kThreads;
+  const int smem = B.dpb == 0 && B.U <= B.nw ? kDepSmem / 2 : kDepSmem / kThreads * threads;
+  const dim3 grid = B.dpb > 0 ? dim3((unsigned)parts(b, B.dpb, true)) : persist_grid(b);
   cudaStream_t st = b->stream;
   const double* z = b->pt.z;
   const double* N = b->pt.N;
@@ -715,15 +747,20 @@ int launch_deposit(emu_box* b, int mode, const double* rnu, const double* rnb, c
   const double* wrow = weight_row(b, shift_row);
   by_order(b->S.order, [&](auto O) {
     constexpr int R = decltype(O)::value;
-    auto go = [&](auto MODE, auto TAB) {
+    auto launch = [&](auto MODE, auto TAB, auto PART) {
       static std::atomic<unsigned> done{0};
-      auto k = k_deposit<decltype(MODE)::value, R, decltype(TAB)::value>;
+      auto k = k_deposit<decltype(MODE)::value, R, decltype(TAB)::value, decltype(PART)::value>;
       if (raise_smem(k, kDepSmem, done) == cudaSuccess)
-        pdl_smem(st, k, grid, B.U > B.nw ? kDepSmem : kDepSmem / 2, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow,
+        pdl_smem(st, k, grid, threads, smem, B, z, N, Nb, rnu, rnb, b->dirtab, shift_row, wrow,
                  frac, b->partial, mode == 0 || mode == 5 ? W : nullptr, b->err);
     };
     using std::false_type;
     using std::true_type;
+    auto go = [&](auto MODE, auto TAB) {
+      if constexpr (decltype(MODE)::value == 3 || decltype(MODE)::value == 5)
+        if (B.dpb > 0) return launch(MODE, TAB, true_type{});
+      launch(MODE, TAB, false_type{});
+    };
     if (mode == 0) go(std::integral_constant<int, 0>{}, false_type{});
     else if (mode == 1) go(std::integral_constant<int, 1>{}, false_type{});
     else if (mode == 2) go(std::integral_constant<int, 2>{}, false_type{});
@@ -737,7 +774,7 @@ int launch_deposit(emu_box* b, int mode, const double* rnu, const double* rnb, c
   });
   if (int rc = after_launch(b, "deposit kernel")) return rc;
   before_launch(b, CLS_COMBINE);
-  const int split = combine_split(b->S, B.nw);
+  const int split = combine_split(b->S, B.nw, false, B.dpb);
   const int rows = mode == 5 ? kNT : kNA;
   const int potential = (mode == 0 || mode == 3 || mode == 5) ? 1 : 0;
   pdl(b->stream, k_combine, dim3(combine_blocks(rows, B.NZ, split)), B, b->partial, out, rows, potential,
@@ -798,7 +835,8 @@ int launch_fused(emu_box* b, int dry, int64_t nsteps) {
   const int maxb = fused_max_blocks(b);
   if (b->blocks > maxb)
     return fail(b, EMU_EINVAL, "the fused step needs all %d blocks resident at once; at most %d fit", b->blocks, maxb);
-  const Batch B = batch_view(b);
+  Batch B = batch_view(b);
+  B.dpb = deposit_part(b, 5);
   StepArgs a{};
   a.dirtab = b->dirtab;
   a.shift = b->shift;
@@ -810,7 +848,7 @@ int launch_fused(emu_box* b, int dry, int64_t nsteps) {
   a.bar = b->bar;
   a.limit_ns = b->limit_ns;
   a.nsteps = nsteps;
-  a.split = combine_split(b->S, B.nw);
+  a.split = combine_split(b->S, B.nw, false, B.dpb);
   a.dry = dry;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = persist_grid(b);
@@ -847,12 +885,14 @@ int launch_rk_on(emu_box* b, int s, const int* srow, int dry, const Parts& pt, c
     constexpr int R = decltype(O)::value;
     const Batch Bv = batch_view(b);
     const double* wrow = weight_row(b, srow);
+    const int threads = Bv.slabs ? kThreads : part_warps(Bv.upb) * kLanes;
+    const dim3 grid = Bv.slabs ? persist_grid(b) : dim3((unsigned)std::min<int64_t>(parts(b, Bv.upb, false), b->blocks));
     auto launch_tiles = [&](auto POT, auto STAGE, auto TILES) {
       static std::atomic<unsigned> done{0};
       constexpr int T = decltype(TILES)::value, smem = (int)sizeof(SlabTable<T>);
       auto k = k_rk_stage<decltype(POT)::value, R, decltype(STAGE)::value, T>;
       if (raise_smem(k, smem, done) == cudaSuccess)
-        pdl_smem(b->stream, k, persist_grid(b), smem, Bv, pt, W, wrow, b->dirtab, srow, At, stage_src, s, dry);
+        pdl_smem(b->stream, k, grid, threads, smem, Bv, pt, W, wrow, b->dirtab, srow, At, stage_src, s, dry);
     };
     by_stage(b->pot, s, [&](auto POT, auto STAGE) {
       if (Bv.slabs) launch_tiles(POT, STAGE, std::integral_constant<int, kSlabTiles>{});
@@ -924,7 +964,7 @@ int rd_prepare(emu_box* b) {
 template <bool POT, int R>
 void launch_rd_stage(emu_box* b, const Batch& Bv, dim3 grid, int s, int dry) {
   auto go = [&](auto kernel) {
-    pdl_smem(b->stream, kernel, grid, kFrameSmem, Bv, b->pt, b->W, b->dirtab, b->shift, b->frame, dry, b->partial,
+    pdl_smem(b->stream, kernel, grid, kThreads, kFrameSmem, Bv, b->pt, b->W, b->dirtab, b->shift, b->frame, dry, b->partial,
              b->err);
   };
   switch (s) {
@@ -945,7 +985,7 @@ int launch_rd(emu_box* b, int s, int dry) {
     constexpr int R = decltype(O)::value;
     if constexpr (R <= 2) {
       if (s == 0)
-        pdl_smem(b->stream, k_rk_deposit<false, R, 0>, grid, kFrameSmem, Bv, b->pt, b->W, b->dirtab, b->shift,
+        pdl_smem(b->stream, k_rk_deposit<false, R, 0>, grid, kThreads, kFrameSmem, Bv, b->pt, b->W, b->dirtab, b->shift,
                  b->frame, 0, b->partial, b->err);
       else if (b->pot)
         launch_rd_stage<true, R>(b, Bv, grid, s, dry);
@@ -2683,6 +2723,7 @@ extern "C" int emu_deposit_static(const emu_config* cfg, const double* z, const 
   B.Ptot = S.Ptot;
   B.U32 = 0;
   B.nw32 = 0;
+  B.slabs = B.upb = B.dpb = 0;
   Parts pt{const_cast<double*>(z), const_cast<double*>(ox), const_cast<double*>(oy), const_cast<double*>(oz),
            const_cast<double*>(N), const_cast<double*>(Nbar), const_cast<double*>(rho),
            const_cast<double*>(rhobar), nullptr, nullptr};
@@ -2694,9 +2735,9 @@ extern "C" int emu_deposit_static(const emu_config* cfg, const double* z, const 
   k_shifts<2><<<(S.MT + kThreads - 1) / kThreads, kThreads, 0, st>>>(B, z, dirtab, f, 1, shift, nullptr);
   if (int rc = check(cudaGetLastError(), "shift kernel")) return rc;
   static std::atomic<unsigned> smem_raised{0};
-  if (int rc = check(raise_smem(k_deposit<0, 2, false>, kDepSmem, smem_raised), "deposit kernel's shared memory"))
+  if (int rc = check(raise_smem(k_deposit<0, 2, false, false>, kDepSmem, smem_raised), "deposit kernel's shared memory"))
     return rc;
-  k_deposit<0, 2, false><<<dim3(kPersistBlocks), kThreads, kDepSmem, st>>>(B, z, N, Nbar, rho, rhobar, dirtab, shift,
+  k_deposit<0, 2, false, false><<<dim3(kPersistBlocks), kThreads, kDepSmem, st>>>(B, z, N, Nbar, rho, rhobar, dirtab, shift,
                                                                           nullptr, 1.0, partial, nullptr, err);
   if (int rc = check(cudaGetLastError(), "deposit kernel")) return rc;
   const int split = combine_split(S, B.nw);

@@ -18,8 +18,8 @@
 #define EMU_RK_DEPOSIT(X, POT, R, S)                                                                                \
   X template __global__ void k_rk_deposit<POT, R, S>(Batch, Parts, double*, const double*, const int*,              \
                                                      const double*, int, double*, int*);
-#define EMU_DEPOSIT(X, MODE, R, TAB)                                                                                \
-  X template __global__ void k_deposit<MODE, R, TAB>(Batch, const double*, const double*, const double*,            \
+#define EMU_DEPOSIT(X, MODE, R, TAB, PART)                                                                                \
+  X template __global__ void k_deposit<MODE, R, TAB, PART>(Batch, const double*, const double*, const double*,            \
                                                      const double*, const double*, const double*, const int*,       \
                                                      const double*, double, double*, double*, int*);
 #define EMU_DEPOSIT_CLUSTER(X, R, TAB, CL)                                                                          \
@@ -40,14 +40,18 @@
 #define EMU_ORDER_INSTANCES(X, R)                                                                                   \
   EMU_POT_INSTANCES(X, false, R)                                                                                    \
   EMU_POT_INSTANCES(X, true, R)                                                                                     \
-  EMU_DEPOSIT(X, 0, R, false)                                                                                       \
-  EMU_DEPOSIT(X, 1, R, false)                                                                                       \
-  EMU_DEPOSIT(X, 2, R, false)                                                                                       \
-  EMU_DEPOSIT(X, 3, R, false)                                                                                       \
-  EMU_DEPOSIT(X, 3, R, true)                                                                                        \
-  EMU_DEPOSIT(X, 4, R, false)                                                                                       \
-  EMU_DEPOSIT(X, 5, R, false)                                                                                       \
-  EMU_DEPOSIT(X, 5, R, true)                                                                                        \
+  EMU_DEPOSIT(X, 0, R, false, false)                                                                                \
+  EMU_DEPOSIT(X, 1, R, false, false)                                                                                \
+  EMU_DEPOSIT(X, 2, R, false, false)                                                                                \
+  EMU_DEPOSIT(X, 3, R, false, false)                                                                                \
+  EMU_DEPOSIT(X, 3, R, false, true)                                                                                 \
+  EMU_DEPOSIT(X, 3, R, true, false)                                                                                 \
+  EMU_DEPOSIT(X, 3, R, true, true)                                                                                  \
+  EMU_DEPOSIT(X, 4, R, false, false)                                                                                \
+  EMU_DEPOSIT(X, 5, R, false, false)                                                                                \
+  EMU_DEPOSIT(X, 5, R, false, true)                                                                                 \
+  EMU_DEPOSIT(X, 5, R, true, false)                                                                                 \
+  EMU_DEPOSIT(X, 5, R, true, true)                                                                                  \
   EMU_DEPOSIT_CLUSTER(X, R, false, 8)                                                                               \
   EMU_DEPOSIT_CLUSTER(X, R, true, 8)                                                                                \
   EMU_DEPOSIT_CLUSTER(X, R, false, 16)                                                                              \

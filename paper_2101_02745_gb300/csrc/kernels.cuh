@@ -98,6 +98,10 @@ struct BoxGeo {
   double vnubar[kNC];
 };
 
+// Warps that share a part of n directions: no more than directions, but 4 at
+// least (they also share the sum over warps and the RK stage's conversions).
+__host__ __device__ inline int part_warps(int n) { return n < 4 ? 4 : n < kWarps ? n : kWarps; }
+
 // Kernel view of a batch (passed by value).
 struct Batch {
   const BoxGeo* box;   // [nbox]
@@ -112,6 +116,7 @@ struct Batch {
   int64_t US;          // total tile units of the RK stage's slabs
   int slabs;           // its work split: 1 = ranges of slabs, 0 = parts of one tile
   int upb;             // directions of a part (slabs 0)
+  int dpb;             // deposit: directions of a block's part of a tile; 0: ranges of units per warp
 };
 
 struct Parts {
@@ -585,7 +590,9 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
                                                   const double* __restrict__ Nbar, const double* r_nu,
                                                   const double* r_nb, const double* __restrict__ dirtab,
                                                   const int* shift, const double* wrow, double frac, double* W,
-                                                  double* buf, int ring2, double (&out)[DepMode<MODE>::NA], int& bad) {
+                                                  double* buf, int ring2, int n,
+                                                  int64_t (&acc)[DepMode<MODE>::NA],
+                                                  int (&ea)[DepMode<MODE>::SETS * DepMode<MODE>::GROUPS], int& bad) {
   namespace w = emu_wide;
   constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T, NW = Sten<ORDER>::NW;
   using D = DepMode<MODE>;
@@ -599,9 +606,7 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
   const bool own = lane >= H && lane < H + T && craw < nz;
   const double pos_dt = frac * B.dt[b];
   const int dbase = g.doff;
-  const int head = max(32 - __clz(dlast - dfirst), 2) - 2;   // headroom beyond the two bits a contribution leaves
-  int64_t acc[D::NA];
-  int ea[D::SETS * D::GROUPS];
+  const int head = max(32 - __clz(n), 2) - 2;   // headroom beyond the two bits a contribution leaves
 #pragma unroll
   for (int c = 0; c < D::NA; ++c) acc[c] = 0;
 #pragma unroll
@@ -749,21 +754,43 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
       }
     }
   }
-  // acc 2^(ea + 4 - kBiasV)
-#pragma unroll
-  for (int sq = 0; sq < D::SETS * D::GROUPS; ++sq) {
-    const int set = sq / D::GROUPS, q = sq % D::GROUPS, nc = q < D::SINGLE ? 1 : 2;
-    const int r0 = set * D::MOM * D::COMP + (q < D::SINGLE ? q : 2 * q - D::SINGLE);
-    const int k = min(max(ea[sq] + 4 - w::kBiasV, -1022), 959);
-#pragma unroll
-    for (int c = 0; c < nc; ++c) {
-#pragma unroll
-      for (int m = 0; m < D::MOM; ++m) {
-        const double v = (double)acc[m * D::COMP + r0 + c];
-        out[m * D::COMP + r0 + c] = ea[sq] >= w::kExpNonFinite ? nan("") : w::scale_nz(v, k);
-      }
+}
+
+// A sum acc 2^(ea + 4 - kBiasV) of deposit_tile as a double.
+__device__ __forceinline__ double deposit_sum(int64_t acc, int ea) {
+  namespace w = emu_wide;
+  if (ea >= w::kExpNonFinite) return nan("");
+  return w::scale_nz((double)acc, min(max(ea + 4 - w::kBiasV, -1022), 959));
+}
+// The exponent group of row c.
+template <int MODE>
+__device__ __forceinline__ constexpr int deposit_group(int c) {
+  using D = DepMode<MODE>;
+  const int k = c % D::COMP, q = k < D::SINGLE ? k : D::SINGLE + (k - D::SINGLE) / 2;
+  return c / (D::MOM * D::COMP) * D::GROUPS + q;
+}
+
+// Part q of the deposit's split into blocks (Batch::dpb > 0): box b, tile and
+// directions [d0, d1); false past the last one.  first_part: the first part of a tile.
+__device__ __forceinline__ bool deposit_part(const Batch& B, int q, int& b, int& tile, int& d0, int& d1) {
+  for (b = 0; b < B.nbox; ++b) {
+    const BoxGeo& g = B.box[b];
+    const int per = (g.M + B.dpb - 1) / B.dpb, all = per * g.ntiles;
+    if (q < all) {
+      tile = q / per;
+      const int i = q - tile * per, len = g.M / per, more = g.M - len * per;   // (the first `more` parts take one more)
+      d0 = i * len + min(i, more);
+      d1 = d0 + len + (i < more);
+      return true;
     }
+    q -= all;
   }
+  return false;
+}
+__device__ __forceinline__ int first_part(const Batch& B, const BoxGeo* box, int tile) {
+  int q = 0;
+  for (const BoxGeo* g = B.box; g < box; ++g) q += (g->M + B.dpb - 1) / B.dpb * g->ntiles;
+  return q + tile * ((box->M + B.dpb - 1) / B.dpb);
 }
 
 // Deposit (Eq. 5), first phase.  MODE 0: B = N rho - Nbar rhobar^* (the
@@ -782,16 +809,61 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
 // every particle of a ring takes the ring's weights: the ring translates
 // rigidly, so its particles share their offset inside the cells (to
 // rounding); each particle's position is still checked against its cell.
-template <int MODE, int ORDER, bool COH>
+template <int MODE, int ORDER, bool COH, bool PART>
 __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lane, const double* z,
                                               const double* __restrict__ N, const double* __restrict__ Nbar,
                                               const double* r_nu, const double* r_nb,
                                               const double* __restrict__ dirtab, const int* shift,
                                               const double* wrow, double frac, double* __restrict__ partial,
                                               double* W, int* err, double* buf = nullptr) {
+  using D = DepMode<MODE>;
+  constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T;
+  int bad = 0;
+  if constexpr (PART) {
+    // few units: a block takes a part of one tile's directions, adds its warps'
+    // sums (as integers, at their largest exponent) and writes one partial
+    const int wib = threadIdx.x >> 5;
+    const int nwarps = part_warps(B.dpb);                         // (the block's, but in k_step)
+    int64_t* sums = (int64_t*)(buf - wib * kDepBuf);              // [warp][row][lane], then the exponents
+    constexpr int kE = D::NA * kLanes;                            // doubles before a warp's exponents
+    static_assert(D::NA * kLanes * 8 + D::SETS * D::GROUPS * kLanes * 4 <= kDepBuf * 8, "a warp's sums fit its buffers");
+    int b, tile, d0, d1;
+    for (int q = blockIdx.x; deposit_part(B, q, b, tile, d0, d1); q += gridDim.x) {
+      const int n = d1 - d0, used = min(n, nwarps);
+      if (wib < used) {
+        const int len = n / nwarps, more = n - len * nwarps;
+        const int w0 = d0 + wib * len + min(wib, more);
+        int64_t acc[D::NA];
+        int ea[D::SETS * D::GROUPS];
+        deposit_tile<MODE, ORDER, COH>(B, b, tile, w0, w0 + len + (wib < more), lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
+                                       wrow, frac, W, buf, 1, n, acc, ea, bad);
+#pragma unroll
+        for (int c = 0; c < D::NA; ++c) sums[wib * kDepBuf + c * kLanes + lane] = acc[c];
+#pragma unroll
+        for (int c = 0; c < D::SETS * D::GROUPS; ++c) ((int*)(sums + wib * kDepBuf + kE))[c * kLanes + lane] = ea[c];
+      }
+      __syncthreads();
+      const int cell = tile * T - H + lane;
+      if (wib < nwarps && lane >= H && lane < H + T && cell < B.box[b].nz) {
+        for (int c = wib; c < D::NA; c += nwarps) {
+          const int* ex = (const int*)(sums + kE) + deposit_group<MODE>(c) * kLanes + lane;
+          int top = 0, e[kWarps];
+#pragma unroll
+          for (int x = 0; x < kWarps; ++x) top = max(top, e[x] = x < used ? ex[x * 2 * kDepBuf] : 0);
+          int64_t v = 0;
+#pragma unroll
+          for (int x = 0; x < kWarps; ++x)
+            if (x < used) v += emu_wide::align(sums[x * kDepBuf + c * kLanes + lane], top - e[x]);
+          partial[(int64_t)q * kSlot + c * T + lane - H] = deposit_sum(v, top);
+        }
+      }
+      __syncthreads();   // (the sums are free for the next part)
+    }
+    if (bad) atomicOr(err, ERR_LATTICE);
+    return;
+  }
   const int64_t u0 = unit_begin(w, B), u1 = unit_begin(w + 1, B);
   if (u0 >= u1) return;
-  int bad = 0;
   int b = box_of_unit(B, u0);
   for (int64_t u = u0; u < u1;) {        // one segment per (box, tile) the warp touches
     while (u >= B.box[b].uoff + (int64_t)B.box[b].ntiles * B.box[b].M) ++b;
@@ -802,10 +874,13 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
     const int64_t ubase = g.uoff + (int64_t)tile * M;
     const int dfirst = (int)(u - ubase), dlast = (int)(uend - ubase);
     u = uend;
-    double acc[DepMode<MODE>::NA];
+    int64_t sum[D::NA];
+    int ea[D::SETS * D::GROUPS];
     deposit_tile<MODE, ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow, frac, W,
-                                   buf, B.U > B.nw, acc, bad);
-    constexpr int H = Sten<ORDER>::H, T = Sten<ORDER>::T;
+                                   buf, B.U > B.nw, dlast - dfirst, sum, ea, bad);
+    double acc[D::NA];
+#pragma unroll
+    for (int c = 0; c < D::NA; ++c) acc[c] = deposit_sum(sum[c], ea[deposit_group<MODE>(c)]);
     flush_tile<ORDER>(acc, g.toff + tile, tile * T - H + lane, g.nz, w, lane, partial);
   }
   if (bad) atomicOr(err, ERR_LATTICE);
@@ -813,7 +888,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
 
 // TAB: the rings' weights from the weight row wrow; otherwise each
 // particle's own (wrow unused, and the table's code compiled out).
-template <int MODE, int ORDER, bool TAB = false>
+template <int MODE, int ORDER, bool TAB, bool PART>
 __global__ void __launch_bounds__(kThreads, 2)
 k_deposit(Batch B, const double* __restrict__ z, const double* __restrict__ N, const double* __restrict__ Nbar,
           const double* __restrict__ r_nu, const double* __restrict__ r_nb, const double* __restrict__ dirtab,
@@ -821,8 +896,8 @@ k_deposit(Batch B, const double* __restrict__ z, const double* __restrict__ N, c
           double* __restrict__ W, int* __restrict__ err) {
   extern __shared__ double dep_sm[];   // kDepSmem bytes (half with one buffer)
   griddep_wait();
-  deposit_phase<MODE, ORDER, false>(B, logical_warp(), threadIdx.x & 31, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                    TAB ? wrow : nullptr, frac, partial, W, err, dep_sm + (threadIdx.x >> 5) * (B.U > B.nw ? kDepBuf : kDepBuf / 2));
+  deposit_phase<MODE, ORDER, false, PART>(B, logical_warp(), threadIdx.x & 31, z, N, Nbar, r_nu, r_nb, dirtab, shift,
+                                    TAB ? wrow : nullptr, frac, partial, W, err, dep_sm + (threadIdx.x >> 5) * (PART || B.U > B.nw ? kDepBuf : kDepBuf / 2));
 }
 
 // ------------------------------------------------------- cluster deposit
@@ -901,14 +976,17 @@ k_deposit_cluster(Batch B, const double* __restrict__ z, const double* __restric
     const BoxGeo& g = B.box[b];
     const int tile = (int)(gt - g.toff);
     const int d0 = (int)((int64_t)gw * g.M / nwc), d1 = (int)((int64_t)(gw + 1) * g.M / nwc);
-    double acc[kNT];
+    int64_t acc[kNT];
+    int ea[DepMode<5>::GROUPS];
 #pragma unroll
-    for (int c = 0; c < kNT; ++c) acc[c] = 0.0;
+    for (int c = 0; c < kNT; ++c) acc[c] = 0;
+#pragma unroll
+    for (int c = 0; c < DepMode<5>::GROUPS; ++c) ea[c] = 0;
     if (d0 < d1)
       deposit_tile<5, ORDER, false>(B, b, tile, d0, d1, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                    TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, 1, acc, bad);
+                                    TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, 1, d1 - d0, acc, ea, bad);
 #pragma unroll
-    for (int c = 0; c < kNT; ++c) red[wib * kDepBuf + c * kLanes + lane] = acc[c];
+    for (int c = 0; c < kNT; ++c) red[wib * kDepBuf + c * kLanes + lane] = deposit_sum(acc[c], ea[deposit_group<5>(c)]);
     __syncthreads();
     for (int e = threadIdx.x; e < NE; e += kThreads) {   // the block's warps, in warp order
       double v = red[e];
@@ -966,9 +1044,16 @@ __device__ __forceinline__ void combine_phase(const Batch& B, const double* part
       g = &B.box[box_of_cell(B, gc)];
       const int lc = gc - g->coff;
       const int tile = lc / B.T, k = lc - tile * B.T;
-      const int64_t gtile = g->toff + tile;
-      const int64_t wf = warp_of_unit(g->uoff + (int64_t)tile * g->M, B);
-      const int64_t wl = warp_of_unit(g->uoff + (int64_t)(tile + 1) * g->M - 1, B);
+      // the slots of the tile's partials: of the warps that own units of it, or of its parts
+      int64_t gtile = g->toff + tile, wf, wl;
+      if (B.dpb > 0) {
+        wf = first_part(B, g, tile);
+        wl = wf + (g->M + B.dpb - 1) / B.dpb - 1;
+        gtile = 0;
+      } else {
+        wf = warp_of_unit(g->uoff + (int64_t)tile * g->M, B);
+        wl = warp_of_unit(g->uoff + (int64_t)(tile + 1) * g->M - 1, B);
+      }
       const double* src = partial + c * B.T + k;
       double a[kCombineILP] = {};
       int64_t q = wf + wi;
@@ -1258,7 +1343,7 @@ __device__ __forceinline__ int potential_operands(const double (&v)[NV], F put) 
 // the whole block: one (cell, exponent group) per thread and round.
 template <bool COH, class Table>
 __device__ __forceinline__ void slab_table(Table& t, const double* A, int NZ, const BoxGeo& g, int c0, int n) {
-  for (int q = threadIdx.x; q < 4 * n; q += kThreads) {
+  for (int q = threadIdx.x; q < 4 * n; q += blockDim.x) {
     const int grp = q / n, c = q - grp * n;
     const double* Aj = A + g.coff + wrapc(c0 + c, g.nz) + (int64_t)2 * grp * NZ;
     double v[8];
@@ -1301,8 +1386,7 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
   constexpr int ny = S == 2 ? 18 : 0, nacc = S == 1 ? 0 : 18, nz_ = S == 4 ? 1 : 0;
   const int narr = 18 + ny + nacc + nz_ + (wrow != nullptr ? 0 : NWS);
   __syncthreads();
-  if (threadIdx.x < (unsigned)narr) {
-    const int a = threadIdx.x;
+  for (int a = threadIdx.x; a < narr; a += blockDim.x) {
     const double* arr;
     if (a < 18) arr = a < 9 ? src_r + a * P : src_b + (a - 9) * P;
     else if (a < 18 + nacc) arr = pt.acc + (a - 18) * P;
@@ -1314,9 +1398,9 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
   }
   // slabs: this block's tile units [x, x1), a (slab, direction) pair belonging
   // to the block its first unit falls to; otherwise its parts part, part + grid, ..
-  int64_t x = (int64_t)blockIdx.x * B.US / gridDim.x;
-  const int64_t x1 = ((int64_t)blockIdx.x + 1) * B.US / gridDim.x;
-  int64_t part = blockIdx.x;
+  int64_t x = B.slabs ? (int64_t)blockIdx.x * B.US / gridDim.x : 0;
+  const int64_t x1 = B.slabs ? ((int64_t)blockIdx.x + 1) * B.US / gridDim.x : 0;
+  int part = blockIdx.x;
   int b = B.slabs && x < x1 ? box_of_slab_unit(B, x) : 0;
   while (true) {
     int slab, d0, d1, sw = 1;
@@ -1338,20 +1422,19 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
       d1 = (int)min((int64_t)M, (int64_t)d0 + (q1 - q));
       x = g.soff + (q + (d1 - d0)) * sw;
     } else {
-      int64_t k = part;
-      int per = 0;
+      int k = part, per = 0;
       for (b = 0; b < B.nbox; ++b) {
         per = (B.box[b].M + B.upb - 1) / B.upb;   // parts of a tile
-        const int64_t all = (int64_t)per * B.box[b].ntiles32;
+        const int all = per * B.box[b].ntiles32;
         if (k < all) break;
         k -= all;
       }
       if (b == B.nbox) break;
       part += gridDim.x;
-      slab = (int)(k / per);
-      const int i = (int)(k - (int64_t)slab * per), M = B.box[b].M;
-      d0 = (int)((int64_t)i * M / per);
-      d1 = (int)((int64_t)(i + 1) * M / per);
+      slab = k / per;
+      const int i = k - slab * per, M = B.box[b].M, len = M / per, more = M - len * per;
+      d0 = i * len + min(i, more);   // (the first `more` parts take one more)
+      d1 = d0 + len + (i < more);
     }
     const BoxGeo& g = B.box[b];
     const int nz = g.nz;
@@ -1362,7 +1445,7 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
     const int tile0 = (wib & (sw - 1)) * kLanes;       // this warp's tile within the slab, in cells
     const int n = min(kLanes, nz - c0 - tile0);
     if (n <= 0) continue;
-    const int dstep = kWarps / sw;
+    const int dstep = (int)(blockDim.x >> 5) / sw;
     double bdt, cdt;
     const double dtb = B.dt[b];
     rk_coefficients(S == 2 ? s : S, dtb, bdt, cdt);
@@ -2112,8 +2195,13 @@ template <int ORDER>
 __device__ __forceinline__ void fused_deposit(const Batch& B, int64_t w, int lane, const Parts& pt, const double* rnu,
                                            const double* rnb, const StepArgs& a, const int* srow,
                                            const double* wrow, double frac, double* buf) {
-  deposit_phase<5, ORDER, true>(B, w, lane, pt.z, pt.N, pt.Nbar, rnu, rnb, a.dirtab, srow, wrow, frac, a.partial,
-                                wrow != nullptr ? nullptr : a.W, a.err, buf);
+  double* W = wrow != nullptr ? nullptr : a.W;
+  if (B.dpb > 0)
+    deposit_phase<5, ORDER, true, true>(B, w, lane, pt.z, pt.N, pt.Nbar, rnu, rnb, a.dirtab, srow, wrow, frac,
+                                        a.partial, W, a.err, buf);
+  else
+    deposit_phase<5, ORDER, true, false>(B, w, lane, pt.z, pt.N, pt.Nbar, rnu, rnb, a.dirtab, srow, wrow, frac,
+                                         a.partial, W, a.err, buf);
 }
 
 __device__ __forceinline__ void fused_combine(const Batch& B, const StepArgs& a) {
