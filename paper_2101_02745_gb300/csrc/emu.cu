@@ -415,6 +415,12 @@ int after_launch(emu_box* b, const char* what) {
 }
 
 dim3 persist_grid(const emu_box* b) { return dim3((unsigned)b->blocks, 1, 1); }
+// Grid and block of the RK stage (and the adjoint's first kernel): the
+// persistent grid with slabs, a block a part (while they last) with parts.
+dim3 rk_grid(const emu_box* b, const Batch& B) {
+  return B.slabs ? persist_grid(b) : dim3((unsigned)std::min<int64_t>(parts(b, B.upb, false), b->blocks));
+}
+int rk_threads(const Batch& B) { return B.slabs ? kThreads : part_warps(B.upb) * kLanes; }
 
 // Warps per group of 32 outputs in k_combine.  Long sums (more than 8
 // partials per tile: small boxes, whose warps own one unit or few) are split
@@ -885,14 +891,12 @@ int launch_rk_on(emu_box* b, int s, const int* srow, int dry, const Parts& pt, c
     constexpr int R = decltype(O)::value;
     const Batch Bv = batch_view(b);
     const double* wrow = weight_row(b, srow);
-    const int threads = Bv.slabs ? kThreads : part_warps(Bv.upb) * kLanes;
-    const dim3 grid = Bv.slabs ? persist_grid(b) : dim3((unsigned)std::min<int64_t>(parts(b, Bv.upb, false), b->blocks));
     auto launch_tiles = [&](auto POT, auto STAGE, auto TILES) {
       static std::atomic<unsigned> done{0};
       constexpr int T = decltype(TILES)::value, smem = (int)sizeof(SlabTable<T>);
       auto k = k_rk_stage<decltype(POT)::value, R, decltype(STAGE)::value, T>;
       if (raise_smem(k, smem, done) == cudaSuccess)
-        pdl_smem(b->stream, k, grid, threads, smem, Bv, pt, W, wrow, b->dirtab, srow, At, stage_src, s, dry);
+        pdl_smem(b->stream, k, rk_grid(b, Bv), rk_threads(Bv), smem, Bv, pt, W, wrow, b->dirtab, srow, At, stage_src, s, dry);
     };
     by_stage(b->pot, s, [&](auto POT, auto STAGE) {
       if (Bv.slabs) launch_tiles(POT, STAGE, std::integral_constant<int, kSlabTiles>{});
@@ -2311,6 +2315,31 @@ int record_step(emu_box* b, double* rec) {
   return EMU_OK;
 }
 
+// First adjoint kernel of stage s: the RK stage's work split.
+int launch_adj_a(emu_box* b, const Parts& ps, const double* W, const int* srow, const double* H, const AdjStage& x,
+                 int s) {
+  before_launch(b, CLS_OTHER);
+  const Batch B = batch_view(b);
+  by_order(b->S.order, [&](auto O) {
+    constexpr int R = decltype(O)::value;
+    auto launch = [&](auto POT, auto TILES) {
+      static std::atomic<unsigned> done{0};
+      constexpr int T = decltype(TILES)::value, smem = (int)sizeof(SlabTable<T>);
+      auto k = k_adj_a<decltype(POT)::value, R, T>;
+      if (raise_smem(k, smem, done) == cudaSuccess)
+        pdl_smem(b->stream, k, rk_grid(b, B), rk_threads(B), smem, B, ps, W, b->dirtab, srow, H, x, s);
+    };
+    auto tiles = [&](auto POT) {
+      if (B.slabs) launch(POT, std::integral_constant<int, kSlabTiles>{});
+      else launch(POT, std::integral_constant<int, 1>{});
+    };
+    if (b->pot) tiles(std::true_type{});
+    else tiles(std::false_type{});
+    return 0;
+  });
+  return after_launch(b, "adjoint stage kernel");
+}
+
 // The backward stages of one adjoint step from a record (no recomputation).
 int adjoint_recorded_body(emu_box* b, const double* rec, double* lambda, double* gN, double* gNbar, void* adj_ws) {
   const size_t P = (size_t)b->S.Ptot;
@@ -2338,18 +2367,7 @@ int adjoint_recorded_body(emu_box* b, const double* rec, double* lambda, double*
     ps.rho = ys;
     ps.rhobar = ysb;
     double* Lcur = (s % 2 == 0) ? La : Lb;
-    before_launch(b, CLS_OTHER);
-    by_order(b->S.order, [&](auto O) {
-      constexpr int R = decltype(O)::value;
-      if (b->pot)
-        pdl(b->stream, k_adj_a<true, R>, persist_grid(b), B, ps, Ws, b->dirtab, srow, Hs, lambda,
-            Lnext, s, Lcur, b->pt.acc);
-      else
-        pdl(b->stream, k_adj_a<false, R>, persist_grid(b), B, ps, Ws, b->dirtab, srow, Hs, lambda,
-            Lnext, s, Lcur, b->pt.acc);
-      return 0;
-    });
-    if (int rc = after_launch(b, "adjoint stage kernel")) return rc;
+    if (int rc = launch_adj_a(b, ps, Ws, srow, Hs, AdjStage{lambda, Lnext, Lcur, b->pt.acc}, s)) return rc;
     if (int rc = launch_deposit(b, 3, b->pt.acc, nullptr, srow, kStageFrac[s - 1], b->mom)) return rc;
     before_launch(b, CLS_OTHER);
     by_order(b->S.order, [&](auto O) {
@@ -2413,18 +2431,7 @@ int adjoint_body(emu_box* b, double* lambda, double* gN, double* gNbar, void* ad
     ps.rho = ys;
     ps.rhobar = ysb;
     double* Lcur = (s % 2 == 0) ? La : Lb;
-    before_launch(b, CLS_OTHER);
-    by_order(b->S.order, [&](auto O) {
-      constexpr int R = decltype(O)::value;
-      if (b->pot)
-        pdl(b->stream, k_adj_a<true, R>, persist_grid(b), B, ps, Ws, b->dirtab, srow, Hs, lambda,
-            Lnext, s, Lcur, b->pt.acc);
-      else
-        pdl(b->stream, k_adj_a<false, R>, persist_grid(b), B, ps, Ws, b->dirtab, srow, Hs, lambda,
-            Lnext, s, Lcur, b->pt.acc);
-      return 0;
-    });
-    if (int rc = after_launch(b, "adjoint stage kernel")) return rc;
+    if (int rc = launch_adj_a(b, ps, Ws, srow, Hs, AdjStage{lambda, Lnext, Lcur, b->pt.acc}, s)) return rc;
     if (int rc = launch_deposit(b, 3, b->pt.acc, nullptr, srow, frac, b->mom)) return rc;
     before_launch(b, CLS_OTHER);
     by_order(b->S.order, [&](auto O) {

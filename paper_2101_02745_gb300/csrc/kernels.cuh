@@ -1237,29 +1237,104 @@ __device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, co
   }
 }
 
-// rk_update of particle p of box g from H in the traceless components as
-// hv[c] 2^(he[c / 2] - kBiasV), |hv| < 2^60.6.
+// H in the traceless components given as hv[c] 2^(he[c / 2] - kBiasV),
+// |hv| < 2^60.6: as doubles, and as the commutator's operand.
+__device__ __forceinline__ void operand_values(const int64_t (&hv)[kNC], const int (&he)[4], double (&Hm)[kNC]) {
+  namespace w = emu_wide;
+#pragma unroll
+  for (int c = 0; c < kNC; ++c)
+    Hm[c] = (double)hv[c] * w::scale(1.0, he[c >> 1] < w::kExpNonFinite ? max(he[c >> 1] - w::kBiasV, -1022) : 1024);
+}
+__device__ __forceinline__ emu_wide::Ham operand_ham(const int64_t (&hv)[kNC], const int (&he)[4]) {
+  namespace w = emu_wide;
+  w::Ham hm;
+  hm.d12 = w::Real{w::split(hv[0]), he[0]};
+  hm.d13 = w::Real{w::split(hv[0] + hv[1]), he[0]};
+  hm.d23 = w::Real{w::split(hv[1]), he[0]};
+  hm.a = w::Cplx{w::split(hv[2]), w::split(hv[3]), he[1]};
+  hm.b = w::Cplx{w::split(hv[4]), w::split(hv[5]), he[2]};
+  hm.c = w::Cplx{w::split(hv[6]), w::split(hv[7]), he[3]};
+  return hm;
+}
+
+// rk_update of particle p of box g from H (hv, he as operand_values).
 template <bool POT, int S, bool COH>
 __device__ __forceinline__ void rk_from_H(const BoxGeo& g, const Parts& pt, const double* src_b, int64_t P, int64_t p,
                                           int dry, double bdt, double cdt, double dtb, const double* vz,
                                           const int64_t (&hv)[kNC], const int (&he)[4], double (&r)[9]) {
-  namespace w = emu_wide;
   if constexpr (POT) {
     double Hm[kNC];
-#pragma unroll
-    for (int c = 0; c < kNC; ++c)
-      Hm[c] = (double)hv[c] * w::scale(1.0, he[c >> 1] < w::kExpNonFinite ? max(he[c >> 1] - w::kBiasV, -1022) : 1024);
+    operand_values(hv, he, Hm);
     rk_particle<POT, S, COH>(g, pt, src_b, P, p, dry, bdt, cdt, dtb, vz, Hm, r);
   } else {
-    w::Ham hm;
-    hm.d12 = w::Real{w::split(hv[0]), he[0]};
-    hm.d13 = w::Real{w::split(hv[0] + hv[1]), he[0]};
-    hm.d23 = w::Real{w::split(hv[1]), he[0]};
-    hm.a = w::Cplx{w::split(hv[2]), w::split(hv[3]), he[1]};
-    hm.b = w::Cplx{w::split(hv[4]), w::split(hv[5]), he[2]};
-    hm.c = w::Cplx{w::split(hv[6]), w::split(hv[7]), he[3]};
+    const emu_wide::Ham hm = operand_ham(hv, he);
     rk_update<S, false, COH>(g.Lz, pt, src_b, P, p, dry, bdt, cdt, dtb, vz, hm, hm, r);
   }
+}
+
+// Arrays of the adjoint's first stage kernel (k_adj_a).
+struct AdjStage {
+  const double *lam, *lamn;   // adjoint of the step's result and of the next stage's state (NULL at stage 4)
+  double *out, *gam;          // adjoint of this stage's state (direct terms), and of its H
+};
+
+// k_adj_a for particle p: r its neutrino matrix (loaded), H as rk_from_H.  The
+// antineutrinos take the neutrinos' operand: with h = H - Vbar^* (H without
+// potentials) -K(Hbar, m) = -conj K(h, m^*) and -conj K(rbar, m) = K(rbar^*, m^*).
+template <bool POT>
+__device__ __forceinline__ void adj_update(const BoxGeo& g, const Parts& pt, int64_t P_, int64_t p, double a, double c,
+                                           const AdjStage& x, const int64_t (&hv)[kNC], const int (&he)[4],
+                                           double (&r)[9]) {
+  namespace w = emu_wide;
+  const unsigned P = (unsigned)P_;
+  double Hm[kNC], Gm[9];
+  w::Ham h;
+  if constexpr (POT) operand_values(hv, he, Hm);
+  else h = operand_ham(hv, he);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) Gm[k] = 0.0;
+#pragma unroll 1
+  for (int which = 0; which < 2; ++which) {
+    const double* lam = row(x.lam, P, which * 9) + p;
+    const double* ln = row(x.lamn, P, which * 9) + p;
+    double* out = row(x.out, P, which * 9) + p;
+    double m2[9], kd[3], ko[6];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const double f = k < 3 ? 2.0 : 1.0;
+      m2[k] = f * a * __ldg(row(lam, P, k));
+      if (x.lamn != nullptr) m2[k] = fma(f * c, __ldg(row(ln, P, k)), m2[k]);
+    }
+    const w::Mat m = w::mat(m2, which);
+    if constexpr (POT) {
+      double v[kNC];
+#pragma unroll
+      for (int k = 0; k < kNC; ++k) {
+        const bool im = k == 3 || k == 5 || k == 7;
+        const double vb = __ldg(g.vnubar + k);
+        v[k] = Hm[k] + (which == 0 ? __ldg(g.vnu + k) : im ? vb : -vb);
+      }
+      h = w::ham(v);
+    }
+    commutator(h, m, kd, ko);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) *row(out, P, k) = -kd[k];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) *row(out, P, 3 + k) = (k & 1) && which ? ko[k] : -ko[k];
+    const double cj = which ? -1.0 : 1.0;
+    const double rt[kNC] = {r[0] - r[1], r[1] - r[2], r[3], cj * r[4], r[5], cj * r[6], r[7], cj * r[8]};
+    w::Ham rh = w::ham(rt);
+    rh.d13 = w::real(r[0] - r[2]);
+    if (which == 0) {   // the antineutrinos' matrix
+#pragma unroll
+      for (int k = 0; k < 9; ++k) r[k] = __ldg(row(pt.rhobar + p, P, k));
+    }
+    commutator(rh, m, kd, ko);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) Gm[k] += k < 3 ? kd[k] : ko[k - 3];
+  }
+#pragma unroll
+  for (int k = 0; k < 9; ++k) *row(x.gam + p, P, k) = Gm[k];
 }
 
 // Box of tile unit x of the slabs (a pair of a slab and a direction counts as
@@ -1372,7 +1447,8 @@ __device__ __forceinline__ int2 table_G(const Table& t, int c, int j, const emu_
 template <bool POT, int ORDER, int S, bool COH, class Table>
 __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const double* W, const double* wrow,
                                          const double* __restrict__ dirtab, const int* shift, const double* A,
-                                         const double* stage_src, int s, int dry, Table& t) {
+                                         const double* stage_src, int s, int dry, Table& t,
+                                         const AdjStage& adj = {}) {
   namespace w = emu_wide;
   constexpr int H = ORDER == 0 ? 0 : Sten<ORDER>::H, NW = ORDER == 0 ? 1 : Sten<ORDER>::NW;
   constexpr int NWS = Sten<ORDER>::NWS;
@@ -1380,16 +1456,18 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
   const int wib = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
   const int64_t P = B.Ptot;
   const int MT = B.MT;
-  const double* src_r = S == 1 ? pt.rho : stage_src;
-  const double* src_b = S == 1 ? pt.rhobar : stage_src + 9 * P;
+  const double* src_r = S <= 1 ? pt.rho : stage_src;
+  const double* src_b = S <= 1 ? pt.rhobar : stage_src + 9 * P;
   // the arrays this stage reads per particle
-  constexpr int ny = S == 2 ? 18 : 0, nacc = S == 1 ? 0 : 18, nz_ = S == 4 ? 1 : 0;
+  const int ny = S == 2 || (S == 0 && adj.lamn != nullptr) ? 18 : 0;
+  constexpr int nacc = S == 1 ? 0 : 18, nz_ = S == 4 ? 1 : 0;
   const int narr = 18 + ny + nacc + nz_ + (wrow != nullptr ? 0 : NWS);
   __syncthreads();
   for (int a = threadIdx.x; a < narr; a += blockDim.x) {
     const double* arr;
     if (a < 18) arr = a < 9 ? src_r + a * P : src_b + (a - 9) * P;
-    else if (a < 18 + nacc) arr = pt.acc + (a - 18) * P;
+    else if (a < 18 + nacc) arr = (S == 0 ? adj.lam : pt.acc) + (a - 18) * P;
+    else if (S == 0 && a < 18 + nacc + ny) arr = adj.lamn + (a - 18 - nacc) * P;
     else if (a < 18 + nacc + ny) arr = a - 18 - nacc < 9 ? pt.rho + (a - 18 - nacc) * P
                                                          : pt.rhobar + (a - 18 - nacc - 9) * P;
     else if (a < 18 + nacc + ny + nz_) arr = pt.z;
@@ -1448,7 +1526,7 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
     const int dstep = (int)(blockDim.x >> 5) / sw;
     double bdt, cdt;
     const double dtb = B.dt[b];
-    rk_coefficients(S == 2 ? s : S, dtb, bdt, cdt);
+    rk_coefficients(S == 2 || S == 0 ? s : S, dtb, bdt, cdt);
     const int64_t poff = g.poff;
     const int doff = g.doff;
     const int tc = tile0 + H + lane;                   // table cell of this lane
@@ -1559,7 +1637,8 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
         }
 #pragma unroll
         for (int grp = 0; grp < 4; ++grp) he[grp] += 2;
-        rk_from_H<POT, S, COH>(g, pt, src_b, P, p, dry, bdt, cdt, dtb, dirtab + 3 * MT + gd, hv, he, r);
+        if constexpr (S == 0) adj_update<POT>(g, pt, P, p, bdt, cdt, adj, hv, he, r);
+        else rk_from_H<POT, S, COH>(g, pt, src_b, P, p, dry, bdt, cdt, dtb, dirtab + 3 * MT + gd, hv, he, r);
       }
       __syncwarp();   // (the unit's G are rewritten by the next)
     }
@@ -2424,91 +2503,20 @@ static __global__ void k_diagnostics(Batch B, const double* __restrict__ mom, do
 // First adjoint launch of stage s.  m = a lam + c lamn, the adjoint of this
 // stage's derivative k_s, with the box's step dt: a = dt/6 (s = 1, 4) or dt/3,
 // c = dt/2 (s = 1, 2) or dt (s = 3), lamn the adjoint of stage s + 1 (NULL
-// for s = 4); writes lam_out = J_rho^T m (direct terms) and Gam = dL/dH_self.
+// for s = 4); writes x.out = J_rho^T m (direct terms) and x.gam = dL/dH_self.
 // pt.rho / pt.rhobar point at the stage state.  The metric D folds into the
 // commutator: D K(X, D^-1 m) is the commutator's raw output (halved diagonal,
 // off-diagonals) for X and m2 = m with its diagonal doubled, so
-//   lam_out = -D K(H, D^-1 m) = raw(-H, m2),   Gamma += S D K(r, D^-1 m) = S raw(r, m2).
-template <bool POT, int ORDER>
+//   out = -D K(H, D^-1 m) = raw(-H, m2),   gam += S D K(r, D^-1 m) = S raw(r, m2).
+// H is formed as in the RK stage (rk_phase: the same work split, tables and
+// integer arithmetic).
+template <bool POT, int ORDER, int TILES>
 __global__ void __launch_bounds__(kThreads, 2)
 k_adj_a(Batch B, Parts pt, const double* __restrict__ W, const double* __restrict__ dirtab,
-        const int* __restrict__ shift, const double* __restrict__ A, const double* __restrict__ lam,
-        const double* __restrict__ lamn, int s, double* __restrict__ lam_out, double* __restrict__ Gam) {
+        const int* __restrict__ shift, const double* __restrict__ A, AdjStage x, int s) {
+  extern __shared__ char smem[];
   griddep_wait();
-  const int lane = threadIdx.x & 31;
-  const int64_t w = logical_warp();
-  const int64_t u0 = unit_begin(w, B), u1 = unit_begin(w + 1, B);
-  if (u0 >= u1) return;
-  const int64_t P = B.Ptot;
-  const int MT = B.MT, NZ = B.NZ;
-  int b = box_of_unit(B, u0);
-  for (int64_t u = u0; u < u1; ++u) {
-    while (u >= B.box[b].uoff + (int64_t)B.box[b].ntiles * B.box[b].M) ++b;
-    const BoxGeo& g = B.box[b];
-    const double dtb = B.dt[b];
-    const double a = (s == 1 || s == 4) ? dtb / 6.0 : dtb / 3.0;
-    const double bc = (s == 3) ? dtb : 0.5 * dtb;
-    const int nz = g.nz, nt = g.ntiles;
-    const int lu = (int)(u - g.uoff);
-    const int d = lu / nt, tile = lu - d * nt;
-    constexpr int Hh = Sten<ORDER>::H, T = Sten<ORDER>::T;
-    const int craw = tile * T - Hh + lane, j = wrapc(craw, nz);
-    const bool active = lane >= Hh && lane < Hh + T && craw < nz;
-    const int gd = g.doff + d;
-    const double ox = __ldg(dirtab + gd), oy = __ldg(dirtab + MT + gd), oz = __ldg(dirtab + 2 * MT + gd);
-    const int64_t p = g.poff + (int64_t)d * nz + wrapc(j - __ldg(shift + gd), nz);
-    double wt[Sten<ORDER>::NW];
-    zero_weights<ORDER>(wt);
-    if (active) load_weights<ORDER>(W, P, p, wt);
-    double H[kNC];   // traceless components of the stage's H
-    const double* Aj = A + g.coff + j;
-#pragma unroll
-    for (int c = 0; c < kNC; ++c) {
-      const double G = fma(-oz, __ldg(Aj + (int64_t)(3 * kNC + c) * NZ),
-                           fma(-oy, __ldg(Aj + (int64_t)(2 * kNC + c) * NZ),
-                               fma(-ox, __ldg(Aj + (int64_t)(kNC + c) * NZ), __ldg(Aj + (int64_t)c * NZ))));
-      H[c] = gather<ORDER>(wt, G);
-    }
-    if (!active) continue;
-    const double a2 = 2.0 * a, bc2 = 2.0 * bc;
-    double Gm[9];
-#pragma unroll
-    for (int which = 0; which < 2; ++which) {
-      double nH[kNC], r[9], m2[9], kd[3], ko[6];   // (the commutators on the integer pipe, as the RK stage's)
-#pragma unroll
-      for (int c = 0; c < kNC; ++c) {                                       // -(S H + V), S for antineutrinos
-        const bool im = (c == 3 || c == 5 || c == 7);
-        const double nsgn = which ? (im ? -1.0 : 1.0) : -1.0;
-        nH[c] = nsgn * H[c] - (POT ? __ldg((which ? g.vnubar : g.vnu) + c) : 0.0);
-      }
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        const double l = lam[(which * 9 + k) * P + p];
-        const double ln = lamn ? lamn[(which * 9 + k) * P + p] : 0.0;
-        m2[k] = k < 3 ? fma(a2, l, bc2 * ln) : fma(a, l, bc * ln);
-        r[k] = (which ? pt.rhobar : pt.rho)[k * P + p];
-      }
-      const emu_wide::Mat mm = emu_wide::mat(m2, false);
-      commutator(emu_wide::ham(nH), mm, kd, ko);
-#pragma unroll
-      for (int k = 0; k < 3; ++k) lam_out[(which * 9 + k) * P + p] = kd[k];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) lam_out[(which * 9 + 3 + k) * P + p] = ko[k];
-      const double rt[kNC] = {r[0] - r[1], r[1] - r[2], r[3], r[4], r[5], r[6], r[7], r[8]};
-      emu_wide::Ham rh = emu_wide::ham(rt);
-      rh.d13 = emu_wide::real(r[0] - r[2]);
-      commutator(rh, mm, kd, ko);
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        const bool im = (k == 4 || k == 6 || k == 8);
-        const double v = k < 3 ? kd[k] : ko[k - 3];
-        if (which == 0) Gm[k] = v;
-        else Gm[k] += (im ? v : -v);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) Gam[k * P + p] = Gm[k];
-  }
+  rk_phase<POT, ORDER, 0, false>(B, pt, W, nullptr, dirtab, shift, A, nullptr, s, 0, *(SlabTable<TILES>*)smem, x);
 }
 
 // Second adjoint launch of one stage: GB = interpolation of the deposited
