@@ -1517,12 +1517,8 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
     const BoxGeo& g = B.box[b];
     const int nz = g.nz;
     const int c0 = slab * sw * kLanes;
-    __syncthreads();   // (the previous slab's table is free, and pf is written)
-    slab_table<COH>(t, A, B.NZ, g, c0 - H, min(sw * kLanes, nz - c0) + 2 * H);
-    __syncthreads();
     const int tile0 = (wib & (sw - 1)) * kLanes;       // this warp's tile within the slab, in cells
     const int n = min(kLanes, nz - c0 - tile0);
-    if (n <= 0) continue;
     const int dstep = (int)(blockDim.x >> 5) / sw;
     double bdt, cdt;
     const double dtb = B.dt[b];
@@ -1540,10 +1536,17 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
       return lane < 3 ? -v : v;
     };
     const int dw = d0 + wib / sw;
-    if (dw >= d1) continue;
-    const bool active = lane < n;
-    double unext = own_number(doff + dw);
-    int shnext = ldi<COH>(shift + doff + dw);
+    const bool active = lane < n, some = n > 0 && dw < d1;
+    double unext = 0.0;
+    int shnext = 0;
+    if (some) {   // (these loads' latency before the table's)
+      unext = own_number(doff + dw);
+      shnext = ldi<COH>(shift + doff + dw);
+    }
+    __syncthreads();   // (the previous slab's table is free, and pf is written)
+    slab_table<COH>(t, A, B.NZ, g, c0 - H, min(sw * kLanes, nz - c0) + 2 * H);
+    __syncthreads();
+    if (!some) continue;
     for (int d = dw; d < d1; d += dstep) {
       const int gd = doff + d;
       const int sh = shnext;
