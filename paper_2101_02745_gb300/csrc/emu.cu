@@ -2564,7 +2564,7 @@ int emu_weight_gradient(emu_box* b, const double* gN, const double* gNbar, doubl
   if (b->is3d) return no_3d(b, "the adjoint");
   if (!gN || !gNbar || !out) return fail(b, EMU_EINVAL, "weight gradient: NULL pointer");
   double* dst = on_host ? b->mom : out;  // staging: the moments buffer holds 72 NZ doubles
-  const int blocks = (b->S.NZ + kThreads - 1) / kThreads;
+  const int blocks = (b->S.NZ + kLanes - 1) / kLanes;
   before_launch(b, CLS_OTHER);
   k_weight_grad<<<blocks, kThreads, 0, b->stream>>>(batch_view(b), gN, gNbar, b->dirtab, dst);
   if (int rc = after_launch(b, "weight gradient kernel")) return rc;
