@@ -1,6 +1,6 @@
 // kernels.cuh -- GB300 (sm_103a) FP64 device code of the particle-in-cell step
 // for the neutrino fast flavour instability (Richers, Willcox, Ford & Myers,
-// arXiv:2101.02745).  Included once, by emu.cu.
+// arXiv:2101.02745).  Included by emu.cu and instances.cuh.
 //
 // A *batch* is a set of independent 1D periodic boxes advanced together; one
 // box is a batch of one.  All arrays of a batch are concatenated:
@@ -25,11 +25,13 @@
 // RK stage has no halo lanes (32-cell tiles, the tile ends through shared
 // memory); its commutators and stencil sums run on the integer pipe (wide.cuh).
 //
-// Persistent schedule.  The step kernels run a fixed grid (2 blocks of 8 warps
-// per SM); the first nw warps split the U units of the batch into equal
-// contiguous ranges.  The deposit's summation order (registers over a warp's
-// directions, one partial per (warp, tile), partials added in warp order by
-// k_combine) depends only on the batch and nw: no atomics, bitwise reproducible.
+// Schedule.  Large boxes run a fixed grid (2 blocks of 8 warps per SM): in the
+// deposit the first nw warps split the U units of the batch into equal contiguous
+// ranges, in the RK stage the blocks split the (slab, direction) pairs.  Small
+// boxes: a block takes a part of one tile's directions.  The deposit's summation
+// order (integer sums over a warp's directions and a part's warps, one partial per
+// (warp, tile) or part, partials added in order by k_combine) depends only on the
+// batch and the grid: no atomics, bitwise reproducible.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -590,7 +592,7 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
                                                   const double* __restrict__ Nbar, const double* r_nu,
                                                   const double* r_nb, const double* __restrict__ dirtab,
                                                   const int* shift, const double* wrow, double frac, double* W,
-                                                  double* buf, int ring2, int n,
+                                                  double* buf, int ring2,
                                                   int64_t (&acc)[DepMode<MODE>::NA],
                                                   int (&ea)[DepMode<MODE>::SETS * DepMode<MODE>::GROUPS], int& bad) {
   namespace w = emu_wide;
@@ -606,7 +608,7 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
   const bool own = lane >= H && lane < H + T && craw < nz;
   const double pos_dt = frac * B.dt[b];
   const int dbase = g.doff;
-  const int head = max(32 - __clz(n), 2) - 2;   // headroom beyond the two bits a contribution leaves
+  const int head = max(32 - __clz(dlast - dfirst), 2) - 2;   // headroom beyond the two bits a contribution leaves
 #pragma unroll
   for (int c = 0; c < D::NA; ++c) acc[c] = 0;
 #pragma unroll
@@ -821,7 +823,8 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
   int bad = 0;
   if constexpr (PART) {
     // few units: a block takes a part of one tile's directions, adds its warps'
-    // sums (as integers, at their largest exponent) and writes one partial
+    // sums (as integers, rounded at their largest exponent: a warp's sum has
+    // headroom for its own directions only) and writes one partial
     const int wib = threadIdx.x >> 5;
     const int nwarps = part_warps(B.dpb);                         // (the block's, but in k_step)
     int64_t* sums = (int64_t*)(buf - wib * kDepBuf);              // [warp][row][lane], then the exponents
@@ -836,7 +839,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
         int64_t acc[D::NA];
         int ea[D::SETS * D::GROUPS];
         deposit_tile<MODE, ORDER, COH>(B, b, tile, w0, w0 + len + (wib < more), lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                       wrow, frac, W, buf, 1, n, acc, ea, bad);
+                                       wrow, frac, W, buf, 1, acc, ea, bad);
 #pragma unroll
         for (int c = 0; c < D::NA; ++c) sums[wib * kDepBuf + c * kLanes + lane] = acc[c];
 #pragma unroll
@@ -850,10 +853,11 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
           int top = 0, e[kWarps];
 #pragma unroll
           for (int x = 0; x < kWarps; ++x) top = max(top, e[x] = x < used ? ex[x * 2 * kDepBuf] : 0);
+          top += 3;   // headroom for 8 warps
           int64_t v = 0;
 #pragma unroll
           for (int x = 0; x < kWarps; ++x)
-            if (x < used) v += emu_wide::align(sums[x * kDepBuf + c * kLanes + lane], top - e[x]);
+            if (x < used) v += emu_wide::align_round(sums[x * kDepBuf + c * kLanes + lane], top - e[x]);
           partial[(int64_t)q * kSlot + c * T + lane - H] = deposit_sum(v, top);
         }
       }
@@ -877,7 +881,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
     int64_t sum[D::NA];
     int ea[D::SETS * D::GROUPS];
     deposit_tile<MODE, ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow, frac, W,
-                                   buf, B.U > B.nw, dlast - dfirst, sum, ea, bad);
+                                   buf, B.U > B.nw, sum, ea, bad);
     double acc[D::NA];
 #pragma unroll
     for (int c = 0; c < D::NA; ++c) acc[c] = deposit_sum(sum[c], ea[deposit_group<MODE>(c)]);
@@ -984,7 +988,7 @@ k_deposit_cluster(Batch B, const double* __restrict__ z, const double* __restric
     for (int c = 0; c < DepMode<5>::GROUPS; ++c) ea[c] = 0;
     if (d0 < d1)
       deposit_tile<5, ORDER, false>(B, b, tile, d0, d1, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                    TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, 1, d1 - d0, acc, ea, bad);
+                                    TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, 1, acc, ea, bad);
 #pragma unroll
     for (int c = 0; c < kNT; ++c) red[wib * kDepBuf + c * kLanes + lane] = deposit_sum(acc[c], ea[deposit_group<5>(c)]);
     __syncthreads();

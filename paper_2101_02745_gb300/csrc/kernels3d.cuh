@@ -1,8 +1,8 @@
 // kernels3d.cuh -- GB300 (sm_103a) FP64 device code of the particle-in-cell step
 // on a 3D periodic grid (the paper's method, Eq. 2, 4-6 and Sec. 2.3, on the 3D
-// grid it names as future work in Sec. 5).  Included once, by emu.cu, after
-// kernels.cuh, whose helpers (shape weights, Spread, gather, commutator,
-// rk_particle, k_combine) it reuses.
+// grid it names as future work in Sec. 5).  Included by emu.cu and
+// instances.cuh after kernels.cuh, whose helpers (shape weights, Spread, gather,
+// rk_from_H, k_combine) it reuses.
 //
 // A 3D box has nx x ny x nz cells (index c = (jx ny + jy) nz + jz; a *row* is
 // the nz cells of one (jx, jy)) and M directions; particle p = d C + site,
@@ -31,11 +31,13 @@
 // offset inside their cells (up to rounding), so their weights on each axis
 // are the direction's (k3_shifts computes them from the site-0 particle), and
 // the deposit of one direction is a 3-tap convolution along z, then y, then x
-// of its B field (k3_spread), summed over directions with (1, Omega) into the
+// of its B field (k3_pass), summed over directions with (1, Omega) into the
 // potential (k3_spread_x_sum); the interpolation of G = A0 - Omega . A is the
-// transposed convolution (k3_gather along x and y, then z by shuffles in
-// k3_rk_stage).  Three 3-tap passes per direction and cell instead of a
-// (2H+1)^2-row gather per particle.
+// transposed convolution (k3_pass along x and y, then z in k3_rk_stage).  Three
+// 3-tap passes per direction and cell instead of a (2H+1)^2-row gather per
+// particle.  The step's fields and weights are fixed-point operands (wide.cuh)
+// throughout: 64^3 x 16 passes 197 -> 116 us, direction sum 454 -> 234 us, step
+// 9.2 -> 6.5 ms against FP64 fields.
 #pragma once
 
 namespace emu_dev {

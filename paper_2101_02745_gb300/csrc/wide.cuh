@@ -231,6 +231,9 @@ EMU_HD int64_t align(int64_t v, int d, int d2) {
 }
 EMU_HD int64_t align(int64_t v, int d) { return align(v, d, max_i(d - 32, 0)); }
 
+// v / 2^d rounded to nearest, d >= 1.
+EMU_HD int64_t align_round(int64_t v, int d) { return (align(v, d - 1) + 1) >> 1; }
+
 // c 2^k for a normal c whose exponent stays normal.
 EMU_HD double scale(double c, int k) { return from_words(hi_word(c) + (int)((unsigned)k << 20), lo_word(c)); }
 // c 2^k for a positive normal c, k not below its smallest normal result; NaN
