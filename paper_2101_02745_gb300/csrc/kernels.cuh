@@ -574,7 +574,7 @@ struct DepMode {
 
 // The direction loop of the deposit for one tile: warp lane `lane` of a tile
 // of box b (lane l owns cell tile * T - H + l) adds the rings dfirst..dlast-1
-// of the tile, in order, to out (MODES as deposit_phase), on the integer pipe.
+// of the tile, in a fixed order, in acc (MODES as deposit_phase), on the integer pipe.
 // B is formed in FP64 (20 instructions a particle, against 85-100 for a deposit
 // with FP64 sums: at 16 cycles each the FP64 pipe bound it); its spread over the
 // stencil and the moments' sums are fixed-point (wide.cuh).  A sum is an
@@ -584,15 +584,22 @@ struct DepMode {
 // bits of headroom, so a contribution keeps 61 - ceil(log2 n) bits below the
 // largest one's leading bit: less error than FP64 sums of n terms, whose
 // rounding follows the partial sums.  Zero contributions add exactly nothing.
+// Bound by integer issue: 16384 x 1000 2467 -> 1040 us a stage against FP64 sums
+// (1256 with plain loads: cp.async hides their latency), 1024 x 378 74 -> 41 us.
 // (buf: this warp's two buffers of kDepRows x 32 doubles in shared memory;
 // ring2 0: only one, when no warp takes more than one direction of a tile.)
+// phase > 0: the directions in cyclic order from the first multiple of phase (a
+// warp's share), so that the warps of neighbouring tiles read the same ring at the
+// same time: a tile's 256-byte rows start anywhere in a 128-byte line, and lines
+// shared with the neighbours came from DRAM twice (268 bytes a particle for 168;
+// 16384 x 1000 1067 -> 1038 us).
 template <int MODE, int ORDER, bool COH>
 __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, int dfirst, int dlast, int lane,
                                                   const double* z, const double* __restrict__ N,
                                                   const double* __restrict__ Nbar, const double* r_nu,
                                                   const double* r_nb, const double* __restrict__ dirtab,
                                                   const int* shift, const double* wrow, double frac, double* W,
-                                                  double* buf, int ring2,
+                                                  double* buf, int ring2, int phase,
                                                   int64_t (&acc)[DepMode<MODE>::NA],
                                                   int (&ea)[DepMode<MODE>::SETS * DepMode<MODE>::GROUPS], int& bad) {
   namespace w = emu_wide;
@@ -615,11 +622,11 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
   for (int q = 0; q < D::SETS * D::GROUPS; ++q) ea[q] = 0;
   // direction d's particle data into buffer d & 1, asynchronously (each lane
   // its own particle's: no exchange between lanes): z, N, Nbar, rho, rhobar
-  auto fetch = [&](int d) -> int64_t {
+  auto fetch = [&](int d, int k) -> int64_t {
     int i = j - ldi<COH>(shift + dbase + d);
     if (i < 0) i += nz;
     const int64_t p = g.poff + (int64_t)d * nz + i;
-    double* dst = buf + (d & ring2) * kDepRows * kLanes + lane;
+    double* dst = buf + (k & ring2) * kDepRows * kLanes + lane;
     cp_async8(dst, z + p);
     if (D::N1) cp_async8(dst + kLanes, N + p);
     if (D::N2) cp_async8(dst + 2 * kLanes, Nbar + p);
@@ -631,17 +638,25 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
     cp_async_commit();
     return p;
   };
-  int64_t pnext = fetch(dfirst);
-  for (int d = dfirst; d < dlast; ++d) {
+  const int n = dlast - dfirst;
+  int dnext = dfirst;
+  if (phase > 0) {   // (no multiple of it among the directions: from dfirst)
+    const int o = (phase - dfirst % phase) % phase;
+    if (o < n) dnext += o;
+  }
+  int64_t pnext = fetch(dnext, 0);
+  for (int k = 0; k < n; ++k) {
+    const int d = dnext;
+    dnext = d + 1 < dlast ? d + 1 : dfirst;
     const int gd = dbase + d;
     const int64_t p = pnext;
-    if (d + 1 < dlast && ring2) {
-      pnext = fetch(d + 1);
+    if (k + 1 < n && ring2) {
+      pnext = fetch(dnext, k + 1);
       cp_async_wait<1>();
     } else {
       cp_async_wait<0>();
     }
-    const double* x = buf + (d & ring2) * kDepRows * kLanes + lane;
+    const double* x = buf + (k & ring2) * kDepRows * kLanes + lane;
     const double n1 = D::N1 ? x[kLanes] : 0.0, n2 = D::N2 ? x[2 * kLanes] : 0.0;
     // component k of the deposited matrix (conj(rhobar) flips the sign of the
     // imaginary components 4, 6, 8)
@@ -839,7 +854,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
         int64_t acc[D::NA];
         int ea[D::SETS * D::GROUPS];
         deposit_tile<MODE, ORDER, COH>(B, b, tile, w0, w0 + len + (wib < more), lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                       wrow, frac, W, buf, 1, acc, ea, bad);
+                                       wrow, frac, W, buf, 1, 0, acc, ea, bad);
 #pragma unroll
         for (int c = 0; c < D::NA; ++c) sums[wib * kDepBuf + c * kLanes + lane] = acc[c];
 #pragma unroll
@@ -868,6 +883,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
   }
   const int64_t u0 = unit_begin(w, B), u1 = unit_begin(w + 1, B);
   if (u0 >= u1) return;
+  const int phase = (int)((B.U + B.nw - 1) / B.nw);
   int b = box_of_unit(B, u0);
   for (int64_t u = u0; u < u1;) {        // one segment per (box, tile) the warp touches
     while (u >= B.box[b].uoff + (int64_t)B.box[b].ntiles * B.box[b].M) ++b;
@@ -881,7 +897,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
     int64_t sum[D::NA];
     int ea[D::SETS * D::GROUPS];
     deposit_tile<MODE, ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow, frac, W,
-                                   buf, B.U > B.nw, sum, ea, bad);
+                                   buf, B.U > B.nw, phase, sum, ea, bad);
     double acc[D::NA];
 #pragma unroll
     for (int c = 0; c < D::NA; ++c) acc[c] = deposit_sum(sum[c], ea[deposit_group<MODE>(c)]);
@@ -988,7 +1004,7 @@ k_deposit_cluster(Batch B, const double* __restrict__ z, const double* __restric
     for (int c = 0; c < DepMode<5>::GROUPS; ++c) ea[c] = 0;
     if (d0 < d1)
       deposit_tile<5, ORDER, false>(B, b, tile, d0, d1, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
-                                    TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, 1, acc, ea, bad);
+                                    TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, 1, 0, acc, ea, bad);
 #pragma unroll
     for (int c = 0; c < kNT; ++c) red[wib * kDepBuf + c * kLanes + lane] = deposit_sum(acc[c], ea[deposit_group<5>(c)]);
     __syncthreads();
@@ -1378,7 +1394,10 @@ __device__ __forceinline__ int box_of_slab_unit(const Batch& B, int64_t x) {
 // adjacent pieces of the same rings (sw = 8: 2 KB of every array).  Per unit a
 // warp forms G = A0 - Omega . A of its cells, the neighbours' G come from
 // shared memory, and the stencil sum is the commutator's operand: everything
-// up to the update runs on the integer pipe.
+// up to the update runs on the integer pipe.  Integer issue and the FP64 pipe
+// (conversions and updates) bound it about equally, HBM runs at 53 %: 16384 x 1000
+// 5.13 -> 2.64 ms a stage against FP64 arithmetic (the FP64 pipe its bound), 1024 x
+// 378 139 -> 73 us.
 constexpr int kSlabTiles = 8;                      // most tiles of a slab
 constexpr int kRowCells = kLanes + 4;              // cells of a unit, likewise
 template <int TILES>                               // of the widest slab
@@ -2516,7 +2535,8 @@ static __global__ void k_diagnostics(Batch B, const double* __restrict__ mom, do
 // off-diagonals) for X and m2 = m with its diagonal doubled, so
 //   out = -D K(H, D^-1 m) = raw(-H, m2),   gam += S D K(r, D^-1 m) = S raw(r, m2).
 // H is formed as in the RK stage (rk_phase: the same work split, tables and
-// integer arithmetic).
+// integer arithmetic; 48 of ~200 FP64 instructions less, the pipe that bounds it):
+// 1024 x 1000, 24 steps, backward from records 103.8 -> 94.2 ms.
 template <bool POT, int ORDER, int TILES>
 __global__ void __launch_bounds__(kThreads, 2)
 k_adj_a(Batch B, Parts pt, const double* __restrict__ W, const double* __restrict__ dirtab,
