@@ -323,10 +323,14 @@ int cuda_check(emu_box* b, cudaError_t e, const char* what) {
 
 // Whether the RK stage's blocks take ranges of slabs (several tiles, rings read
 // in pieces of up to 2 KB) or parts of single tiles: slabs when the batch has
-// at least 16 32-cell units per block of the default grid or more tiles than
-// blocks, unless a form was chosen; parts spread few units evenly.
+// at least 32 32-cell units per block of the default grid or more tiles than
+// blocks, unless a form was chosen; parts spread few units evenly and let other
+// boxes' kernels in.  us a step, parts / slabs: 777 x 130 (11 units a block) 147 /
+// 149 for three boxes in turn, 173 / 206 alone; 1024 x 152 (16) 195 / 199, 242 /
+// 228; 1024 x 200 (21) 231 / 240, 282 / 300; 777 x 300 (25) 272 / 274, 324 / 339;
+// 1024 x 378 (40) 381 / 383, 456 / 451; 2048 x 300 (63) 570 / 571, 703 / 667.
 int use_slabs(const emu_box* b) {
-  return b->rk_form >= 0 ? b->rk_form : b->S.U32 >= 16 * (int64_t)kPersistBlocks || b->S.NT32 > b->blocks;
+  return b->rk_form >= 0 ? b->rk_form : b->S.U32 >= 32 * (int64_t)kPersistBlocks || b->S.NT32 > b->blocks;
 }
 
 // Work split of small boxes, in the RK stage and the deposit: a block takes a
