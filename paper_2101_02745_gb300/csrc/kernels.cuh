@@ -100,9 +100,10 @@ struct BoxGeo {
   double vnubar[kNC];
 };
 
-// Warps that share a part of n directions: no more than directions, but 4 at
-// least (they also share the sum over warps and the RK stage's conversions).
-__host__ __device__ inline int part_warps(int n) { return n < 4 ? 4 : n < kWarps ? n : kWarps; }
+// Warps that share a part of n directions: no more than directions, but all 8 in
+// the smallest boxes (parts of less than 6: few blocks), where they only share the
+// sum over warps and the RK stage's conversions.
+__host__ __device__ inline int part_warps(int n) { return n < 6 || n > kWarps ? kWarps : n; }
 
 // Kernel view of a batch (passed by value).
 struct Batch {
