@@ -339,8 +339,9 @@ int emu_get_layout(emu_box* box, int32_t* general);
 int emu_set_barrier_timeout(emu_box* box, int64_t ns);
 
 /* Deposit of the step's stages in step form 0 and of emu_rk_stage (Eq. 5;
- * step forms 1 and 2 keep their own): 0 = every warp sums its rings of a tile
- * and writes a partial sum, a second launch adds the partials of each cell
+ * step forms 1 and 2 keep their own): 0 = every warp (in small boxes every
+ * block) sums its rings of a tile and writes a partial sum, a second launch adds
+ * the partials of each cell
  * (the default); 1, 2 = thread-block clusters of 8 or 16 blocks (64 or 128
  * warps) take one tile at a time, split its rings, add their sums through
  * shared and distributed shared memory and write the potential in the same
@@ -359,7 +360,8 @@ int emu_set_deposit_form(emu_box* box, int32_t form);
  * and emu_set_grid set it too).  Errors: EMU_EINVAL. */
 int emu_set_rk_form(emu_box* box, int32_t form);
 
-/* Set the grid of the step kernels to `blocks` blocks of 256 threads (1..608;
+/* Set the grid of the step kernels to at most `blocks` blocks of at most 256
+ * threads (small boxes launch fewer and smaller ones; 1..608;
  * the default is 304, two per SM; emu_autotune picks among 152, 304 and 608),
  * for callers that share the GPU with other work.  The blocks' warps split the
  * work, so the choice changes the deposit's summation order (results stay
