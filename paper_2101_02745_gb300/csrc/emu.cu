@@ -2270,6 +2270,16 @@ int emu_set_oscillation(emu_box* b, int32_t box, const emu_oscillation* osc) {
       g.n_e = ne;
     }
     for (int c = 0; c < kNC; ++c) any = any || g.vnu[c] != 0.0 || g.vnubar[c] != 0.0;
+    for (int sp = 0; sp < 2; ++sp) {
+      const double* v = sp ? g.vnubar : g.vnu;
+      for (int q = 0; q < 4; ++q) {   // the diagonal differences, each complex off-diagonal
+        namespace w = emu_wide;
+        const int e0 = w::exponent(v[2 * q]), e1 = w::exponent(v[2 * q + 1]), top = std::max(e0, e1);
+        g.ve[sp][q] = top;
+        g.vq[sp][2 * q] = w::join(w::limbs(v[2 * q], e0, top));
+        g.vq[sp][2 * q + 1] = w::join(w::limbs(v[2 * q + 1], e1, top));
+      }
+    }
   }
   b->pot = any;
   b->step_valid = false;
