@@ -1260,14 +1260,8 @@ __device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, co
   }
 }
 
-// H in the traceless components given as hv[c] 2^(he[c / 2] - kBiasV),
-// |hv| < 2^60.6: as doubles, and as the commutator's operand.
-__device__ __forceinline__ void operand_values(const int64_t (&hv)[kNC], const int (&he)[4], double (&Hm)[kNC]) {
-  namespace w = emu_wide;
-#pragma unroll
-  for (int c = 0; c < kNC; ++c)
-    Hm[c] = (double)hv[c] * w::scale(1.0, he[c >> 1] < w::kExpNonFinite ? max(he[c >> 1] - w::kBiasV, -1022) : 1024);
-}
+// The commutator's operand from H in the traceless components, given as
+// hv[c] 2^(he[c / 2] - kBiasV), |hv| < 2^60.6.
 __device__ __forceinline__ emu_wide::Ham operand_ham(const int64_t (&hv)[kNC], const int (&he)[4]) {
   namespace w = emu_wide;
   w::Ham hm;
@@ -1304,7 +1298,7 @@ __device__ __forceinline__ emu_wide::Ham operand_sum(const int64_t (&hv)[kNC], c
   return operand_ham(s, e);
 }
 
-// rk_update of particle p of box g from H (hv, he as operand_values).
+// rk_update of particle p of box g from H (hv, he as operand_ham).
 template <bool POT, int S, bool COH>
 __device__ __forceinline__ void rk_from_H(const BoxGeo& g, const Parts& pt, const double* src_b, int64_t P, int64_t p,
                                           int dry, double bdt, double cdt, double dtb, const double* vz,

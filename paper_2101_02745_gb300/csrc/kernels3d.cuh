@@ -56,7 +56,7 @@ struct Box3 {
   double alpha;
   uint64_t seed;
   const double* dt;    // the box's step size (device)
-  const BoxGeo* g;     // device copy: vacuum and matter terms (vnu, vnubar) and Lz, for rk_particle
+  const BoxGeo* g;     // device copy: vacuum and matter terms and Lz, for rk_from_H
 };
 
 __device__ __forceinline__ int64_t unit3_begin(int64_t w, const Box3& b) { return w >= b.nw ? b.U : w * b.U / b.nw; }
