@@ -790,6 +790,18 @@ __device__ __forceinline__ constexpr int deposit_group(int c) {
   return c / (D::MOM * D::COMP) * D::GROUPS + q;
 }
 
+// Where a part's warp keeps the exponents of its sums (deposit_phase), in 32-bit
+// words: two a row, in the 8-byte column of their lane.  The warp's buffer still
+// holds particle data there, and each lane reads and writes its own column only:
+// no lane's store can pass another's reads.
+__host__ __device__ constexpr int part_exponent(int c, int lane) { return 2 * ((c >> 1) * kLanes + lane) + (c & 1); }
+__host__ __device__ constexpr bool part_exponents_in_column(int groups) {
+  for (int c = 0; c < groups; ++c)
+    for (int lane = 0; lane < kLanes; ++lane)
+      if (part_exponent(c, lane) / 2 % kLanes != lane) return false;
+  return true;
+}
+
 // Part q of the deposit's split into blocks (Batch::dpb > 0): box b, tile and
 // directions [d0, d1); false past the last one.  first_part: the first part of a tile.
 __device__ __forceinline__ bool deposit_part(const Batch& B, int q, int& b, int& tile, int& d0, int& d1) {
@@ -847,7 +859,9 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
     const int nwarps = part_warps(B.dpb);                         // (the block's, but in k_step)
     int64_t* sums = (int64_t*)(buf - wib * kDepBuf);              // [warp][row][lane], then the exponents
     constexpr int kE = D::NA * kLanes;                            // doubles before a warp's exponents
-    static_assert(D::NA * kLanes * 8 + D::SETS * D::GROUPS * kLanes * 4 <= kDepBuf * 8, "a warp's sums fit its buffers");
+    constexpr int NE = D::SETS * D::GROUPS;
+    static_assert(D::NA + (NE + 1) / 2 <= kDepBuf / kLanes, "a warp's sums fit its buffers");
+    static_assert(part_exponents_in_column(NE), "a lane's exponents lie in its own column");
     int b, tile, d0, d1;
     for (int q = blockIdx.x; deposit_part(B, q, b, tile, d0, d1); q += gridDim.x) {
       const int n = d1 - d0, used = min(n, nwarps);
@@ -861,13 +875,13 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
 #pragma unroll
         for (int c = 0; c < D::NA; ++c) sums[wib * kDepBuf + c * kLanes + lane] = acc[c];
 #pragma unroll
-        for (int c = 0; c < D::SETS * D::GROUPS; ++c) ((int*)(sums + wib * kDepBuf + kE))[c * kLanes + lane] = ea[c];
+        for (int c = 0; c < NE; ++c) ((int*)(sums + wib * kDepBuf + kE))[part_exponent(c, lane)] = ea[c];
       }
       __syncthreads();
       const int cell = tile * T - H + lane;
       if (wib < nwarps && lane >= H && lane < H + T && cell < B.box[b].nz) {
         for (int c = wib; c < D::NA; c += nwarps) {
-          const int* ex = (const int*)(sums + kE) + deposit_group<MODE>(c) * kLanes + lane;
+          const int* ex = (const int*)(sums + kE) + part_exponent(deposit_group<MODE>(c), lane);
           int top = 0, e[kWarps];
 #pragma unroll
           for (int x = 0; x < kWarps; ++x) top = max(top, e[x] = x < used ? ex[x * 2 * kDepBuf] : 0);
