@@ -545,6 +545,18 @@ __device__ __forceinline__ int from_lane(int v, int o) {
   return o > 0 ? __shfl_up_sync(kFull, v, o) : __shfl_down_sync(kFull, v, -o);
 }
 
+// Limbs of u in every lane: a direction's components in lanes 0-2, there scaled by
+// 2^-ko (direction_excess), other numbers up to 1 in the rest.
+__device__ __forceinline__ emu_wide::Limbs direction_limbs(double u, int lane, int& ko) {
+  emu_wide::Limbs l = emu_wide::unit_limbs(u);
+  ko = 0;
+  if (__reduce_add_sync(kFull, lane < 3 ? emu_wide::unit_magnitude(u) : 0) > emu_wide::kDotLimit) {
+    ko = max(__reduce_max_sync(kFull, lane < 3 ? emu_wide::unit_excess(u) : 0), 1);
+    if (lane < 3) l = emu_wide::unit_limbs(u, ko);
+  }
+  return l;
+}
+
 // Asynchronous copies of 8 bytes from global to shared memory, by the thread
 // that reads them: its copies of all but the last N groups are done after
 // cp_async_wait<N>.
@@ -1275,7 +1287,7 @@ __device__ __forceinline__ void rk_particle(const BoxGeo& g, const Parts& pt, co
 }
 
 // The commutator's operand from H in the traceless components, given as
-// hv[c] 2^(he[c / 2] - kBiasV), |hv| < 2^60.6.
+// hv[c] 2^(he[c / 2] - kBiasV), |hv| < 2^60.8.
 __device__ __forceinline__ emu_wide::Ham operand_ham(const int64_t (&hv)[kNC], const int (&he)[4]) {
   namespace w = emu_wide;
   w::Ham hm;
@@ -1625,9 +1637,9 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
 #pragma unroll
         for (int o = 0; o < NW; ++o) wd[o] = ldp<COH>(row(W + p, (unsigned)P, o));
       }
-      // directions above 1 (not unit vectors) are scaled by 2^-ko
-      const int ko = __reduce_max_sync(kFull, lane < 3 ? w::unit_excess(u) : 0);
-      const w::Limbs ul = w::unit_limbs(u, lane < 3 ? ko : 0);
+      // (longer directions than unit vectors are scaled by 2^-ko)
+      int ko;
+      const w::Limbs ul = direction_limbs(u, lane, ko);
       const w::Limbs om[3] = {bcast(ul, 0), bcast(ul, 1), bcast(ul, 2)};
       // G of this lane's cell and of the H cells on each side of the tile
       if (active) {
@@ -1780,8 +1792,8 @@ k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ 
       if (active)
         bad |= shape_weights<ORDER>(fma(pos_dt, __ldg(dirtab + 3 * MT + gd), z[p]), (double)j + 0.5, g.inv_dz, g.nz_d,
                                     wt);
-      const int ko = __reduce_max_sync(kFull, w::unit_excess(u));
-      const w::Limbs ul = w::unit_limbs(u, ko);
+      int ko;
+      const w::Limbs ul = direction_limbs(u, lane, ko);
       const w::Limbs om[3] = {bcast(ul, 0), bcast(ul, 1), bcast(ul, 2)};
       auto G = [&](int c, int x) {
         return operand_G(t.a[c][x], t.a[9 + c][x], t.a[18 + c][x], t.a[27 + c][x], om, ko);

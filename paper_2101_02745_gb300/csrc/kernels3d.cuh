@@ -134,7 +134,7 @@ __global__ void k3_shifts(Box3 b, const double* __restrict__ x, const double* __
   }
   if (wtab != nullptr) {
     const double om[3] = {dirtab[d], dirtab[b.M + d], dirtab[2 * b.M + d]};
-    const int ko = max(max(emu_wide::unit_excess(om[0]), emu_wide::unit_excess(om[1])), emu_wide::unit_excess(om[2]));
+    const int ko = emu_wide::direction_excess(om[0], om[1], om[2]);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const emu_wide::Limbs l = emu_wide::unit_limbs(om[a], ko);

@@ -518,7 +518,7 @@ k_grk_stage(Batch B, Parts pt, const int2* __restrict__ At, const int2* __restri
   const int hc = wrapc((int)floor(zs * g.inv_dz), g.nz);
   double wt[NW];
   shape_weights<ORDER>(zs, (double)hc + 0.5, g.inv_dz, g.nz_d, wt);
-  const int ko = max(max(w::unit_excess(ox), w::unit_excess(oy)), w::unit_excess(oz));
+  const int ko = w::direction_excess(ox, oy, oz);
   const w::Limbs om[3] = {w::unit_limbs(-ox, ko), w::unit_limbs(-oy, ko), w::unit_limbs(-oz, ko)};
   int cell[NW], e[NW][4], he[4] = {0, 0, 0, 0};
 #pragma unroll

@@ -158,6 +158,18 @@ EMU_HD int unit_excess(double x) {
   return a > 0x3ff00001 ? (a >> 20) - 1021 : 0;
 }
 constexpr int kMaxExcess = 29;   // larger directions (above 2^27) count as infinite
+// dot3 needs components whose magnitudes add up to at most 2.25 (unit vectors:
+// 1.74): |x| in units of 2^-20, one that has an excess as more than that limit.
+constexpr int kDotLimit = 9 << 18;
+EMU_HD int unit_magnitude(double x) {
+  const int a = hi_word(x) & 0x7fffffff;
+  return a > 0x3ff00001 ? 1 << 24 : (int)shr((unsigned)(a & 0xfffff) | 0x100000u, 1023 - (a >> 20));
+}
+// The k of a direction (x, y, z) in dot3.
+EMU_HD int direction_excess(double x, double y, double z) {
+  const int k = max_i(max_i(unit_excess(x), unit_excess(y)), unit_excess(z));
+  return k == 0 && unit_magnitude(x) + unit_magnitude(y) + unit_magnitude(z) > kDotLimit ? 1 : k;
+}
 // Limbs of an int64 below 2^61 in magnitude, and back.
 EMU_HD Limbs split(int64_t v) { return Limbs{(int)(v >> 32), (int)((unsigned)v >> 1)}; }
 EMU_HD int64_t join(Limbs a) { return (int64_t)(((uint64_t)(uint32_t)a.h << 32) + 2 * (int64_t)a.l); }
@@ -214,8 +226,10 @@ EMU_HD int64_t mul2_down(Limbs a, Limbs b, Limbs c, Limbs d) {
   return mad((int)(m >> 32), two(), mad(a.h, b.h, prod(c.h, d.h)));
 }
 
-// q + (a1 b1 + a2 b2 + a3 b3) / 2^64 for |a| < 2^61, |q| < 2^59 and |b| <= 2^62
-// with b1^2 + b2^2 + b3^2 <= 2^124: below 2^60.6.
+// q + (a1 b1 + a2 b2 + a3 b3) / 2^64 for |a| < 2^61, |q| < 2^59 and |b1| + |b2| +
+// |b3| <= 2.25 2^62 (direction_excess): the middle sum stays below 3 2^60 +
+// 2.25 2^61 < 2^63, the result below 2^60.71.  (Components just below 1 each, a
+// length of 1.73, wrapped it: 6e-9 of G.)
 EMU_HD int64_t dot3(int64_t q, Limbs a1, Limbs b1, Limbs a2, Limbs b2, Limbs a3, Limbs b3) {
   const int64_t m =
       mad(a1.h, b1.l, mad(a1.l, b1.h, mad(a2.h, b2.l, mad(a2.l, b2.h, mad(a3.h, b3.l, mad(a3.l, b3.h, half_unit()))))));
