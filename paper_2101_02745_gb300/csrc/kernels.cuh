@@ -197,6 +197,12 @@ __device__ __forceinline__ int box_of_direction(const Batch& B, int d) {
 // test, one more instruction of the FP64 pipe, only behind it.
 __device__ __forceinline__ bool half_or_more(double d) { return (__double2hiint(d) & 0x7fffffff) >= 0x3fe00000; }
 
+// The error of a particle at the offset d from its cell's centre: none, off its
+// site, or no finite position (an infinite one's image reduction is NaN).
+__device__ __forceinline__ int site_error(double d) {
+  return fabs(d) <= 0.5 + kLatticeTol ? 0 : isnan(d) ? ERR_NONFINITE : ERR_LATTICE;
+}
+
 // Shape weights (Sec. 2.2.1) of order ORDER of a particle at (unwrapped)
 // position zs whose lattice site is cell h (hp = h + 1/2): the offset
 // d = zs/dz - hp, reduced to the nearest periodic image, lies in [-1/2, 1/2),
@@ -209,15 +215,17 @@ __device__ __forceinline__ bool half_or_more(double d) { return (__double2hiint(
 //            f = d - (j0 - h) in [0, 1): (1-f)^3/6, 2/3 - f^2 + f^3/2,
 //            2/3 - (1-f)^2 + (1-f)^3/2, f^3/6 on cells j0-1 .. j0+2.
 // The image reduction is only needed next to the domain ends, so it sits
-// behind the lattice test.  Returns nonzero if the particle is off its site.
+// behind the lattice test.  Returns 0, ERR_LATTICE if the particle is off its
+// site, or ERR_NONFINITE if its position is not finite (then w is not either,
+// but for order 0).
 template <int ORDER>
 __device__ __forceinline__ int shape_weights(double zs, double hp, double inv_dz, double nz_d,
                                              double (&w)[Sten<ORDER>::NW]) {
   double d = fma(zs, inv_dz, -hp);
   int bad = 0;
-  if (half_or_more(d) && fabs(d) > 0.5 + kLatticeTol) {
+  if (half_or_more(d) && !(fabs(d) <= 0.5 + kLatticeTol)) {
     d -= nz_d * rint(d / nz_d);
-    bad = fabs(d) > 0.5 + kLatticeTol;
+    bad = site_error(d);
   }
   if constexpr (ORDER == 0) {
     w[0] = 0.0; w[1] = 1.0; w[2] = 0.0;
@@ -246,13 +254,13 @@ __device__ __forceinline__ int shape_weights(double zs, double hp, double inv_dz
   return bad;
 }
 
-// The lattice test of shape_weights alone: nonzero if the particle at zs is
-// off the cell whose centre is hp (in cells), up to the periodic image.
+// The lattice test of shape_weights alone, for the particle at zs and the cell
+// whose centre is hp (in cells), up to the periodic image.
 __device__ __forceinline__ int off_site(double zs, double hp, double inv_dz, double nz_d) {
   double d = fma(zs, inv_dz, -hp);
-  if (half_or_more(d) && fabs(d) > 0.5 + kLatticeTol) {
+  if (half_or_more(d) && !(fabs(d) <= 0.5 + kLatticeTol)) {
     d -= nz_d * rint(d / nz_d);
-    return fabs(d) > 0.5 + kLatticeTol;
+    return site_error(d);
   }
   return 0;
 }
@@ -546,12 +554,14 @@ __device__ __forceinline__ int from_lane(int v, int o) {
 }
 
 // Limbs of u in every lane: a direction's components in lanes 0-2, there scaled by
-// 2^-ko (direction_excess), other numbers up to 1 in the rest.
+// 2^-ko (direction_excess), other numbers up to 1 in the rest (one that is not
+// finite counts as an infinite direction).
 __device__ __forceinline__ emu_wide::Limbs direction_limbs(double u, int lane, int& ko) {
   emu_wide::Limbs l = emu_wide::unit_limbs(u);
   ko = 0;
-  if (__reduce_add_sync(kFull, lane < 3 ? emu_wide::unit_magnitude(u) : 0) > emu_wide::kDotLimit) {
-    ko = max(__reduce_max_sync(kFull, lane < 3 ? emu_wide::unit_excess(u) : 0), 1);
+  const int m = emu_wide::unit_magnitude(u);
+  if (__reduce_add_sync(kFull, lane < 3 || m > emu_wide::kDotLimit ? m : 0) > emu_wide::kDotLimit) {
+    ko = max(__reduce_max_sync(kFull, emu_wide::unit_excess(u)), 1);
     if (lane < 3) l = emu_wide::unit_limbs(u, ko);
   }
   return l;
@@ -690,18 +700,23 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
     const double zs = fma(pos_dt, __ldg(dirtab + 3 * MT + gd), x[0]);
     w::Limbs wl[NW];   // the weight slot o of the particle that gives it to this lane's cell
     double wt[NW];
+    int site;          // the lattice test's error
     if (wrow != nullptr) {
       if (ORDER > 0 && lane >= 3 && lane < 3 + NW) u = ldp<COH>(wrow + (lane - 3) * MT + gd);
-      bad |= off_site(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d));
+      site = off_site(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d));
     } else {
-      bad |= shape_weights<ORDER>(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d), wt);
+      site = shape_weights<ORDER>(zs, hp, __ldg(&g.inv_dz), __ldg(&g.nz_d), wt);
       if ((MODE == 0 || MODE == 5) && W != nullptr && own) {   // the RK stage of these positions reads them back
 #pragma unroll
         for (int q = 0; q < Sten<ORDER>::NWS; ++q) *row(W + p, P, q) = wt[q];
       }
     }
+    bad |= site;
+    // weights have no exponent: a particle without a finite position counts as
+    // an infinite B, a ring without finite weights as an infinite direction
+    const int enf = site & ERR_NONFINITE ? w::kExpNonFinite : 0;
     // directions above 1 (not unit vectors) are scaled by 2^-ko
-    const int ko = __reduce_max_sync(kFull, lane < 3 ? w::unit_excess(u) : 0);
+    const int ko = __reduce_max_sync(kFull, w::unit_excess(u));
     const w::Limbs ul = w::unit_limbs(u, lane < 3 ? ko : 0);
     const w::Limbs om[3] = {bcast(ul, 0), bcast(ul, 1), bcast(ul, 2)};
     if constexpr (ORDER > 0) {
@@ -736,7 +751,7 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
         bv[0] = value(set, k);
         if (nc > 1) bv[1] = value(set, k + 1);
       }
-      const int e0 = w::exponent(bv[0]), e1 = nc > 1 ? w::exponent(bv[1]) : 0, e = max(e0, e1);
+      const int e0 = w::exponent(bv[0]), e1 = nc > 1 ? w::exponent(bv[1]) : 0, e = max(max(e0, e1), enf);
       w::Limbs bl[2];
       bl[0] = nc > 1 ? w::limbs(bv[0], e0, e) : w::limbs(bv[0], e);
       if (nc > 1) bl[1] = w::limbs(bv[1], e1, e);
@@ -907,7 +922,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
       }
       __syncthreads();   // (the sums are free for the next part)
     }
-    if (bad) atomicOr(err, ERR_LATTICE);
+    if (bad) atomicOr(err, bad);
     return;
   }
   const int64_t u0 = unit_begin(w, B), u1 = unit_begin(w + 1, B);
@@ -932,7 +947,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
     for (int c = 0; c < D::NA; ++c) acc[c] = deposit_sum(sum[c], ea[deposit_group<MODE>(c)]);
     flush_tile<ORDER>(acc, g.toff + tile, tile * T - H + lane, g.nz, w, lane, partial);
   }
-  if (bad) atomicOr(err, ERR_LATTICE);
+  if (bad) atomicOr(err, bad);
 }
 
 // TAB: the rings' weights from the weight row wrow; otherwise each
@@ -1058,7 +1073,7 @@ k_deposit_cluster(Batch B, const double* __restrict__ z, const double* __restric
     }
     cluster_sync();   // the slots are free for the next tile, and no block leaves while read
   }
-  if (bad) atomicOr(err, ERR_LATTICE);
+  if (bad) atomicOr(err, bad);
   if (nonfinite) atomicOr(err, ERR_NONFINITE);
 }
 
@@ -1695,10 +1710,13 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
             }
           }
         }
-        // hv[c] 2^(he + 2 - kBiasV) = H_c, then he + 2 -> he
-        if (ko != 0) {
+        // hv[c] 2^(he + 2 - kBiasV) = H_c, then he + 2 -> he (weights that are
+        // not finite have no exponent)
+        int kx = ko;
+        if (ORDER > 0 && !ring && w::exponent(wd[H]) >= w::kExpNonFinite) kx = w::kMaxExcess + 1;
+        if (kx != 0) {
 #pragma unroll
-          for (int grp = 0; grp < 4; ++grp) he[grp] = ko <= w::kMaxExcess ? he[grp] + ko : w::kExpNonFinite;
+          for (int grp = 0; grp < 4; ++grp) he[grp] = kx <= w::kMaxExcess ? he[grp] + kx : w::kExpNonFinite;
         }
 #pragma unroll
         for (int grp = 0; grp < 4; ++grp) he[grp] += 2;
@@ -1789,9 +1807,11 @@ k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ 
       const double u = lane < 3 ? -__ldg(dirtab + lane * MT + gd) : 0.0;
       double wt[Sten<ORDER>::NW];
       zero_weights<ORDER>(wt);
+      int site = 0;
       if (active)
-        bad |= shape_weights<ORDER>(fma(pos_dt, __ldg(dirtab + 3 * MT + gd), z[p]), (double)j + 0.5, g.inv_dz, g.nz_d,
+        site = shape_weights<ORDER>(fma(pos_dt, __ldg(dirtab + 3 * MT + gd), z[p]), (double)j + 0.5, g.inv_dz, g.nz_d,
                                     wt);
+      bad |= site;
       int ko;
       const w::Limbs ul = direction_limbs(u, lane, ko);
       const w::Limbs om[3] = {bcast(ul, 0), bcast(ul, 1), bcast(ul, 2)};
@@ -1823,7 +1843,7 @@ k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ 
             he = max(he, e[o]);
           }
           const int k2 = min(max(he + 2 + ko - w::kBiasV, -1022), 959);
-          const bool inf = he >= w::kExpNonFinite || ko > w::kMaxExcess;
+          const bool inf = he >= w::kExpNonFinite || ko > w::kMaxExcess || (site & ERR_NONFINITE);
 #pragma unroll
           for (int c = k0; c < k0 + nc; ++c) {
             int64_t v = 0;
@@ -1842,7 +1862,7 @@ k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ 
       __syncwarp();   // (the unit's G are rewritten by the next)
     }
   }
-  if (bad) atomicOr(err, ERR_LATTICE);
+  if (bad) atomicOr(err, bad);
 }
 
 // ------------------------------------------- RK stage with the next deposit
@@ -2192,7 +2212,7 @@ k_rk_deposit(Batch B, Parts pt, double* __restrict__ W, const double* __restrict
     __syncwarp();
   }
   flush_frame(acc, partial + (w + stile) * kSlotF, lane);
-  if (lat) atomicOr(err, ERR_LATTICE);
+  if (lat) atomicOr(err, lat);
   if (far) atomicOr(err, ERR_STEP);
 }
 
@@ -2747,7 +2767,7 @@ k_adj_seed(Batch B, Parts pt, const double* __restrict__ dirtab, const int* __re
       }
     }
   }
-  if (bad) atomicOr(err, ERR_LATTICE);
+  if (bad) atomicOr(err, bad);
 }
 
 // Chain rule through Eq. 8, N_p = (n_c + 3 f_c . Omega_p) dV / M with c the

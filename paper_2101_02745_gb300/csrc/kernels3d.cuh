@@ -113,6 +113,7 @@ __global__ void k3_shifts(Box3 b, const double* __restrict__ x, const double* __
   const int64_t p0 = (int64_t)d * b.C;
   const double pos[3] = {x[p0], y[p0], z[p0]};
   const double dt = *b.dt;
+  bool finite = true;   // (weights have no exponent: without a finite position the direction counts as infinite)
 #pragma unroll
   for (int s = 0; s < 4; ++s) {
     if (s >= nrows) break;
@@ -123,7 +124,7 @@ __global__ void k3_shifts(Box3 b, const double* __restrict__ x, const double* __
       shift[(s * 3 + a) * b.M + d] = cell;
       if (wtab != nullptr) {
         double w[NW];
-        (void)shape_weights<ORDER>(xs, (double)cell + 0.5, b.inv_h[a], b.n_d[a], w);
+        finite = finite && !(shape_weights<ORDER>(xs, (double)cell + 0.5, b.inv_h[a], b.n_d[a], w) & ERR_NONFINITE);
 #pragma unroll
         for (int q = 0; q < NW; ++q) {
           const emu_wide::Limbs l = emu_wide::unit_limbs(w[q]);
@@ -134,7 +135,7 @@ __global__ void k3_shifts(Box3 b, const double* __restrict__ x, const double* __
   }
   if (wtab != nullptr) {
     const double om[3] = {dirtab[d], dirtab[b.M + d], dirtab[2 * b.M + d]};
-    const int ko = emu_wide::direction_excess(om[0], om[1], om[2]);
+    const int ko = finite ? emu_wide::direction_excess(om[0], om[1], om[2]) : emu_wide::kMaxExcess + 1;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const emu_wide::Limbs l = emu_wide::unit_limbs(om[a], ko);
@@ -268,7 +269,7 @@ k3_deposit(Box3 b, const double* __restrict__ x, const double* __restrict__ y, c
     }
     flush_tile<ORDER>(acc, gtile, craw, nz, w, lane, partial);
   }
-  if (bad) atomicOr(err, ERR_LATTICE);
+  if (bad) atomicOr(err, bad);
 }
 
 // off_site for cell j: first whether the position lies in the cell itself, from
@@ -328,10 +329,10 @@ k3_prep(Box3 b, const double* __restrict__ x, const double* __restrict__ y, cons
     const emu_wide::Cplx l = emu_wide::cplx(bv[0], bv[1]);
     Bf.f[(int64_t)(2 * q) * P + out] = make_int2(l.r.h, l.r.l);
     Bf.f[(int64_t)(2 * q + 1) * P + out] = make_int2(l.i.h, l.i.l);
-    eg[q] = l.e;
+    eg[q] = bad & ERR_NONFINITE ? emu_wide::kExpNonFinite : l.e;
   }
   Bf.e[out] = pack_exponents(eg);
-  if (bad) atomicOr(err, ERR_LATTICE);
+  if (bad) atomicOr(err, bad);
 }
 
 // sum_q w[q] V_q of a field's values at the sites nb, for its NG exponent groups
@@ -683,7 +684,7 @@ k3_interpolate(Box3 b, const double* __restrict__ x, const double* __restrict__ 
       for (int k = 0; k < 9; ++k) Hout[k * P + p] = Hf[k];
     }
   }
-  if (bad) atomicOr(err, ERR_LATTICE);
+  if (bad) atomicOr(err, bad);
 }
 
 // Initial particles on the 3D lattice (Sec. 3.1, Eq. 8, 9; as k_init):

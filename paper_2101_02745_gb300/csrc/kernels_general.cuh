@@ -258,13 +258,12 @@ k_gdeposit(Batch B, Parts pt, const double* __restrict__ r_nu, const double* __r
     for (int c = 0; c < NA; ++c) {
       const double v = warp_sum(acc[c]) * scale;
       if (lane == (c & 31)) {
-        bad |= !isfinite(v) ? 2 : 0;
+        bad |= !isfinite(v) ? ERR_NONFINITE : 0;
         out[(int64_t)c * B.NZ + gc] = v;
       }
     }
   }
-  if (bad & 1) atomicOr(err, ERR_LATTICE);
-  if (bad & 2) atomicOr(err, ERR_NONFINITE);
+  if (bad) atomicOr(err, bad);
 }
 
 // The step's deposit (MODE 5) in two parts.  k_gprep: one thread per sorted
@@ -323,11 +322,11 @@ k_gprep(Batch B, Parts pt, const double* __restrict__ r_nu, const double* __rest
     const w::Cplx l = w::cplx(bv[0], bv[1]);
     put(S.b + (int64_t)(2 * q) * P + i, l.r);
     put(S.b + (int64_t)(2 * q + 1) * P + i, l.i);
-    eg[q] = ko <= w::kMaxExcess ? l.e : w::kExpNonFinite;
+    eg[q] = ko <= w::kMaxExcess && !(bad & ERR_NONFINITE) ? l.e : w::kExpNonFinite;
   }
   if (ko > w::kMaxExcess) ko = 0;
   S.e[i] = make_int2(eg[0] | ko << 11 | eg[1] << 16, eg[2] | eg[3] << 16);
-  if (bad) atomicOr(err, ERR_LATTICE);
+  if (bad) atomicOr(err, bad);
 }
 
 // The step's deposit from k_gprep's sorted data: kGSplit warps per global
@@ -517,8 +516,8 @@ k_grk_stage(Batch B, Parts pt, const int2* __restrict__ At, const int2* __restri
   const double zs = fma(stage_frac(s - 1) * dt, vz, pt.z[p]);
   const int hc = wrapc((int)floor(zs * g.inv_dz), g.nz);
   double wt[NW];
-  shape_weights<ORDER>(zs, (double)hc + 0.5, g.inv_dz, g.nz_d, wt);
-  const int ko = w::direction_excess(ox, oy, oz);
+  const int site = shape_weights<ORDER>(zs, (double)hc + 0.5, g.inv_dz, g.nz_d, wt);
+  const int ko = site & ERR_NONFINITE ? w::kMaxExcess + 1 : w::direction_excess(ox, oy, oz);
   const w::Limbs om[3] = {w::unit_limbs(-ox, ko), w::unit_limbs(-oy, ko), w::unit_limbs(-oz, ko)};
   int cell[NW], e[NW][4], he[4] = {0, 0, 0, 0};
 #pragma unroll
