@@ -605,9 +605,8 @@ struct DepMode {
 // stencil and the moments' sums are fixed-point (wide.cuh).  A sum is an
 // int64 per lane; the components of one group share the exponent ea of
 // their sums, which grows when a direction's contribution asks for it (the
-// sums are then shifted).  A tile's sums of n directions leave ceil(log2 n)
-// bits of headroom, so a contribution keeps 61 - ceil(log2 n) bits below the
-// largest one's leading bit: less error than FP64 sums of n terms, whose
+// sums are then shifted).  Sums of n directions have headroom for n contributions
+// and round them without a bias (sum_headroom): less error than FP64 sums, whose
 // rounding follows the partial sums.  Zero contributions add exactly nothing.
 // Bound by integer issue: 16384 x 1000 2467 -> 1040 us a stage against FP64 sums
 // (1256 with plain loads: cp.async hides their latency), 1024 x 378 74 -> 41 us.
@@ -640,7 +639,7 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
   const bool own = lane >= H && lane < H + T && craw < nz;
   const double pos_dt = frac * B.dt[b];
   const int dbase = g.doff;
-  const int head = max(32 - __clz(dlast - dfirst), 2) - 2;   // headroom beyond the two bits a contribution leaves
+  const int head = w::sum_headroom(dlast - dfirst);
 #pragma unroll
   for (int c = 0; c < D::NA; ++c) acc[c] = 0;
 #pragma unroll
@@ -716,9 +715,16 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
     // an infinite B, a ring without finite weights as an infinite direction
     const int enf = site & ERR_NONFINITE ? w::kExpNonFinite : 0;
     // directions above 1 (not unit vectors) are scaled by 2^-ko
-    const int ko = __reduce_max_sync(kFull, w::unit_excess(u));
+    const int ko = __reduce_max_sync(kFull, w::unit_excess(u)), half = w::sum_half(ko);
     const w::Limbs ul = w::unit_limbs(u, lane < 3 ? ko : 0);
-    const w::Limbs om[3] = {bcast(ul, 0), bcast(ul, 1), bcast(ul, 2)};
+    const w::Factor uf = w::factor(w::join(ul));
+    w::Factor om[3];
+    int64_t mh[3];   // (order 3 has no registers left for them: it adds the half unit as one every second term)
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      om[m] = w::Factor{__shfl_sync(kFull, uf.h, m), __shfl_sync(kFull, uf.l, m)};
+      mh[m] = w::moment_half(om[m]);
+    }
     if constexpr (ORDER > 0) {
       if (wrow != nullptr) {
         if ((MODE == 0 || MODE == 5) && W != nullptr && own) {
@@ -793,11 +799,11 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
 #pragma unroll
       for (int c = 0; c < nc; ++c) {
         const int64_t v = w::align(cv[c], dd, df);
-        const w::Limbs l = w::split(v);
-        acc[r0 + c] += w::align(v, 2 + ko, 0);
+        const w::Factor f = w::factor(ORDER == 3 ? v + (k & 1) : v);
+        acc[r0 + c] += w::zeroth_moment(v, ko, half);
 #pragma unroll
         for (int m = 1; m < D::MOM; ++m)
-          acc[m * D::COMP + r0 + c] = w::mul_add(l, om[m - 1], acc[m * D::COMP + r0 + c]);
+          acc[m * D::COMP + r0 + c] = w::moment_add(f, om[m - 1], ORDER == 3 ? w::half_unit() : mh[m - 1], acc[m * D::COMP + r0 + c]);
       }
     }
   }

@@ -100,8 +100,9 @@ static __global__ void k3_dirtable(Box3 b, Parts pt, double* __restrict__ dirtab
 // shape weights there, the direction's weights on each axis (all its
 // particles share the offset inside their cells): wtab[((s * 3 + axis) * 5 +
 // q) * M + d], q < NW, as operands (unit_limbs); then the directions as
-// operands, rows 60-62 Omega and row 63 (their scale 2^-x, 0).
-constexpr int kOpRows = 64;   // rows of the operand table
+// operands, rows 60-62 Omega, row 63 (their scale 2^-x, 0) and rows 64-66 Omega as
+// the factors of the direction sum.
+constexpr int kOpRows = 67;   // rows of the operand table
 template <int ORDER>
 __global__ void k3_shifts(Box3 b, const double* __restrict__ x, const double* __restrict__ y,
                           const double* __restrict__ z, const double* __restrict__ dirtab, Fracs fr, int nrows,
@@ -139,7 +140,9 @@ __global__ void k3_shifts(Box3 b, const double* __restrict__ x, const double* __
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const emu_wide::Limbs l = emu_wide::unit_limbs(om[a], ko);
+      const emu_wide::Factor f = emu_wide::factor(emu_wide::join(l));
       wtab[(60 + a) * b.M + d] = make_int2(l.h, l.l);
+      wtab[(64 + a) * b.M + d] = make_int2(f.h, f.l);
     }
     wtab[63 * b.M + d] = make_int2(ko, 0);
   }
@@ -465,7 +468,7 @@ k3_spread_x_sum(Box3 b, Field3 in, const int2* __restrict__ wrow, const int2* __
     if (jn < 0 || jn >= b.n[0]) jn = wrapn(jn, b.n[0]);
     nb[q] = cell + (jn - jx) * stride;
   }
-  const int head = max(32 - __clz(M), 2) - 2;   // headroom (deposit_tile)
+  const int head = w::sum_headroom(M);
   int64_t acc[4 * 2 * NG];
   int ea[NG];
 #pragma unroll
@@ -476,8 +479,15 @@ k3_spread_x_sum(Box3 b, Field3 in, const int2* __restrict__ wrow, const int2* __
     w::Limbs wl[NW];
 #pragma unroll
     for (int q = 0; q < NW; ++q) wl[q] = operand(wrow + q * M, d);
-    const w::Limbs om[3] = {operand(ops + 60 * M, d), operand(ops + 61 * M, d), operand(ops + 62 * M, d)};
-    const int ko = __ldg(&ops[63 * M + d].x);
+    w::Factor om[3];
+    int64_t mh[3];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const int2 o = __ldg(ops + (64 + m) * M + d);
+      om[m] = w::Factor{o.x, o.y};
+      mh[m] = w::moment_half(om[m]);
+    }
+    const int ko = __ldg(&ops[63 * M + d].x), half = w::sum_half(ko);
     int64_t cv[2 * NG];
     int eg[NG];
     field_taps<NW, NW == 3 ? 2 : 1, NG>(in, P, (int64_t)d * b.C, nb, wl, cv, eg, g0);
@@ -497,10 +507,10 @@ k3_spread_x_sum(Box3 b, Field3 in, const int2* __restrict__ wrow, const int2* __
 #pragma unroll
       for (int c = 2 * g; c < 2 * g + 2; ++c) {
         const int64_t v = w::align(cv[c], dd, df);
-        const w::Limbs l = w::split(v);
-        acc[c] += w::align(v, 2 + ko, 0);
+        const w::Factor f = w::factor(v);
+        acc[c] += w::zeroth_moment(v, ko, half);
 #pragma unroll
-        for (int m = 0; m < 3; ++m) acc[(m + 1) * 2 * NG + c] = w::mul_add(l, om[m], acc[(m + 1) * 2 * NG + c]);
+        for (int m = 0; m < 3; ++m) acc[(m + 1) * 2 * NG + c] = w::moment_add(f, om[m], mh[m], acc[(m + 1) * 2 * NG + c]);
       }
     }
   }

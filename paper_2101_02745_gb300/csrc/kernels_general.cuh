@@ -275,7 +275,7 @@ k_gdeposit(Batch B, Parts pt, const double* __restrict__ r_nu, const double* __r
 // that gathers it.
 struct Sorted {
   int2* b;   // [kNC][P] B
-  int2* o;   // [3][P] Omega 2^-ko
+  int2* o;   // [3][P] Omega 2^-ko, factors of the direction sum
   int2* e;   // [P] exponents of B (diagonal pair, three complex components), 16 bits each; ko in bits 11-15
 };
 template <int ORDER>
@@ -301,7 +301,10 @@ k_gprep(Batch B, Parts pt, const double* __restrict__ r_nu, const double* __rest
   for (int q = 0; q < NWS; ++q) put(Ws + q * P + i, w::unit_limbs(wt[q]));
   int ko = max(max(w::unit_excess(om[0]), w::unit_excess(om[1])), w::unit_excess(om[2]));
 #pragma unroll
-  for (int a = 0; a < 3; ++a) put(S.o + a * P + i, w::unit_limbs(om[a], ko));
+  for (int a = 0; a < 3; ++a) {
+    const w::Factor f = w::factor(w::join(w::unit_limbs(om[a], ko)));
+    S.o[a * P + i] = make_int2(f.h, f.l);
+  }
   const double n1 = pt.N[p], n2 = pt.Nbar[p];
   // conj(rhobar) flips the sign of the imaginary components 4, 6, 8
   auto value = [&](int k) {
@@ -376,7 +379,7 @@ k_gdeposit_sorted(Batch B, const int2* __restrict__ Ws, Sorted S, const int* __r
         const int sc = g->coff + wrapc(j - o, g->nz);
         n += (start[sc + 1] - start[sc] + kGSplit * kLanes - 1) / (kGSplit * kLanes);
       }
-      const int head = max(32 - __clz(n), 2) - 2;   // headroom (deposit_tile)
+      const int head = w::sum_headroom(n);
       for (int o = -H; o <= H; ++o) {           // source cells j - o: their particles' weight slot H + o
         if (ORDER == 0 && o != 0) continue;
         const int sc = g->coff + wrapc(j - o, g->nz);
@@ -384,10 +387,14 @@ k_gdeposit_sorted(Batch B, const int2* __restrict__ Ws, Sorted S, const int* __r
         for (int i = i0 + k * kLanes + lane; i < i1; i += kGSplit * kLanes) {
           w::Limbs wl{0, 0};
           if (ORDER > 0) wl = limbs_of(__ldg(Ws + (int64_t)(H + o) * P + i));
-          const w::Limbs om[3] = {limbs_of(__ldg(S.o + i)), limbs_of(__ldg(S.o + P + i)),
-                                  limbs_of(__ldg(S.o + 2 * P + i))};
+          w::Factor om[3];
+#pragma unroll
+          for (int m = 0; m < 3; ++m) {
+            const int2 o2 = __ldg(S.o + m * P + i);
+            om[m] = w::Factor{o2.x, o2.y};
+          }
           const int2 ex = __ldg(S.e + i);
-          const int ko = (ex.x >> 11) & 31, e[4] = {ex.x & 0x7ff, ex.x >> 16, ex.y & 0xffff, ex.y >> 16};
+          const int ko = (ex.x >> 11) & 31, half = w::sum_half(ko), e[4] = {ex.x & 0x7ff, ex.x >> 16, ex.y & 0xffff, ex.y >> 16};
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const int es = e[q] + ko;
@@ -405,10 +412,11 @@ k_gdeposit_sorted(Batch B, const int2* __restrict__ Ws, Sorted S, const int* __r
             for (int c = 2 * q; c < 2 * q + 2; ++c) {
               const w::Limbs bl = limbs_of(__ldg((const int2*)row((const double*)S.b + i, (unsigned)P, c)));
               const int64_t v = w::align(ORDER == 0 ? w::join(bl) >> 2 : w::mul(bl, wl), dd, df);
-              const w::Limbs l = w::split(v);
-              acc[c] += w::align(v + 2, 2 + ko, 0);   // (rounded: thousands of terms would add up a bias)
+              const w::Factor f = w::factor(v);
+              acc[c] += w::zeroth_moment(v, ko, half);
 #pragma unroll
-              for (int m = 0; m < 3; ++m) acc[(m + 1) * kNC + c] = w::mul_add(l, om[m], acc[(m + 1) * kNC + c]);
+              for (int m = 0; m < 3; ++m)   // (a lane's few terms: the floors' bias stays below their rounding)
+                acc[(m + 1) * kNC + c] = w::moment_add(f, om[m], w::half_unit(), acc[(m + 1) * kNC + c]);
             }
           }
         }

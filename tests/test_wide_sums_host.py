@@ -24,6 +24,33 @@ int64_t dot(const double* A, const double* o, int* e) {
   *e = top + 2 + ko - kBiasV;
   return join(split(dot3(align(join(a[0]) >> 2, ko, 0), a[1], b[0], a[2], b[1], a[3], b[2])));
 }
+// Zeroth and first moment of n terms, each the sum of three taps w v, as a deposit adds
+// them; om: the terms' direction component (scaled by 2^-ko): value 2^(*ea + 4 - kBiasV).
+// alternate: half a unit for the first moment as one every second term
+void sums(const double* v, const double* wt, const double* om, int n, int ko, int alternate, int64_t* acc, int* ea) {
+  const int head = sum_headroom(n), half = sum_half(ko);
+  acc[0] = acc[1] = 0;
+  *ea = 0;
+  for (int d = 0; d < n; ++d) {
+    int e[3], et = 0;
+    for (int k = 0; k < 3; ++k) et = max_i(et, e[k] = exponent(v[3 * d + k]));
+    int64_t cv = 0;
+    for (int k = 0; k < 3; ++k) cv += align(mul(limbs(v[3 * d + k], e[k]), unit_limbs(wt[3 * d + k])), et - e[k]);
+    const int es = et + ko;
+    if (es + head > *ea) {
+      const int sh = es + head - *ea;
+      *ea += sh;
+      acc[0] = align(acc[0], sh);
+      acc[1] = align(acc[1], sh);
+    }
+    const int dd = *ea - es;
+    const int64_t x = align(cv, dd);
+    const Factor f = factor(join(unit_limbs(om[d], ko)));
+    acc[0] += zeroth_moment(x, ko, half);
+    acc[1] = alternate ? moment_add(factor(x + (d & 1)), f, half_unit(), acc[1])
+                       : moment_add(factor(x), f, moment_half(f), acc[1]);
+  }
+}
 }
 '''
 
@@ -73,3 +100,69 @@ def test_dot_product_of_any_direction(lib, kind, operands):
         ref = F(a[0]) - sum(F(x) * F(y) for x, y in zip(a[1:], d))
         scale = F(np.abs(a).max()) * F(max(2.0, 4 * np.abs(d).max()))
         assert abs(got - ref) <= 9 * F(2) ** -58 * scale, (a, d, float(got - ref))
+
+
+def _sums(lib, v, w, om, ko=0, alternate=0):
+    """(got, exact, FP64 chain) of both moments, and the largest term."""
+    acc, ea = np.zeros(2, np.int64), ctypes.c_int()
+    v, w, om = (np.ascontiguousarray(a, float) for a in (v, w, om))
+    lib.sums(_ptr(v), _ptr(w), _ptr(om), len(om), ko, alternate, _ptr(acc), ctypes.byref(ea))
+    got = [F(float(a)) * F(2) ** (ea.value + 4 - 1083) for a in acc.astype(float)]
+    exact, f0, f1, big = [F(0), F(0)], 0.0, 0.0, 0.0
+    for vv, ww, o in zip(v, w, om):
+        c = 0.0
+        for x, y in zip(vv, ww):
+            c = float(F(c) + F(x) * F(y))       # (a multiply-add rounds once)
+        f0, f1 = f0 + c, float(F(f1) + F(o) * F(c))
+        t = sum(F(x) * F(y) for x, y in zip(vv, ww))
+        exact[0] += t
+        exact[1] += t * F(o)
+        big = max(big, abs(float(t)))
+    return got, exact, (f0, f1), big
+
+
+@pytest.mark.parametrize("n", [1, 8, 31, 32, 225, 1000])
+@pytest.mark.parametrize("kind", ["random signs", "one sign", "forward"])
+@pytest.mark.parametrize("alternate", [0, 1])
+def test_sums_err_no_more_than_double_precision(lib, alternate, kind, n):
+    """The rms error of both moments of n terms is at most that of FP64 multiply-adds, and its mean is
+    that of unbiased rounding (within five standard errors)."""
+    rng = np.random.default_rng(n)
+    trials = 40 if n > 100 else 100
+    ours, chain = np.zeros((trials, 2)), np.zeros((trials, 2))
+    for t in range(trials):
+        d = rng.uniform(-0.5, 0.5, n)
+        w = np.stack([0.5 * (0.5 - d) ** 2, 0.75 - d * d, 0.5 * (0.5 + d) ** 2], axis=1)
+        v = rng.uniform(0.2, 1.2, (n, 3)) * (1.0 if kind == "one sign" else rng.choice([-1.0, 1.0], (n, 3)))
+        om = rng.uniform(0.9, 1.0, n) if kind == "forward" else rng.uniform(-1.0, 1.0, n)
+        got, exact, fp64, big = _sums(lib, v, w, om, 0, alternate)
+        ours[t] = [float(g - x) / big for g, x in zip(got, exact)]
+        chain[t] = [float(F(g) - x) / big for g, x in zip(fp64, exact)]
+    rms, ref = (np.sqrt((a ** 2).mean(axis=0)) for a in (ours, chain))
+    assert np.all(rms <= ref), (rms, ref)
+    assert np.all(np.abs(ours.mean(axis=0)) <= 5 * rms / np.sqrt(trials)), (ours.mean(axis=0), rms)
+
+
+@pytest.mark.parametrize("alternate", [0, 1])
+@pytest.mark.parametrize("ko", [0, 1, 7])
+@pytest.mark.parametrize("n", [1, 31, 32, 63, 64, 1023, 1024])
+def test_sums_of_the_largest_terms_fit(lib, n, ko, alternate):
+    """n terms of one sign at the largest significand, taps that add up to 2: within 2^-50 of the sum."""
+    v = np.full((n, 3), -(2 - 2.0 ** -52))
+    w = np.tile([0.5, 1.0, 0.5], (n, 1))
+    got, exact, _, _ = _sums(lib, v, w, np.full(n, 2.0 ** ko), ko, alternate)
+    for g, x in zip(got, exact):
+        assert abs(g - x) <= F(2) ** -50 * abs(x) * (2 ** ko if x is exact[0] else 1)
+
+
+@pytest.mark.parametrize("alternate", [0, 1])
+def test_zero_terms_add_nothing(lib, alternate):
+    n = 64
+    v = np.zeros((n, 3))
+    v[5] = [0.25, -1.5, 0.75]
+    w = np.tile([0.125, 0.75, 0.125], (n, 1))
+    om = np.linspace(-1, 1, n)
+    got, exact, _, _ = _sums(lib, v, w, om, 0, alternate)
+    assert got[0] == exact[0]                     # (few bits: exact)
+    one, _, _, _ = _sums(lib, v[5:6], w[5:6], om[5:6], 0, alternate)
+    assert abs(got[1] - exact[1]) <= F(2) ** -52 and abs(one[1] - exact[1]) <= F(2) ** -55
