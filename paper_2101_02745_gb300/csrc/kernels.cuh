@@ -809,11 +809,15 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
   }
 }
 
+// Exponents of sums that are not finite, lie at an end of the range of doubles or are
+// zero (the smallest).
+__device__ __forceinline__ bool far_exponent(int ea) { return (unsigned)(ea - 64) > 1966u; }
 // A sum acc 2^(ea + 4 - kBiasV) of deposit_tile as a double.
 __device__ __forceinline__ double deposit_sum(int64_t acc, int ea) {
   namespace w = emu_wide;
-  if (ea >= w::kExpNonFinite) return nan("");
-  return w::scale_nz((double)acc, min(max(ea + 4 - w::kBiasV, -1022), 959));
+  if (far_exponent(ea) && (acc != 0 || ea >= w::kExpNonFinite))
+    return ea >= w::kExpNonFinite ? nan("") : w::scaled(acc, ea + 4 - w::kBiasV);
+  return w::scaled_near(acc, ea + 4 - w::kBiasV);
 }
 // The exponent group of row c.
 template <int MODE>
@@ -821,6 +825,35 @@ __device__ __forceinline__ constexpr int deposit_group(int c) {
   using D = DepMode<MODE>;
   const int k = c % D::COMP, q = k < D::SINGLE ? k : D::SINGLE + (k - D::SINGLE) / 2;
   return c / (D::MOM * D::COMP) * D::GROUPS + q;
+}
+
+// deposit_sum of a tile's sums, with one branch for all of them.
+template <int MODE>
+__device__ __forceinline__ void deposit_sums(const int64_t (&sum)[DepMode<MODE>::NA],
+                                             const int (&ea)[DepMode<MODE>::SETS * DepMode<MODE>::GROUPS],
+                                             double (&acc)[DepMode<MODE>::NA]) {
+  namespace w = emu_wide;
+  using D = DepMode<MODE>;
+  int64_t far = 0;
+#pragma unroll
+  for (int q = 0; q < D::SETS * D::GROUPS; ++q) {
+    if (far_exponent(ea[q])) {
+      far |= ea[q] >= w::kExpNonFinite;
+#pragma unroll
+      for (int c = 0; c < D::NA; ++c)
+        if (deposit_group<MODE>(c) == q) far |= sum[c];
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < D::NA; ++c)
+    acc[c] = w::scaled_near(sum[c], w::near(ea[deposit_group<MODE>(c)] + 4 - w::kBiasV));
+  if (far != 0) {
+#pragma unroll
+    for (int c = 0; c < D::NA; ++c) {
+      const int e = ea[deposit_group<MODE>(c)];
+      acc[c] = e >= w::kExpNonFinite ? nan("") : acc[c] * w::far_factor(e + 4 - w::kBiasV);
+    }
+  }
 }
 
 // Where a part's warp keeps the exponents of its sums (deposit_phase), in 32-bit
@@ -949,8 +982,7 @@ __device__ __forceinline__ void deposit_phase(const Batch& B, int64_t w, int lan
     deposit_tile<MODE, ORDER, COH>(B, b, tile, dfirst, dlast, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift, wrow, frac, W,
                                    buf, B.U > B.nw, phase, sum, ea, bad);
     double acc[D::NA];
-#pragma unroll
-    for (int c = 0; c < D::NA; ++c) acc[c] = deposit_sum(sum[c], ea[deposit_group<MODE>(c)]);
+    deposit_sums<MODE>(sum, ea, acc);
     flush_tile<ORDER>(acc, g.toff + tile, tile * T - H + lane, g.nz, w, lane, partial);
   }
   if (bad) atomicOr(err, bad);
@@ -1055,8 +1087,10 @@ k_deposit_cluster(Batch B, const double* __restrict__ z, const double* __restric
     if (d0 < d1)
       deposit_tile<5, ORDER, false>(B, b, tile, d0, d1, lane, z, N, Nbar, r_nu, r_nb, dirtab, shift,
                                     TAB ? wrow : nullptr, frac, W, red + wib * kDepBuf, 1, 0, acc, ea, bad);
+    double sum[kNT];
+    deposit_sums<5>(acc, ea, sum);
 #pragma unroll
-    for (int c = 0; c < kNT; ++c) red[wib * kDepBuf + c * kLanes + lane] = deposit_sum(acc[c], ea[deposit_group<5>(c)]);
+    for (int c = 0; c < kNT; ++c) red[wib * kDepBuf + c * kLanes + lane] = sum[c];
     __syncthreads();
     for (int e = threadIdx.x; e < NE; e += kThreads) {   // the block's warps, in warp order
       double v = red[e];
@@ -1784,23 +1818,33 @@ k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ 
     q += d1 - d0;
     const int c0 = slab * InterpTable::kTiles * kLanes, ncell = min(InterpTable::kTiles * kLanes, nz - c0) + 2 * H;
     __syncthreads();
+    int far = 0;   // whether a cell's exponent takes H to an end of the range of doubles
     for (int x = threadIdx.x; x < 6 * ncell; x += kThreads) {
       const int grp = x / ncell, c = x - grp * ncell;
       const double* Aj = A + wrapc(c0 - H + c, nz);
+      int e, some = 0;
       if (grp < 3) {
         double v[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = __ldg(Aj + (int64_t)(9 * k + grp) * NZ);
-        t.e[grp][c] = potential_operands<4>(v, [&](int k, int2 o) { t.a[9 * k + grp][c] = o; });
+        for (int k = 0; k < 4; ++k) {
+          v[k] = __ldg(Aj + (int64_t)(9 * k + grp) * NZ);
+          some |= (__double2hiint(v[k]) & 0x7fffffff) | __double2loint(v[k]);
+        }
+        e = potential_operands<4>(v, [&](int k, int2 o) { t.a[9 * k + grp][c] = o; });
       } else {
         const int k0 = 2 * grp - 3;
         double v[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = __ldg(Aj + (int64_t)(9 * (k >> 1) + k0 + (k & 1)) * NZ);
-        t.e[grp][c] = potential_operands<8>(v, [&](int k, int2 o) { t.a[9 * (k >> 1) + k0 + (k & 1)][c] = o; });
+        for (int k = 0; k < 8; ++k) {
+          v[k] = __ldg(Aj + (int64_t)(9 * (k >> 1) + k0 + (k & 1)) * NZ);
+          some |= (__double2hiint(v[k]) & 0x7fffffff) | __double2loint(v[k]);
+        }
+        e = potential_operands<8>(v, [&](int k, int2 o) { t.a[9 * (k >> 1) + k0 + (k & 1)][c] = o; });
       }
+      t.e[grp][c] = e;
+      far |= e > 2000 || (e < 64 && some != 0);
     }
-    __syncthreads();
+    far = __syncthreads_or(far);
     const int tile0 = (wib & (InterpTable::kTiles - 1)) * kLanes, n = min(kLanes, nz - c0 - tile0);
     if (n <= 0) continue;
     const int j = c0 + tile0 + lane, tc = tile0 + H + lane;
@@ -1848,7 +1892,7 @@ k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ 
             e[o] = t.e[grp][tc - H + o];
             he = max(he, e[o]);
           }
-          const int k2 = min(max(he + 2 + ko - w::kBiasV, -1022), 959);
+          const int k2 = w::near(he + 2 + ko - w::kBiasV);
           const bool inf = he >= w::kExpNonFinite || ko > w::kMaxExcess || (site & ERR_NONFINITE);
 #pragma unroll
           for (int c = k0; c < k0 + nc; ++c) {
@@ -1861,7 +1905,15 @@ k_interpolate(Batch B, const double* __restrict__ z, const double* __restrict__ 
                 v += w::align(w::mul(limbs_of(t.g[wib][c][lane + o]), wl[o]), he - e[o]);
               v *= 4;
             }
-            *row(Hout + p, P, c) = inf ? nan("") : w::scale_nz((double)v, k2);
+            *row(Hout + p, P, c) = inf ? nan("") : w::scaled_near(v, k2);
+          }
+        }
+        if (far) {   // (in place: read back by the thread that wrote them)
+#pragma unroll 1
+          for (int c = 0; c < 9; ++c) {
+            int he = 0;
+            for (int o = 0; o < NW; ++o) he = max(he, t.e[c < 3 ? c : (c + 3) / 2][tc - H + o]);
+            *row(Hout + p, P, c) *= w::far_factor(he + 2 + ko - w::kBiasV);
           }
         }
       }

@@ -517,14 +517,17 @@ k3_spread_x_sum(Box3 b, Field3 in, const int2* __restrict__ wrow, const int2* __
   int bad = 0, eo[NG];
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
-    const int k = min(max(ea[g] + 4 - w::kBiasV, -1022), 959);
     double v[8];
+    if (far_exponent(ea[g])) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const double x = w::scale_nz((double)acc[(q >> 1) * 2 * NG + 2 * g + (q & 1)], k) * b.kappa_dV;
-      v[q] = ea[g] >= w::kExpNonFinite ? nan("") : x;
-      bad |= !isfinite(v[q]);
+      for (int q = 0; q < 8; ++q) v[q] = deposit_sum(acc[(q >> 1) * 2 * NG + 2 * g + (q & 1)], ea[g]) * b.kappa_dV;
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        v[q] = w::scaled_near(acc[(q >> 1) * 2 * NG + 2 * g + (q & 1)], ea[g] + 4 - w::kBiasV) * b.kappa_dV;
     }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) bad |= !isfinite(v[q]);
     eo[g] = potential_operands(
         v, [&](int q, int2 x) { At[(int64_t)((q >> 1) * kNC + 2 * (g0 + g) + (q & 1)) * b.C + cell] = x; });
   }

@@ -24,6 +24,7 @@ int64_t dot(const double* A, const double* o, int* e) {
   *e = top + 2 + ko - kBiasV;
   return join(split(dot3(align(join(a[0]) >> 2, ko, 0), a[1], b[0], a[2], b[1], a[3], b[2])));
 }
+double scaled_of(int64_t v, int k) { return scaled(v, k); }
 // Zeroth and first moment of n terms, each the sum of three taps w v, as a deposit adds
 // them; om: the terms' direction component (scaled by 2^-ko): value 2^(*ea + 4 - kBiasV).
 // alternate: half a unit for the first moment as one every second term
@@ -64,6 +65,8 @@ def lib(tmp_path_factory):
                            str(d / "h.so"), str(d / "h.cpp")])
     lib = ctypes.CDLL(str(d / "h.so"))
     lib.dot.restype = ctypes.c_int64
+    lib.scaled_of.restype = ctypes.c_double
+    lib.scaled_of.argtypes = [ctypes.c_int64, ctypes.c_int]
     return lib
 
 
@@ -166,3 +169,12 @@ def test_zero_terms_add_nothing(lib, alternate):
     assert got[0] == exact[0]                     # (few bits: exact)
     one, _, _, _ = _sums(lib, v[5:6], w[5:6], om[5:6], 0, alternate)
     assert abs(got[1] - exact[1]) <= F(2) ** -52 and abs(one[1] - exact[1]) <= F(2) ** -55
+
+
+def test_scaled_results(lib):
+    """v 2^k over every exponent a sum can have: exact, rounded once where subnormal, infinite where too large."""
+    for v in (0, 1, -3, 2 ** 53 - 1, -(2 ** 62 + 2 ** 20), 2 ** 63 - 1, -2 ** 63):
+        for k in (-1079, -1078, -1075, -1060, -1023, -1022, -1021, 0, 900, 958, 959, 960, 961, 967, 970, 1000):
+            with np.errstate(over="ignore"):
+                want = np.ldexp(np.float64(v), k)
+            assert lib.scaled_of(v, k) == want, (v, k)
