@@ -345,17 +345,19 @@ int64_t parts(const emu_box* b, int64_t upb, bool deposit) {
 }
 
 // Directions of a part: the fewest that leave no more parts than blocks (all
-// of a tile's directions when the tiles alone are more), but at least 6 (4 in
-// boxes of less than 1.5 units a block): parts of 3 directions of a 256 x 96 box
-// fill all SMs with half-idle blocks and three such boxes at a time take 254 us
-// per 4 steps, parts of 6 directions 188 us (one box alone the same).  Parts of
-// 4 / 6, us a step: 120 x 90 (1.2 units a block) 35.0 / 35.4 for three boxes in
-// turn, 86 / 97 alone; 200 x 80 (1.8) 44 / 40, 87 / 97.
+// of a tile's directions when the tiles alone are more), but at least 6: parts of 3
+// directions of a 256 x 96 box fill all SMs with half-idle blocks and three such boxes
+// at a time take 254 us per 4 steps, parts of 6 directions 188 us (one box alone the
+// same).  At least 4 in boxes of less than 1.5 units a block and, in the deposit, of
+// less than 2: fewer directions an SM serve one box alone.  us a step with parts of
+// 4 / 6: 120 x 90 (1.2 units a block) 35.0 / 35.4 for three boxes in turn, 86 / 97
+// alone; the deposit's of 200 x 80 (1.8) 41.0 / 40.0 and 90.5 / 98.7, with vacuum and
+// matter terms 43.1 / 42.2 and 96.6 / 104.8 (both kernels' 44.8 / 40.0 and 88.2 / 98.7).
 int part_directions(const emu_box* b, bool deposit) {
   const int64_t units = deposit ? b->S.U : b->S.U32;
   int64_t upb = std::max<int64_t>((units + b->blocks - 1) / b->blocks, 1);
   while (upb < b->S.Mmax && parts(b, upb, deposit) > b->blocks) ++upb;
-  return (int)std::max<int64_t>(upb, std::min(2 * units < 3 * b->blocks ? 4 : 6, b->S.Mmax));
+  return (int)std::max<int64_t>(upb, std::min(2 * units < (deposit ? 4 : 3) * b->blocks ? 4 : 6, b->S.Mmax));
 }
 
 // Directions of a block's part in the deposit (Batch::dpb), 0 for ranges of
