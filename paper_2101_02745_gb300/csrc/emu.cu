@@ -1509,7 +1509,7 @@ int gsort(emu_box* b, double frac, const int** ids_out) {
   return EMU_OK;
 }
 
-// Deposit of particles anywhere (modes as k_deposit) into out.
+// Deposit of particles anywhere (modes 0, 1, 2 and 4 of k_deposit) into out.
 int launch_gdeposit(emu_box* b, int mode, const double* rnu, const double* rnb, double frac, double* out) {
   const int* ids = nullptr;
   if (int rc = gsort(b, frac, &ids)) return rc;
@@ -1524,8 +1524,7 @@ int launch_gdeposit(emu_box* b, int mode, const double* rnu, const double* rnb, 
     if (mode == 0) pdl(st, k_gdeposit<0, R>, grid, B, b->pt, rnu, rnb, frac, ids, start, out, b->err);
     else if (mode == 1) pdl(st, k_gdeposit<1, R>, grid, B, b->pt, rnu, rnb, frac, ids, start, out, b->err);
     else if (mode == 2) pdl(st, k_gdeposit<2, R>, grid, B, b->pt, rnu, rnb, frac, ids, start, out, b->err);
-    else if (mode == 4) pdl(st, k_gdeposit<4, R>, grid, B, b->pt, rnu, rnb, frac, ids, start, out, b->err);
-    else pdl(st, k_gdeposit<5, R>, grid, B, b->pt, rnu, rnb, frac, ids, start, out, b->err);
+    else pdl(st, k_gdeposit<4, R>, grid, B, b->pt, rnu, rnb, frac, ids, start, out, b->err);
     return 0;
   });
   return after_launch(b, "deposit kernel (particles anywhere)");

@@ -1,6 +1,6 @@
 // instances.cuh -- the heavy kernels' instances of one shape order R, so that
 // each order compiles in a translation unit of its own (instances_<R>.cu) and
-// emu.cu only declares them (EMU_EXTERN extern).
+// emu.cu only declares them (X empty here, extern there).
 #pragma once
 
 #include "kernels.cuh"

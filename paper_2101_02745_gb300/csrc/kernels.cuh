@@ -608,8 +608,9 @@ struct DepMode {
 // sums are then shifted).  Sums of n directions have headroom for n contributions
 // and round them without a bias (sum_headroom): less error than FP64 sums, whose
 // rounding follows the partial sums.  Zero contributions add exactly nothing.
-// Bound by integer issue: 16384 x 1000 2467 -> 1040 us a stage against FP64 sums
-// (1256 with plain loads: cp.async hides their latency), 1024 x 378 74 -> 41 us.
+// Bound by latency at four warps a scheduler (issue slots 48 %, FP64 pipe 58 %
+// busy): 16384 x 1000 2467 -> 1040 us a stage against FP64 sums (1256 with plain
+// loads: cp.async hides their latency), 1024 x 378 74 -> 41 us.
 // (buf: this warp's two buffers of kDepRows x 32 doubles in shared memory;
 // ring2 0: only one, when no warp takes more than one direction of a tile.)
 // phase > 0: the directions in cyclic order from the first multiple of phase (a
@@ -1488,10 +1489,11 @@ __device__ __forceinline__ int box_of_slab_unit(const Batch& B, int64_t x) {
 // adjacent pieces of the same rings (sw = 8: 2 KB of every array).  Per unit a
 // warp forms G = A0 - Omega . A of its cells, the neighbours' G come from
 // shared memory, and the stencil sum is the commutator's operand: everything
-// up to the update runs on the integer pipe.  Integer issue and the FP64 pipe
-// (conversions and updates) bound it about equally, HBM runs at 53 %: 16384 x 1000
-// 5.13 -> 2.64 ms a stage against FP64 arithmetic (the FP64 pipe its bound), 1024 x
-// 378 139 -> 73 us.
+// up to the update runs on the integer pipe.  Latency bounds it: four warps a
+// scheduler (126 registers), issue slots 45-49 % busy, fixed-latency waits and
+// memory the largest stalls, the FP64 pipe (conversions and updates) busiest at
+// 56-71 %, HBM at 53 %.  16384 x 1000 5.13 -> 2.64 ms a stage against FP64 arithmetic
+// (the FP64 pipe its bound), 1024 x 378 139 -> 73 us.
 constexpr int kSlabTiles = 8;                      // most tiles of a slab
 constexpr int kRowCells = kLanes + 4;              // cells of a unit, likewise
 template <int TILES>                               // of the widest slab
@@ -1786,8 +1788,8 @@ k_rk_stage(Batch B, Parts pt, const double* __restrict__ W, const double* __rest
 // particles at z + frac dt v_z, each with its own weights, from the potential
 // A[36][NZ].  As rk_phase up to H: a block takes a range of (slab of 4 tiles,
 // direction) pairs and converts the slab's potential once; the diagonal entries
-// have an exponent each.  (With FP64 G and taps 63 FP64 instructions a particle,
-// now 18: 270 us for 2048 x 1000.)
+// have an exponent each.  (18 FP64 instructions a particle for 63 with FP64 G and
+// taps: 2048 x 1000 262 -> 116 us.)
 struct InterpTable {
   static constexpr int kTiles = 4, kCells = kTiles * kLanes + 4;
   int2 a[kNA][kCells];

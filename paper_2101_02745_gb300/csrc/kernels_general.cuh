@@ -164,7 +164,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // Deposit (Eq. 5) of particles anywhere: one warp per global cell (grid-
-// stride), MODE as k_deposit (0, 1, 2, 4, 5); out as the lattice deposit's
+// stride), MODE as k_deposit (0, 1, 2, 4); out as the lattice deposit's
 // combination writes it (rows x NZ, scaled by kappa/dV or 1/dV).
 template <int MODE, int ORDER>
 __global__ void __launch_bounds__(kThreads)
@@ -173,7 +173,7 @@ k_gdeposit(Batch B, Parts pt, const double* __restrict__ r_nu, const double* __r
            int* __restrict__ err) {
   griddep_wait();
   constexpr int H = Sten<ORDER>::H, NW = Sten<ORDER>::NW;
-  constexpr int NA = MODE == 5 ? kNT : kNA;
+  constexpr int NA = kNA;
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = (int64_t)gridDim.x * kWarps;
   const int64_t P = B.Ptot;
@@ -200,28 +200,7 @@ k_gdeposit(Batch B, Parts pt, const double* __restrict__ r_nu, const double* __r
         double w = wt[0];
 #pragma unroll
         for (int s = 1; s < NW; ++s) w = (s == H + o) ? wt[s] : w;
-        if constexpr (MODE == 5) {
-          const double n1 = w * pt.N[p], n2 = w * pt.Nbar[p];
-          double bprev = 0.0;
-#pragma unroll
-          for (int c = 0; c < kNC; ++c) {
-            double bv;
-            if (c < 2) {
-              if (c == 0) bprev = fma(-n2, r_nb[p], n1 * r_nu[p]);
-              const double bn = fma(-n2, r_nb[(c + 1) * P + p], n1 * r_nu[(c + 1) * P + p]);
-              bv = bprev - bn;
-              bprev = bn;
-            } else {
-              const int k = c + 1;
-              const double xv = r_nu[k * P + p], yv = r_nb[k * P + p];
-              bv = (k == 4 || k == 6 || k == 8) ? fma(n2, yv, n1 * xv) : fma(-n2, yv, n1 * xv);
-            }
-            acc[c] += bv;
-            acc[kNC + c] = fma(ox, bv, acc[kNC + c]);
-            acc[2 * kNC + c] = fma(oy, bv, acc[2 * kNC + c]);
-            acc[3 * kNC + c] = fma(oz, bv, acc[3 * kNC + c]);
-          }
-        } else if constexpr (MODE == 4) {
+        if constexpr (MODE == 4) {
 #pragma unroll
           for (int k = 0; k < 9; ++k) {
             const double c1 = w * pt.N[p] * r_nu[k * P + p];
@@ -253,7 +232,7 @@ k_gdeposit(Batch B, Parts pt, const double* __restrict__ r_nu, const double* __r
         }
       }
     }
-    const double scale = (MODE == 0 || MODE == 5) ? g.kappa_dV : g.inv_dV;
+    const double scale = MODE == 0 ? g.kappa_dV : g.inv_dV;
 #pragma unroll
     for (int c = 0; c < NA; ++c) {
       const double v = warp_sum(acc[c]) * scale;

@@ -213,14 +213,10 @@ EMU_HD int one() {
   return 1;
 #endif
 }
-// a b / 2^64 and c + a b / 2^64.  |V| < 2^61 keeps every partial sum in 63 bits.
+// a b / 2^64.  |V| < 2^61 keeps every partial sum in 63 bits.
 EMU_HD int64_t mul(Limbs a, Limbs b) {
   const int64_t m = mad(a.h, b.l, mad(a.l, b.h, half_unit()));
   return mad((int)(m >> 32), two(), prod(a.h, b.h));
-}
-EMU_HD int64_t mul_add(Limbs a, Limbs b, int64_t c) {
-  const int64_t m = mad(a.h, b.l, mad(a.l, b.h, half_unit()));
-  return mad((int)(m >> 32), two(), mad(a.h, b.h, c));
 }
 // The same with the middle term rounded down (two instructions less each: the
 // rounding addend costs a 64-bit add).  For sums with as many subtracted as
@@ -287,8 +283,6 @@ EMU_HD int64_t moment_add(Factor v, Factor om, int64_t half, int64_t c) {
 // v / 2^d rounded to nearest, d >= 1.
 EMU_HD int64_t align_round(int64_t v, int d) { return (align(v, d - 1) + 1) >> 1; }
 
-// c 2^k for a normal c whose exponent stays normal.
-EMU_HD double scale(double c, int k) { return from_words(hi_word(c) + (int)((unsigned)k << 20), lo_word(c)); }
 // c 2^k for a positive normal c, k not below its smallest normal result; NaN
 // where the result is out of range (k at most 3000).
 EMU_HD double scale_up(double c, int k) {
