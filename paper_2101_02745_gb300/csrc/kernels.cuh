@@ -681,24 +681,12 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
     } else {
       cp_async_wait<0>();
     }
-    const double* x = buf + (k & ring2) * kDepRows * kLanes + lane;
-    const double n1 = D::N1 ? x[kLanes] : 0.0, n2 = D::N2 ? x[2 * kLanes] : 0.0;
-    // component k of the deposited matrix (conj(rhobar) flips the sign of the
-    // imaginary components 4, 6, 8)
-    auto value = [&](int set, int k) -> double {
-      const bool im = k == 4 || k == 6 || k == 8;
-      const double a = D::RNU ? x[(3 + k) * kLanes] : 0.0, c = D::RNB ? x[(12 + k) * kLanes] : 0.0;
-      if (MODE == 3) return a;
-      if (MODE == 1 || (MODE == 4 && set == 0)) return n1 * a;
-      if (MODE == 2 || MODE == 4) return n2 * c;
-      return fma(im ? n2 : -n2, c, n1 * a);
-    };
+    double* x = buf + (k & ring2) * kDepRows * kLanes + lane;
     // Omega, and the ring's weights when every particle takes them: lane q
     // converts one of them
     double u = 0.0;
     if (lane < 3) u = __ldg(dirtab + lane * MT + gd);
     const double zs = fma(pos_dt, __ldg(dirtab + 3 * MT + gd), x[0]);
-    w::Limbs wl[NW];   // the weight slot o of the particle that gives it to this lane's cell
     double wt[NW];
     int site;          // the lattice test's error
     if (wrow != nullptr) {
@@ -711,10 +699,27 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
         for (int q = 0; q < Sten<ORDER>::NWS; ++q) *row(W + p, P, q) = wt[q];
       }
     }
-    bad |= site;
     // weights have no exponent: a particle without a finite position counts as
-    // an infinite B, a ring without finite weights as an infinite direction
-    const int enf = site & ERR_NONFINITE ? w::kExpNonFinite : 0;
+    // one of infinite B, a ring without finite weights as an infinite direction
+    if (site != 0) {
+      bad |= site;
+      if (site & ERR_NONFINITE) {
+#pragma unroll 1
+        for (int q = 1; q < kDepRows; ++q) x[q * kLanes] = nan("");
+      }
+    }
+    const double n1 = D::N1 ? x[kLanes] : 0.0, n2 = D::N2 ? x[2 * kLanes] : 0.0;
+    // component k of the deposited matrix (conj(rhobar) flips the sign of the
+    // imaginary components 4, 6, 8)
+    auto value = [&](int set, int k) -> double {
+      const bool im = k == 4 || k == 6 || k == 8;
+      const double a = D::RNU ? x[(3 + k) * kLanes] : 0.0, c = D::RNB ? x[(12 + k) * kLanes] : 0.0;
+      if (MODE == 3) return a;
+      if (MODE == 1 || (MODE == 4 && set == 0)) return n1 * a;
+      if (MODE == 2 || MODE == 4) return n2 * c;
+      return fma(im ? n2 : -n2, c, n1 * a);
+    };
+    w::Limbs wl[NW];   // the weight slot o of the particle that gives it to this lane's cell
     // directions above 1 (not unit vectors) are scaled by 2^-ko
     const int ko = __reduce_max_sync(kFull, w::unit_excess(u)), half = w::sum_half(ko);
     const w::Limbs ul = w::unit_limbs(u, lane < 3 ? ko : 0);
@@ -758,7 +763,7 @@ __device__ __forceinline__ void deposit_tile(const Batch& B, int b, int tile, in
         bv[0] = value(set, k);
         if (nc > 1) bv[1] = value(set, k + 1);
       }
-      const int e0 = w::exponent(bv[0]), e1 = nc > 1 ? w::exponent(bv[1]) : 0, e = max(max(e0, e1), enf);
+      const int e0 = w::exponent(bv[0]), e1 = nc > 1 ? w::exponent(bv[1]) : 0, e = max(e0, e1);
       w::Limbs bl[2];
       bl[0] = nc > 1 ? w::limbs(bv[0], e0, e) : w::limbs(bv[0], e);
       if (nc > 1) bl[1] = w::limbs(bv[1], e1, e);
@@ -1752,13 +1757,11 @@ __device__ __forceinline__ void rk_phase(const Batch& B, const Parts& pt, const 
             }
           }
         }
-        // hv[c] 2^(he + 2 - kBiasV) = H_c, then he + 2 -> he (weights that are
-        // not finite have no exponent)
-        int kx = ko;
-        if (ORDER > 0 && !ring && w::exponent(wd[H]) >= w::kExpNonFinite) kx = w::kMaxExcess + 1;
-        if (kx != 0) {
+        // hv[c] 2^(he + 2 - kBiasV) = H_c, then he + 2 -> he (a particle's own weights
+        // need no test: where they are not finite, the deposit's potential is not)
+        if (ko != 0) {
 #pragma unroll
-          for (int grp = 0; grp < 4; ++grp) he[grp] = kx <= w::kMaxExcess ? he[grp] + kx : w::kExpNonFinite;
+          for (int grp = 0; grp < 4; ++grp) he[grp] = ko <= w::kMaxExcess ? he[grp] + ko : w::kExpNonFinite;
         }
 #pragma unroll
         for (int grp = 0; grp < 4; ++grp) he[grp] += 2;
