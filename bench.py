@@ -470,7 +470,7 @@ def run_gpu(args, rank, world, local_rank):
     roofline = {"bound": "hbm", "achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
                 "traffic": traffic, "traffic_unit": "bytes per launch (ncu dram read + write, scaled by particles)",
                 "kernel": kname, "bytes_per_launch": bytes_, "avg_launch_ms": avg_ms,
-                "limited_by": "integer issue and the FP64 pipe (conversions, updates) about equally",
+                "limited_by": "latency at four warps a scheduler (FP64 pipe 56-71 % busy, issue slots 45-49 %)",
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs" if "hbm_gbs" in peaks else "fallback",
                 "fp64_equivalent": {"tflops": achieved, "flops_per_launch": flops, "of_fp64_peak": achieved / peak,
                                     "fp64_peak": peak,

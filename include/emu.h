@@ -70,7 +70,7 @@ extern "C" {
 #define EMU_OK 0
 #define EMU_EINVAL (-1)    /* bad argument: null pointer, size, unsupported option */
 #define EMU_ECUDA (-2)     /* a CUDA runtime call failed */
-#define EMU_ENUMERIC (-3)  /* a non-finite value appeared on the grid */
+#define EMU_ENUMERIC (-3)  /* a non-finite value appeared on the grid, or a position is not finite */
 #define EMU_ETIMEOUT (-4)  /* a bounded device-side wait (a grid barrier of the fused step) gave up */
 #define EMU_ELATTICE (-5)  /* particles violate the lattice contract */
 

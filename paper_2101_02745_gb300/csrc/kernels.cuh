@@ -609,7 +609,7 @@ struct DepMode {
 // and round them without a bias (sum_headroom): less error than FP64 sums, whose
 // rounding follows the partial sums.  Zero contributions add exactly nothing.
 // Bound by latency at four warps a scheduler (issue slots 48 %, FP64 pipe 58 %
-// busy): 16384 x 1000 2467 -> 1040 us a stage against FP64 sums (1256 with plain
+// busy): 16384 x 1000 2467 -> 1050 us a stage against FP64 sums (1256 with plain
 // loads: cp.async hides their latency), 1024 x 378 74 -> 41 us.
 // (buf: this warp's two buffers of kDepRows x 32 doubles in shared memory;
 // ring2 0: only one, when no warp takes more than one direction of a tile.)

@@ -36,8 +36,8 @@
 // transposed convolution (k3_pass along x and y, then z in k3_rk_stage).  Three
 // 3-tap passes per direction and cell instead of a (2H+1)^2-row gather per
 // particle.  The step's fields and weights are fixed-point operands (wide.cuh)
-// throughout: 64^3 x 16 passes 197 -> 116 us, direction sum 454 -> 234 us, step
-// 9.2 -> 6.5 ms against FP64 fields.
+// throughout: 64^3 x 16 passes 197 -> 116 us, direction sum 454 -> 241 us, step
+// 9.2 -> 6.6 ms against FP64 fields.
 #pragma once
 
 namespace emu_dev {

@@ -23,9 +23,10 @@
 // Zero operands stay exactly zero, so zero products add exactly nothing.
 // Subnormal inputs count as half their value (their field's exponent is that of
 // the smallest normal numbers less one).  An infinite or
-// NaN input is not represented: callers test exponents for kExpNonFinite.
+// NaN input is not represented: callers test exponents for kExpNonFinite (shape
+// weights and directions, which have none, are tested where they are formed).
 //
-// The same code compiles for the host (g++), where the test runs it.
+// The same code compiles for the host (g++), where the tests run it.
 #pragma once
 
 #include <cstdint>
@@ -256,9 +257,8 @@ EMU_HD int64_t align(int64_t v, int d) { return align(v, d, max_i(d - 32, 0)); }
 // half a unit in the mean.  The zeroth moment's quarter, rounded up from half,
 // makes up for it, and so does half a unit times Omega in the rounding of the
 // others': no bias is left.  (Floors alone left half a unit a term: 20 times the
-// error of an FP64 sum for 225 terms of random sign, 90 times for 1000; now a
-// tenth to half of it, tests/test_wide_sums_host.py.)  A zero contribution adds
-// exactly nothing.
+// error of an FP64 sum for 225 terms of random sign, 90 times for 1000; now 0.1 to
+// 0.8 of it for 1 to 4000 terms.)  A zero contribution adds exactly nothing.
 EMU_HD int sum_headroom(int n) {
 #ifdef __CUDA_ARCH__
   return max_i(32 - __clz(n), 5) - 5;
